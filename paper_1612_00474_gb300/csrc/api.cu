@@ -318,7 +318,8 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
         return RPB_ENOMEM;
     }
     if ((rc = cuda_fail(cudaMemsetAsync(w.lz, 0, lanczos_state_elems(max_iter) * sizeof(double), c->stream),
-                        "memset"))) {
+                        "memset")) ||
+        (rc = lanczos_upload(w.lz, max_iter, c->stream))) {
         free_ws(w);
         delete c;
         return rc;

@@ -9,8 +9,8 @@
 //
 //   pair products : one 128-target block of one instance per CTA, all of that instance's sources
 //                   in 128-source tiles; the float64 self term and s_i/(8 pi eta) in the epilogue.
-//   Lanczos       : per-instance dot products / Gram-Schmidt (one CTA per instance), one warp per
-//                   instance for the tridiagonal step, instances drop out as they converge.
+//   Lanczos       : per-instance dot products / Gram-Schmidt and tridiagonal step (one CTA per
+//                   instance), instances drop out as they converge.
 //   noise         : Philox keyed by each instance's seed, counter (k/2, step_b, stream, 0) -- the
 //                   same numbers the single-suspension path draws for that seed and step.
 #include <algorithm>
@@ -536,21 +536,18 @@ __global__ void batch_scale_kernel(const double *__restrict__ w, const InstDesc 
     }
 }
 
-// One warp per instance (4 per block): the tridiagonal step; converged instances leave the active set.
-__global__ void __launch_bounds__(128) batch_tail_kernel(double *__restrict__ lz, size_t lz_stride, LzLayout L, int k,
-                                                         double tol, const double *__restrict__ norm2, int B,
-                                                         int *__restrict__ active, int *__restrict__ n_active)
+// One block per instance: the tridiagonal step; converged instances leave the active set.
+__global__ void __launch_bounds__(kTailThreads) batch_tail_kernel(double *__restrict__ lz, size_t lz_stride, LzLayout L,
+                                                                  int k, double tol, const double *__restrict__ norm2,
+                                                                  const double *__restrict__ nodes,
+                                                                  int *__restrict__ active, int *__restrict__ n_active)
 {
-    __shared__ double q0[4][kMaxIter];
-    __shared__ double sl[4][kMaxIter];
-    __shared__ double red[4][32];
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.x * 4 + wid;
-    if (b >= B || !active[b]) return;  // whole warp leaves together
+    __shared__ TailShared sh;
+    const int b = blockIdx.x;
+    if (!active[b]) return;  // the whole block leaves together
     double *lzb = lz + (size_t)b * lz_stride;
-    lanczos_tail_warp(lzb, L, k, tol, lzb[L.c1 + k] + lzb[L.c2 + k], sqrt(norm2[b]), q0[wid], sl[wid], red[wid]);
-    __syncwarp();
-    if (lane == 0) {
+    lanczos_tail_block(lzb, L, k, tol, lzb[L.c1 + k] + lzb[L.c2 + k], sqrt(norm2[b]), nodes, sh);
+    if (threadIdx.x == 0) {
         double *st = lzb + L.status;
         st[6] = k + 1;
         if (st[ST_STOP] != 0.0) {
@@ -600,6 +597,7 @@ struct rpb_batch {
     double *lz = nullptr;
     double *red = nullptr;
     double *norm2 = nullptr;
+    double *nodes = nullptr;  // nodes and weights of the Lanczos square root
     // host (pinned)
     InstDesc *h_inst = nullptr;
     BlockDesc *h_blocks = nullptr;
@@ -639,7 +637,7 @@ enum { V_POS, V_UP, V_F, V_T, V_UN, V_W, V_WT, V_G, V_DRIFT, V_PA, V_PB, V_WORK 
 static void batch_free(rpb_batch *bt)
 {
     void *dev[] = {bt->d_inst, bt->d_blocks, bt->d_inst_of, bt->d_active, bt->d_nactive, bt->src, bt->V, bt->lz, bt->red,
-                   bt->norm2, bt->d_left};
+                   bt->norm2, bt->nodes, bt->d_left};
     for (void *p : dev)
         if (p) cudaFree(p);
     for (double *p : bt->vec)
@@ -852,8 +850,8 @@ static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, doub
             rc = cuda_fail(cudaMemsetAsync(bt->d_nactive, 0, sizeof(int), st), "memset");
         }
         if (!rc) {
-            batch_tail_kernel<<<(B + 3) / 4, 128, 0, st>>>(bt->lz, bt->lz_stride, L, k, tol, bt->norm2, B,
-                                                           bt->d_active, bt->d_nactive);
+            batch_tail_kernel<<<B, kTailThreads, 0, st>>>(bt->lz, bt->lz_stride, L, k, tol, bt->norm2, bt->nodes,
+                                                          bt->d_active, bt->d_nactive);
             count_launches(5);
             if (graph) {
                 const bool has_next = k + 1 < max_iter;
@@ -1106,6 +1104,7 @@ int rpb_batch_create(rpb_batch **out, const rpb_params *p, int64_t max_total_N, 
               cudaMalloc(&bt->lz, (size_t)max_B * L.total * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&bt->red, (size_t)(max_iter + 2) * max_B * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&bt->norm2, (size_t)max_B * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&bt->nodes, 2 * kSqrtNodes * sizeof(double)) == cudaSuccess &&
               cudaMallocHost(&bt->h_inst, max_B * sizeof(InstDesc)) == cudaSuccess &&
               cudaMallocHost(&bt->h_blocks, max_blocks * sizeof(BlockDesc)) == cudaSuccess &&
               cudaMallocHost(&bt->h_nactive, sizeof(int)) == cudaSuccess &&
@@ -1127,7 +1126,8 @@ int rpb_batch_create(rpb_batch **out, const rpb_params *p, int64_t max_total_N, 
         delete bt;
         return RPB_ENOMEM;
     }
-    if (cuda_fail(cudaMemsetAsync(bt->lz, 0, (size_t)max_B * L.total * sizeof(double), bt->stream), "memset")) {
+    if (cuda_fail(cudaMemsetAsync(bt->lz, 0, (size_t)max_B * L.total * sizeof(double), bt->stream), "memset") ||
+        upload_sqrt_nodes(bt->nodes, bt->stream)) {
         batch_free(bt);
         delete bt;
         return RPB_ECUDA;

@@ -28,7 +28,22 @@ constexpr int kBlasThreads = 256;
 
 size_t lanczos_state_elems(int max_iter)
 {
-    return LzLayout(max_iter).total;
+    return LzLayout(max_iter).total + 2 * kSqrtNodes;  // the state block, then the square root's nodes
+}
+
+int upload_sqrt_nodes(double *nodes, cudaStream_t st)
+{
+    static const SqrtNodes host = sqrt_nodes();
+    int rc;
+    if ((rc = cuda_fail(cudaMemcpyAsync(nodes, host.s, sizeof(host.s), cudaMemcpyHostToDevice, st), "square root nodes")))
+        return rc;
+    return cuda_fail(cudaMemcpyAsync(nodes + kSqrtNodes, host.w, sizeof(host.w), cudaMemcpyHostToDevice, st),
+                     "square root weights");
+}
+
+int lanczos_upload(double *lz, int max_iter, cudaStream_t st)
+{
+    return upload_sqrt_nodes(lz + LzLayout(max_iter).total, st);
 }
 
 static int blas_grid(int64_t n, int num_sms)
@@ -157,21 +172,20 @@ __global__ void norm_init_kernel(const double *__restrict__ red, int G, double *
     }
 }
 
-// One warp: the tridiagonal step for the single Krylov space (see lanczos_tail_warp).  Inside a
-// replayed graph (runs != null) lane 0 then counts this run of iteration k, records m = k + 1 and lets
-// the conditional node of iteration k + 1 run only if the iteration has not stopped.
-__global__ void __launch_bounds__(32) lanczos_tail_kernel(double *__restrict__ lz, LzLayout L, int k, double tol,
-                                                          const double *__restrict__ red_norm, int Gred,
-                                                          cudaGraphConditionalHandle next = 0ull, int has_next = 0,
-                                                          unsigned long long *__restrict__ runs = nullptr,
-                                                          int *__restrict__ m_out = nullptr)
+// The tridiagonal step for the single Krylov space (see lanczos_tail_block).  Inside a replayed graph
+// (runs != null) thread 0 then counts this run of iteration k, records m = k + 1 and lets the
+// conditional node of iteration k + 1 run only if the iteration has not stopped.
+__global__ void __launch_bounds__(kTailThreads) lanczos_tail_kernel(double *__restrict__ lz, LzLayout L, int k,
+                                                                    double tol, const double *__restrict__ red_norm,
+                                                                    int Gred, cudaGraphConditionalHandle next = 0ull,
+                                                                    int has_next = 0,
+                                                                    unsigned long long *__restrict__ runs = nullptr,
+                                                                    int *__restrict__ m_out = nullptr)
 {
-    __shared__ double q0[kMaxIter];
-    __shared__ double sl[kMaxIter];
-    __shared__ double red[32];
-    const double bn = warp_sum_partials(red_norm, Gred);  // the same value in every lane
-    lanczos_tail_warp(lz, L, k, tol, lz[L.c1 + k] + lz[L.c2 + k], sqrt(bn), q0, sl, red);
-    if (runs && threadIdx.x == 0) {  // lane 0 wrote the status words
+    __shared__ TailShared sh;
+    const double bn = warp_sum_partials(red_norm, Gred);  // the same value in every thread
+    lanczos_tail_block(lz, L, k, tol, lz[L.c1 + k] + lz[L.c2 + k], sqrt(bn), lz + L.total, sh);
+    if (runs && threadIdx.x == 0) {  // thread 0 wrote the status words
         *runs += 1ull;
         *m_out = k + 1;
         if (has_next) cudaGraphSetConditional(next, lz[L.status + ST_STOP] == 0.0 ? 1u : 0u);
@@ -373,7 +387,7 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
             if ((rc = cuda_fail(cudaEventRecord(ctx->lz_ev_a, main_st), "event record")) ||
                 (rc = cuda_fail(cudaStreamWaitEvent(ctx->lz_side, ctx->lz_ev_a, 0), "stream wait")))
                 return rc;
-            lanczos_tail_kernel<<<1, 32, 0, ctx->lz_side>>>(lz, L, k, tol, rn, G);
+            lanczos_tail_kernel<<<1, kTailThreads, 0, ctx->lz_side>>>(lz, L, k, tol, rn, G);
             count_launches(5);
             if ((rc = cuda_fail(cudaMemcpyAsync(hs, status, 8 * sizeof(double), cudaMemcpyDeviceToHost, ctx->lz_side),
                                 "status copy")) ||
@@ -424,7 +438,7 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
                 !(rc = cuda_fail(cudaStreamWaitEvent(side, gr->ev_fork, 0), "stream wait")))
                 tail_st = side;
             if (!rc) {
-                lanczos_tail_kernel<<<1, 32, 0, tail_st>>>(lz, L, k, tol, red_norm, G,
+                lanczos_tail_kernel<<<1, kTailThreads, 0, tail_st>>>(lz, L, k, tol, red_norm, G,
                                                            has_next ? gr->hnd[k + 1] : 0ull, has_next ? 1 : 0,
                                                            gr->state->iter_runs + k, &gr->state->m);
                 count_launches(1);

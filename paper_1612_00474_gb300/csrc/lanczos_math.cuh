@@ -1,11 +1,14 @@
-// lanczos_math.cuh -- per-warp step of the Lanczos square root shared by the single and batched
-// kernels: the Ritz data of the tridiagonal T_{k+1}, the update y_k = |W| Q sqrt(Lambda) Q^T e_1,
-// the error estimate eps_k and the stopping decision (Sec. II.C).
+// lanczos_math.cuh -- tridiagonal step of the Lanczos square root shared by the single and batched
+// kernels: y_k = |W| T_{k+1}^{1/2} e_1 for the tridiagonal T_{k+1}, the error estimate eps_k and the
+// stopping decision (Sec. II.C).  One 128-thread block per Krylov space evaluates a rational
+// approximation of the square root, one node per thread; a T that is not positive definite takes the
+// eigen-decomposition, one warp.
 #pragma once
 
 #include <cfloat>
 
 #include "rpb_internal.cuh"
+#include "sqrt_nodes.h"
 
 namespace rpb {
 
@@ -36,25 +39,20 @@ enum { ST_EPS = 0, ST_INV_BETA = 1, ST_NW = 2, ST_INV_NW = 3, ST_STOP = 4, ST_BR
 // (Bowdler, Martin, Reinsch & Wilkinson), then y = |W| Q sqrt(max(Lambda, 0)) Q^T e_1.
 // Called by one full warp: every lane runs the (identical) scalar recurrence on private copies of d
 // and e and applies the rotations to its own rows (lane, lane + 32) of Q, so no lane reads another's
-// data until the end.  lz: this Krylov space's state block; alpha_k, beta_k: the new coefficients;
-// q0, sl, red: warp-private shared scratch (kMaxIter, kMaxIter, 32 doubles).
-__device__ __forceinline__ void lanczos_tail_warp(double *__restrict__ lz, const LzLayout &L, int k, double tol,
-                                                  double alpha_k, double beta_k, double *q0, double *sl,
-                                                  double *red)
+// data until the end.  alpha, beta: the entries of T (k + 1 and k of them); q0, sl: shared scratch
+// (kMaxIter doubles each).  Lane i returns entries i and i + 32 of y in y0, y1.
+static __device__ __noinline__ void tridiag_sqrt_ql(const double *alpha, const double *beta, int k, double nW, double *q0,
+                                             double *sl, double *y_out0, double *y_out1)
 {
     const int lane = threadIdx.x & 31;
-    double *status = lz + L.status;
     const int n = k + 1;
     double d[kMaxIter], e[kMaxIter], z0[kMaxIter], z1[kMaxIter];
     for (int i = 0; i < n; ++i) {
-        d[i] = (i == k) ? alpha_k : lz[L.alpha + i];
-        e[i] = (i < k) ? lz[L.beta + i] : 0.0;
+        d[i] = alpha[i];
+        e[i] = (i < k) ? beta[i] : 0.0;
         z0[i] = (i == lane) ? 1.0 : 0.0;
         z1[i] = (i == lane + 32) ? 1.0 : 0.0;
     }
-    double tnorm = 0.0;
-    for (int i = 0; i < n; ++i) tnorm = fmax(tnorm, fmax(fabs(d[i]), fabs(e[i])));
-    tnorm = fmax(tnorm, beta_k);
     for (int l = 0; l < n; ++l) {
         for (int iter = 0; iter < 100; ++iter) {
             int m = l;
@@ -113,46 +111,155 @@ __device__ __forceinline__ void lanczos_tail_warp(double *__restrict__ lz, const
     if (lane < n) sl[lane] = sqrt(fmax(d[lane], 0.0));
     if (lane + 32 < n) sl[lane + 32] = sqrt(fmax(d[lane + 32], 0.0));
     __syncwarp();
-    const double nW = status[ST_NW];
     double y0 = 0.0, y1 = 0.0;
     for (int j = 0; j < n; ++j) {
         const double cj = sl[j] * q0[j];
         y0 = fma(z0[j], cj, y0);
         if (n > 32) y1 = fma(z1[j], cj, y1);
     }
-    y0 *= nW;
-    y1 *= nW;
+    *y_out0 = y0 * nW;
+    *y_out1 = y1 * nW;
+}
+
+// 1/d for a positive normal d: the hardware's approximation (relative error below 2^-23) and one
+// third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - d y.
+__device__ __forceinline__ double rcp_pos(double d)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+constexpr int kTailThreads = kSqrtNodes;  // one node per thread
+constexpr int kTailRows = 16;             // entries of y summed over the nodes at a time
+struct TailShared {
+    double al[kMaxIter], be[kMaxIter], b2[kMaxIter];  // the entries of T, beta^2
+    double y[kMaxIter];
+    double q0[kMaxIter], sl[kMaxIter];                // eigen-decomposition
+    double z[kTailRows][kSqrtNodes + 8];              // the nodes' terms (padded: the sums read 8 columns of
+                                                      // four rows at a time)
+};
+
+// Largest of the lanes' non-negative values: the bit patterns of non-negative doubles order as integers,
+// so this leaves the float64 pipe alone.
+__device__ __forceinline__ double warp_max_pos(double v)
+{
+    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long q = __shfl_xor_sync(0xffffffffu, b, o);
+        b = q > b ? q : b;
+    }
+    return __longlong_as_double((long long)b);
+}
+
+// The tridiagonal step of one Krylov space by one block of kTailThreads threads: stores alpha_k,
+// beta_k, y, eps and the stopping decision in its state block lz.  nodes: kSqrtNodes shifts, then as
+// many weights (sqrt_nodes.h).
+//
+// With T = tridiag(beta, alpha, beta) scaled by its Gershgorin bound M, y = |W| T^{1/2} e_1 ~
+// |W| sqrt(M) sum_j w_j T (T + M s_j)^{-1} e_1.  Thread j solves its shifted system by eliminating from
+// the last row up: c_i = alpha_i - beta_i^2 / d_{i+1}, d_i = c_i + s; then x_0 = 1/d_0,
+// x_{i+1} = -(beta_i / d_{i+1}) x_i, and (T x)_0 = c_0 x_0, (T x)_i = -s x_i, with no cancellation.
+// Everything is backward stable for a positive definite T (relative errors of a few 1e-16 in y, against
+// 1e-15 to 1e-13 of an eigen-decomposition); a pivot that is not positive (or not finite) in some
+// thread shows a T that is not, and the block takes the eigen-decomposition instead, whose negative
+// eigenvalues (rounding of a semi-definite mobility) are clamped to 0.
+//
+// What bounds it: the float64 chain of one elimination, about 7 instructions per row and thread, each
+// 64 cycles of a scheduler whatever the active lanes.  The eigen-decomposition is a chain of about
+// 1.7 k^2 / 2 rotations of 28 such instructions on one warp: 48 us per launch on average over the
+// iterations of a converging solve of 8 dimensions and 164 us over one of 19; with the nodes a
+// 3001-sphere free-space solve (18 iterations, float32 pairs) went from 3251 to 1211 us and a step of 4096
+// spheres from 1103 to 1004 us.
+__device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, const LzLayout &L, int k, double tol,
+                                                   double alpha_k, double beta_k, const double *__restrict__ nodes,
+                                                   TailShared &sh)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    double *status = lz + L.status;
+    const int n = k + 1;
+    if (tid < n) {
+        const double b = tid < k ? lz[L.beta + tid] : 0.0;
+        sh.al[tid] = tid < k ? lz[L.alpha + tid] : alpha_k;
+        sh.be[tid] = b;
+        sh.b2[tid] = b * b;
+    }
+    const double sj = nodes[tid], wj = nodes[kSqrtNodes + tid];
+    const double nW = status[ST_NW];
+    __syncthreads();
+    // Gershgorin bound and largest entry (every warp, over the entries lane and lane + 32)
+    double mb = 0.0, mt = fabs(beta_k);
+    for (int i = lane; i < n; i += 32) {
+        const double a = fabs(sh.al[i]), b = fabs(sh.be[i]);
+        mb = fmax(mb, a + b + (i > 0 ? fabs(sh.be[i - 1]) : 0.0));
+        mt = fmax(mt, fmax(a, b));
+    }
+    const double M = warp_max_pos(mb);
+    const double tnorm = warp_max_pos(mt);
+    const double s = M * sj;
+    double r[kMaxIter];
+    double c = sh.al[k];
+    double d = c + s;
+    // positive and normal, below 2^1000: on the exponent bits (false for NaN)
+    auto fine = [](double v) { return (unsigned)(__double2hiint(v) - 0x00100000) < 0x7e600000u; };
+    bool ok = fine(d);
+    double ri = rcp_pos(d);
+    r[k] = ri;
+    for (int i = k - 1; i >= 0; --i) {
+        c = fma(-sh.b2[i], ri, sh.al[i]);
+        d = c + s;
+        ok = ok && fine(d);
+        ri = rcp_pos(d);
+        r[i] = ri;
+    }
+    if (__syncthreads_or(!ok)) {
+        if (tid >= 32) return;  // (no barrier follows for the first warp on this path)
+        double y0, y1;
+        tridiag_sqrt_ql(sh.al, sh.be, k, nW, sh.q0, sh.sl, &y0, &y1);
+        if (lane < n) sh.y[lane] = y0;
+        if (lane + 32 < n) sh.y[lane + 32] = y1;
+        __syncwarp();
+    } else {
+        const double scale = sqrt(M) * nW;
+        const double x0 = wj * ri;
+        double z = -(s * x0);
+        for (int base = 0; base < n; base += kTailRows) {
+            const int m = min(kTailRows, n - base);
+            for (int i = 0; i < m; ++i) {
+                if (base + i > 0) z = -(sh.be[base + i - 1] * r[base + i]) * z;
+                sh.z[i][tid] = base + i > 0 ? z : c * x0;
+            }
+            __syncthreads();
+            // eight threads per entry: 16 nodes each, then three butterfly levels (a fixed order)
+            const int row = tid >> 3, p = tid & 7;
+            double v = 0.0;
+            if (row < m)
+                for (int u = 0; u < kSqrtNodes / 8; ++u) v += sh.z[row][p + 8 * u];
+            for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (p == 0 && row < m) sh.y[base + row] = v * scale;
+            __syncthreads();
+        }
+        if (tid >= 32) return;
+    }
     // eps_k = |y - (yprev, 0)| / |yprev|
     double num = 0.0, den = 0.0;
-    if (lane < n) {
-        const double p0 = (lane < k) ? lz[L.yprev + lane] : 0.0;
-        num += (y0 - p0) * (y0 - p0);
-        den += p0 * p0;
-    }
-    if (lane + 32 < n) {
-        const double p1 = (lane + 32 < k) ? lz[L.yprev + lane + 32] : 0.0;
-        num += (y1 - p1) * (y1 - p1);
-        den += p1 * p1;
+    for (int i = lane; i < n; i += 32) {
+        const double y = sh.y[i], p = i < k ? lz[L.yprev + i] : 0.0;
+        num += (y - p) * (y - p);
+        den += p * p;
+        lz[L.y + i] = y;
+        lz[L.yprev + i] = y;
     }
     // warp sums by a butterfly (a fixed order; every lane ends with the same totals)
-    double snum = num, sden = den;
     for (int o = 16; o > 0; o >>= 1) {
-        snum += __shfl_xor_sync(0xffffffffu, snum, o);
-        sden += __shfl_xor_sync(0xffffffffu, sden, o);
-    }
-    (void)red;
-    if (lane < n) {
-        lz[L.y + lane] = y0;
-        lz[L.yprev + lane] = y0;
-    }
-    if (lane + 32 < n) {
-        lz[L.y + lane + 32] = y1;
-        lz[L.yprev + lane + 32] = y1;
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
     }
     if (lane == 0) {
         lz[L.alpha + k] = alpha_k;
         lz[L.beta + k] = beta_k;
-        const double eps = (k >= 1 && sden > 0.0) ? sqrt(snum / sden) : -1.0;
+        const double eps = (k >= 1 && den > 0.0) ? sqrt(num / den) : -1.0;
         const bool brk = beta_k <= 1e-14 * tnorm;
         const bool conv = (tol > 0.0 && k >= 1 && eps <= tol);
         status[ST_EPS] = eps;

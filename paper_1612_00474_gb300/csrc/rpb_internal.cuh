@@ -344,8 +344,13 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
 // Streams and device state of graph-replayed runs (run.cu), released by rpb_destroy.
 void run_free(rpb_ctx *ctx);
 
-// Sizes of the Lanczos small-state block (doubles) for max_iter.
+// Copy the nodes and weights of the square root (sqrt_nodes.h: all shifts, then all weights) to the
+// device; the copies are complete or staged when it returns.
+int upload_sqrt_nodes(double *nodes, cudaStream_t st);
+// Sizes of the Lanczos small-state block (doubles) for max_iter; the square root's nodes follow the
+// state (at LzLayout::total).
 size_t lanczos_state_elems(int max_iter);
+int lanczos_upload(double *lz, int max_iter, cudaStream_t st);  // the nodes into a state block
 size_t lanczos_red_elems(int max_iter);
 
 }  // namespace rpb
