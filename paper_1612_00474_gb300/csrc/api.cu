@@ -9,6 +9,7 @@
 #include <new>
 
 #include "rpb_internal.cuh"
+#include "sym64_plan.h"
 
 namespace rpb {
 
@@ -73,7 +74,7 @@ static void free_ws(Workspace &w)
 {
     void *dev[] = {w.src, w.partial, w.V, w.w, w.red, w.lz, w.pos_a, w.pos_b, w.pos_w, w.cells,
                    w.vec_a, w.vec_b, w.vec_c, w.vec_d, w.vec_e, w.vec_f, w.vec_g,
-                   w.sym_index, w.sym_tgt, w.sym_src, w.src2, w.pc, w.pcx};
+                   w.sym_index, w.sym_tgt, w.sym_src, w.sym64, w.src2, w.pc, w.pcx};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (w.host_status) cudaFreeHost(w.host_status);
@@ -308,6 +309,19 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
                 delete c;
                 return RPB_ENOMEM;
             }
+        }
+    }
+    if (p->precision == RPB_FP64) {
+        // the float64 symmetric pass keeps a triangle of column partials (~3 N^2/8 bytes); used while that
+        // stays below 8 GB too, the one-way kernel beyond
+        const size_t bytes =
+            sizeof(double) * (size_t)(sym64_tgt_elems(max_N, c->num_sms) + sym64_src_elems(max_N, c->num_sms));
+        if (bytes <= ((size_t)8 << 30) && cudaMalloc(&w.sym64, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            set_error("cudaMalloc of the symmetric-pass scratch (%zu bytes) failed", bytes);
+            free_ws(w);
+            delete c;
+            return RPB_ENOMEM;
         }
     }
     if (cudaMallocHost((void **)&w.host_status, 8 * sizeof(double)) != cudaSuccess) {

@@ -366,9 +366,9 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
     }
     // Speculate only where a product is short: one product is wasted per solve (after the stopping
     // iteration) and about one tridiagonal step (~55 us) is saved per iteration; the estimate uses the
-    // measured per-pair times of the one-way float64 and symmetric float32 kernels on this part.
+    // measured per-pair times of the symmetric float64 and float32 kernels on this part.
     const double t_product = (ctx->Lx > 0.0 ? 9.0 : 1.0) * (double)N * (double)N *
-                             (ctx->p.precision == RPB_FP64 ? 5e-10 : 1.3e-12);
+                             (ctx->p.precision == RPB_FP64 ? 8e-11 : 1.3e-12);
     const bool speculate = t_product < 3e-4;
     bool have_product = false;  // w already holds M v_k (the speculative product of iteration k - 1)
     for (int k = 0; k < max_iter; ++k) {

@@ -22,6 +22,8 @@
 //   - float32 mode: positions split x = x_hi + x_lo (two floats), so near-pair offsets keep float32
 //     relative accuracy anywhere in a large box; per-tile float32 sums are added with Kahan
 //     compensation.
+// The float64 products with forces take the symmetric pass of pair64.cu; pair_f64_kernel serves torque-only
+// products, row ranges, the allocation-free product and contexts too large for that pass's scratch.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -1480,6 +1482,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
     const int N = (int)N64;
     if (ctx->sym_enabled && ctx->p.wall && !(ctx->Lx > 0.0) && F && N >= 2 * kTile && (!T || ctx->sym_fused))
         return mobility_sym(ctx, N, pos, F, T, U);
+    if (mobility_sym64_ok(ctx, F)) return mobility_sym64(ctx, N, pos, F, T, U);
     cudaStream_t st = ctx->stream;
     const double a = ctx->p.a;
     int splits;

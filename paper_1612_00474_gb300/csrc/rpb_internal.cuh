@@ -173,6 +173,7 @@ struct Workspace {
     float *sym_src = nullptr;
     size_t sym_src_bytes = 0;
     void *src2 = nullptr;          // second right-hand side of the two-RHS symmetric pass (float4 per sphere)
+    double *sym64 = nullptr;       // float64 contexts: row and column partials of the symmetric pass (pair64.cu)
     SymSched sym;       // the whole triangle
     SymSched sym_part;  // one share of it (rpb_mobility_apply_part)
 };
@@ -253,6 +254,10 @@ int mobility_rows_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double 
 // Share `part` of `nparts` of the product (rpb_mobility_apply_part); never goes through the product hook.
 int mobility_part_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *F, const double *T, int part,
                        int nparts, double *U);
+// The float64 product with each unordered pair evaluated once (pair64.cu): whether it can be taken (a
+// float64 context with its scratch, forces given, no periodic images), and the product.
+bool mobility_sym64_ok(const rpb_ctx *ctx, const double *F);
+int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U);
 // Whether mobility_apply2_impl can take this product (float32 symmetric pass with two right-hand sides).
 bool mobility_apply2_ok(const rpb_ctx *ctx, int64_t N);
 // U = M_tt F + M_tr T and U2 = M_tt P in one symmetric pass (F, T, P non-null).
