@@ -20,7 +20,7 @@
 #include <new>
 #include <vector>
 
-#include "lanczos_math.cuh"
+#include "gs.cuh"
 #include "pair_math.cuh"
 
 namespace rpb {
@@ -41,7 +41,6 @@ struct BlockDesc {
     int first;  // first target (instance-local) of this 128-target block
 };
 
-constexpr int kBThreads = 256;
 
 // ------------------------------------------------------------------ layout kernels
 __global__ void inst_of_kernel(const InstDesc *__restrict__ inst, int B, int *__restrict__ inst_of)
@@ -435,92 +434,104 @@ __global__ void batch_rfd_combine_kernel(double *__restrict__ up_drift, const do
 }
 
 // ------------------------------------------------------------------ batched Lanczos
-__device__ __forceinline__ double block_sum_b(double v, double *sh)
+// Every instance's spheres are cut into chunks of kGsChunk, one block each (gs.cuh), numbered instance by
+// instance; a reduction writes one partial per chunk and the next kernel adds an instance's own in a
+// fixed order, so nothing depends on the companions.  (One block per instance left the largest instances
+// to one SM: of a served mix with suspensions of up to 32768 spheres, 24 instances, the dot products and
+// projections took 18% of a step; 7.7 of 42 ms.)
+struct ChunkDesc {
+    int inst, first;    // instance, its first sphere (instance-local)
+    int chunk0, count;  // the instance's first chunk and its number of chunks
+};
+
+__device__ __forceinline__ GsSpan chunk_span(const ChunkDesc &c, const InstDesc &d, int64_t total)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0)
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r += sh[k];
-    __syncthreads();
-    return r;
+    return GsSpan{d.off + c.first, total, min(kGsChunk, d.N - c.first)};
 }
 
-// red[k * B + b] = <V[k], w> over instance b's 3 N_b rows; grid (B, nvec).
-__global__ void __launch_bounds__(kBThreads) batch_dots_kernel(const double *__restrict__ V, size_t ld,
-                                                               const double *__restrict__ w,
-                                                               const InstDesc *__restrict__ inst,
-                                                               const int *__restrict__ active, int64_t total, int B,
-                                                               double *__restrict__ red)
+// red[j nchunks + chunk] = the chunk's part of <V_j, w>, j < nvec
+__global__ void __launch_bounds__(kGsThreads) batch_dots_kernel(const double *__restrict__ V, size_t ld, int nvec,
+                                                                const double *__restrict__ w,
+                                                                const InstDesc *__restrict__ inst,
+                                                                const ChunkDesc *__restrict__ chunks,
+                                                                const int *__restrict__ active, int64_t total,
+                                                                double *__restrict__ red)
 {
-    __shared__ double sh[kBThreads / 32];
-    const int b = blockIdx.x;
-    if (active && !active[b]) return;  // uniform per block
-    const InstDesc d = inst[b];
-    const double *v = V + (size_t)blockIdx.y * ld;
-    double acc = 0.0;
-    for (int c = 0; c < 3; ++c)
-        for (int il = threadIdx.x; il < d.N; il += blockDim.x) {
-            const int64_t r = c * total + d.off + il;
-            acc = fma(v[r], w[r], acc);
-        }
-    acc = block_sum_b(acc, sh);
-    if (threadIdx.x == 0) red[(size_t)blockIdx.y * B + b] = acc;
+    __shared__ double sh[kGsWarps][kMaxIter + 8];
+    const ChunkDesc c = chunks[blockIdx.x];
+    if (active && !active[c.inst]) return;  // uniform per block
+    int64_t row[kGsRows];
+    double x[kGsRows];
+    gs_rows(chunk_span(c, inst[c.inst], total), row);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) x[u] = row[u] >= 0 ? w[row[u]] : 0.0;
+    const double s = gs_dots(V, ld, nvec, row, x, sh);
+    if (threadIdx.x < nvec) red[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s;
 }
 
-// w -= sum_k coef_k V[k] over instance b's rows (coef_k = red[k B + b]); block b also stores the
-// coefficients in its state block (lz_b + coef_off) and, if norm_out, |w|^2 in norm_out[b].
-__global__ void __launch_bounds__(kBThreads) batch_project_kernel(const double *__restrict__ V, size_t ld,
-                                                                  double *__restrict__ w,
-                                                                  const InstDesc *__restrict__ inst,
-                                                                  const int *__restrict__ active, int64_t total, int B,
-                                                                  int nvec, const double *__restrict__ red,
-                                                                  double *__restrict__ lz, size_t lz_stride,
-                                                                  size_t coef_off, double *__restrict__ norm_out)
+// w -= sum_j c_j V_j with c_j from the partials `red`; the instance's first chunk stores c in its state block
+// (lz_b + coef_off).  Then, with red2, the dot products of the new w (the second pass of Gram-Schmidt) as
+// batch_dots_kernel, or the chunk's part of |w|^2 in norm2.
+__global__ void __launch_bounds__(kGsThreads) batch_project_kernel(const double *__restrict__ V, size_t ld, int nvec,
+                                                                   double *__restrict__ w,
+                                                                   const InstDesc *__restrict__ inst,
+                                                                   const ChunkDesc *__restrict__ chunks,
+                                                                   const int *__restrict__ active, int64_t total,
+                                                                   const double *__restrict__ red,
+                                                                   double *__restrict__ lz, size_t lz_stride,
+                                                                   size_t coef_off, double *__restrict__ red2,
+                                                                   double *__restrict__ norm2)
 {
-    __shared__ double coef[kMaxIter + 1];
-    __shared__ double sh[kBThreads / 32];
-    const int b = blockIdx.x;
-    if (active && !active[b]) return;
-    const InstDesc d = inst[b];
-    for (int k = threadIdx.x; k < nvec; k += blockDim.x) {
-        coef[k] = red[(size_t)k * B + b];
-        lz[(size_t)b * lz_stride + coef_off + k] = coef[k];
-    }
-    __syncthreads();
-    double acc = 0.0;
-    for (int c = 0; c < 3; ++c)
-        for (int il = threadIdx.x; il < d.N; il += blockDim.x) {
-            const int64_t r = c * total + d.off + il;
-            double x = w[r];
-            for (int k = 0; k < nvec; ++k) x -= coef[k] * V[(size_t)k * ld + r];
-            w[r] = x;
-            acc = fma(x, x, acc);
-        }
-    if (norm_out) {
-        acc = block_sum_b(acc, sh);
-        if (threadIdx.x == 0) norm_out[b] = acc;
+    __shared__ double sh[kGsWarps][kMaxIter + 8];
+    __shared__ double coef[kMaxIter];
+    const ChunkDesc c = chunks[blockIdx.x];
+    if (active && !active[c.inst]) return;
+    int64_t row[kGsRows];
+    double x[kGsRows];
+    gs_rows(chunk_span(c, inst[c.inst], total), row);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) x[u] = row[u] >= 0 ? w[row[u]] : 0.0;
+    gs_coefs(red + c.chunk0, gridDim.x, c.count, nvec, coef);
+    if (c.first == 0 && threadIdx.x < nvec) lz[(size_t)c.inst * lz_stride + coef_off + threadIdx.x] = coef[threadIdx.x];
+    gs_project(V, ld, nvec, row, coef, x);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u)
+        if (row[u] >= 0) w[row[u]] = x[u];
+    if (red2) {
+        const double s = gs_dots(V, ld, nvec, row, x, sh);
+        if (threadIdx.x < nvec) red2[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s;
+    } else {
+        double s = 0.0;
+#pragma unroll
+        for (int u = 0; u < kGsRows; ++u) s = fma(x[u], x[u], s);
+        s = gs_block_sum(s, sh[0]);
+        if (threadIdx.x == 0) norm2[blockIdx.x] = s;
     }
 }
 
-// |W_b| per instance from red[b] (the squared norms); v_0 scale factors; activity.
-__global__ void batch_norm_init_kernel(const double *__restrict__ red, int B, double *__restrict__ lz, size_t lz_stride,
-                                       size_t status_off, int *__restrict__ active)
+// |W_b| per instance from the chunks' squared norms, one warp each; v_0 scale factors; activity.
+__global__ void __launch_bounds__(128) batch_norm_init_kernel(const double *__restrict__ red,
+                                                              const int2 *__restrict__ inst_chunks, int B,
+                                                              double *__restrict__ lz, size_t lz_stride,
+                                                              size_t status_off, int *__restrict__ active)
 {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) {
-        double *st = lz + (size_t)b * lz_stride + status_off;
-        const double nw = sqrt(red[b]);
-        st[ST_NW] = nw;
-        st[ST_INV_NW] = nw > 0.0 ? 1.0 / nw : 0.0;
-        st[ST_EPS] = -1.0;
-        st[ST_STOP] = nw > 0.0 ? 0.0 : 1.0;
-        st[ST_BREAK] = 0.0;
-        st[6] = 0.0;  // m (iterations used)
-        st[7] = nw > 0.0 ? 0.0 : 1.0;  // converged flag
-        active[b] = nw > 0.0 ? 1 : 0;
-    }
+    const int b = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (b >= B) return;
+    const int2 c = inst_chunks[b];
+    double s = 0.0;
+    for (int k = lane; k < c.y; k += 32) s += red[c.x + k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane != 0) return;
+    double *st = lz + (size_t)b * lz_stride + status_off;
+    const double nw = sqrt(s);
+    st[ST_NW] = nw;
+    st[ST_INV_NW] = nw > 0.0 ? 1.0 / nw : 0.0;
+    st[ST_EPS] = -1.0;
+    st[ST_STOP] = nw > 0.0 ? 0.0 : 1.0;
+    st[ST_BREAK] = 0.0;
+    st[6] = 0.0;  // m (iterations used)
+    st[7] = nw > 0.0 ? 0.0 : 1.0;  // converged flag
+    active[b] = nw > 0.0 ? 1 : 0;
 }
 
 // v[r] = w[r] * status_b[idx] for rows of active instances (all instances when active is null).
@@ -539,6 +550,7 @@ __global__ void batch_scale_kernel(const double *__restrict__ w, const InstDesc 
 // One block per instance: the tridiagonal step; converged instances leave the active set.
 __global__ void __launch_bounds__(kTailThreads) batch_tail_kernel(double *__restrict__ lz, size_t lz_stride, LzLayout L,
                                                                   int k, double tol, const double *__restrict__ norm2,
+                                                                  const int2 *__restrict__ inst_chunks,
                                                                   const double *__restrict__ nodes,
                                                                   int *__restrict__ active, int *__restrict__ n_active)
 {
@@ -546,7 +558,11 @@ __global__ void __launch_bounds__(kTailThreads) batch_tail_kernel(double *__rest
     const int b = blockIdx.x;
     if (!active[b]) return;  // the whole block leaves together
     double *lzb = lz + (size_t)b * lz_stride;
-    lanczos_tail_block(lzb, L, k, tol, lzb[L.c1 + k] + lzb[L.c2 + k], sqrt(norm2[b]), nodes, sh);
+    const int2 c = inst_chunks[b];
+    double s = 0.0;  // |w|^2 from the chunks' parts (every warp, the same in every thread)
+    for (int q = threadIdx.x & 31; q < c.y; q += 32) s += norm2[c.x + q];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    lanczos_tail_block(lzb, L, k, tol, lzb[L.c1 + k] + lzb[L.c2 + k], sqrt(s), nodes, sh);
     if (threadIdx.x == 0) {
         double *st = lzb + L.status;
         st[6] = k + 1;
@@ -588,6 +604,8 @@ struct rpb_batch {
     // device
     InstDesc *d_inst = nullptr;
     BlockDesc *d_blocks = nullptr;
+    ChunkDesc *d_chunks = nullptr;   // chunks of the Gram-Schmidt kernels, and each instance's (first, count)
+    int2 *d_inst_chunks = nullptr;
     int *d_inst_of = nullptr;
     int *d_active = nullptr;
     int *d_nactive = nullptr;
@@ -601,11 +619,13 @@ struct rpb_batch {
     // host (pinned)
     InstDesc *h_inst = nullptr;
     BlockDesc *h_blocks = nullptr;
+    ChunkDesc *h_chunks = nullptr;
+    int2 *h_inst_chunks = nullptr;
     int *h_nactive = nullptr;
     double *h_lz = nullptr;
     int64_t total = 0;
     int B = 0;
-    int nblocks = 0;
+    int nblocks = 0, nchunks = 0;
     // multi-step runs: a private stream to capture and replay the step graph on, joined to the
     // caller's stream by an event; a device counter of unconverged instance-steps
     cudaStream_t cap = nullptr;
@@ -636,13 +656,13 @@ enum { V_POS, V_UP, V_F, V_T, V_UN, V_W, V_WT, V_G, V_DRIFT, V_PA, V_PB, V_WORK 
 
 static void batch_free(rpb_batch *bt)
 {
-    void *dev[] = {bt->d_inst, bt->d_blocks, bt->d_inst_of, bt->d_active, bt->d_nactive, bt->src, bt->V, bt->lz, bt->red,
+    void *dev[] = {bt->d_inst, bt->d_blocks, bt->d_chunks, bt->d_inst_chunks, bt->d_inst_of, bt->d_active, bt->d_nactive, bt->src, bt->V, bt->lz, bt->red,
                    bt->norm2, bt->nodes, bt->d_left};
     for (void *p : dev)
         if (p) cudaFree(p);
     for (double *p : bt->vec)
         if (p) cudaFree(p);
-    void *host[] = {bt->h_inst, bt->h_blocks, bt->h_nactive, bt->h_lz, bt->h_unconv};
+    void *host[] = {bt->h_inst, bt->h_blocks, bt->h_chunks, bt->h_inst_chunks, bt->h_nactive, bt->h_lz, bt->h_unconv};
     for (void *p : host)
         if (p) cudaFreeHost(p);
     if (bt->d_unconv) cudaFree(bt->d_unconv);
@@ -709,10 +729,24 @@ static int batch_setup(rpb_batch *bt, int B, const int64_t *N, const int64_t *st
     int k = 0;
     for (int b : order)
         for (int64_t f = 0; f < N[b]; f += kTile) bt->h_blocks[k++] = BlockDesc{b, (int)f};
+    int nc = 0;
+    for (int b = 0; b < B; ++b) {
+        const int cnt = (int)((N[b] + kGsChunk - 1) / kGsChunk), c0 = nc;
+        bt->h_inst_chunks[b] = make_int2(c0, cnt);
+        for (int q = 0; q < cnt; ++q) bt->h_chunks[nc++] = ChunkDesc{b, q * kGsChunk, c0, cnt};
+    }
     bt->total = total;
     bt->B = B;
     bt->nblocks = nblk;
+    bt->nchunks = nc;
     int rc;
+    if ((rc = cuda_fail(cudaMemcpyAsync(bt->d_chunks, bt->h_chunks, nc * sizeof(ChunkDesc), cudaMemcpyHostToDevice,
+                                        bt->stream),
+                        "batch chunks")) ||
+        (rc = cuda_fail(cudaMemcpyAsync(bt->d_inst_chunks, bt->h_inst_chunks, B * sizeof(int2), cudaMemcpyHostToDevice,
+                                        bt->stream),
+                        "batch chunks")))
+        return rc;
     if ((rc = cuda_fail(cudaMemcpyAsync(bt->d_inst, bt->h_inst, B * sizeof(InstDesc), cudaMemcpyHostToDevice, bt->stream),
                         "batch descriptors")))
         return rc;
@@ -823,9 +857,11 @@ static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, doub
             count_launches(1);
         }
     }
-    batch_dots_kernel<<<dim3(B, 1), kBThreads, 0, main_st>>>(W, 0, W, bt->d_inst, nullptr, total, B, bt->red);
-    batch_norm_init_kernel<<<(B + 127) / 128, 128, 0, main_st>>>(bt->red, B, bt->lz, bt->lz_stride, L.status,
-                                                                bt->d_active);
+    const int nc = bt->nchunks;
+    double *red2 = bt->red + (size_t)bt->max_iter * nc;
+    batch_dots_kernel<<<nc, kGsThreads, 0, main_st>>>(W, 0, 1, W, bt->d_inst, bt->d_chunks, nullptr, total, bt->red);
+    batch_norm_init_kernel<<<(B + 3) / 4, 128, 0, main_st>>>(bt->red, bt->d_inst_chunks, B, bt->lz, bt->lz_stride,
+                                                             L.status, bt->d_active);
     batch_scale_kernel<<<ge, 256, 0, main_st>>>(W, bt->d_inst, bt->d_inst_of, nullptr, total, bt->lz, bt->lz_stride,
                                                 L.status, ST_INV_NW, V);
     count_launches(3);
@@ -841,18 +877,18 @@ static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, doub
         rc = batch_product(bt, pos, vk, nullptr, w, bt->d_active);
         const int nv = k + 1;
         if (!rc) {
-            batch_dots_kernel<<<dim3(B, nv), kBThreads, 0, st>>>(V, ld, w, bt->d_inst, bt->d_active, total, B, bt->red);
-            batch_project_kernel<<<B, kBThreads, 0, st>>>(V, ld, w, bt->d_inst, bt->d_active, total, B, nv, bt->red,
-                                                          bt->lz, bt->lz_stride, L.c1, nullptr);
-            batch_dots_kernel<<<dim3(B, nv), kBThreads, 0, st>>>(V, ld, w, bt->d_inst, bt->d_active, total, B, bt->red);
-            batch_project_kernel<<<B, kBThreads, 0, st>>>(V, ld, w, bt->d_inst, bt->d_active, total, B, nv, bt->red,
-                                                          bt->lz, bt->lz_stride, L.c2, bt->norm2);
+            batch_dots_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, nv, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
+                                                         bt->red);
+            batch_project_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, nv, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
+                                                            bt->red, bt->lz, bt->lz_stride, L.c1, red2, nullptr);
+            batch_project_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, nv, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
+                                                            red2, bt->lz, bt->lz_stride, L.c2, nullptr, bt->norm2);
             rc = cuda_fail(cudaMemsetAsync(bt->d_nactive, 0, sizeof(int), st), "memset");
         }
         if (!rc) {
-            batch_tail_kernel<<<B, kTailThreads, 0, st>>>(bt->lz, bt->lz_stride, L, k, tol, bt->norm2, bt->nodes,
-                                                          bt->d_active, bt->d_nactive);
-            count_launches(5);
+            batch_tail_kernel<<<B, kTailThreads, 0, st>>>(bt->lz, bt->lz_stride, L, k, tol, bt->norm2,
+                                                          bt->d_inst_chunks, bt->nodes, bt->d_active, bt->d_nactive);
+            count_launches(4);
             if (graph) {
                 const bool has_next = k + 1 < max_iter;
                 batch_iter_kernel<<<1, 1, 0, st>>>(has_next ? hnd[k + 1] : 0ull, has_next ? 1 : 0, bt->d_nactive,
@@ -1093,7 +1129,7 @@ int rpb_batch_create(rpb_batch **out, const rpb_params *p, int64_t max_total_N, 
     const LzLayout L(max_iter);
     bt->lz_stride = L.total;
     const size_t vb = (size_t)3 * max_total_N * sizeof(double);
-    const int64_t max_blocks = max_total_N / kTile + max_B + 1;
+    const int64_t max_blocks = max_total_N / kTile + max_B + 1, max_chunks = max_total_N / kGsChunk + max_B + 1;
     bool ok = cudaMalloc(&bt->d_inst, max_B * sizeof(InstDesc)) == cudaSuccess &&
               cudaMalloc(&bt->d_blocks, max_blocks * sizeof(BlockDesc)) == cudaSuccess &&
               cudaMalloc(&bt->d_inst_of, max_total_N * sizeof(int)) == cudaSuccess &&
@@ -1102,8 +1138,12 @@ int rpb_batch_create(rpb_batch **out, const rpb_params *p, int64_t max_total_N, 
               cudaMalloc(&bt->src, max_total_N * sizeof(SrcF64)) == cudaSuccess &&
               cudaMalloc(&bt->V, vb * (max_iter + 1)) == cudaSuccess &&
               cudaMalloc(&bt->lz, (size_t)max_B * L.total * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&bt->red, (size_t)(max_iter + 2) * max_B * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&bt->norm2, (size_t)max_B * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&bt->red, (size_t)2 * max_iter * max_chunks * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&bt->norm2, (size_t)max_chunks * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&bt->d_chunks, max_chunks * sizeof(ChunkDesc)) == cudaSuccess &&
+              cudaMalloc(&bt->d_inst_chunks, max_B * sizeof(int2)) == cudaSuccess &&
+              cudaMallocHost(&bt->h_chunks, max_chunks * sizeof(ChunkDesc)) == cudaSuccess &&
+              cudaMallocHost(&bt->h_inst_chunks, max_B * sizeof(int2)) == cudaSuccess &&
               cudaMalloc(&bt->nodes, 2 * kSqrtNodes * sizeof(double)) == cudaSuccess &&
               cudaMallocHost(&bt->h_inst, max_B * sizeof(InstDesc)) == cudaSuccess &&
               cudaMallocHost(&bt->h_blocks, max_blocks * sizeof(BlockDesc)) == cudaSuccess &&

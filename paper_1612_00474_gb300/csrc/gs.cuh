@@ -1,0 +1,119 @@
+// gs.cuh -- device side of the Gram-Schmidt steps of the Lanczos iteration (classical Gram-Schmidt
+// applied twice, Sec. II.C), on blocks of kGsThreads threads that each own a chunk of spheres.
+//
+// What bounds them: float64 instructions (64 cycles of a scheduler per warp instruction), not memory.  A
+// thread keeps its rows of w in registers; dot products are taken eight basis vectors at a time, so
+// that summing them over a warp costs nine additions for the eight (a reduce-scatter over the lanes)
+// instead of forty.
+#pragma once
+
+#include "lanczos_math.cuh"
+
+namespace rpb {
+
+constexpr int kGsThreads = 256;
+constexpr int kGsWarps = kGsThreads / 32;
+constexpr int kGsChunk = 256;                              // spheres of a chunk at most
+constexpr int kGsRows = 3 * kGsChunk / kGsThreads;         // rows (sphere, component) of a thread
+
+// Rows of a chunk: components x, y, z of `cnt` spheres at offsets base + c stride + i.
+struct GsSpan {
+    int64_t base, stride;
+    int cnt;
+};
+
+// Offsets of this thread's rows (component-major in the chunk); -1 past the end.
+__device__ __forceinline__ void gs_rows(const GsSpan &s, int64_t (&row)[kGsRows])
+{
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) {
+        const int r = threadIdx.x + u * kGsThreads;
+        const int c = r < s.cnt ? 0 : (r < 2 * s.cnt ? 1 : 2);
+        row[u] = r < 3 * s.cnt ? s.base + c * s.stride + (r - c * s.cnt) : -1;
+    }
+}
+
+// Sums over the warp of eight values per lane: lane l returns the sum of v[l >> 2] (a fixed order).
+__device__ __forceinline__ double warp_sum8(double (&v)[8])
+{
+    const int lane = threadIdx.x & 31;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+    double a[4], b[2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = (b4 ? v[q + 4] : v[q]) + __shfl_xor_sync(0xffffffffu, b4 ? v[q] : v[q + 4], 16);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) b[q] = (b3 ? a[q + 2] : a[q]) + __shfl_xor_sync(0xffffffffu, b3 ? a[q] : a[q + 2], 8);
+    double s = (b2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, b2 ? b[0] : b[1], 4);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    return s + __shfl_xor_sync(0xffffffffu, s, 1);
+}
+
+// Sum over the block of one value per thread, in every thread; sh: kGsWarps doubles.
+__device__ __forceinline__ double gs_block_sum(double v, double *sh)
+{
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    for (int k = 0; k < kGsWarps; ++k) s += sh[k];
+    __syncthreads();
+    return s;
+}
+
+// The block's part of <V_j, w>, j < nvec: thread j < nvec returns it (nvec <= kGsThreads).
+// sh: kGsWarps x (kMaxIter + 8) doubles.
+__device__ __forceinline__ double gs_dots(const double *__restrict__ V, size_t ld, int nvec, const int64_t (&row)[kGsRows],
+                                          const double (&w)[kGsRows], double (*sh)[kMaxIter + 8])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int j0 = 0; j0 < nvec; j0 += 8) {
+        double acc[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            acc[q] = 0.0;
+            if (j0 + q < nvec) {
+                const double *v = V + (size_t)(j0 + q) * ld;
+#pragma unroll
+                for (int u = 0; u < kGsRows; ++u)
+                    if (row[u] >= 0) acc[q] = fma(v[row[u]], w[u], acc[q]);
+            }
+        }
+        const double s = warp_sum8(acc);
+        if ((lane & 3) == 0) sh[warp][j0 + (lane >> 2)] = s;
+    }
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < nvec)
+        for (int k = 0; k < kGsWarps; ++k) s += sh[k][threadIdx.x];
+    return s;
+}
+
+// w -= sum_j coef_j V_j
+__device__ __forceinline__ void gs_project(const double *__restrict__ V, size_t ld, int nvec, const int64_t (&row)[kGsRows],
+                                           const double *coef, double (&w)[kGsRows])
+{
+#pragma unroll 4
+    for (int j = 0; j < nvec; ++j) {
+        const double *v = V + (size_t)j * ld;
+        const double m = -coef[j];
+#pragma unroll
+        for (int u = 0; u < kGsRows; ++u)
+            if (row[u] >= 0) w[u] = fma(m, v[row[u]], w[u]);
+    }
+}
+
+// coef_j = sum of n partials red[j rs + k], j < nvec, by one warp per vector in a fixed order; ends with a
+// block barrier.
+__device__ __forceinline__ void gs_coefs(const double *__restrict__ red, size_t rs, int n, int nvec, double *coef)
+{
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x >> 5; j < nvec; j += kGsWarps) {
+        double s = 0.0;
+        for (int k = lane; k < n; k += 32) s += red[(size_t)j * rs + k];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) coef[j] = s;
+    }
+    __syncthreads();
+}
+
+}  // namespace rpb
