@@ -615,6 +615,7 @@ struct rpb_batch {
     double *lz = nullptr;
     double *red = nullptr;
     double *norm2 = nullptr;
+    double *selfc = nullptr;  // self coefficients of the packed positions (SelfCoefs), 4 max_total_N
     double *nodes = nullptr;  // nodes and weights of the Lanczos square root
     // host (pinned)
     InstDesc *h_inst = nullptr;
@@ -657,7 +658,7 @@ enum { V_POS, V_UP, V_F, V_T, V_UN, V_W, V_WT, V_G, V_DRIFT, V_PA, V_PB, V_WORK 
 static void batch_free(rpb_batch *bt)
 {
     void *dev[] = {bt->d_inst, bt->d_blocks, bt->d_chunks, bt->d_inst_chunks, bt->d_inst_of, bt->d_active, bt->d_nactive, bt->src, bt->V, bt->lz, bt->red,
-                   bt->norm2, bt->nodes, bt->d_left};
+                   bt->norm2, bt->selfc, bt->nodes, bt->d_left};
     for (void *p : dev)
         if (p) cudaFree(p);
     for (double *p : bt->vec)
@@ -779,14 +780,16 @@ static int batch_product(rpb_batch *bt, const double *pos, const double *F, cons
     const double scale = 1.0 / (8.0 * kPi * bt->p.eta);
     const int pb = 256;
     const int gpack = (int)((total + pb - 1) / pb);
+    const SelfCoefs none = {nullptr, 0, 0.0, PairConsts<double>{}};  // the one-way kernels evaluate their self terms
     if (bt->p.precision == RPB_FP32 && bt->sym_ok) {
         SrcF32 *src = (SrcF32 *)bt->src;
-        pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src);
+        const SelfCoefs sc = {bt->selfc, total, scale, make_consts<double>(a)};
+        pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, sc);
         count_launches(1);
-        return batch_sym_apply(bt->sym, bt->stream, src, total, pos, F, T, U, active, a, bt->p.eta);
+        return batch_sym_apply(bt->sym, bt->stream, src, total, F, T, U, active, a, sc);
     } else if (bt->p.precision == RPB_FP32) {
         SrcF32 *src = (SrcF32 *)bt->src;
-        pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src);
+        pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, none);
         const X2Consts c = make_x2_consts(a);
         const PairConsts<double> cd = make_consts<double>(a);
         if (T)
@@ -797,7 +800,7 @@ static int batch_product(rpb_batch *bt, const double *pos, const double *F, cons
                 src, bt->d_inst, bt->d_blocks, active, total, c, cd, a, scale, pos, F, T, U);
     } else {
         SrcF64 *src = (SrcF64 *)bt->src;
-        pack_f64_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src);
+        pack_f64_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, none);
         const PairConsts<double> c = make_consts<double>(a);
         if (T)
             batch_pair_f64_kernel<true><<<bt->nblocks, kPairThreads, 0, bt->stream>>>(
@@ -1144,6 +1147,7 @@ int rpb_batch_create(rpb_batch **out, const rpb_params *p, int64_t max_total_N, 
               cudaMalloc(&bt->d_inst_chunks, max_B * sizeof(int2)) == cudaSuccess &&
               cudaMallocHost(&bt->h_chunks, max_chunks * sizeof(ChunkDesc)) == cudaSuccess &&
               cudaMallocHost(&bt->h_inst_chunks, max_B * sizeof(int2)) == cudaSuccess &&
+              cudaMalloc(&bt->selfc, (size_t)4 * max_total_N * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&bt->nodes, 2 * kSqrtNodes * sizeof(double)) == cudaSuccess &&
               cudaMallocHost(&bt->h_inst, max_B * sizeof(InstDesc)) == cudaSuccess &&
               cudaMallocHost(&bt->h_blocks, max_blocks * sizeof(BlockDesc)) == cudaSuccess &&

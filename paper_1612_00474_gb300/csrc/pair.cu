@@ -38,7 +38,8 @@ namespace rpb {
 
 // ------------------------------------------------------------------ packing
 __global__ void pack_f32_kernel(const double *__restrict__ pos, const double *__restrict__ F,
-                                const double *__restrict__ T, int N, double a, int wall, SrcF32 *__restrict__ out)
+                                const double *__restrict__ T, int N, double a, int wall, SrcF32 *__restrict__ out,
+                                SelfCoefs sc)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -52,6 +53,7 @@ __global__ void pack_f32_kernel(const double *__restrict__ pos, const double *__
     o.t = make_float4(T ? (float)(s * T[i]) : 0.f, T ? (float)(s * T[N + i]) : 0.f, T ? (float)(s * T[2 * N + i]) : 0.f,
                       0.f);
     out[i] = o;
+    if (sc.s) store_self_coefs(sc, i, s, wall ? fmax(z, a) : z, wall);
 }
 
 // Second right-hand side of the two-RHS symmetric pass: s_j P_j as float32 (x, y, z, 0).
@@ -65,7 +67,8 @@ __global__ void pack_rhs2_kernel(const double *__restrict__ pos, const double *_
 }
 
 __global__ void pack_f64_kernel(const double *__restrict__ pos, const double *__restrict__ F,
-                                const double *__restrict__ T, int N, double a, int wall, SrcF64 *__restrict__ out)
+                                const double *__restrict__ T, int N, double a, int wall, SrcF64 *__restrict__ out,
+                                SelfCoefs sc)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -78,6 +81,18 @@ __global__ void pack_f64_kernel(const double *__restrict__ pos, const double *__
     o.s = make_double2(T ? s * T[i] : 0.0, T ? s * T[N + i] : 0.0);
     o.u = make_double2(T ? s * T[2 * N + i] : 0.0, 0.0);
     out[i] = o;
+    if (sc.s) store_self_coefs(sc, i, s, wall ? fmax(z, a) : z, wall);
+}
+
+// The self coefficients of a context's products, or none (the row-range and allocation-free products
+// evaluate their self terms themselves).
+SelfCoefs self_coefs(const rpb_ctx *ctx, int64_t N)
+{
+    return SelfCoefs{ctx->ws.selfc, N, 1.0 / (8.0 * kPi * ctx->p.eta), make_consts<double>(ctx->p.a)};
+}
+static SelfCoefs no_self_coefs()
+{
+    return SelfCoefs{nullptr, 0, 0.0, PairConsts<double>{}};
 }
 
 // ------------------------------------------------------------------ pair kernels
@@ -641,32 +656,30 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
     }
 }
 
-// Row partials of the targets plus column partials of the sources, fixed order; float64 self term
-// (with the torque's wall self coupling when T is given; left out when self_term is 0, for all but
-// one share of a shared product); s_i / (8 pi eta).  col_rows: the rows [r0, r1) of each column that
-// the schedule wrote (null: all rows above the diagonal).  NC = 6: the partials also
-// carry a second translation-translation right-hand side P, written to U2 with its own self term.
+// Row partials of the targets plus column partials of the sources, fixed order, and the float64 self term
+// from the spheres' coefficients (left out when self_term is 0, for all but one share of a shared
+// product).  col_rows: the rows [r0, r1) of each column that the schedule wrote (null: all rows above the
+// diagonal).  NC = 6: the partials also carry a second translation-translation right-hand side P,
+// written to U2 with its own self term.
 // BATCH: tiles of many suspensions (tile_inst: the suspension of each tile; sinst as in the pair
 // kernel); the column of tile b holds the rows tile0 .. b - 1 of its suspension, summed in an order
 // relative to tile0 so that a suspension's result does not depend on its companions.
+// What bounds it: float64 instructions for the batched form (they were about 400 warp instructions a
+// tile, most of them the self terms and the conversions of the compensated sums; now about 100), a chain
+// of loads and additions for a single small suspension.
 template <int NC, bool BATCH = false>
-__global__ void __launch_bounds__(BATCH ? 384 : 768, BATCH ? 5 : 2) pair_sym_reduce_kernel(const double *__restrict__ tgt_part, const float *__restrict__ src_part,
-                                       const int *__restrict__ row_seg, const int *__restrict__ col_start, int N,
-                                       const double *__restrict__ pos, const double *__restrict__ F,
-                                       const double *__restrict__ T, PairConsts<double> c, double a, double scale,
-                                       double *__restrict__ U, const double *__restrict__ P = nullptr,
-                                       double *__restrict__ U2 = nullptr,
-                                       const SymInst *__restrict__ sinst = nullptr,
-                                       const int *__restrict__ tile_inst = nullptr,
-                                       const int *__restrict__ active = nullptr,
-                                       const int *__restrict__ col_rows = nullptr, int self_term = 1)
+__global__ void __launch_bounds__(BATCH ? 384 : 768, BATCH ? 5 : 2) pair_sym_reduce_kernel(
+    const double *__restrict__ tgt_part, const float *__restrict__ src_part, const int *__restrict__ row_seg,
+    const int *__restrict__ col_start, int N, const double *__restrict__ F, const double *__restrict__ T, SelfCoefs sc,
+    double *__restrict__ U, const double *__restrict__ P = nullptr, double *__restrict__ U2 = nullptr,
+    const SymInst *__restrict__ sinst = nullptr, const int *__restrict__ tile_inst = nullptr,
+    const int *__restrict__ active = nullptr, const int *__restrict__ col_rows = nullptr, int self_term = 1)
 {
     // one CTA of 768 threads (384 batched) per 128-sphere tile, the longest columns first; thread (half, q, l):
-    // component q of sphere l, rows of its column congruent to `half` modulo HALVES
+    // component q of sphere l, rows of its column and segments of its row congruent to `half` modulo HALVES
     // (a batched suspension's columns are at most a few tiles long: one thread per (q, l) there, so
     // that twice as many tiles are resident at once)
     constexpr int HALVES = BATCH ? 1 : 6 / NC;
-    __shared__ double s[NC][kTile];
     __shared__ double s1[NC][kTile];
     const int nb = gridDim.x;
     const int b = BATCH ? (int)blockIdx.x : nb - 1 - (int)blockIdx.x;
@@ -703,44 +716,31 @@ __global__ void __launch_bounds__(BATCH ? 384 : 768, BATCH ? 5 : 2) pair_sym_red
             }
         }
     }
-    double v = 0.0;
+    // the four sums as one float32 pair (Knuth's exact two-sum, the errors gathered in the low part:
+    // 2^-48 of the largest), so that one sum, not eight numbers, is converted
+    float hi = cs[0], lo = -cc[0];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v += (double)cs[u] - (double)cc[u];
-    if (HALVES == 2 && half == 1) s1[q][l] = v;
-    __syncthreads();
-    if (half == 0) {
-        double acc = 0.0;
-        for (int k = row_seg[b]; k < row_seg[b + 1]; ++k) acc += tgt_part[((size_t)k * NC + q) * kTile + l];
-        s[q][l] = acc + (HALVES == 2 ? v + s1[q][l] : v);
+    for (int u = 1; u < 4; ++u) {
+        const float t = hi + cs[u], z = t - hi;
+        lo += (hi - (t - z)) + (cs[u] - z) - cc[u];
+        hi = t;
     }
-    __syncthreads();
+    double v = (double)hi + (double)lo;
+#pragma unroll 4
+    for (int k = row_seg[b] + half; k < row_seg[b + 1]; k += HALVES) v += tgt_part[((size_t)k * NC + q) * kTile + l];
+    if (HALVES == 2) {
+        if (half == 1) s1[q][l] = v;
+        __syncthreads();
+        if (half == 0) v += s1[q][l];
+    }
     const int lb = (b - tb) * kTile + l;
-    if (half != 0 || lb >= Ni || (q != 0 && q != 3)) return;
+    if (half != 0 || lb >= Ni) return;
     const long long i = off + lb;
-    const double z = pos[2 * N + i];
-    const double si = H0(z / a);
-    const double zc = fmax(z, a);
-    const double k = si * scale;
-    if (q == 0) {
-        double ux = s[0][l], uy = s[1][l], uz = s[2][l];
-        if (!BATCH && !self_term)
-            ;
-        else if (T)
-            self_velocity<true>(zc, si * F[i], si * F[N + i], si * F[2 * N + i], si * T[i], si * T[N + i], c, ux, uy,
-                                uz);
-        else
-            self_velocity<false>(zc, si * F[i], si * F[N + i], si * F[2 * N + i], 0.0, 0.0, c, ux, uy, uz);
-        U[i] = k * ux;
-        U[N + i] = k * uy;
-        U[2 * N + i] = k * uz;
-    } else if (NC == 6) {
-        double ux = s[3 % NC][l], uy = s[4 % NC][l], uz = s[5 % NC][l];
-        if (BATCH || self_term)
-            self_velocity<false>(zc, si * P[i], si * P[N + i], si * P[2 * N + i], 0.0, 0.0, c, ux, uy, uz);
-        U2[i] = k * ux;
-        U2[N + i] = k * uy;
-        U2[2 * N + i] = k * uz;
-    }
+    if (NC == 6 && q >= 3)
+        U2[(q - 3) * (int64_t)N + i] = sc.velocity(i, q - 3, v, P, nullptr, N);
+    else
+        U[q * (int64_t)N + i] =
+            BATCH || self_term ? sc.velocity(i, q, v, F, T, N) : sc.s[i] * sc.scale * v;
 }
 
 constexpr int kTtMinBlocks = 5;     // resident CTAs per SM of the translation-translation form (up to 102 registers:
@@ -836,7 +836,8 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
     const double a = ctx->p.a;
     SrcF32 *src = (SrcF32 *)w.src;
     const int pb = 256;
-    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src);
+    const SelfCoefs self = self_coefs(ctx, N);
+    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, self);
     const SymCta *ctas = (const SymCta *)sc->index;
     const SymSeg *segs = (const SymSeg *)(sc->index + sc->seg_off);
     const X2Consts c = make_x2_consts(a);
@@ -850,9 +851,8 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
                                                                                           w.sym_tgt, w.sym_src);
     }
     pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
-        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, pos, F, T, make_consts<double>(a), a,
-        1.0 / (8.0 * kPi * ctx->p.eta), U, nullptr, nullptr, nullptr, nullptr, nullptr, sc->index + sc->rows_off,
-        part == 0);
+        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
+        sc->index + sc->rows_off, part == 0);
     count_launches(sc->ncta > 0 ? 3 : 2);
     return cuda_fail(cudaGetLastError(), "symmetric pair kernels");
 }
@@ -870,7 +870,8 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
     const double a = ctx->p.a;
     SrcF32 *src = (SrcF32 *)w.src;
     const int pb = 256;
-    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos_w, F, T, N, a, 1, src);
+    const SelfCoefs self = self_coefs(ctx, N);
+    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos_w, F, T, N, a, 1, src, self);
     const SymCta *ctas = (const SymCta *)sc->index;
     const SymSeg *segs = (const SymSeg *)(sc->index + sc->seg_off);
     const X2Consts c = make_x2_consts(a);
@@ -891,9 +892,8 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
                 src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, pl);
     }
     pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
-        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, pos, F, T, make_consts<double>(a), a,
-        1.0 / (8.0 * kPi * ctx->p.eta), U, nullptr, nullptr, nullptr, nullptr, nullptr, sc->index + sc->rows_off,
-        part == 0);
+        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
+        sc->index + sc->rows_off, part == 0);
     count_launches(sc->ncta > 0 ? 3 : 2);
     return cuda_fail(cudaGetLastError(), "periodic symmetric pair kernels");
 }
@@ -995,8 +995,8 @@ int batch_sym_plan(BatchSymPlan &pl, int B, const int64_t *N, cudaStream_t st, b
     return RPB_OK;
 }
 
-int batch_sym_apply(const BatchSymPlan &pl, cudaStream_t st, const SrcF32 *src, int64_t total, const double *pos,
-                    const double *F, const double *T, double *U, const int *active, double a, double eta)
+int batch_sym_apply(const BatchSymPlan &pl, cudaStream_t st, const SrcF32 *src, int64_t total, const double *F,
+                    const double *T, double *U, const int *active, double a, const SelfCoefs &sc)
 {
     const SymCta *ctas = (const SymCta *)pl.index;
     const SymSeg *segs = (const SymSeg *)(pl.index + pl.seg_off);
@@ -1013,8 +1013,8 @@ int batch_sym_apply(const BatchSymPlan &pl, cudaStream_t st, const SrcF32 *src, 
         pair_f32x2_sym_kernel<5, false, false, false, true><<<pl.ncta, kPairThreads, 0, st>>>(
             src, n, ctas, segs, c, cs, pl.tgt, pl.srcp, nullptr, PerLen{}, pl.sinst, active);
     pair_sym_reduce_kernel<3, true><<<pl.ntiles, 3 * kTile, 0, st>>>(
-        pl.tgt, pl.srcp, pl.index + pl.row_off, cs, n, pos, F, T, make_consts<double>(a), a, 1.0 / (8.0 * kPi * eta),
-        U, nullptr, nullptr, pl.sinst, pl.index + pl.inst_off, active);
+        pl.tgt, pl.srcp, pl.index + pl.row_off, cs, n, F, T, sc, U, nullptr, nullptr, pl.sinst, pl.index + pl.inst_off,
+        active);
     count_launches(2);
     return cuda_fail(cudaGetLastError(), "batched symmetric kernels");
 }
@@ -1042,7 +1042,8 @@ int mobility_apply2_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const dou
     SrcF32 *src = (SrcF32 *)w.src;
     float4 *src2 = (float4 *)w.src2;
     const int pb = 256;
-    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src);
+    const SelfCoefs self = self_coefs(ctx, N);
+    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, self);
     pack_rhs2_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, P, N, a, src2);
     const SymCta *ctas = (const SymCta *)sc->index;
     const SymSeg *segs = (const SymSeg *)(sc->index + sc->seg_off);
@@ -1050,8 +1051,8 @@ int mobility_apply2_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const dou
     pair_f32x2_sym_kernel<kRhs2MinBlocks, true, true><<<sc->ncta, kPairThreads, 0, st>>>(
         src, N, ctas, segs, make_x2_consts(a), cs, w.sym_tgt, w.sym_src, src2);
     pair_sym_reduce_kernel<6><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
-        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, pos, F, T, make_consts<double>(a), a,
-        1.0 / (8.0 * kPi * ctx->p.eta), U, P, U2, nullptr, nullptr, nullptr, sc->index + sc->rows_off);
+        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, P, U2, nullptr, nullptr, nullptr,
+        sc->index + sc->rows_off);
     count_launches(4);
     return cuda_fail(cudaGetLastError(), "two-right-hand-side symmetric kernels");
 }
@@ -1252,11 +1253,8 @@ __global__ void __launch_bounds__(kPairThreads) pair_periodic_f32_kernel(const S
 // stride nt, U with component stride ldu (ldu < 0: nt).
 __global__ void pair_reduce_kernel(const double *__restrict__ part, int splits, int N, const double *__restrict__ pos,
                                    const double *__restrict__ F, const double *__restrict__ T, PairConsts<double> c,
-                                   double a, double scale, double *__restrict__ U, int wall = 1, int t0 = 0,
-                                   int nt = -1, int ldu = -1)
+                                   double a, double scale, double *__restrict__ U, int wall, int t0, int nt, int ldu)
 {
-    if (nt < 0) nt = N;
-    if (ldu < 0) ldu = nt;
     const int li = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = t0 + li;
     if (li >= nt || i >= N) return;
@@ -1395,7 +1393,7 @@ int mobility_rows_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
     const bool torque = T != nullptr;
     if (fp64) {
         SrcF64 *src = (SrcF64 *)ctx->ws.src;
-        pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src);
+        pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, no_self_coefs());
         const PairConsts<double> c = make_consts<double>(a);
         if (!ctx->p.wall) {
             if (torque)
@@ -1409,7 +1407,7 @@ int mobility_rows_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
         }
     } else {
         SrcF32 *src = (SrcF32 *)ctx->ws.src;
-        pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src);
+        pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, no_self_coefs());
         const X2Consts c = make_x2_consts(a);
         if (torque)
             pair_f32x2_kernel<true><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part, (int)t0, nt);
@@ -1507,7 +1505,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
         }
         if (ctx->p.precision == RPB_FP32) {
             SrcF32 *src = (SrcF32 *)ctx->ws.src;
-            pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src);
+            pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src, no_self_coefs());
             const PairConsts<float> c = make_consts<float>(a);
             const float Lxh = (float)Lx, Lyh = (float)Ly;
             const float Lxl = (float)(Lx - (double)Lxh), Lyl = (float)(Ly - (double)Lyh);
@@ -1521,7 +1519,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
                 pair_periodic_f32_kernel<false, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, Lxh, Lxl, Lyh, Lyl, part);
         } else {
             SrcF64 *src = (SrcF64 *)ctx->ws.src;
-            pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src);
+            pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src, no_self_coefs());
             const PairConsts<double> c = make_consts<double>(a);
             if (torque && ctx->p.wall)
                 pair_periodic_f64_kernel<true, true><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, Lx, Ly, part);
@@ -1538,7 +1536,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
     }
     if (ctx->p.precision == RPB_FP32) {
         SrcF32 *src = (SrcF32 *)ctx->ws.src;
-        pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src);
+        pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, no_self_coefs());
         if (!ctx->p.wall) {
             const PairConsts<float> c = make_consts<float>(a);
             if (torque)
@@ -1560,7 +1558,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
         }
     } else {
         SrcF64 *src = (SrcF64 *)ctx->ws.src;
-        pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src);
+        pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, no_self_coefs());
         const PairConsts<double> c = make_consts<double>(a);
         if (!ctx->p.wall) {
             if (torque)
@@ -2048,7 +2046,7 @@ extern "C" int rpb_mobility_apply_noalloc(int64_t N64, const double *pos, const 
     const double a = p->a;
     if (p->precision == RPB_FP32) {
         SrcF32 *src = (SrcF32 *)base;
-        pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src);
+        pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, no_self_coefs());
         const PairConsts<float> c = make_consts<float>(a);
         if (T)
             pair_f32_kernel<true><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
@@ -2056,7 +2054,7 @@ extern "C" int rpb_mobility_apply_noalloc(int64_t N64, const double *pos, const 
             pair_f32_kernel<false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
     } else {
         SrcF64 *src = (SrcF64 *)base;
-        pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src);
+        pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, no_self_coefs());
         const PairConsts<double> c = make_consts<double>(a);
         if (T)
             pair_f64_kernel<true><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);

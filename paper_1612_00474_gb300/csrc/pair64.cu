@@ -259,50 +259,34 @@ __global__ void __launch_bounds__(32 * kSym64Warps) pair_sym64_kernel(const SrcF
     }
 }
 
-// One CTA per tile: the tile's row and column partials in a fixed order, eight threads per sum, while one
-// more warp evaluates the self terms; U = s_i / (8 pi eta) (sum + self).
+// One CTA per tile: the tile's row and column partials in a fixed order, eight threads per sum, and the
+// self term.
 constexpr int kRed64Groups = 8;
-constexpr int kRed64Threads = 96 * kRed64Groups + 32;
+constexpr int kRed64Threads = 96 * kRed64Groups;
 
-template <bool WALL>
 __global__ void __launch_bounds__(kRed64Threads) pair_sym64_reduce_kernel(
     const double *__restrict__ tgt_part, const double *__restrict__ src_part, Sym64Plan pl, int N,
-    const double *__restrict__ pos, const double *__restrict__ F, const double *__restrict__ T, PairConsts<double> c,
-    double a, double scale, double *__restrict__ U)
+    const double *__restrict__ F, const double *__restrict__ T, SelfCoefs sc, double *__restrict__ U)
 {
     __shared__ double sum[kRed64Groups][96];
-    __shared__ double self[4][kTile64];  // the self term, and s_i scale
     const int b = pl.nb - 1 - (int)blockIdx.x;  // the longest columns first
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int i = b * kTile64 + lane;
-    if (tid >= 96 * kRed64Groups) {
-        const int k = min(i, N - 1);
-        const double z = pos[2 * (int64_t)N + k];
-        const double si = WALL ? H0(z / a) : 1.0;
-        double x = 0.0, y = 0.0, w = 0.0;
-        self_velocity<true, WALL>(WALL ? fmax(z, a) : z, si * F[k], si * F[N + (int64_t)k], si * F[2 * (int64_t)N + k],
-                                  T ? si * T[k] : 0.0, T ? si * T[N + (int64_t)k] : 0.0, c, x, y, w);
-        self[0][lane] = x;
-        self[1][lane] = y;
-        self[2][lane] = w;
-        self[3][lane] = si * scale;
-    } else {
-        const int g = tid / 96, e = tid - 96 * g;
-        const int64_t r0 = sym64_row_run(pl, b) * pl.qs;
-        const int nr = (int)((pl.nb - b + pl.L - 1) / pl.L) * pl.qs, nc = b * pl.qs;
-        const double *row = tgt_part + r0 * 96 + e, *col = src_part + sym64_col_slot(pl, 0, b, 0) * 96 + e;
-        double x[2] = {0.0, 0.0};
+    const int tid = threadIdx.x;
+    const int g = tid / 96, e = tid - 96 * g;
+    const int64_t r0 = sym64_row_run(pl, b) * pl.qs;
+    const int nr = (int)((pl.nb - b + pl.L - 1) / pl.L) * pl.qs, nc = b * pl.qs;
+    const double *row = tgt_part + r0 * 96 + e, *col = src_part + sym64_col_slot(pl, 0, b, 0) * 96 + e;
+    double x[2] = {0.0, 0.0};
 #pragma unroll 4
-        for (int k = g; k < nr; k += kRed64Groups) x[0] += row[(int64_t)k * 96];
+    for (int k = g; k < nr; k += kRed64Groups) x[0] += row[(int64_t)k * 96];
 #pragma unroll 4
-        for (int k = g; k < nc; k += kRed64Groups) x[1] += col[(int64_t)k * 96];
-        sum[g][e] = x[0] + x[1];
-    }
+    for (int k = g; k < nc; k += kRed64Groups) x[1] += col[(int64_t)k * 96];
+    sum[g][e] = x[0] + x[1];
     __syncthreads();
+    const int i = b * kTile64 + (tid & 31);
     if (tid < 96 && i < N) {
-        double x = 0.0;
-        for (int g = 0; g < kRed64Groups; ++g) x += sum[g][tid];
-        U[(int64_t)(tid >> 5) * N + i] = self[3][lane] * (x + self[tid >> 5][lane]);
+        double s = 0.0;
+        for (int k = 0; k < kRed64Groups; ++k) s += sum[k][tid];
+        U[(int64_t)(tid >> 5) * N + i] = sc.velocity(i, tid >> 5, s, F, T, N);
     }
 }
 
@@ -315,12 +299,12 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
 {
     cudaStream_t st = ctx->stream;
     const double a = ctx->p.a;
-    const PairConsts<double> c = make_consts<double>(a);
+    const SelfCoefs self = self_coefs(ctx, N);
     const Sym64Consts c64 = make_sym64_consts(a);
     const Sym64Plan pl = sym64_plan(N, ctx->num_sms);
     double *tgt = ctx->ws.sym64, *col = tgt + sym64_tgt_elems(ctx->max_N, ctx->num_sms);
     SrcF64 *src = (SrcF64 *)ctx->ws.src;
-    pack_f64_kernel<<<(N + 255) / 256, 256, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src);
+    pack_f64_kernel<<<(N + 255) / 256, 256, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
     const dim3 grid((unsigned)pl.runs, (unsigned)pl.qs);
     const int nt = 32 * kSym64Warps;
     if (ctx->p.wall && T)
@@ -331,11 +315,7 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
         pair_sym64_kernel<true, false><<<grid, nt, 0, st>>>(src, N, pl, c64, tgt, col);
     else
         pair_sym64_kernel<false, false><<<grid, nt, 0, st>>>(src, N, pl, c64, tgt, col);
-    const double scale = 1.0 / (8.0 * kPi * ctx->p.eta);
-    if (ctx->p.wall)
-        pair_sym64_reduce_kernel<true><<<pl.nb, kRed64Threads, 0, st>>>(tgt, col, pl, N, pos, F, T, c, a, scale, U);
-    else
-        pair_sym64_reduce_kernel<false><<<pl.nb, kRed64Threads, 0, st>>>(tgt, col, pl, N, pos, F, T, c, a, scale, U);
+    pair_sym64_reduce_kernel<<<pl.nb, kRed64Threads, 0, st>>>(tgt, col, pl, N, F, T, self, U);
     count_launches(3);
     return cuda_fail(cudaGetLastError(), "float64 symmetric pair kernels");
 }

@@ -210,6 +210,45 @@ __device__ __forceinline__ void self_velocity(double h, double Fx, double Fy, do
     }
 }
 
+// The self term and the target's factor at one position, ready to use: s_i = H0(z/a), and s_i^2 / (8 pi eta)
+// times the parallel and normal self mobilities and the torque's self coupling of self_velocity
+// (scale = 1/(8 pi eta)).  Stored by the pack kernels in four arrays of n (SelfCoefs), so that the reduce
+// kernels, which are bound by float64 instructions, spend two per output on it instead of about 45 a
+// sphere, and the products of a Lanczos solve share one evaluation.
+struct SelfCoefs {
+    double *s;       // s_i | parallel | normal | torque coupling
+    int64_t n;       // stride of the four arrays
+    double scale;
+    PairConsts<double> c;
+    // component q (0, 1, 2) of the velocity from the pair sum x of sphere i and its own load
+    __device__ __forceinline__ double velocity(int64_t i, int q, double x, const double *__restrict__ F,
+                                               const double *__restrict__ T, int64_t ld) const
+    {
+        double u = fma(s[i] * scale, x, s[(q == 2 ? 2 : 1) * n + i] * F[q * ld + i]);
+        if (T && q < 2) u = fma(q == 0 ? s[3 * n + i] : -s[3 * n + i], T[(1 - q) * ld + i], u);
+        return u;
+    }
+};
+
+SelfCoefs self_coefs(const rpb_ctx *ctx, int64_t N);  // of a context's products (pair.cu)
+
+__device__ __forceinline__ void store_self_coefs(const SelfCoefs &k, int64_t i, double s, double h, int wall)
+{
+    const PairConsts<double> &c = k.c;
+    double ux = 0.0, uy = 0.0, uz = 0.0, tx = 0.0, ty = 0.0, tz = 0.0;
+    const double f = s * s * k.scale;
+    if (wall) {
+        self_velocity<false, true>(h, 1.0, 0.0, 1.0, 0.0, 0.0, c, ux, uy, uz);
+        self_velocity<true, true>(h, 0.0, 0.0, 0.0, 0.0, 1.0, c, tx, ty, tz);
+    } else {
+        self_velocity<false, false>(h, 1.0, 0.0, 1.0, 0.0, 0.0, c, ux, uy, uz);
+    }
+    k.s[i] = s;
+    k.s[k.n + i] = f * ux;
+    k.s[2 * k.n + i] = f * uz;
+    k.s[3 * k.n + i] = f * tx;
+}
+
 // Float32 form of pair_velocity for the hot loop, hand-fused and algebraically rearranged (same
 // mathematics): the wall terms use the unnormalised image vector R, the free-space c1 and wall A/|R|
 // share one multiply-add into F, r.F and R.F share their in-plane part, the free-space rotlet

@@ -155,6 +155,7 @@ struct Workspace {
     double *pos_b = nullptr;
     double *pos_w = nullptr;      // positions folded into the unit cell (pseudo-periodic mode), 3 max_N
     void *cells = nullptr;        // cell lists of the force pass (cell_lists_bytes)
+    double *selfc = nullptr;      // self coefficients of the packed positions (SelfCoefs), 4 max_N
     double *vec_a = nullptr;      // 3 max_N scratch vectors for the AB step
     double *vec_b = nullptr;
     double *vec_c = nullptr;
@@ -264,11 +265,15 @@ bool mobility_apply2_ok(const rpb_ctx *ctx, int64_t N);
 int mobility_apply2_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *F, const double *T,
                          const double *P, double *U, double *U2);
 
-// Packed source records from float64 SoA inputs (pair.cu); also used by the batched path.
+// Packed source records from float64 SoA inputs (pair.cu), and the spheres' self coefficients where
+// sc.s is given; also used by the batched path.
+struct SelfCoefs;
 __global__ void pack_f32_kernel(const double *__restrict__ pos, const double *__restrict__ F,
-                                const double *__restrict__ T, int N, double a, int wall, SrcF32 *__restrict__ out);
+                                const double *__restrict__ T, int N, double a, int wall, SrcF32 *__restrict__ out,
+                                SelfCoefs sc);
 __global__ void pack_f64_kernel(const double *__restrict__ pos, const double *__restrict__ F,
-                                const double *__restrict__ T, int N, double a, int wall, SrcF64 *__restrict__ out);
+                                const double *__restrict__ T, int N, double a, int wall, SrcF64 *__restrict__ out,
+                                SelfCoefs sc);
 
 // Number of column splits and chunk length the pair kernel uses for N targets.
 // slots: resident CTAs of the float32 kernel over the GPU (0: unknown, fixed rule).
@@ -291,8 +296,8 @@ int batch_sym_plan(BatchSymPlan &pl, int B, const int64_t *N, cudaStream_t st, b
 void batch_sym_free(BatchSymPlan &pl);
 // U_b = M_tt F_b (+ M_tr T_b) for every suspension of the plan, from packed float32 sources; active
 // masks suspensions (null: all).
-int batch_sym_apply(const BatchSymPlan &pl, cudaStream_t st, const SrcF32 *src, int64_t total, const double *pos,
-                    const double *F, const double *T, double *U, const int *active, double a, double eta);
+int batch_sym_apply(const BatchSymPlan &pl, cudaStream_t st, const SrcF32 *src, int64_t total, const double *F,
+                    const double *T, double *U, const int *active, double a, const SelfCoefs &sc);
 // d_step (optional): a device word to read the step index from instead of `step` (graph replays).
 int philox_impl(rpb_ctx *ctx, int64_t N, uint64_t seed, uint32_t step, uint32_t stream_id, uint32_t instance,
                 double *out, const unsigned int *d_step = nullptr);
