@@ -109,7 +109,7 @@ int rpb_set_periodic(rpb_ctx *ctx, double Lx, double Ly);
  * wall), rpb_lanczos_sqrt_apply and the Brownian part of rpb_ab_step / rpb_step run the iteration on
  * P M P with P = D^{-1/2} (0 where D = 0) and return g = D^{1/2} y: a sample with covariance M, but
  * not M^{1/2} W itself.  iters_out / lanczos_iters count the products with P M P, and the error
- * estimate and the stopping test are taken on y.  Allocates 2 vectors of 3 max_N doubles on the first
+ * estimate and the stopping test are taken on y.  Allocates a vector of 3 max_N doubles on the first
  * switch-on (RPB_ENOMEM if that fails; the setting is then unchanged); RPB_EINVAL for an unknown
  * kind.  Batch contexts do not use it. */
 #define RPB_PRECOND_NONE 0
@@ -183,10 +183,8 @@ int rpb_mobility_apply2(rpb_ctx *ctx, int64_t N, const double *pos, const double
  * tol <= 0, runs exactly max_iter iterations (for comparisons at equal m).  Stops early (exact
  * result) if the Krylov space becomes invariant.  max_iter must be in [1, context max_iter].
  * W = 0 gives g = 0, m = 0.  W, g: 3N; g must not alias W or pos.  iters_out, err_out: host
- * pointers (may be NULL).  Waits on the host once per iteration for the stopping test (the
- * tridiagonal step and its status copy run on a side stream of the context, ordered after the
- * iteration's work by events; short products of the next iteration may already be enqueued then and
- * are discarded at the stop), and orders the stream after that side stream before returning.  Returns RPB_ENOCONV
+ * pointers (may be NULL).  Waits on the host once per iteration for the stopping test (short products of
+ * the next iteration may already be enqueued then and are discarded at the stop).  Returns RPB_ENOCONV
  * if tol > 0 and max_iter was reached without convergence (g is still written). */
 int rpb_lanczos_sqrt_apply(rpb_ctx *ctx, int64_t N, const double *pos, const double *W, double *g,
                            double tol, int max_iter, int *iters_out, double *err_out);
@@ -245,12 +243,11 @@ int rpb_step(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, int64_t step,
 /* nsteps time steps of one suspension, as nsteps calls of rpb_step with step indices step, step + 1,
  * ... (Eq. AB or Eq. EM; Sec. II.A-C for the drift and the Lanczos square root), with the same results
  * bit for bit: the step is captured once as the body of a loop (WHILE) node of a CUDA graph and the
- * graph is launched once, running nsteps steps with no host synchronisation in between.  Each
- * Lanczos iteration after the first is a conditional node that runs only while the stopping test of
+ * graph is launched once, running nsteps steps with no host synchronisation in between.  The
+ * Lanczos iterations after the first are the body of a loop node that runs while the stopping test of
  * Sec. II.C (eps_m <= tol, or an invariant Krylov space) has not been met, decided on the device by
- * the previous iteration, so a replay runs the iterations a host-driven step would, up to max_iter;
- * for short products the tridiagonal step of an iteration runs beside the next iteration's product
- * (a graph branch; the product is unused after the last iteration).  The step index keying the noise and the first-step flag
+ * the previous iteration, so a replay runs the iterations a host-driven step would, up to max_iter.
+ * The step index keying the noise and the first-step flag
  * (step == 0 starts with an Euler-Maruyama step) advance on the device.
  *   - The work runs on a stream the context creates on first use (with a few hundred bytes of
  *     device state), ordered after the context's stream; the context's stream is ordered after the

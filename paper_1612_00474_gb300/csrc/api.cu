@@ -72,9 +72,7 @@ static int check_vec(const void *p, const char *name, bool nullable)
 
 static void free_ws(Workspace &w)
 {
-    void *dev[] = {w.src, w.partial, w.V, w.w, w.red, w.lz, w.pos_a, w.pos_b, w.pos_w, w.cells, w.selfc,
-                   w.vec_a, w.vec_b, w.vec_c, w.vec_d, w.vec_e, w.vec_f, w.vec_g,
-                   w.sym_index, w.sym_tgt, w.sym_src, w.sym64, w.src2, w.pc, w.pcx};
+    void *dev[] = {w.slab, w.sym_index, w.sym_tgt, w.sym_src, w.src2, w.pc};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (w.host_status) cudaFreeHost(w.host_status);
@@ -130,29 +128,13 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
         if ((rc = philox_impl(ctx, N, seed, step, 1u, 0u, Wt, d_step))) return rc;
         if (mobility_apply2_ok(ctx, N)) {
             // the deterministic velocity and the first Lanczos product M v_0 share one pair pass
-            // (with the preconditioner: M P v_0, scaled by P afterwards)
-            bool zero = false;
-            if ((rc = lanczos_precond_prepare(ctx, N, pos)) || (rc = lanczos_init(ctx, N, W, &zero, gr != nullptr)))
+            if ((rc = lanczos_precond_prepare(ctx, N, pos)) || (rc = lanczos_init(ctx, N, W, false, gr)) ||
+                (rc = mobility_apply2_impl(ctx, N, pos, F, T, w.vf, Un, w.w)))
                 return rc;
-            if (zero) {
-                if ((rc = mobility_apply_impl(ctx, N, pos, F, T, Un))) return rc;
-                if ((rc = cuda_fail(cudaMemsetAsync(g, 0, 3 * N * sizeof(double), ctx->stream), "zero g")))
-                    return rc;
-                conv = 1;
-            } else {
-                if (ctx->precond) {
-                    if ((rc = precond_scale(ctx, N, w.V, w.pcx, false)) ||
-                        (rc = mobility_apply2_impl(ctx, N, pos, F, T, w.pcx, Un, w.w)) ||
-                        (rc = precond_scale(ctx, N, w.w, w.w, false)))
-                        return rc;
-                } else if ((rc = mobility_apply2_impl(ctx, N, pos, F, T, w.V, Un, w.w))) {
-                    return rc;
-                }
-                lrc = lanczos_run(ctx, N, pos, g, tol, max_iter, true, &iters, &err, &conv, gr);
-            }
+            lrc = lanczos_run(ctx, N, pos, g, tol, max_iter, true, true, &iters, &err, &conv, gr);
         } else {
             if ((rc = mobility_apply_impl(ctx, N, pos, F, T, Un))) return rc;
-            lrc = lanczos_impl(ctx, N, pos, W, g, tol, max_iter, &iters, &err, &conv, gr);
+            lrc = lanczos_impl(ctx, N, pos, W, g, tol, max_iter, ctx->hook == nullptr, &iters, &err, &conv, gr);
         }
         if (lrc != RPB_OK && lrc != RPB_ENOCONV) return lrc;
         if ((rc = rfd_impl(ctx, N, pos, Wt, delta, drift, rfd == RPB_RFD_ONE_SIDED))) return rc;
@@ -241,7 +223,7 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
     if ((rc = cuda_fail(cudaGetDevice(&c->device), "cudaGetDevice")) ||
         (rc = cuda_fail(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device),
                         "cudaDeviceGetAttribute")) ||
-        (rc = pair_occupancy(c))) {
+        (rc = pair_occupancy(c)) || (rc = lanczos_setup(c))) {
         delete c;
         return rc;
     }
@@ -249,7 +231,14 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
     const size_t n3 = (size_t)3 * max_N;
     const size_t vb = n3 * sizeof(double);
     w.partial_bytes = pair_partial_bytes(max_N, c->num_sms);
-    w.red_elems = lanczos_red_elems(max_iter);
+    w.red_elems = lanczos_red_elems(max_N, max_iter);
+    // the float64 symmetric pass keeps a triangle of column partials (~3 N^2/8 bytes); used while that
+    // stays below 8 GB, the one-way kernel beyond
+    size_t sym64_bytes = 0;
+    if (p->precision == RPB_FP64) {
+        sym64_bytes = sizeof(double) * (size_t)(sym64_tgt_elems(max_N, c->num_sms) + sym64_src_elems(max_N, c->num_sms));
+        if (sym64_bytes > ((size_t)8 << 30)) sym64_bytes = 0;
+    }
     struct {
         void **ptr;
         size_t bytes;
@@ -258,6 +247,7 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
         {&w.partial, w.partial_bytes},
         {(void **)&w.V, vb * (size_t)(max_iter + 1)},
         {(void **)&w.w, vb},
+        {(void **)&w.vf, vb},
         {(void **)&w.red, w.red_elems * sizeof(double)},
         {(void **)&w.lz, lanczos_state_elems(max_iter) * sizeof(double)},
         {(void **)&w.pos_a, vb},
@@ -272,16 +262,23 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
         {(void **)&w.vec_e, vb},
         {(void **)&w.vec_f, vb},
         {(void **)&w.vec_g, vb},
+        {(void **)&w.sym64, sym64_bytes},
     };
+    // one allocation, each array on a 256-byte boundary
+    size_t total = 0;
+    for (auto &a : allocs) total += (a.bytes + 255) / 256 * 256;
+    cudaError_t e = cudaMalloc(&w.slab, total);
+    if (e != cudaSuccess) {
+        set_error("cudaMalloc of %zu bytes failed: %s", total, cudaGetErrorString(e));
+        cudaGetLastError();
+        free_ws(w);
+        delete c;
+        return RPB_ENOMEM;
+    }
+    total = 0;
     for (auto &a : allocs) {
-        cudaError_t e = cudaMalloc(a.ptr, a.bytes);
-        if (e != cudaSuccess) {
-            set_error("cudaMalloc of %zu bytes failed: %s", a.bytes, cudaGetErrorString(e));
-            cudaGetLastError();
-            free_ws(w);
-            delete c;
-            return RPB_ENOMEM;
-        }
+        *a.ptr = a.bytes ? (char *)w.slab + total : nullptr;
+        total += (a.bytes + 255) / 256 * 256;
     }
     {
         // the symmetric float32 translation-translation pass needs a triangle of column partials
@@ -312,19 +309,6 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
             }
         }
     }
-    if (p->precision == RPB_FP64) {
-        // the float64 symmetric pass keeps a triangle of column partials (~3 N^2/8 bytes); used while that
-        // stays below 8 GB too, the one-way kernel beyond
-        const size_t bytes =
-            sizeof(double) * (size_t)(sym64_tgt_elems(max_N, c->num_sms) + sym64_src_elems(max_N, c->num_sms));
-        if (bytes <= ((size_t)8 << 30) && cudaMalloc(&w.sym64, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            set_error("cudaMalloc of the symmetric-pass scratch (%zu bytes) failed", bytes);
-            free_ws(w);
-            delete c;
-            return RPB_ENOMEM;
-        }
-    }
     if (cudaMallocHost((void **)&w.host_status, 8 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         set_error("pinned host allocation failed");
@@ -349,10 +333,7 @@ int rpb_destroy(rpb_ctx *ctx)
     g_err[0] = 0;
     int rc = cuda_fail(cudaStreamSynchronize(ctx->stream), "rpb_destroy sync");
     run_free(ctx);
-    if (ctx->lz_side) cudaStreamSynchronize(ctx->lz_side);
-    if (ctx->lz_ev_a) cudaEventDestroy(ctx->lz_ev_a);
-    if (ctx->lz_ev_t) cudaEventDestroy(ctx->lz_ev_t);
-    if (ctx->lz_side) cudaStreamDestroy(ctx->lz_side);
+    if (ctx->lz_ev) cudaEventDestroy(ctx->lz_ev);
     free_ws(ctx->ws);
     delete ctx;
     return rc;
@@ -399,12 +380,10 @@ int rpb_set_preconditioner(rpb_ctx *ctx, int kind)
     Workspace &w = ctx->ws;
     if (kind != RPB_PRECOND_NONE && !w.pc) {
         const size_t vb = (size_t)3 * ctx->max_N * sizeof(double);
-        if (cudaMalloc(&w.pc, vb) != cudaSuccess || cudaMalloc(&w.pcx, vb) != cudaSuccess) {
+        if (cudaMalloc(&w.pc, vb) != cudaSuccess) {
             cudaGetLastError();
-            if (w.pc) cudaFree(w.pc);
-            if (w.pcx) cudaFree(w.pcx);
-            w.pc = w.pcx = nullptr;
-            set_error("cudaMalloc of the preconditioner vectors (2 x %zu bytes) failed", vb);
+            w.pc = nullptr;
+            set_error("cudaMalloc of the preconditioner vector (%zu bytes) failed", vb);
             return RPB_ENOMEM;
         }
     }
@@ -525,7 +504,7 @@ int rpb_lanczos_sqrt_apply(rpb_ctx *ctx, int64_t N, const double *pos, const dou
         set_error("g aliases an input");
         return RPB_EINVAL;
     }
-    return lanczos_impl(ctx, N, pos, W, g, tol, max_iter, iters_out, err_out, nullptr);
+    return lanczos_impl(ctx, N, pos, W, g, tol, max_iter, false, iters_out, err_out, nullptr);
 }
 
 int rpb_rfd_drift(rpb_ctx *ctx, int64_t N, const double *pos, const double *Wt, double delta, double *drift)

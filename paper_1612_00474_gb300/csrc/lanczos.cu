@@ -5,26 +5,51 @@
 //   c = V_{0..k}^T w ;  w -= V c                (classical Gram-Schmidt, pass 1; c_k = alpha_k)
 //   c' = V_{0..k}^T w ; w -= V c'               (pass 2: full reorthogonalisation)
 //   alpha_k = c_k + c'_k ;  beta_k = |w| ;  v_{k+1} = w / beta_k
-//   T_{k+1} = tridiag(beta, alpha, beta) -> eigenpairs (implicit QL, one warp) ->
-//   y_k = |W| Q sqrt(Lambda) Q^T e_1 ;  g_k = V_{0..k} y_k
+//   T_{k+1} = tridiag(beta, alpha, beta);  y_k = |W| T_{k+1}^{1/2} e_1 ;  g_k = V_{0..k} y_k
 //   eps_k = |y_k - (y_{k-1}, 0)| / |y_{k-1}|  (equals |g_k - g_{k-1}| / |g_{k-1}| while V stays
 //   orthonormal, which the reorthogonalisation maintains), first defined at k = 1.
 // The first subtraction of pass 1 already removes alpha_k v_k and beta_{k-1} v_{k-1}, i.e. the
 // three-term recurrence is a subset of the reorthogonalisation.
-// Reductions are two-level (per-block partials, then a fixed-order sum): results do not depend on
-// scheduling.  The stopping decision is read back once per iteration (one small device-to-host
-// copy and a stream synchronisation), or, inside a graph-replayed run, taken on the device: each
-// iteration after the first is a conditional node that the previous iteration enables.
+//
+// What bounds it: for a small suspension the chain of launches, reductions and float64 latencies of
+// an iteration, so everything after the product is one kernel: a thread-block cluster holds w in
+// registers, exchanges the partial dot products through distributed shared memory, scales v_{k+1},
+// writes it into the packed sources of the next product (whose positions stay packed), and its first
+// block does the tridiagonal step.  Separate kernels for the two projections, their dot products, the
+// scaling, the packing and the tridiagonal step were seven launches, about 25 us of an iteration at 256
+// spheres; 20 steps of 256 spheres in float64 went from 13.7 to 8.8 ms, a step of 4096 in float32 from 960 to
+// 849 us.  Larger suspensions spread the same steps over the GPU (gs.cuh).
+// Reductions are summed in a fixed order: results do not depend on scheduling.  The stopping decision
+// is written to pinned host memory, or, inside a graph-replayed run, taken on the device: the
+// iterations after the first are the body of a loop node that each iteration keeps running or ends.
+#include <cooperative_groups.h>
+
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <mutex>
 
-#include "lanczos_math.cuh"
+#include "gs.cuh"
 #include "pair_math.cuh"
 
 namespace rpb {
 
+namespace cg = cooperative_groups;
+
 constexpr int kBlasThreads = 256;
 
+// Spheres of a chunk in the kernels for larger suspensions: small enough to fill the GPU, at most
+// 256 partial sums per dot product up to 65536 spheres.
+static int64_t gs_chunk(int64_t N)
+{
+    return N > 32768 ? 256 : (N > 12288 ? 128 : 64);
+}
+
+size_t lanczos_red_elems(int64_t max_N, int max_iter)
+{
+    // partials of the dot products of both passes and of a norm: 12288/64, 32768/128 or N/256 chunks
+    return (size_t)(2 * max_iter + 1) * (size_t)std::max<int64_t>(256, (max_N + 255) / 256);
+}
 
 size_t lanczos_state_elems(int max_iter)
 {
@@ -33,12 +58,9 @@ size_t lanczos_state_elems(int max_iter)
 
 int upload_sqrt_nodes(double *nodes, cudaStream_t st)
 {
-    static const SqrtNodes host = sqrt_nodes();
-    int rc;
-    if ((rc = cuda_fail(cudaMemcpyAsync(nodes, host.s, sizeof(host.s), cudaMemcpyHostToDevice, st), "square root nodes")))
-        return rc;
-    return cuda_fail(cudaMemcpyAsync(nodes + kSqrtNodes, host.w, sizeof(host.w), cudaMemcpyHostToDevice, st),
-                     "square root weights");
+    static const SqrtNodes host = sqrt_nodes();  // shifts, then weights
+    static_assert(sizeof(host) == 2 * kSqrtNodes * sizeof(double), "contiguous");
+    return cuda_fail(cudaMemcpyAsync(nodes, &host, sizeof(host), cudaMemcpyHostToDevice, st), "square root nodes");
 }
 
 int lanczos_upload(double *lz, int max_iter, cudaStream_t st)
@@ -55,141 +77,238 @@ static int blas_grid(int64_t n, int num_sms)
     return (int)g;
 }
 
-size_t lanczos_red_elems(int max_iter)
-{
-    // (max_iter + 1) dot products + one norm, each with up to 2 * SMs partials (SM count <= 1024)
-    return (size_t)(max_iter + 3) * 2048;
-}
-
-__device__ __forceinline__ double block_sum(double v, double *sh)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r += sh[k];
+// What the kernels of an iteration work on.
+struct GsArgs {
+    double *V;         // Krylov basis, rows of ld
+    size_t ld;
+    int64_t N;
+    double *w;         // the product M v_k (with the preconditioner, before its second scaling)
+    const double *W;   // initialisation: the vector whose square root product is wanted
+    double *vf;        // the load of the next product: v_{k+1}, times P with the preconditioner
+    const double *P;   // preconditioner (or null)
+    const double *sc;  // s_i (SelfCoefs), for the packed sources
+    void *src;         // packed sources whose loads the next product reads (null: it packs itself)
+    int fp64;
+    double *lz;
+    LzLayout L;
+    double *red, *red2, *norm2;  // partials (larger suspensions)
+    double tol;
+    int k, max_iter;
+    double *hs;        // pinned host copy of the status words (null: none)
+    RunState *rs;      // graph-replayed run: k and the loop's state live here
+    cudaGraphConditionalHandle loop;
+    __device__ __forceinline__ int iter() const { return rs ? rs->k : k; }
+    // v_{k+1} (row r = c N + i, i a sphere of component c) into the basis and the next product's load
+    __device__ __forceinline__ void store(double *v, int64_t r, double x) const
+    {
+        v[r] = x;
+        const double f = P ? x * P[r] : x;
+        vf[r] = f;
+        if (!src) return;
+        const int c = r < N ? 0 : (r < 2 * N ? 1 : 2);
+        const int64_t i = r - c * N;
+        const double s = sc[i] * f;
+        if (fp64)
+            reinterpret_cast<double *>((SrcF64 *)src + i)[3 + c] = s;
+        else
+            reinterpret_cast<float *>((SrcF32 *)src + i)[5 + c] = (float)s;
     }
-    __syncthreads();
-    return r;  // valid in thread 0
-}
-
-// Sum of n partials by one warp in a fixed order (lane-strided sums, then a butterfly); every lane
-// returns the total.
-__device__ __forceinline__ double warp_sum_partials(const double *__restrict__ p, int n)
-{
-    const int lane = threadIdx.x & 31;
-    double v = 0.0;
-    for (int b = lane; b < n; b += 32) v += p[b];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// red[k * G + b] = sum over block b's rows of V[k][r] * w[r], k = 0 .. nvec-1 (grid = (G, nvec)).
-__global__ void __launch_bounds__(kBlasThreads) dots_kernel(const double *__restrict__ V, size_t ld, int64_t n,
-                                                             const double *__restrict__ w, double *__restrict__ red)
-{
-    __shared__ double sh[kBlasThreads / 32];
-    const int G = gridDim.x;
-    const double *v = V + (size_t)blockIdx.y * ld;
-    double acc = 0.0;
-    for (int64_t r = (int64_t)blockIdx.x * kBlasThreads + threadIdx.x; r < n; r += (int64_t)G * kBlasThreads)
-        acc = fma(v[r], w[r], acc);
-    acc = block_sum(acc, sh);
-    if (threadIdx.x == 0) red[(size_t)blockIdx.y * G + blockIdx.x] = acc;
-}
-
-// Reduce the dots partials for k = 0 .. nvec-1 (fixed order), then w -= sum_k coef_k V[k].
-// Block 0 stores the coefficients in coef_out.  With norm_out != null also writes per-block partial
-// sums of the updated w^2 to norm_out[b].
-__global__ void __launch_bounds__(kBlasThreads) project_out_kernel(const double *__restrict__ V, size_t ld, int64_t n,
-                                                                    int nvec, const double *__restrict__ red, int Gred,
-                                                                    double *__restrict__ w,
-                                                                    double *__restrict__ coef_out,
-                                                                    double *__restrict__ norm_out)
-{
-    __shared__ double coef[kMaxIter + 1];
-    __shared__ double sh[kBlasThreads / 32];
-    const int warp = threadIdx.x >> 5;
-    for (int k = warp; k < nvec; k += kBlasThreads / 32) {
-        const double s = warp_sum_partials(red + (size_t)k * Gred, Gred);
-        if ((threadIdx.x & 31) == 0) {
-            coef[k] = s;
-            if (blockIdx.x == 0) coef_out[k] = s;
-        }
-    }
-    __syncthreads();
-    double acc = 0.0;
-    for (int64_t r = (int64_t)blockIdx.x * kBlasThreads + threadIdx.x; r < n; r += (int64_t)gridDim.x * kBlasThreads) {
-        double x = w[r];
-        for (int k = 0; k < nvec; ++k) x -= coef[k] * V[(size_t)k * ld + r];
-        w[r] = x;
-        acc = fma(x, x, acc);
-    }
-    if (norm_out) {
-        acc = block_sum(acc, sh);
-        if (threadIdx.x == 0) norm_out[blockIdx.x] = acc;
-    }
-}
-
-// v[r] = w[r] * status[idx]
-__global__ void scale_kernel(const double *__restrict__ w, int64_t n, const double *__restrict__ status, int idx,
-                             double *__restrict__ v)
-{
-    const double s = status[idx];
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-        v[r] = w[r] * s;
-}
-
-// v[r] = w[r] / |w|, |w|^2 summed from the norm partials by one warp in the fixed order the
-// tridiagonal kernel uses for beta_k (so 1/|w| is bitwise its 1/beta_k).
-__global__ void scale_norm_kernel(const double *__restrict__ w, int64_t n, const double *__restrict__ red_norm,
-                                  int Gred, double *__restrict__ v)
-{
-    __shared__ double inv;
-    if (threadIdx.x < 32) {
-        const double bn = warp_sum_partials(red_norm, Gred);
-        if (threadIdx.x == 0) inv = 1.0 / sqrt(bn);
-    }
-    __syncthreads();
-    const double s = inv;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-        v[r] = w[r] * s;
-}
-
-// |W| from its squared-norm partials.
-__global__ void norm_init_kernel(const double *__restrict__ red, int G, double *__restrict__ status)
-{
-    const double s = warp_sum_partials(red, G);  // launched as one warp
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+    // status words of a new Krylov space, |W|^2 = s
+    __device__ __forceinline__ void begin(double s) const
+    {
+        double *status = lz + L.status;
         const double nw = sqrt(s);
         status[ST_NW] = nw;
         status[ST_INV_NW] = nw > 0.0 ? 1.0 / nw : 0.0;
         status[ST_EPS] = -1.0;
         status[ST_STOP] = 0.0;
         status[ST_BREAK] = 0.0;
+        if (rs) rs->k = 0;
+    }
+    // after the tridiagonal step of iteration k, by the thread that wrote the status words
+    __device__ __forceinline__ void end(int k) const
+    {
+        const double *status = lz + L.status;
+        if (hs)
+            for (int q = 0; q < 8; ++q) hs[q] = status[q];
+        if (rs) {
+            rs->m = k + 1;
+            rs->k = k + 1;
+            if (k > 0) rs->loops += 1ull;
+            if (max_iter > 1) cudaGraphSetConditional(loop, status[ST_STOP] == 0.0 && k + 1 < max_iter ? 1u : 0u);
+        }
+    }
+};
+// record layout that GsArgs::store writes into: floats 5 .. 7 of SrcF32, doubles 3 .. 5 of SrcF64 hold s F
+static_assert(sizeof(SrcF32) == 48 && sizeof(SrcF64) == 80, "packed source records");
+
+// ------------------------------------------------------------------ small suspensions: one cluster
+constexpr int kGsCluster = 16;  // blocks of the cluster at most (8 where the device schedules no 16)
+
+// coef_j = sum over the cluster's blocks of their part[j], four threads per j; ends with a block barrier
+__device__ __forceinline__ void cluster_coefs(cg::cluster_group &cl, double *part, int nvec, double *coef)
+{
+    const int j = threadIdx.x >> 2, q = threadIdx.x & 3, n = (int)cl.num_blocks();
+    double s = 0.0;
+    if (j < nvec)
+        for (int r = q; r < n; r += 4) s += cl.map_shared_rank(part, r)[j];
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if (q == 0 && j < nvec) coef[j] = s;
+    __syncthreads();
+}
+
+// One cluster, block r holding spheres [r per, (r + 1) per): Gram-Schmidt on w, v_{k+1}, and the tridiagonal
+// step in the first block.  init: v_0 = W / |W| instead.
+__global__ void __launch_bounds__(kGsThreads) gs_cluster_kernel(GsArgs A, int per, int init)
+{
+    static_assert(kGsThreads >= 4 * kMaxIter, "four threads per coefficient");
+    __shared__ double sh[kGsWarps][kMaxIter + 8];
+    __shared__ double part[2][kMaxIter], norm[1], coef[kMaxIter];
+    __shared__ TailShared ts;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+    const int k = init ? -1 : A.iter();
+    const int first = rank * per;
+    const int left = (int)A.N - first;
+    int64_t row[kGsRows];
+    double x[kGsRows];
+    gs_rows(GsSpan{first, A.N, max(0, min(per, left))}, row);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) {
+        x[u] = row[u] < 0 ? 0.0 : (init ? A.W[row[u]] : A.w[row[u]]);
+        if (A.P && !init && row[u] >= 0) x[u] *= A.P[row[u]];
+    }
+    for (int pass = 0; pass < 2 && !init; ++pass) {
+        const double s = gs_dots(A.V, A.ld, k + 1, row, x, sh);
+        if (tid <= k) part[pass][tid] = s;
+        cl.sync();
+        cluster_coefs(cl, part[pass], k + 1, coef);
+        if (rank == 0 && tid <= k) A.lz[(pass ? A.L.c2 : A.L.c1) + tid] = coef[tid];
+        gs_project(A.V, A.ld, k + 1, row, coef, x);
+    }
+    double s = 0.0;
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) s = fma(x[u], x[u], s);
+    s = gs_block_sum(s, sh[0]);
+    if (tid == 0) norm[0] = s;
+    cl.sync();
+    const int lane = tid & 31;
+    double bn = lane < (int)cl.num_blocks() ? cl.map_shared_rank(norm, lane)[0] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) bn += __shfl_xor_sync(0xffffffffu, bn, o);
+    cl.barrier_arrive();  // nothing of another block's memory is read from here on
+    const double nb = sqrt(bn);
+    const double inv = init && !(nb > 0.0) ? 0.0 : 1.0 / nb;
+    double *v = A.V + (size_t)(k + 1) * A.ld;
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u)
+        if (row[u] >= 0) A.store(v, row[u], x[u] * inv);
+    if (rank == 0) {
+        if (init) {
+            if (tid == 0) A.begin(bn);
+        } else if (tid < kTailThreads) {
+            // (c1 and c2 of the last vector were stored by other threads of this block, before a barrier)
+            lanczos_tail_block(A.lz, A.L, k, A.tol, A.lz[A.L.c1 + k] + A.lz[A.L.c2 + k], nb, A.lz + A.L.total, ts);
+            if (tid == 0) A.end(k);
+        }
+    }
+    cl.barrier_wait();
+}
+
+// ------------------------------------------------------------------ larger suspensions: chunks over the GPU
+__device__ __forceinline__ void gs_chunk_rows(const GsArgs &A, int chunk, int64_t (&row)[kGsRows])
+{
+    const int64_t first = (int64_t)blockIdx.x * chunk;
+    gs_rows(GsSpan{first, A.N, (int)min((int64_t)chunk, A.N - first)}, row);
+}
+
+// partials of <V_j, w>, j <= k (w scaled by the preconditioner first)
+__global__ void __launch_bounds__(kGsThreads) gs_dots_kernel(GsArgs A, int chunk)
+{
+    __shared__ double sh[kGsWarps][kMaxIter + 8];
+    const int k = A.iter();
+    int64_t row[kGsRows];
+    double x[kGsRows];
+    gs_chunk_rows(A, chunk, row);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) {
+        x[u] = row[u] >= 0 ? A.w[row[u]] : 0.0;
+        if (A.P && row[u] >= 0) A.w[row[u]] = x[u] *= A.P[row[u]];
+    }
+    const double s = gs_dots(A.V, A.ld, k + 1, row, x, sh);
+    if (threadIdx.x <= k) A.red[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s;
+}
+
+// w -= V c; pass 0: then the dot products of pass 2; pass 1: then the partials of |w|^2
+__global__ void __launch_bounds__(kGsThreads) gs_project_kernel(GsArgs A, int chunk, int pass)
+{
+    __shared__ double sh[kGsWarps][kMaxIter + 8];
+    __shared__ double coef[kMaxIter];
+    const int k = A.iter(), tid = threadIdx.x;
+    int64_t row[kGsRows];
+    double x[kGsRows];
+    gs_chunk_rows(A, chunk, row);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) x[u] = row[u] >= 0 ? A.w[row[u]] : 0.0;
+    gs_coefs(pass ? A.red2 : A.red, gridDim.x, gridDim.x, k + 1, coef);
+    if (blockIdx.x == 0 && tid <= k) A.lz[(pass ? A.L.c2 : A.L.c1) + tid] = coef[tid];
+    gs_project(A.V, A.ld, k + 1, row, coef, x);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u)
+        if (row[u] >= 0) A.w[row[u]] = x[u];
+    if (pass == 0) {
+        const double s = gs_dots(A.V, A.ld, k + 1, row, x, sh);
+        if (tid <= k) A.red2[(size_t)tid * gridDim.x + blockIdx.x] = s;
+    } else {
+        double s = 0.0;
+#pragma unroll
+        for (int u = 0; u < kGsRows; ++u) s = fma(x[u], x[u], s);
+        s = gs_block_sum(s, sh[0]);
+        if (tid == 0) A.norm2[blockIdx.x] = s;
     }
 }
 
-// The tridiagonal step for the single Krylov space (see lanczos_tail_block).  Inside a replayed graph
-// (runs != null) thread 0 then counts this run of iteration k, records m = k + 1 and lets the
-// conditional node of iteration k + 1 run only if the iteration has not stopped.
-__global__ void __launch_bounds__(kTailThreads) lanczos_tail_kernel(double *__restrict__ lz, LzLayout L, int k,
-                                                                    double tol, const double *__restrict__ red_norm,
-                                                                    int Gred, cudaGraphConditionalHandle next = 0ull,
-                                                                    int has_next = 0,
-                                                                    unsigned long long *__restrict__ runs = nullptr,
-                                                                    int *__restrict__ m_out = nullptr)
+// partials of |W|^2
+__global__ void __launch_bounds__(kGsThreads) gs_norm_kernel(GsArgs A, int chunk)
 {
-    __shared__ TailShared sh;
-    const double bn = warp_sum_partials(red_norm, Gred);  // the same value in every thread
-    lanczos_tail_block(lz, L, k, tol, lz[L.c1 + k] + lz[L.c2 + k], sqrt(bn), lz + L.total, sh);
-    if (runs && threadIdx.x == 0) {  // thread 0 wrote the status words
-        *runs += 1ull;
-        *m_out = k + 1;
-        if (has_next) cudaGraphSetConditional(next, lz[L.status + ST_STOP] == 0.0 ? 1u : 0u);
-    }
+    __shared__ double sh[kGsWarps];
+    int64_t row[kGsRows];
+    gs_chunk_rows(A, chunk, row);
+    double s = 0.0;
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u)
+        if (row[u] >= 0) s = fma(A.W[row[u]], A.W[row[u]], s);
+    s = gs_block_sum(s, sh);
+    if (threadIdx.x == 0) A.norm2[blockIdx.x] = s;
+}
+
+// v_{k+1} = w / |w| (init: v_0 = W / |W|)
+__global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(GsArgs A, int chunk, int init)
+{
+    __shared__ double bn;
+    gs_coefs(A.norm2, 0, gridDim.x, 1, &bn);
+    const double nb = sqrt(bn);
+    const double inv = init && !(nb > 0.0) ? 0.0 : 1.0 / nb;
+    const int k = init ? -1 : A.iter();
+    int64_t row[kGsRows];
+    gs_chunk_rows(A, chunk, row);
+    double *v = A.V + (size_t)(k + 1) * A.ld;
+    const double *w = init ? A.W : A.w;
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u)
+        if (row[u] >= 0) A.store(v, row[u], w[row[u]] * inv);
+    if (init && blockIdx.x == 0 && threadIdx.x == 0) A.begin(bn);
+}
+
+__global__ void __launch_bounds__(kTailThreads) lanczos_tail_kernel(GsArgs A, int parts)
+{
+    __shared__ TailShared ts;
+    const int k = A.iter();
+    double bn = 0.0;  // the same in every warp
+    for (int b = threadIdx.x & 31; b < parts; b += 32) bn += A.norm2[b];
+    for (int o = 16; o > 0; o >>= 1) bn += __shfl_xor_sync(0xffffffffu, bn, o);
+    lanczos_tail_block(A.lz, A.L, k, A.tol, A.lz[A.L.c1 + k] + A.lz[A.L.c2 + k], sqrt(bn), A.lz + A.L.total, ts);
+    if (threadIdx.x == 0) A.end(k);
 }
 
 // g[r] = sum_{k < m} y[k] V[k][r]   (y already carries |W|); d_m (optional): read m from the device
@@ -254,7 +373,7 @@ int lanczos_precond_prepare(rpb_ctx *ctx, int64_t N, const double *pos)
     return cuda_fail(cudaGetLastError(), "preconditioner");
 }
 
-int precond_scale(rpb_ctx *ctx, int64_t N, const double *x, double *out, bool inverse)
+static int precond_scale(rpb_ctx *ctx, int64_t N, const double *x, double *out, bool inverse)
 {
     precond_scale_kernel<<<blas_grid(3 * N, ctx->num_sms), kBlasThreads, 0, ctx->stream>>>(x, ctx->ws.pc, 3 * N,
                                                                                          inverse ? 1 : 0, out);
@@ -262,221 +381,212 @@ int precond_scale(rpb_ctx *ctx, int64_t N, const double *x, double *out, bool in
     return cuda_fail(cudaGetLastError(), "preconditioner scale");
 }
 
-int lanczos_init(rpb_ctx *ctx, int64_t N, const double *W, bool *nw_zero, bool graph)
+// Blocks of the cluster that the device can schedule: 16 (beyond the portable 8) where it offers them,
+// asked once per device.
+static int query_cluster()
 {
-    cudaStream_t st = ctx->stream;
-    const int64_t n = 3 * N;
-    const LzLayout L(ctx->max_iter);
-    double *status = ctx->ws.lz + L.status;
-    double *red = ctx->ws.red;
-    double *hs = ctx->ws.host_status;
-    const int G = blas_grid(n, ctx->num_sms);
-    int rc;
-    // |W| and v_0 = W / |W|
-    dots_kernel<<<dim3(G, 1), kBlasThreads, 0, st>>>(W, 0, n, W, red);
-    norm_init_kernel<<<1, 32, 0, st>>>(red, G, status);
-    scale_kernel<<<G, kBlasThreads, 0, st>>>(W, n, status, ST_INV_NW, ctx->ws.V);
-    count_launches(3);
-    if (graph) {
-        *nw_zero = false;
-        return cuda_fail(cudaGetLastError(), "lanczos init");
+    int n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kGsCluster);
+    cfg.blockDim = dim3(kGsThreads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kGsCluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(gs_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, gs_cluster_kernel, &cfg) == cudaSuccess && n >= 1)
+        return kGsCluster;
+    cudaGetLastError();
+    return 8;
+}
+
+int lanczos_setup(rpb_ctx *ctx)
+{
+    static std::mutex mu;
+    static int blocks[64] = {};  // per device ordinal, 0: not asked yet
+    std::lock_guard<std::mutex> lock(mu);
+    if (ctx->device < 0 || ctx->device >= 64) {
+        ctx->gs_cluster = query_cluster();
+        return RPB_OK;
     }
-    if ((rc = cuda_fail(cudaMemcpyAsync(hs, status, 8 * sizeof(double), cudaMemcpyDeviceToHost, st), "status copy")))
-        return rc;
-    if ((rc = cuda_fail(cudaStreamSynchronize(st), "lanczos init"))) return rc;
-    *nw_zero = hs[ST_NW] == 0.0;
+    if (!blocks[ctx->device]) blocks[ctx->device] = query_cluster();
+    ctx->gs_cluster = blocks[ctx->device];
     return RPB_OK;
 }
 
-int lanczos_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *W, double *g, double tol, int max_iter,
-                 int *iters_out, double *err_out, int *converged_out, LzGraph *gr)
+// Blocks of the cluster for N spheres, 0 for the kernels over the whole GPU.  Up to kGsChunk spheres a
+// block; 64 and fewer for a small suspension, whose time is the latency of the steps and not their
+// arithmetic.
+static int gs_cluster_blocks(const rpb_ctx *ctx, int64_t N)
 {
-    bool zero = false;
-    int rc;
-    if ((rc = lanczos_precond_prepare(ctx, N, pos)) || (rc = lanczos_init(ctx, N, W, &zero, gr != nullptr))) return rc;
-    if (zero) {
-        if ((rc = cuda_fail(cudaMemsetAsync(g, 0, 3 * N * sizeof(double), ctx->stream), "zero g"))) return rc;
-        if (iters_out) *iters_out = 0;
-        if (err_out) *err_out = -1.0;
-        if (converged_out) *converged_out = 1;
-        return RPB_OK;
-    }
-    return lanczos_run(ctx, N, pos, g, tol, max_iter, false, iters_out, err_out, converged_out, gr);
+    if (N <= 32) return 1;
+    if (N <= 512) return 8;
+    return N <= (int64_t)ctx->gs_cluster * kGsChunk ? ctx->gs_cluster : 0;
 }
 
-// w = M v (with the preconditioner: P M P v), on the context's stream
-static int lanczos_product(rpb_ctx *ctx, int64_t N, const double *pos, const double *v, double *w)
+static GsArgs gs_args(rpb_ctx *ctx, int64_t N, bool pack, LzGraph *gr)
+{
+    const Workspace &w = ctx->ws;
+    GsArgs A = {w.V, (size_t)3 * ctx->max_N, N, w.w, nullptr, w.vf, ctx->precond ? w.pc : nullptr, w.selfc,
+                pack ? w.src : nullptr, ctx->p.precision == RPB_FP64, w.lz, LzLayout(ctx->max_iter)};
+    const size_t nch = (size_t)((N + gs_chunk(N) - 1) / gs_chunk(N));
+    A.red = w.red;
+    A.red2 = A.red + (size_t)ctx->max_iter * nch;
+    A.norm2 = A.red2 + (size_t)ctx->max_iter * nch;
+    A.tol = 0.0;
+    A.k = 0;
+    A.max_iter = 1;
+    A.hs = nullptr;
+    A.rs = gr ? gr->state : nullptr;
+    A.loop = 0;
+    return A;
+}
+
+static int gs_cluster_launch(cudaStream_t st, const GsArgs &A, int blocks, int init)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kGsThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    count_launches(1);
+    return cuda_fail(cudaLaunchKernelEx(&cfg, gs_cluster_kernel, A, (int)((A.N + blocks - 1) / blocks), init),
+                     "lanczos cluster kernel");
+}
+
+// Everything of an iteration after its product, on the context's stream.
+static int gs_iteration(rpb_ctx *ctx, const GsArgs &A)
+{
+    cudaStream_t st = ctx->stream;
+    if (const int blocks = gs_cluster_blocks(ctx, A.N)) return gs_cluster_launch(st, A, blocks, 0);
+    const int chunk = (int)gs_chunk(A.N);
+    const int nch = (int)((A.N + chunk - 1) / chunk);
+    gs_dots_kernel<<<nch, kGsThreads, 0, st>>>(A, chunk);
+    gs_project_kernel<<<nch, kGsThreads, 0, st>>>(A, chunk, 0);
+    gs_project_kernel<<<nch, kGsThreads, 0, st>>>(A, chunk, 1);
+    gs_scale_kernel<<<nch, kGsThreads, 0, st>>>(A, chunk, 0);
+    lanczos_tail_kernel<<<1, kTailThreads, 0, st>>>(A, nch);
+    count_launches(5);
+    return cuda_fail(cudaGetLastError(), "lanczos kernels");
+}
+
+int lanczos_init(rpb_ctx *ctx, int64_t N, const double *W, bool packed, LzGraph *gr)
+{
+    cudaStream_t st = ctx->stream;
+    GsArgs A = gs_args(ctx, N, packed, gr);
+    A.W = W;
+    if (const int blocks = gs_cluster_blocks(ctx, N)) return gs_cluster_launch(st, A, blocks, 1);
+    const int chunk = (int)gs_chunk(N);
+    const int nch = (int)((N + chunk - 1) / chunk);
+    gs_norm_kernel<<<nch, kGsThreads, 0, st>>>(A, chunk);
+    gs_scale_kernel<<<nch, kGsThreads, 0, st>>>(A, chunk, 1);
+    count_launches(2);
+    return cuda_fail(cudaGetLastError(), "lanczos init");
+}
+
+int lanczos_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *W, double *g, double tol, int max_iter,
+                 bool packed, int *iters_out, double *err_out, int *converged_out, LzGraph *gr)
 {
     int rc;
-    if (!ctx->precond) return mobility_apply_impl(ctx, N, pos, v, nullptr, w);
-    if ((rc = precond_scale(ctx, N, v, ctx->ws.pcx, false)) ||
-        (rc = mobility_apply_impl(ctx, N, pos, ctx->ws.pcx, nullptr, w)))
-        return rc;
-    return precond_scale(ctx, N, w, w, false);
+    if ((rc = lanczos_precond_prepare(ctx, N, pos)) || (rc = lanczos_init(ctx, N, W, packed, gr))) return rc;
+    return lanczos_run(ctx, N, pos, g, tol, max_iter, false, packed, iters_out, err_out, converged_out, gr);
 }
 
 int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double tol, int max_iter, bool first_done,
-                int *iters_out, double *err_out, int *converged_out, LzGraph *gr)
+                bool packed, int *iters_out, double *err_out, int *converged_out, LzGraph *gr)
 {
     const cudaStream_t main_st = ctx->stream;
     const int64_t n = 3 * N;
-    const size_t ld = (size_t)3 * ctx->max_N;
-    const LzLayout L(ctx->max_iter);
-    double *lz = ctx->ws.lz;
-    double *status = lz + L.status;
-    double *red = ctx->ws.red;
-    double *V = ctx->ws.V;
-    double *w = ctx->ws.w;
-    double *hs = ctx->ws.host_status;
-    const int G = blas_grid(n, ctx->num_sms);
-    double *red_norm = red + (size_t)(ctx->max_iter + 1) * G;
+    Workspace &w = ctx->ws;
+    const double *hs = w.host_status;
     int rc;
     int m = 0;
     bool stopped = false;
     double eps = -1.0;
-    if (gr) {  // one conditional handle per iteration after the first, on the graph being captured
-        cudaStreamCaptureStatus cs;
-        cudaGraph_t cg = nullptr;
-        if ((rc = cuda_fail(cudaStreamGetCaptureInfo(main_st, &cs, nullptr, &cg, nullptr, nullptr, nullptr),
-                            "capture info")))
-            return rc;
-        CondSet cs_all = {};
-        for (int k = 1; k < max_iter; ++k) {
-            gr->iter_launches[k] = 0;
-            if ((rc = cuda_fail(cudaGraphConditionalHandleCreate(&gr->hnd[k], cg, 0u, cudaGraphCondAssignDefault),
+    // after the first product the positions are packed and each iteration writes the next load beside
+    // them (unless the products are the caller's)
+    const bool pk = ctx->hook == nullptr;
+    GsArgs A = gs_args(ctx, N, pk, gr);
+    A.tol = tol;
+    A.max_iter = max_iter;
+    auto product = [&](bool is_packed) {
+        return mobility_apply_impl(ctx, N, pos, w.vf, nullptr, w.w, is_packed && pk);
+    };
+    if (gr) {
+        // iteration 0 with the step; the others are the body of a loop node that an iteration's
+        // tridiagonal step keeps running (its condition is set in every step before the node is met)
+        gr->body_launches = 0;
+        if (max_iter > 1) {
+            cudaStreamCaptureStatus cs;
+            cudaGraph_t cg_ = nullptr;
+            if ((rc = cuda_fail(cudaStreamGetCaptureInfo(main_st, &cs, nullptr, &cg_, nullptr, nullptr, nullptr),
+                                "capture info")) ||
+                (rc = cuda_fail(cudaGraphConditionalHandleCreate(&A.loop, cg_, 0u, cudaGraphCondAssignDefault),
                                 "conditional handle")))
                 return rc;
-            cs_all.h[k - 1] = gr->hnd[k];
         }
-        // the iterations' conditions start at 0 in every step (the graph may run the step in a loop)
+        if ((!first_done && (rc = product(packed))) || (rc = gs_iteration(ctx, A))) return rc;
         if (max_iter > 1) {
-            graph_reset_conds_kernel<<<1, 64, 0, main_st>>>(cs_all, max_iter - 1);
-            count_launches(1);
-        }
-    }
-    // Host-driven: the tridiagonal step of iteration k runs on a side stream while the context's
-    // stream goes on with v_{k+1} = w / |w| and, for short products, the product M v_{k+1} (discarded if
-    // iteration k stopped); the norm partials alternate between two buffers so that the side stream's
-    // reads never meet the next iteration's writes.
-    if (!gr && !ctx->lz_side) {
-        if ((rc = cuda_fail(cudaStreamCreateWithFlags(&ctx->lz_side, cudaStreamNonBlocking), "lanczos side stream")) ||
-            (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->lz_ev_a, cudaEventDisableTiming), "lanczos event")) ||
-            (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->lz_ev_t, cudaEventDisableTiming), "lanczos event")))
-            return rc;
-    }
-    // Speculate only where a product is short: one product is wasted per solve (after the stopping
-    // iteration) and about one tridiagonal step (~55 us) is saved per iteration; the estimate uses the
-    // measured per-pair times of the symmetric float64 and float32 kernels on this part.
-    const double t_product = (ctx->Lx > 0.0 ? 9.0 : 1.0) * (double)N * (double)N *
-                             (ctx->p.precision == RPB_FP64 ? 8e-11 : 1.3e-12);
-    const bool speculate = t_product < 3e-4;
-    bool have_product = false;  // w already holds M v_k (the speculative product of iteration k - 1)
-    for (int k = 0; k < max_iter; ++k) {
-        if (!gr) {
-            const double *vk = V + (size_t)k * ld;
-            double *rn = red + (size_t)(ctx->max_iter + 1 + (k & 1)) * G;
-            rc = RPB_OK;
-            if (!(k == 0 && first_done) && !have_product) rc = lanczos_product(ctx, N, pos, vk, w);
-            have_product = false;
-            if (rc) return rc;
-            const int nv = k + 1;
-            dots_kernel<<<dim3(G, nv), kBlasThreads, 0, main_st>>>(V, ld, n, w, red);
-            project_out_kernel<<<G, kBlasThreads, 0, main_st>>>(V, ld, n, nv, red, G, w, lz + L.c1, nullptr);
-            dots_kernel<<<dim3(G, nv), kBlasThreads, 0, main_st>>>(V, ld, n, w, red);
-            project_out_kernel<<<G, kBlasThreads, 0, main_st>>>(V, ld, n, nv, red, G, w, lz + L.c2, rn);
-            if ((rc = cuda_fail(cudaEventRecord(ctx->lz_ev_a, main_st), "event record")) ||
-                (rc = cuda_fail(cudaStreamWaitEvent(ctx->lz_side, ctx->lz_ev_a, 0), "stream wait")))
-                return rc;
-            lanczos_tail_kernel<<<1, kTailThreads, 0, ctx->lz_side>>>(lz, L, k, tol, rn, G);
-            count_launches(5);
-            if ((rc = cuda_fail(cudaMemcpyAsync(hs, status, 8 * sizeof(double), cudaMemcpyDeviceToHost, ctx->lz_side),
-                                "status copy")) ||
-                (rc = cuda_fail(cudaEventRecord(ctx->lz_ev_t, ctx->lz_side), "event record")))
-                return rc;
-            if (k + 1 < max_iter) {  // v_{k+1} (unused if this iteration stops)
-                scale_norm_kernel<<<G, kBlasThreads, 0, main_st>>>(w, n, rn, G, V + (size_t)(k + 1) * ld);
-                count_launches(1);
-                if (speculate) {
-                    if ((rc = lanczos_product(ctx, N, pos, V + (size_t)(k + 1) * ld, w))) return rc;
-                    have_product = true;
-                }
-            }
-            if ((rc = cuda_fail(cudaEventSynchronize(ctx->lz_ev_t), "lanczos iteration"))) return rc;
-            m = k + 1;
-            eps = hs[ST_EPS];
-            if (hs[ST_STOP] != 0.0) {
-                stopped = true;
-                break;
-            }
-            continue;
-        }
-        const bool cond = gr && k >= 1;
-        if (cond) {
-            if ((rc = graph_begin_if(main_st, gr->body, gr->hnd[k]))) return rc;
+            if ((rc = graph_begin_cond(main_st, gr->body, A.loop, cudaGraphCondTypeWhile))) return rc;
             ctx->stream = gr->body;
-        }
-        cudaStream_t st = ctx->stream;
-        const uint64_t before = rpb_launch_count();
-        const double *vk = V + (size_t)k * ld;
-        // graph branch: iteration k's tridiagonal step beside v_{k+1} and its product M v_{k+1}, which
-        // the body of iteration k + 1 then finds in w (discarded if iteration k stopped)
-        cudaStream_t side = k == 0 ? gr->side0 : gr->side;
-        const bool branch = speculate && gr->side0 != nullptr && gr->side != nullptr;
-        rc = RPB_OK;
-        if (!(k == 0 && first_done) && !(branch && k >= 1)) rc = lanczos_product(ctx, N, pos, vk, w);
-        if (!rc) {
-            const int nv = k + 1;
-            dots_kernel<<<dim3(G, nv), kBlasThreads, 0, st>>>(V, ld, n, w, red);
-            project_out_kernel<<<G, kBlasThreads, 0, st>>>(V, ld, n, nv, red, G, w, lz + L.c1, nullptr);
-            dots_kernel<<<dim3(G, nv), kBlasThreads, 0, st>>>(V, ld, n, w, red);
-            project_out_kernel<<<G, kBlasThreads, 0, st>>>(V, ld, n, nv, red, G, w, lz + L.c2, red_norm);
-            count_launches(4);
-            const bool has_next = k + 1 < max_iter;
-            cudaStream_t tail_st = st;
-            if (branch && has_next &&
-                !(rc = cuda_fail(cudaEventRecord(gr->ev_fork, st), "event record")) &&
-                !(rc = cuda_fail(cudaStreamWaitEvent(side, gr->ev_fork, 0), "stream wait")))
-                tail_st = side;
-            if (!rc) {
-                lanczos_tail_kernel<<<1, kTailThreads, 0, tail_st>>>(lz, L, k, tol, red_norm, G,
-                                                           has_next ? gr->hnd[k + 1] : 0ull, has_next ? 1 : 0,
-                                                           gr->state->iter_runs + k, &gr->state->m);
-                count_launches(1);
-            }
-            if (!rc && has_next) {  // v_{k+1} (unused when this iteration stopped)
-                scale_norm_kernel<<<G, kBlasThreads, 0, st>>>(w, n, red_norm, G, V + (size_t)(k + 1) * ld);
-                count_launches(1);
-                if (tail_st != st) {
-                    rc = lanczos_product(ctx, N, pos, V + (size_t)(k + 1) * ld, w);
-                    const int jrc = cuda_fail(cudaEventRecord(gr->ev_join, side), "event record");
-                    const int wrc = jrc ? jrc : cuda_fail(cudaStreamWaitEvent(st, gr->ev_join, 0), "stream wait");
-                    if (!rc) rc = wrc;
-                }
-            }
-            if (!rc) rc = cuda_fail(cudaGetLastError(), "lanczos kernels");
-        }
-        if (cond) {
-            gr->iter_launches[k] = (int)(rpb_launch_count() - before);
-            cudaGraph_t body_graph = nullptr;
+            const uint64_t before = rpb_launch_count();
+            rc = product(true);
+            if (!rc) rc = gs_iteration(ctx, A);
+            gr->body_launches = (int)(rpb_launch_count() - before);
+            cudaGraph_t body_graph = nullptr;  // owned by the node
             const int erc = cuda_fail(cudaStreamEndCapture(gr->body, &body_graph), "body capture end");
             ctx->stream = main_st;
-            if (!rc) rc = erc;
+            if (rc || (rc = erc)) return rc;
         }
-        if (rc) return rc;
-        if (stopped) break;
+    } else {
+        // Host-driven: the tridiagonal step leaves its status in pinned memory and an event tells when.  Where
+        // a product is short the next one is enqueued before the host knows whether this iteration
+        // stopped (then it is discarded): the stream would otherwise idle for the host's answer, about 15 us
+        // an iteration.  The estimate uses the measured per-pair times of the symmetric kernels.
+        if (!ctx->lz_ev &&
+            (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->lz_ev, cudaEventDisableTiming), "lanczos event")))
+            return rc;
+        const double t_product = (ctx->Lx > 0.0 ? 9.0 : 1.0) * (double)N * (double)N *
+                                 (ctx->p.precision == RPB_FP64 ? 8e-11 : 1.3e-12);
+        const bool speculate = t_product < 1e-4;
+        A.hs = w.host_status;
+        bool have = first_done;
+        for (int k = 0; k < max_iter && !stopped; ++k) {
+            A.k = k;
+            if (!have && (rc = product(k == 0 ? packed : true))) return rc;
+            if ((rc = gs_iteration(ctx, A)) || (rc = cuda_fail(cudaEventRecord(ctx->lz_ev, main_st), "event record")))
+                return rc;
+            have = speculate && k + 1 < max_iter;
+            if (have && (rc = product(true))) return rc;
+            if ((rc = cuda_fail(cudaEventSynchronize(ctx->lz_ev), "lanczos iteration"))) return rc;
+            if (k == 0 && hs[ST_NW] == 0.0) {  // W = 0
+                if (iters_out) *iters_out = 0;
+                if (err_out) *err_out = -1.0;
+                if (converged_out) *converged_out = 1;
+                return cuda_fail(cudaMemsetAsync(g, 0, n * sizeof(double), main_st), "zero g");
+            }
+            m = k + 1;
+            eps = hs[ST_EPS];
+            stopped = hs[ST_STOP] != 0.0;
+        }
     }
-    // the combination reads y, which the side stream's tridiagonal step wrote
-    if (!gr && (rc = cuda_fail(cudaStreamWaitEvent(main_st, ctx->lz_ev_t, 0), "stream wait"))) return rc;
-    combine_kernel<<<G, kBlasThreads, 0, main_st>>>(V, ld, n, m, lz + L.y, g, gr ? &gr->state->m : nullptr);
+    combine_kernel<<<blas_grid(n, ctx->num_sms), kBlasThreads, 0, main_st>>>(
+        w.V, A.ld, n, m, w.lz + A.L.y, g, gr ? &gr->state->m : nullptr);
     count_launches(1);
     if (ctx->precond && (rc = precond_scale(ctx, N, g, g, true))) return rc;  // g = D^{1/2} y
     if ((rc = cuda_fail(cudaGetLastError(), "lanczos kernels"))) return rc;
     if (gr) return RPB_OK;
     if (iters_out) *iters_out = m;
     if (err_out) *err_out = eps;
-    const bool converged = stopped;
-    if (converged_out) *converged_out = converged ? 1 : 0;
-    if (tol > 0.0 && !converged) {
+    if (converged_out) *converged_out = stopped ? 1 : 0;
+    if (tol > 0.0 && !stopped) {
         set_error("lanczos: no convergence in %d iterations (eps=%g, tol=%g)", m, eps, tol);
         return RPB_ENOCONV;
     }

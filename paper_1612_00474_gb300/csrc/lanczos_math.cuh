@@ -1,6 +1,6 @@
 // lanczos_math.cuh -- tridiagonal step of the Lanczos square root shared by the single and batched
 // kernels: y_k = |W| T_{k+1}^{1/2} e_1 for the tridiagonal T_{k+1}, the error estimate eps_k and the
-// stopping decision (Sec. II.C).  One 128-thread block per Krylov space evaluates a rational
+// stopping decision (Sec. II.C).  128 threads per Krylov space evaluate a rational
 // approximation of the square root, one node per thread; a T that is not positive definite takes the
 // eigen-decomposition, one warp.
 #pragma once
@@ -153,7 +153,24 @@ __device__ __forceinline__ double warp_max_pos(double v)
     return __longlong_as_double((long long)b);
 }
 
-// The tridiagonal step of one Krylov space by one block of kTailThreads threads: stores alpha_k,
+// Barrier 1 among the kTailThreads threads of a tridiagonal step (their block may have more), and the
+// or of a predicate over them.
+__device__ __forceinline__ void tail_sync()
+{
+    asm volatile("bar.sync 1, %0;" ::"n"(kTailThreads) : "memory");
+}
+__device__ __forceinline__ bool tail_any(bool p)
+{
+    unsigned r;
+    asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.u32 a, %1, 0;\n\tbar.red.or.pred b, 1, %2, a;\n\t"
+                 "selp.u32 %0, 1, 0, b;\n\t}"
+                 : "=r"(r)
+                 : "r"((unsigned)p), "n"(kTailThreads)
+                 : "memory");
+    return r != 0;
+}
+
+// The tridiagonal step of one Krylov space by the first kTailThreads threads of a block: stores alpha_k,
 // beta_k, y, eps and the stopping decision in its state block lz.  nodes: kSqrtNodes shifts, then as
 // many weights (sqrt_nodes.h).
 //
@@ -187,7 +204,7 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
     }
     const double sj = nodes[tid], wj = nodes[kSqrtNodes + tid];
     const double nW = status[ST_NW];
-    __syncthreads();
+    tail_sync();
     // Gershgorin bound and largest entry (every warp, over the entries lane and lane + 32)
     double mb = 0.0, mt = fabs(beta_k);
     for (int i = lane; i < n; i += 32) {
@@ -213,7 +230,7 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
         ri = rcp_pos(d);
         r[i] = ri;
     }
-    if (__syncthreads_or(!ok)) {
+    if (tail_any(!ok)) {
         if (tid >= 32) return;  // (no barrier follows for the first warp on this path)
         double y0, y1;
         tridiag_sqrt_ql(sh.al, sh.be, k, nW, sh.q0, sh.sl, &y0, &y1);
@@ -230,7 +247,7 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
                 if (base + i > 0) z = -(sh.be[base + i - 1] * r[base + i]) * z;
                 sh.z[i][tid] = base + i > 0 ? z : c * x0;
             }
-            __syncthreads();
+            tail_sync();
             // eight threads per entry: 16 nodes each, then three butterfly levels (a fixed order)
             const int row = tid >> 3, p = tid & 7;
             double v = 0.0;
@@ -238,7 +255,7 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
                 for (int u = 0; u < kSqrtNodes / 8; ++u) v += sh.z[row][p + 8 * u];
             for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (p == 0 && row < m) sh.y[base + row] = v * scale;
-            __syncthreads();
+            tail_sync();
         }
         if (tid >= 32) return;
     }

@@ -826,7 +826,7 @@ int pair_prepare(rpb_ctx *ctx, int64_t N)
 // requires ctx->ws.sym_* scratch.  With nparts > 1: share `part` of the triangle's pairs, the self
 // terms with share 0 only (the shares add up to the product).
 static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U,
-                        int part = 0, int nparts = 1)
+                        bool packed = false, int part = 0, int nparts = 1)
 {
     cudaStream_t st = ctx->stream;
     Workspace &w = ctx->ws;
@@ -837,7 +837,7 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
     SrcF32 *src = (SrcF32 *)w.src;
     const int pb = 256;
     const SelfCoefs self = self_coefs(ctx, N);
-    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, self);
+    if (!packed) pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, self);
     const SymCta *ctas = (const SymCta *)sc->index;
     const SymSeg *segs = (const SymSeg *)(sc->index + sc->seg_off);
     const X2Consts c = make_x2_consts(a);
@@ -853,14 +853,14 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
     pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
         w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
         sc->index + sc->rows_off, part == 0);
-    count_launches(sc->ncta > 0 ? 3 : 2);
+    count_launches((sc->ncta > 0 ? 2 : 1) + !packed);
     return cuda_fail(cudaGetLastError(), "symmetric pair kernels");
 }
 
 // The symmetric product in pseudo-periodic mode: positions already folded into the unit cell
 // (pos_w; the self terms use the heights of pos, which the fold leaves unchanged); shares as above.
 static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const double *pos, const double *F,
-                                 const double *T, double *U, int part = 0, int nparts = 1)
+                                 const double *T, double *U, bool packed = false, int part = 0, int nparts = 1)
 {
     cudaStream_t st = ctx->stream;
     Workspace &w = ctx->ws;
@@ -871,7 +871,7 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
     SrcF32 *src = (SrcF32 *)w.src;
     const int pb = 256;
     const SelfCoefs self = self_coefs(ctx, N);
-    pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos_w, F, T, N, a, 1, src, self);
+    if (!packed) pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos_w, F, T, N, a, 1, src, self);
     const SymCta *ctas = (const SymCta *)sc->index;
     const SymSeg *segs = (const SymSeg *)(sc->index + sc->seg_off);
     const X2Consts c = make_x2_consts(a);
@@ -894,7 +894,7 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
     pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
         w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
         sc->index + sc->rows_off, part == 0);
-    count_launches(sc->ncta > 0 ? 3 : 2);
+    count_launches((sc->ncta > 0 ? 2 : 1) + !packed);
     return cuda_fail(cudaGetLastError(), "periodic symmetric pair kernels");
 }
 
@@ -1253,7 +1253,8 @@ __global__ void __launch_bounds__(kPairThreads) pair_periodic_f32_kernel(const S
 // stride nt, U with component stride ldu (ldu < 0: nt).
 __global__ void pair_reduce_kernel(const double *__restrict__ part, int splits, int N, const double *__restrict__ pos,
                                    const double *__restrict__ F, const double *__restrict__ T, PairConsts<double> c,
-                                   double a, double scale, double *__restrict__ U, int wall, int t0, int nt, int ldu)
+                                   double a, double scale, double *__restrict__ U, int wall, int t0, int nt, int ldu,
+                                   SelfCoefs sc)
 {
     const int li = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = t0 + li;
@@ -1264,6 +1265,12 @@ __global__ void pair_reduce_kernel(const double *__restrict__ part, int splits, 
         ux += part[o + li];
         uy += part[o + nt + li];
         uz += part[o + 2 * nt + li];
+    }
+    if (sc.s) {
+        U[li] = sc.velocity(i, 0, ux, F, T, N);
+        U[ldu + li] = sc.velocity(i, 1, uy, F, T, N);
+        U[2 * ldu + li] = sc.velocity(i, 2, uz, F, T, N);
+        return;
     }
     const double z = pos[2 * N + i];
     const double si = wall ? H0(z / a) : 1.0;
@@ -1289,7 +1296,7 @@ __global__ void __launch_bounds__(128) pair_reduce_warp_kernel(const double *__r
                                                                const double *__restrict__ F,
                                                                const double *__restrict__ T, PairConsts<double> c,
                                                                double a, double scale, double *__restrict__ U,
-                                                               int wall, int t0, int nt, int ldu)
+                                                               int wall, int t0, int nt, int ldu, SelfCoefs sc)
 {
     const int lane = threadIdx.x & 31;
     const int li = blockIdx.x * 4 + (threadIdx.x >> 5);
@@ -1306,6 +1313,11 @@ __global__ void __launch_bounds__(128) pair_reduce_warp_kernel(const double *__r
         ux += __shfl_xor_sync(0xffffffffu, ux, m);
         uy += __shfl_xor_sync(0xffffffffu, uy, m);
         uz += __shfl_xor_sync(0xffffffffu, uz, m);
+    }
+    if (sc.s) {
+        const int q = lane;  // every lane holds the sums
+        if (q < 3) U[q * ldu + li] = sc.velocity(i, q, q == 0 ? ux : (q == 1 ? uy : uz), F, T, N);
+        return;
     }
     if (lane != 0) return;
     const double z = pos[2 * N + i];
@@ -1324,22 +1336,23 @@ __global__ void __launch_bounds__(128) pair_reduce_warp_kernel(const double *__r
 }
 
 // Chunk partials -> U (targets t0 .. t0 + nt - 1, nt < 0: all N; U's component stride ldu, ldu < 0:
-// nt): a thread per target for few chunks (coalesced loads), a warp per target for many.
+// nt): a thread per target for few chunks (coalesced loads), a warp per target for many.  With the
+// spheres' self coefficients in sc, or without (sc.s null) evaluating the self terms.
 static void launch_pair_reduce(cudaStream_t st, const double *part, int splits, int N, const double *pos,
-                               const double *F, const double *T, double a, double scale, double *U, int wall,
-                               int t0 = 0, int nt = -1, int ldu = -1)
+                               const double *F, const double *T, double a, double scale, double *U, int wall, int t0,
+                               int nt, int ldu, const SelfCoefs &sc)
 {
     if (nt < 0) nt = N;
     if (ldu < 0) ldu = nt;
     const PairConsts<double> c = make_consts<double>(a);
     if (splits >= 16) {
         pair_reduce_warp_kernel<<<(unsigned)((nt + 3) / 4), 128, 0, st>>>(part, splits, N, pos, F, T, c, a, scale, U,
-                                                                          wall, t0, nt, ldu);
+                                                                          wall, t0, nt, ldu, sc);
     } else {
         // 64-target CTAs: the float64 self terms of a small product then spread over several SMs
         const int rb = 64;
         pair_reduce_kernel<<<(unsigned)((nt + rb - 1) / rb), rb, 0, st>>>(part, splits, N, pos, F, T, c, a, scale, U,
-                                                                          wall, t0, nt, ldu);
+                                                                          wall, t0, nt, ldu, sc);
     }
 }
 
@@ -1415,15 +1428,16 @@ int mobility_rows_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
             pair_f32x2_kernel<false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part, (int)t0, nt);
     }
     launch_pair_reduce(st, part, splits, N, pos, F, T, a, 1.0 / (8.0 * kPi * ctx->p.eta), U_rows, ctx->p.wall,
-                       (int)t0, nt, (int)ldu);
+                       (int)t0, nt, (int)ldu, no_self_coefs());
     count_launches(3);
     return cuda_fail(cudaGetLastError(), "row pair kernels");
 }
 
 static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const double *F, const double *T,
-                           double *U);
+                           double *U, bool packed = false);
 
-int mobility_apply_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const double *F, const double *T, double *U)
+int mobility_apply_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const double *F, const double *T, double *U,
+                        bool packed)
 {
     if (ctx->hook && !ctx->in_hook) {  // the product is delegated (e.g. shared out among processes)
         ctx->in_hook = 1;
@@ -1432,7 +1446,7 @@ int mobility_apply_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doub
         if (rc != RPB_OK && rpb_last_error()[0] == 0) set_error("product hook returned %d", rc);
         return rc;
     }
-    return mobility_direct(ctx, N64, pos, F, T, U);
+    return mobility_direct(ctx, N64, pos, F, T, U, packed);
 }
 
 // Rows [r0, r1) of share `part` of `nparts`: whole 128-row tiles, as equal as the tiles allow.
@@ -1453,12 +1467,12 @@ int mobility_part_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
     const int N = (int)N64;
     cudaStream_t st = ctx->stream;
     const bool sym = ctx->sym_enabled && ctx->p.wall && F && N >= 2 * kTile && (!T || ctx->sym_fused);
-    if (sym && !(ctx->Lx > 0.0)) return mobility_sym(ctx, N, pos, F, T, U, part, nparts);
+    if (sym && !(ctx->Lx > 0.0)) return mobility_sym(ctx, N, pos, F, T, U, false, part, nparts);
     if (sym && ctx->p.precision == RPB_FP32) {
         const int pb = 256;
         wrap_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, N, ctx->Lx, ctx->Ly, ctx->ws.pos_w);
         count_launches(1);
-        return mobility_sym_periodic(ctx, N, ctx->ws.pos_w, pos, F, T, U, part, nparts);
+        return mobility_sym_periodic(ctx, N, ctx->ws.pos_w, pos, F, T, U, false, part, nparts);
     }
     int rc;
     if ((rc = cuda_fail(cudaMemsetAsync(U, 0, (size_t)3 * N * sizeof(double), st), "part product zero fill")))
@@ -1475,12 +1489,12 @@ int mobility_part_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
 }
 
 static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const double *F, const double *T,
-                           double *U)
+                           double *U, bool packed)
 {
     const int N = (int)N64;
     if (ctx->sym_enabled && ctx->p.wall && !(ctx->Lx > 0.0) && F && N >= 2 * kTile && (!T || ctx->sym_fused))
-        return mobility_sym(ctx, N, pos, F, T, U);
-    if (mobility_sym64_ok(ctx, F)) return mobility_sym64(ctx, N, pos, F, T, U);
+        return mobility_sym(ctx, N, pos, F, T, U, packed);
+    if (mobility_sym64_ok(ctx, F)) return mobility_sym64(ctx, N, pos, F, T, U, packed);
     cudaStream_t st = ctx->stream;
     const double a = ctx->p.a;
     int splits;
@@ -1494,18 +1508,19 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
     const int pb = 256;
     const dim3 grid((unsigned)((N + kPairThreads - 1) / kPairThreads), (unsigned)splits);
     const bool torque = T != nullptr;
+    const SelfCoefs self = self_coefs(ctx, N);
     if (ctx->Lx > 0.0) {  // pseudo-periodic: wrap into the unit cell, pack, nine shifts per source
         const double Lx = ctx->Lx, Ly = ctx->Ly;
-        wrap_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, N, Lx, Ly, ctx->ws.pos_w);
+        if (!packed) wrap_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, N, Lx, Ly, ctx->ws.pos_w);
         const double *pw = ctx->ws.pos_w;
         if (ctx->p.precision == RPB_FP32 && ctx->sym_enabled && ctx->p.wall && F && N >= 2 * kTile &&
             (!T || ctx->sym_fused)) {
-            count_launches(1);
-            return mobility_sym_periodic(ctx, N, pw, pos, F, T, U);
+            count_launches(!packed);
+            return mobility_sym_periodic(ctx, N, pw, pos, F, T, U, packed);
         }
         if (ctx->p.precision == RPB_FP32) {
             SrcF32 *src = (SrcF32 *)ctx->ws.src;
-            pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src, no_self_coefs());
+            if (!packed) pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src, self);
             const PairConsts<float> c = make_consts<float>(a);
             const float Lxh = (float)Lx, Lyh = (float)Ly;
             const float Lxl = (float)(Lx - (double)Lxh), Lyl = (float)(Ly - (double)Lyh);
@@ -1519,7 +1534,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
                 pair_periodic_f32_kernel<false, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, Lxh, Lxl, Lyh, Lyl, part);
         } else {
             SrcF64 *src = (SrcF64 *)ctx->ws.src;
-            pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src, no_self_coefs());
+            if (!packed) pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pw, F, T, N, a, ctx->p.wall, src, self);
             const PairConsts<double> c = make_consts<double>(a);
             if (torque && ctx->p.wall)
                 pair_periodic_f64_kernel<true, true><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, Lx, Ly, part);
@@ -1530,13 +1545,13 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
             else
                 pair_periodic_f64_kernel<false, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, Lx, Ly, part);
         }
-        launch_pair_reduce(st, part, splits, N, pos, F, T, a, 1.0 / (8.0 * kPi * ctx->p.eta), U, ctx->p.wall);
-        count_launches(4);
+        launch_pair_reduce(st, part, splits, N, nullptr, F, T, a, 0.0, U, 0, 0, -1, -1, self);
+        count_launches(packed ? 2 : 4);
         return cuda_fail(cudaGetLastError(), "periodic pair kernels");
     }
     if (ctx->p.precision == RPB_FP32) {
         SrcF32 *src = (SrcF32 *)ctx->ws.src;
-        pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, no_self_coefs());
+        if (!packed) pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
         if (!ctx->p.wall) {
             const PairConsts<float> c = make_consts<float>(a);
             if (torque)
@@ -1558,7 +1573,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
         }
     } else {
         SrcF64 *src = (SrcF64 *)ctx->ws.src;
-        pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, no_self_coefs());
+        if (!packed) pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
         const PairConsts<double> c = make_consts<double>(a);
         if (!ctx->p.wall) {
             if (torque)
@@ -1571,8 +1586,8 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
             pair_f64_kernel<false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
         }
     }
-    launch_pair_reduce(st, part, splits, N, pos, F, T, a, 1.0 / (8.0 * kPi * ctx->p.eta), U, ctx->p.wall);
-    count_launches(3);
+    launch_pair_reduce(st, part, splits, N, nullptr, F, T, a, 0.0, U, 0, 0, -1, -1, self);
+    count_launches(packed ? 2 : 3);
     return cuda_fail(cudaGetLastError(), "pair kernels");
 }
 
@@ -2061,7 +2076,7 @@ extern "C" int rpb_mobility_apply_noalloc(int64_t N64, const double *pos, const 
         else
             pair_f64_kernel<false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
     }
-    launch_pair_reduce(st, part, splits, N, pos, F, T, a, 1.0 / (8.0 * kPi * p->eta), U, 1);
+    launch_pair_reduce(st, part, splits, N, pos, F, T, a, 1.0 / (8.0 * kPi * p->eta), U, 1, 0, -1, -1, no_self_coefs());
     count_launches(3);
     return cuda_fail(cudaGetLastError(), "rpb_mobility_apply_noalloc kernels");
 }

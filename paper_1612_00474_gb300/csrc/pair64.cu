@@ -295,7 +295,7 @@ bool mobility_sym64_ok(const rpb_ctx *ctx, const double *F)
     return ctx->ws.sym64 != nullptr && F != nullptr && !(ctx->Lx > 0.0);
 }
 
-int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U)
+int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U, bool packed)
 {
     cudaStream_t st = ctx->stream;
     const double a = ctx->p.a;
@@ -304,7 +304,7 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
     const Sym64Plan pl = sym64_plan(N, ctx->num_sms);
     double *tgt = ctx->ws.sym64, *col = tgt + sym64_tgt_elems(ctx->max_N, ctx->num_sms);
     SrcF64 *src = (SrcF64 *)ctx->ws.src;
-    pack_f64_kernel<<<(N + 255) / 256, 256, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
+    if (!packed) pack_f64_kernel<<<(N + 255) / 256, 256, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
     const dim3 grid((unsigned)pl.runs, (unsigned)pl.qs);
     const int nt = 32 * kSym64Warps;
     if (ctx->p.wall && T)
@@ -316,7 +316,7 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
     else
         pair_sym64_kernel<false, false><<<grid, nt, 0, st>>>(src, N, pl, c64, tgt, col);
     pair_sym64_reduce_kernel<<<pl.nb, kRed64Threads, 0, st>>>(tgt, col, pl, N, F, T, self, U);
-    count_launches(3);
+    count_launches(packed ? 2 : 3);
     return cuda_fail(cudaGetLastError(), "float64 symmetric pair kernels");
 }
 

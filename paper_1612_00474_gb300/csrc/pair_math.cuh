@@ -224,7 +224,8 @@ struct SelfCoefs {
     __device__ __forceinline__ double velocity(int64_t i, int q, double x, const double *__restrict__ F,
                                                const double *__restrict__ T, int64_t ld) const
     {
-        double u = fma(s[i] * scale, x, s[(q == 2 ? 2 : 1) * n + i] * F[q * ld + i]);
+        double u = s[i] * scale * x;
+        if (F) u = fma(s[(q == 2 ? 2 : 1) * n + i], F[q * ld + i], u);
         if (T && q < 2) u = fma(q == 0 ? s[3 * n + i] : -s[3 * n + i], T[(1 - q) * ld + i], u);
         return u;
     }

@@ -143,11 +143,13 @@ struct SymSched {
 
 // Scratch owned by a context.
 struct Workspace {
+    void *slab = nullptr;         // the allocation of the arrays down to vec_g, and of sym64
     void *src = nullptr;          // packed sources, max_N records (SrcF64 size)
     void *partial = nullptr;      // pair-kernel partial sums
     size_t partial_bytes = 0;
     double *V = nullptr;          // Lanczos basis, (max_iter + 1) x 3 max_N
     double *w = nullptr;          // Lanczos work vector, 3 max_N
+    double *vf = nullptr;         // load of the next Lanczos product (the Krylov vector, scaled by the preconditioner)
     double *red = nullptr;        // reduction partials
     size_t red_elems = 0;
     double *lz = nullptr;         // Lanczos small state (alpha, beta, y, y_prev, coefficients, status)
@@ -165,7 +167,6 @@ struct Workspace {
     double *vec_g = nullptr;
     double *host_status = nullptr; // pinned host copy of the Lanczos status word
     double *pc = nullptr;          // block-diagonal preconditioner D^{-1/2} (3 max_N), rpb_set_preconditioner
-    double *pcx = nullptr;         // a Krylov vector scaled by it
     // symmetric translation-translation pass (float32 contexts): schedules, row and column partials
     int *sym_index = nullptr;      // room for two schedules of sym_index_ints each (sym.index, sym_part.index)
     size_t sym_index_ints = 0;
@@ -182,32 +183,28 @@ struct Workspace {
 constexpr int kRunMaxIter = 64;  // = kMaxIter of the Lanczos state
 
 // Device state of a graph-replayed run (rpb_run): the step index the noise is drawn with, whether the
-// coming step is a first (Euler-Maruyama) step, the Lanczos dimension m of the latest step, and counters
-// of the instance-steps that did not converge and of the runs of each Lanczos iteration.
+// coming step is a first (Euler-Maruyama) step, the Lanczos dimension m of the latest step and the
+// iteration it is at, and counters of the steps that did not converge and of the iterations run in the
+// loop node (all but each step's first).
 struct RunState {
     unsigned int step;
     int first;
     int m;
     int left;  // steps left in the run
+    int k;
+    int pad;
     unsigned long long unconv;
-    unsigned long long iter_runs[kRunMaxIter];
+    unsigned long long loops;
 };
 struct RunCtx;  // run.cu
 
-// Capture of the Lanczos iterations into a CUDA graph (rpb_run): iteration k >= 1 is the body of a
-// conditional node hnd[k], captured on `body`; the last kernel of iteration k - 1 sets its condition on
-// the device from the stopping test, and records m in state.
+// Capture of the Lanczos iterations into a CUDA graph (rpb_run): the iterations after the first are the
+// body of a loop (WHILE) node captured on `body`; the last kernel of an iteration sets its condition on
+// the device from the stopping test, and records m and the iteration in state.
 struct LzGraph {
     cudaStream_t body = nullptr;
     RunState *state = nullptr;
-    // a second branch inside an iteration: the tridiagonal step beside the next iteration's product
-    // (short products only; null: no branch).  A stream joined into a capture stays in it until the
-    // capture ends, so the first iteration (captured with the step) and the conditional bodies (each
-    // a capture of its own) fork onto different streams: side0 and side.
-    cudaStream_t side0 = nullptr, side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    cudaGraphConditionalHandle hnd[kRunMaxIter] = {};
-    int iter_launches[kRunMaxIter] = {};  // kernels captured into iteration k's body
+    int body_launches = 0;  // kernels captured into the loop's body
 };
 
 }  // namespace rpb
@@ -231,9 +228,8 @@ struct rpb_ctx {
     rpb_product_hook hook = nullptr;  // products delegated to the caller (rpb_set_product_hook)
     void *hook_user = nullptr;
     int in_hook = 0;                  // inside the hook: products are computed here
-    // host-driven Lanczos: the side stream its tridiagonal steps run on, and its two events
-    cudaStream_t lz_side = nullptr;
-    cudaEvent_t lz_ev_a = nullptr, lz_ev_t = nullptr;
+    int gs_cluster = 8;               // blocks of the Lanczos cluster kernel at most (lanczos_setup)
+    cudaEvent_t lz_ev = nullptr;      // host-driven Lanczos: an iteration's status has been written
 };
 
 namespace rpb {
@@ -245,9 +241,10 @@ void count_launches(int n);
 int cuda_fail(cudaError_t e, const char *what);
 
 // Pair product: U = M_tt F + M_tr T with the context's precision.  F or T may be null.
-// All pointers device, SoA float64.  Enqueued on ctx->stream.
+// All pointers device, SoA float64.  Enqueued on ctx->stream.  packed: the context's packed sources hold
+// these positions and s F already (F is still read for the self terms; T must be null).
 int mobility_apply_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *F, const double *T,
-                        double *U);
+                        double *U, bool packed = false);
 // Rows t0 .. t1 - 1 of the product (component stride ldu, ldu < 0: t1 - t0), one-way kernels over a
 // target range.
 int mobility_rows_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *F, const double *T, int64_t t0,
@@ -258,7 +255,7 @@ int mobility_part_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double 
 // The float64 product with each unordered pair evaluated once (pair64.cu): whether it can be taken (a
 // float64 context with its scratch, forces given, no periodic images), and the product.
 bool mobility_sym64_ok(const rpb_ctx *ctx, const double *F);
-int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U);
+int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U, bool packed);
 // Whether mobility_apply2_impl can take this product (float32 symmetric pass with two right-hand sides).
 bool mobility_apply2_ok(const rpb_ctx *ctx, int64_t N);
 // U = M_tt F + M_tr T and U2 = M_tt P in one symmetric pass (F, T, P non-null).
@@ -301,8 +298,8 @@ int batch_sym_apply(const BatchSymPlan &pl, cudaStream_t st, const SrcF32 *src, 
 // d_step (optional): a device word to read the step index from instead of `step` (graph replays).
 int philox_impl(rpb_ctx *ctx, int64_t N, uint64_t seed, uint32_t step, uint32_t stream_id, uint32_t instance,
                 double *out, const unsigned int *d_step = nullptr);
-// Open a conditional (IF) node after the work captured so far on `st` and start capturing its body on
-// `body`; the node runs its body when `h` was set non-zero during this launch of the graph.
+// Open a conditional node after the work captured so far on `st` and start capturing its body on
+// `body`; an IF node runs its body when `h` was set non-zero, a WHILE node as long as it is.
 int graph_begin_if(cudaStream_t st, cudaStream_t body, cudaGraphConditionalHandle h);
 int graph_begin_cond(cudaStream_t st, cudaStream_t body, cudaGraphConditionalHandle h,
                      cudaGraphConditionalNodeType type);
@@ -323,22 +320,20 @@ __global__ void graph_loop_tail_kernel(int *left, cudaGraphConditionalHandle h);
 // Host-side preparation a product at this N needs (the symmetric pass's schedule), done before a
 // stream capture so that the captured products find it in place.
 int pair_prepare(rpb_ctx *ctx, int64_t N);
+// packed: the positions are packed already (a product at these positions was the last one)
 int lanczos_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *W, double *g, double tol, int max_iter,
-                 int *iters_out, double *err_out, int *converged_out, LzGraph *gr = nullptr);
-// The two halves of lanczos_impl: |W| and v_0 = W/|W| into ws.V (synchronises; *nw_zero when W = 0),
-// then the iterations; with first_done the first product M v_0 is already in ws.w (with the
-// preconditioner on: P M P v_0, see lanczos_precond_prepare).
-// graph: inside a stream capture; nothing is read back (*nw_zero false: the noise W of a step is never 0).
-int lanczos_init(rpb_ctx *ctx, int64_t N, const double *W, bool *nw_zero, bool graph = false);
+                 bool packed, int *iters_out, double *err_out, int *converged_out, LzGraph *gr = nullptr);
+// The two halves of lanczos_impl: v_0 = W/|W| into ws.V and, times the preconditioner, into ws.vf (packed:
+// into the packed sources too); then the iterations.  first_done: the product M vf is already in ws.w.
+int lanczos_init(rpb_ctx *ctx, int64_t N, const double *W, bool packed, LzGraph *gr);
 // With ctx->precond set: P = D^{-1/2} at these positions into ws.pc (D: diagonal of the self blocks),
-// so that the iteration runs on P M P and returns g = D^{1/2} y.  precond_scale: out = x * P
-// elementwise (inverse: x / P, 0 where P = 0).
+// so that the iteration runs on P M P and returns g = D^{1/2} y.
 int lanczos_precond_prepare(rpb_ctx *ctx, int64_t N, const double *pos);
-int precond_scale(rpb_ctx *ctx, int64_t N, const double *x, double *out, bool inverse);
-// gr: inside a stream capture, the iterations after the first in conditional nodes (see LzGraph); the
-// host outputs are then not written.
+// gr: inside a stream capture, the iterations after the first in a loop node (see LzGraph); the host
+// outputs are then not written (the noise W of a step is never 0).
 int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double tol, int max_iter, bool first_done,
-                int *iters_out, double *err_out, int *converged_out, LzGraph *gr = nullptr);
+                bool packed, int *iters_out, double *err_out, int *converged_out, LzGraph *gr = nullptr);
+int lanczos_setup(rpb_ctx *ctx);
 int rfd_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *Wt, double delta, double *drift,
              int one_sided = 0);
 // d_first (optional): a device word that, when non-zero, makes the update a first step (graph replays).
@@ -361,6 +356,6 @@ int upload_sqrt_nodes(double *nodes, cudaStream_t st);
 // state (at LzLayout::total).
 size_t lanczos_state_elems(int max_iter);
 int lanczos_upload(double *lz, int max_iter, cudaStream_t st);  // the nodes into a state block
-size_t lanczos_red_elems(int max_iter);
+size_t lanczos_red_elems(int64_t max_N, int max_iter);
 
 }  // namespace rpb

@@ -4,9 +4,11 @@
 // Sec. II.A and the update of Eq. AB) is captured once as the body of a WHILE node of a graph on a
 // stream the context owns, and the graph is launched once: the body runs nsteps times with no host
 // synchronisation in between, the last kernel of a step counting the steps down.  Each Lanczos
-// iteration after the first is a conditional (IF) node inside that body whose condition the previous
-// iteration sets on the device from the stopping test, so a replay runs exactly the iterations a
-// host-driven step runs; the step index that keys the noise and the first-step flag live on the device
+// iteration after the first is a pass of a loop (WHILE) node inside that body whose condition the
+// previous iteration sets on the device from the stopping test, so a replay runs exactly the iterations a
+// host-driven step runs, and the graph holds one iteration's kernels whatever max_iter (with one IF node per
+// iteration, the nodes after the stop cost 2.3 us a step each, and 64 of them 3 ms of capture and
+// instantiation a call); the step index that keys the noise and the first-step flag live on the device
 // and advance at the end of each step.
 // The kernels, their arguments and their order are those of rpb_step, so the results are the same
 // bit for bit.
@@ -22,11 +24,8 @@ static_assert(kRunMaxIter == kMaxIter, "run state sized for the Lanczos dimensio
 struct RunCtx {
     cudaStream_t st = nullptr;    // capture and replay
     cudaStream_t loop = nullptr;  // the body of the loop over the steps is captured here
-    cudaStream_t body = nullptr;  // the Lanczos iterations' conditional bodies are captured here
-    cudaStream_t side0 = nullptr, side = nullptr;  // a second branch inside a Lanczos iteration (the tridiagonal
-                                                   // step): in the first iteration, in the conditional ones
+    cudaStream_t body = nullptr;  // the body of the loop over the Lanczos iterations is captured here
     cudaEvent_t ev = nullptr;     // orders the run after the context's stream and back
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;  // fork and join of that branch in the capture
     RunState *state = nullptr;    // device
     RunState *h_state = nullptr;  // pinned host copy
     double *h_status = nullptr;   // pinned host copy of the Lanczos status words
@@ -96,10 +95,9 @@ void run_free(rpb_ctx *ctx)
 {
     RunCtx *r = ctx->run;
     if (!r) return;
-    for (cudaStream_t q : {r->st, r->loop, r->body, r->side0, r->side})
+    for (cudaStream_t q : {r->st, r->loop, r->body})
         if (q) cudaStreamDestroy(q);
-    for (cudaEvent_t e : {r->ev, r->ev_fork, r->ev_join})
-        if (e) cudaEventDestroy(e);
+    if (r->ev) cudaEventDestroy(r->ev);
     if (r->state) cudaFree(r->state);
     if (r->h_state) cudaFreeHost(r->h_state);
     if (r->h_status) cudaFreeHost(r->h_status);
@@ -121,11 +119,7 @@ static int run_setup(rpb_ctx *ctx)
     if ((rc = cuda_fail(cudaStreamCreateWithFlags(&r->st, cudaStreamNonBlocking), "run stream")) ||
         (rc = cuda_fail(cudaStreamCreateWithFlags(&r->loop, cudaStreamNonBlocking), "run loop stream")) ||
         (rc = cuda_fail(cudaStreamCreateWithFlags(&r->body, cudaStreamNonBlocking), "run body stream")) ||
-        (rc = cuda_fail(cudaStreamCreateWithFlags(&r->side0, cudaStreamNonBlocking), "run side stream")) ||
-        (rc = cuda_fail(cudaStreamCreateWithFlags(&r->side, cudaStreamNonBlocking), "run side stream")) ||
-        (rc = cuda_fail(cudaEventCreateWithFlags(&r->ev, cudaEventDisableTiming), "run event")) ||
-        (rc = cuda_fail(cudaEventCreateWithFlags(&r->ev_fork, cudaEventDisableTiming), "run event")) ||
-        (rc = cuda_fail(cudaEventCreateWithFlags(&r->ev_join, cudaEventDisableTiming), "run event"))) {
+        (rc = cuda_fail(cudaEventCreateWithFlags(&r->ev, cudaEventDisableTiming), "run event"))) {
         run_free(ctx);
         return rc;
     }
@@ -147,7 +141,8 @@ __global__ void run_init_kernel(RunState *s, unsigned int step, int nsteps)
     s->m = 0;
     s->left = nsteps;
     s->unconv = 0ull;
-    for (int k = 0; k < kRunMaxIter; ++k) s->iter_runs[k] = 0ull;
+    s->k = 0;
+    s->loops = 0ull;
 }
 
 // End of a replayed step: the next step's index, no longer a first step, whether this step's Lanczos
@@ -198,10 +193,6 @@ extern "C" int rpb_run(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, int
     LzGraph gr;
     gr.body = r->body;
     gr.state = r->state;
-    gr.side0 = r->side0;
-    gr.side = r->side;
-    gr.ev_fork = r->ev_fork;
-    gr.ev_join = r->ev_join;
     const LzLayout L(ctx->max_iter);
     const double *status = ctx->ws.lz + L.status;
     const bool lanczos = ctx->p.kT > 0.0;
@@ -251,13 +242,9 @@ extern "C" int rpb_run(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, int
     cudaGraphExecDestroy(exec);
     cudaGraphDestroy(graph);
     if (rc) return rc;
-    // kernels executed: the unconditional part every step, each iteration body once per run of it
-    int64_t cond_part = 0, executed = 0;
-    for (int k = 1; k < kRunMaxIter; ++k) {
-        cond_part += gr.iter_launches[k];
-        executed += (int64_t)gr.iter_launches[k] * (int64_t)r->h_state->iter_runs[k];
-    }
-    count_launches((int)((per_step - cond_part) * (int64_t)nsteps + executed));
+    // kernels executed: the unconditional part every step, the loop's body once per run of it
+    count_launches((int)((int64_t)(per_step - gr.body_launches) * nsteps +
+                         (int64_t)gr.body_launches * (int64_t)r->h_state->loops));
     const int64_t unconv = (int64_t)r->h_state->unconv;
     if (unconverged) *unconverged = unconv;
     if (stats) {
