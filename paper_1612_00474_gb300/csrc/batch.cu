@@ -462,10 +462,11 @@ __global__ void __launch_bounds__(kGsThreads) batch_dots_kernel(const double *__
     if (active && !active[c.inst]) return;  // uniform per block
     int64_t row[kGsRows];
     double x[kGsRows];
-    gs_rows(chunk_span(c, inst[c.inst], total), row);
+    const GsSpan span = chunk_span(c, inst[c.inst], total);
+    const int nu = gs_rows(span, row), nw = gs_warps(span);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) x[u] = row[u] >= 0 ? w[row[u]] : 0.0;
-    const double s = gs_dots(V, ld, nvec, row, x, sh);
+    const double s = gs_dots(V, ld, nvec, row, nu, nw, x, sh);
     if (threadIdx.x < nvec) red[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s;
 }
 
@@ -488,23 +489,24 @@ __global__ void __launch_bounds__(kGsThreads) batch_project_kernel(const double 
     if (active && !active[c.inst]) return;
     int64_t row[kGsRows];
     double x[kGsRows];
-    gs_rows(chunk_span(c, inst[c.inst], total), row);
+    const GsSpan span = chunk_span(c, inst[c.inst], total);
+    const int nu = gs_rows(span, row), nw = gs_warps(span);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) x[u] = row[u] >= 0 ? w[row[u]] : 0.0;
     gs_coefs(red + c.chunk0, gridDim.x, c.count, nvec, coef);
     if (c.first == 0 && threadIdx.x < nvec) lz[(size_t)c.inst * lz_stride + coef_off + threadIdx.x] = coef[threadIdx.x];
-    gs_project(V, ld, nvec, row, coef, x);
+    gs_project(V, ld, nvec, row, nu, coef, x);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u)
         if (row[u] >= 0) w[row[u]] = x[u];
     if (red2) {
-        const double s = gs_dots(V, ld, nvec, row, x, sh);
+        const double s = gs_dots(V, ld, nvec, row, nu, nw, x, sh);
         if (threadIdx.x < nvec) red2[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s;
     } else {
         double s = 0.0;
 #pragma unroll
         for (int u = 0; u < kGsRows; ++u) s = fma(x[u], x[u], s);
-        s = gs_block_sum(s, sh[0]);
+        s = gs_block_sum(s, nu, nw, sh[0]);
         if (threadIdx.x == 0) norm2[blockIdx.x] = s;
     }
 }

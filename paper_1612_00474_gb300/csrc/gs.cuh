@@ -22,8 +22,10 @@ struct GsSpan {
     int cnt;
 };
 
-// Offsets of this thread's rows (component-major in the chunk); -1 past the end.
-__device__ __forceinline__ void gs_rows(const GsSpan &s, int64_t (&row)[kGsRows])
+// Offsets of this thread's rows (component-major in the chunk); -1 past the end.  Returns the number of rows that
+// some lane of the warp has: the loops over the rows run to it, since a float64 instruction costs the same
+// with no lane active.
+__device__ __forceinline__ int gs_rows(const GsSpan &s, int64_t (&row)[kGsRows])
 {
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) {
@@ -31,6 +33,13 @@ __device__ __forceinline__ void gs_rows(const GsSpan &s, int64_t (&row)[kGsRows]
         const int c = r < s.cnt ? 0 : (r < 2 * s.cnt ? 1 : 2);
         row[u] = r < 3 * s.cnt ? s.base + c * s.stride + (r - c * s.cnt) : -1;
     }
+    const int left = 3 * s.cnt - (int)(threadIdx.x & ~31u);
+    return left <= 0 ? 0 : min(kGsRows, (left + kGsThreads - 1) / kGsThreads);
+}
+// Warps of the block that have rows.
+__device__ __forceinline__ int gs_warps(const GsSpan &s)
+{
+    return min(kGsWarps, (3 * s.cnt + 31) / 32);
 }
 
 // Sums over the warp of eight values per lane: lane l returns the sum of v[l >> 2] (a fixed order).
@@ -48,24 +57,28 @@ __device__ __forceinline__ double warp_sum8(double (&v)[8])
     return s + __shfl_xor_sync(0xffffffffu, s, 1);
 }
 
-// Sum over the block of one value per thread, in every thread; sh: kGsWarps doubles.
-__device__ __forceinline__ double gs_block_sum(double v, double *sh)
+// Sum over the block of one value per thread, in the first warp's threads; sh: kGsWarps doubles.
+__device__ __forceinline__ double gs_block_sum(double v, int nu, int nw, double *sh)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    const int lane = threadIdx.x & 31;
+    if (nu > 0) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) sh[threadIdx.x >> 5] = v;
+    }
     __syncthreads();
     double s = 0.0;
-    for (int k = 0; k < kGsWarps; ++k) s += sh[k];
-    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = lane < nw ? sh[lane] : 0.0;
+        for (int o = kGsWarps / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
     return s;
 }
 
-// The block's part of <V_j, w>, j < nvec: thread j < nvec returns it (nvec <= kGsThreads).
-// sh: kGsWarps x (kMaxIter + 8) doubles.
-__device__ __forceinline__ double gs_dots(const double *__restrict__ V, size_t ld, int nvec, const int64_t (&row)[kGsRows],
-                                          const double (&w)[kGsRows], double (*sh)[kMaxIter + 8])
+template <int NU>
+__device__ __forceinline__ void gs_dots_rows(const double *__restrict__ V, size_t ld, int nvec,
+                                             const int64_t (&row)[kGsRows], const double (&w)[kGsRows], double *sh)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     for (int j0 = 0; j0 < nvec; j0 += 8) {
         double acc[8];
 #pragma unroll
@@ -74,32 +87,59 @@ __device__ __forceinline__ double gs_dots(const double *__restrict__ V, size_t l
             if (j0 + q < nvec) {
                 const double *v = V + (size_t)(j0 + q) * ld;
 #pragma unroll
-                for (int u = 0; u < kGsRows; ++u)
+                for (int u = 0; u < NU; ++u)
                     if (row[u] >= 0) acc[q] = fma(v[row[u]], w[u], acc[q]);
             }
         }
         const double s = warp_sum8(acc);
-        if ((lane & 3) == 0) sh[warp][j0 + (lane >> 2)] = s;
+        if ((lane & 3) == 0) sh[j0 + (lane >> 2)] = s;
     }
+}
+
+// The block's part of <V_j, w>, j < nvec: thread j < nvec returns it (nvec <= kGsThreads).
+// sh: kGsWarps x (kMaxIter + 8) doubles; nu, nw: gs_rows, gs_warps.
+__device__ __forceinline__ double gs_dots(const double *__restrict__ V, size_t ld, int nvec, const int64_t (&row)[kGsRows],
+                                          int nu, int nw, const double (&w)[kGsRows], double (*sh)[kMaxIter + 8])
+{
+    static_assert(kGsRows == 3, "one case per number of rows");
+    double *mine = sh[threadIdx.x >> 5];
+    if (nu == 1)
+        gs_dots_rows<1>(V, ld, nvec, row, w, mine);
+    else if (nu == 2)
+        gs_dots_rows<2>(V, ld, nvec, row, w, mine);
+    else if (nu == 3)
+        gs_dots_rows<3>(V, ld, nvec, row, w, mine);
     __syncthreads();
     double s = 0.0;
     if (threadIdx.x < nvec)
-        for (int k = 0; k < kGsWarps; ++k) s += sh[k][threadIdx.x];
+        for (int k = 0; k < nw; ++k) s += sh[k][threadIdx.x];
     return s;
 }
 
-// w -= sum_j coef_j V_j
-__device__ __forceinline__ void gs_project(const double *__restrict__ V, size_t ld, int nvec, const int64_t (&row)[kGsRows],
-                                           const double *coef, double (&w)[kGsRows])
+template <int NU>
+__device__ __forceinline__ void gs_project_rows(const double *__restrict__ V, size_t ld, int nvec,
+                                                const int64_t (&row)[kGsRows], const double *coef, double (&w)[kGsRows])
 {
 #pragma unroll 4
     for (int j = 0; j < nvec; ++j) {
         const double *v = V + (size_t)j * ld;
         const double m = -coef[j];
 #pragma unroll
-        for (int u = 0; u < kGsRows; ++u)
+        for (int u = 0; u < NU; ++u)
             if (row[u] >= 0) w[u] = fma(m, v[row[u]], w[u]);
     }
+}
+
+// w -= sum_j coef_j V_j
+__device__ __forceinline__ void gs_project(const double *__restrict__ V, size_t ld, int nvec, const int64_t (&row)[kGsRows],
+                                           int nu, const double *coef, double (&w)[kGsRows])
+{
+    if (nu == 1)
+        gs_project_rows<1>(V, ld, nvec, row, coef, w);
+    else if (nu == 2)
+        gs_project_rows<2>(V, ld, nvec, row, coef, w);
+    else if (nu == 3)
+        gs_project_rows<3>(V, ld, nvec, row, coef, w);
 }
 
 // coef_j = sum of n partials red[j rs + k], j < nvec, by one warp per vector in a fixed order; ends with a

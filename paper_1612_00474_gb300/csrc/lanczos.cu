@@ -173,32 +173,34 @@ __global__ void __launch_bounds__(kGsThreads) gs_cluster_kernel(GsArgs A, int pe
     const int left = (int)A.N - first;
     int64_t row[kGsRows];
     double x[kGsRows];
-    gs_rows(GsSpan{first, A.N, max(0, min(per, left))}, row);
+    const GsSpan span = {first, A.N, max(0, min(per, left))};
+    const int nu = gs_rows(span, row), nw = gs_warps(span);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) {
         x[u] = row[u] < 0 ? 0.0 : (init ? A.W[row[u]] : A.w[row[u]]);
         if (A.P && !init && row[u] >= 0) x[u] *= A.P[row[u]];
     }
     for (int pass = 0; pass < 2 && !init; ++pass) {
-        const double s = gs_dots(A.V, A.ld, k + 1, row, x, sh);
+        const double s = gs_dots(A.V, A.ld, k + 1, row, nu, nw, x, sh);
         if (tid <= k) part[pass][tid] = s;
         cl.sync();
         cluster_coefs(cl, part[pass], k + 1, coef);
         if (rank == 0 && tid <= k) A.lz[(pass ? A.L.c2 : A.L.c1) + tid] = coef[tid];
-        gs_project(A.V, A.ld, k + 1, row, coef, x);
+        gs_project(A.V, A.ld, k + 1, row, nu, coef, x);
     }
     double s = 0.0;
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) s = fma(x[u], x[u], s);
-    s = gs_block_sum(s, sh[0]);
+    s = gs_block_sum(s, nu, nw, sh[0]);
     if (tid == 0) norm[0] = s;
     cl.sync();
-    const int lane = tid & 31;
+    const int lane = tid & (kGsCluster - 1);
     double bn = lane < (int)cl.num_blocks() ? cl.map_shared_rank(norm, lane)[0] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) bn += __shfl_xor_sync(0xffffffffu, bn, o);
+    for (int o = kGsCluster / 2; o > 0; o >>= 1) bn += __shfl_xor_sync(0xffffffffu, bn, o);
     cl.barrier_arrive();  // nothing of another block's memory is read from here on
-    const double nb = sqrt(bn);
-    const double inv = init && !(nb > 0.0) ? 0.0 : 1.0 / nb;
+    double nb, inv;
+    root_and_inverse(bn, &nb, &inv);
+    if (init && !(nb > 0.0)) inv = 0.0;
     double *v = A.V + (size_t)(k + 1) * A.ld;
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u)
@@ -216,10 +218,10 @@ __global__ void __launch_bounds__(kGsThreads) gs_cluster_kernel(GsArgs A, int pe
 }
 
 // ------------------------------------------------------------------ larger suspensions: chunks over the GPU
-__device__ __forceinline__ void gs_chunk_rows(const GsArgs &A, int chunk, int64_t (&row)[kGsRows])
+__device__ __forceinline__ GsSpan gs_chunk_span(const GsArgs &A, int chunk)
 {
     const int64_t first = (int64_t)blockIdx.x * chunk;
-    gs_rows(GsSpan{first, A.N, (int)min((int64_t)chunk, A.N - first)}, row);
+    return GsSpan{first, A.N, (int)min((int64_t)chunk, A.N - first)};
 }
 
 // partials of <V_j, w>, j <= k (w scaled by the preconditioner first)
@@ -229,13 +231,14 @@ __global__ void __launch_bounds__(kGsThreads) gs_dots_kernel(GsArgs A, int chunk
     const int k = A.iter();
     int64_t row[kGsRows];
     double x[kGsRows];
-    gs_chunk_rows(A, chunk, row);
+    const GsSpan span = gs_chunk_span(A, chunk);
+    const int nu = gs_rows(span, row), nw = gs_warps(span);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) {
         x[u] = row[u] >= 0 ? A.w[row[u]] : 0.0;
         if (A.P && row[u] >= 0) A.w[row[u]] = x[u] *= A.P[row[u]];
     }
-    const double s = gs_dots(A.V, A.ld, k + 1, row, x, sh);
+    const double s = gs_dots(A.V, A.ld, k + 1, row, nu, nw, x, sh);
     if (threadIdx.x <= k) A.red[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = s;
 }
 
@@ -247,23 +250,24 @@ __global__ void __launch_bounds__(kGsThreads) gs_project_kernel(GsArgs A, int ch
     const int k = A.iter(), tid = threadIdx.x;
     int64_t row[kGsRows];
     double x[kGsRows];
-    gs_chunk_rows(A, chunk, row);
+    const GsSpan span = gs_chunk_span(A, chunk);
+    const int nu = gs_rows(span, row), nw = gs_warps(span);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) x[u] = row[u] >= 0 ? A.w[row[u]] : 0.0;
     gs_coefs(pass ? A.red2 : A.red, gridDim.x, gridDim.x, k + 1, coef);
     if (blockIdx.x == 0 && tid <= k) A.lz[(pass ? A.L.c2 : A.L.c1) + tid] = coef[tid];
-    gs_project(A.V, A.ld, k + 1, row, coef, x);
+    gs_project(A.V, A.ld, k + 1, row, nu, coef, x);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u)
         if (row[u] >= 0) A.w[row[u]] = x[u];
     if (pass == 0) {
-        const double s = gs_dots(A.V, A.ld, k + 1, row, x, sh);
+        const double s = gs_dots(A.V, A.ld, k + 1, row, nu, nw, x, sh);
         if (tid <= k) A.red2[(size_t)tid * gridDim.x + blockIdx.x] = s;
     } else {
         double s = 0.0;
 #pragma unroll
         for (int u = 0; u < kGsRows; ++u) s = fma(x[u], x[u], s);
-        s = gs_block_sum(s, sh[0]);
+        s = gs_block_sum(s, nu, nw, sh[0]);
         if (tid == 0) A.norm2[blockIdx.x] = s;
     }
 }
@@ -273,12 +277,13 @@ __global__ void __launch_bounds__(kGsThreads) gs_norm_kernel(GsArgs A, int chunk
 {
     __shared__ double sh[kGsWarps];
     int64_t row[kGsRows];
-    gs_chunk_rows(A, chunk, row);
+    const GsSpan span = gs_chunk_span(A, chunk);
+    const int nu = gs_rows(span, row), nw = gs_warps(span);
     double s = 0.0;
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u)
         if (row[u] >= 0) s = fma(A.W[row[u]], A.W[row[u]], s);
-    s = gs_block_sum(s, sh);
+    s = gs_block_sum(s, nu, nw, sh);
     if (threadIdx.x == 0) A.norm2[blockIdx.x] = s;
 }
 
@@ -287,11 +292,12 @@ __global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(GsArgs A, int chun
 {
     __shared__ double bn;
     gs_coefs(A.norm2, 0, gridDim.x, 1, &bn);
-    const double nb = sqrt(bn);
-    const double inv = init && !(nb > 0.0) ? 0.0 : 1.0 / nb;
+    double nb, inv;
+    root_and_inverse(bn, &nb, &inv);
+    if (init && !(nb > 0.0)) inv = 0.0;
     const int k = init ? -1 : A.iter();
     int64_t row[kGsRows];
-    gs_chunk_rows(A, chunk, row);
+    gs_rows(gs_chunk_span(A, chunk), row);
     double *v = A.V + (size_t)(k + 1) * A.ld;
     const double *w = init ? A.W : A.w;
 #pragma unroll

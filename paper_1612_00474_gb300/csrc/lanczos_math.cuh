@@ -121,16 +121,6 @@ static __device__ __noinline__ void tridiag_sqrt_ql(const double *alpha, const d
     *y_out1 = y1 * nW;
 }
 
-// 1/d for a positive normal d: the hardware's approximation (relative error below 2^-23) and one
-// third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - d y.
-__device__ __forceinline__ double rcp_pos(double d)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    const double e = fma(-d, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
 constexpr int kTailThreads = kSqrtNodes;  // one node per thread
 constexpr int kTailRows = 16;             // entries of y summed over the nodes at a time
 struct TailShared {
@@ -174,8 +164,8 @@ __device__ __forceinline__ bool tail_any(bool p)
 // beta_k, y, eps and the stopping decision in its state block lz.  nodes: kSqrtNodes shifts, then as
 // many weights (sqrt_nodes.h).
 //
-// With T = tridiag(beta, alpha, beta) scaled by its Gershgorin bound M, y = |W| T^{1/2} e_1 ~
-// |W| sqrt(M) sum_j w_j T (T + M s_j)^{-1} e_1.  Thread j solves its shifted system by eliminating from
+// With T = tridiag(beta, alpha, beta) scaled by M, the power of four above its Gershgorin bound (its square
+// root is exact and costs nothing), y = |W| T^{1/2} e_1 ~ |W| sqrt(M) sum_j w_j T (T + M s_j)^{-1} e_1.  Thread j solves its shifted system by eliminating from
 // the last row up: c_i = alpha_i - beta_i^2 / d_{i+1}, d_i = c_i + s; then x_0 = 1/d_0,
 // x_{i+1} = -(beta_i / d_{i+1}) x_i, and (T x)_0 = c_0 x_0, (T x)_i = -s x_i, with no cancellation.
 // Everything is backward stable for a positive definite T (relative errors of a few 1e-16 in y, against
@@ -212,21 +202,22 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
         mb = fmax(mb, a + b + (i > 0 ? fabs(sh.be[i - 1]) : 0.0));
         mt = fmax(mt, fmax(a, b));
     }
-    const double M = warp_max_pos(mb);
+    // M = 4^e >= the bound, sqrt(M) = 2^e (a bound that is not a plain positive number fails the pivots' test)
+    const double bound = warp_max_pos(mb);
+    const int e4 = plain_pos(bound) ? ((__double2hiint(bound) >> 20) - 1023 + 2) >> 1 : 0;
+    const double M = __hiloint2double((1023 + 2 * e4) << 20, 0), rootM = __hiloint2double((1023 + e4) << 20, 0);
     const double tnorm = warp_max_pos(mt);
     const double s = M * sj;
     double r[kMaxIter];
     double c = sh.al[k];
     double d = c + s;
-    // positive and normal, below 2^1000: on the exponent bits (false for NaN)
-    auto fine = [](double v) { return (unsigned)(__double2hiint(v) - 0x00100000) < 0x7e600000u; };
-    bool ok = fine(d);
+    bool ok = plain_pos(d) && plain_pos(bound);
     double ri = rcp_pos(d);
     r[k] = ri;
     for (int i = k - 1; i >= 0; --i) {
         c = fma(-sh.b2[i], ri, sh.al[i]);
         d = c + s;
-        ok = ok && fine(d);
+        ok = ok && plain_pos(d);
         ri = rcp_pos(d);
         r[i] = ri;
     }
@@ -238,7 +229,7 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
         if (lane + 32 < n) sh.y[lane + 32] = y1;
         __syncwarp();
     } else {
-        const double scale = sqrt(M) * nW;
+        const double scale = rootM * nW;
         const double x0 = wj * ri;
         double z = -(s * x0);
         for (int base = 0; base < n; base += kTailRows) {
@@ -248,41 +239,46 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
                 sh.z[i][tid] = base + i > 0 ? z : c * x0;
             }
             tail_sync();
-            // eight threads per entry: 16 nodes each, then three butterfly levels (a fixed order)
-            const int row = tid >> 3, p = tid & 7;
+            // eight threads per entry, 16 for up to eight entries: 16 or 8 nodes each, then the butterfly
+            // levels (a fixed order)
+            const int lg = n <= 8 ? 4 : 3, row = tid >> lg, p = tid & ((1 << lg) - 1);
             double v = 0.0;
             if (row < m)
-                for (int u = 0; u < kSqrtNodes / 8; ++u) v += sh.z[row][p + 8 * u];
+                for (int u = p; u < kSqrtNodes; u += 1 << lg) v += sh.z[row][u];
+            if (lg == 4) v += __shfl_xor_sync(0xffffffffu, v, 8);
             for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (p == 0 && row < m) sh.y[base + row] = v * scale;
             tail_sync();
         }
         if (tid >= 32) return;
     }
-    // eps_k = |y - (yprev, 0)| / |yprev|
-    double num = 0.0, den = 0.0;
-    for (int i = lane; i < n; i += 32) {
-        const double y = sh.y[i], p = i < k ? lz[L.yprev + i] : 0.0;
-        num += (y - p) * (y - p);
-        den += p * p;
-        lz[L.y + i] = y;
-        lz[L.yprev + i] = y;
+    // eps_k = |y - (yprev, 0)| / |yprev|: lanes 0 .. 15 sum the numerator, 16 .. 31 the denominator
+    const bool upper = lane >= 16;
+    double sq = 0.0;
+    for (int i = lane & 15; i < n; i += 16) {
+        const double p = i < k ? lz[L.yprev + i] : 0.0;
+        const double d = upper ? p : sh.y[i] - p;
+        sq = fma(d, d, sq);
     }
-    // warp sums by a butterfly (a fixed order; every lane ends with the same totals)
-    for (int o = 16; o > 0; o >>= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, o);
-        den += __shfl_xor_sync(0xffffffffu, den, o);
-    }
+    __syncwarp();  // yprev has been read
+    for (int i = lane; i < n; i += 32) lz[L.y + i] = lz[L.yprev + i] = sh.y[i];
+    for (int o = 8; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    const double den = __shfl_sync(0xffffffffu, sq, 16);
+    const double num = sq;  // in lane 0
     if (lane == 0) {
         lz[L.alpha + k] = alpha_k;
         lz[L.beta + k] = beta_k;
-        const double eps = (k >= 1 && den > 0.0) ? sqrt(num / den) : -1.0;
+        double eps = -1.0;
+        if (k >= 1 && den > 0.0) {
+            const double q = plain_pos(den) ? num * rcp_pos(den) : num / den;
+            eps = plain_pos(q) ? q * rsqrt_pos(q) : sqrt(q);
+        }
         const bool brk = beta_k <= 1e-14 * tnorm;
         const bool conv = (tol > 0.0 && k >= 1 && eps <= tol);
         status[ST_EPS] = eps;
         status[ST_BREAK] = brk ? 1.0 : 0.0;
         status[ST_STOP] = (brk || conv) ? 1.0 : 0.0;
-        status[ST_INV_BETA] = brk ? 0.0 : 1.0 / beta_k;
+        status[ST_INV_BETA] = brk ? 0.0 : (plain_pos(beta_k) ? rcp_pos(beta_k) : 1.0 / beta_k);
     }
 }
 

@@ -19,17 +19,6 @@
 
 namespace rpb {
 
-// 1/sqrt(x) for a positive normal x: the hardware's approximation, then one fourth-order step of the
-// binomial series, y (1 + e/2 + 3 e^2/8 + 5 e^3/16) with e = 1 - x y^2 (Householder's iteration).
-__device__ __forceinline__ double rsqrt_pos(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
-    const double p = fma(e, fma(e, 0.3125, 0.375), 0.5);
-    return fma(e * y, p, y);
-}
-
 // a < b for non-negative doubles, on the bit patterns (off the float64 pipe)
 __device__ __forceinline__ bool less_bits(double a, double b)
 {

@@ -29,6 +29,48 @@ struct alignas(16) SrcF64 {
     double2 u;  // s Tz, 0
 };
 
+#ifdef __CUDACC__
+// 1/sqrt(x) for a positive normal x: the hardware's approximation, then one fourth-order step of the
+// binomial series, y (1 + e/2 + 3 e^2/8 + 5 e^3/16) with e = 1 - x y^2 (Householder's iteration).
+__device__ __forceinline__ double rsqrt_pos(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    const double p = fma(e, fma(e, 0.3125, 0.375), 0.5);
+    return fma(e * y, p, y);
+}
+
+// 1/d for a positive normal d: the hardware's approximation (relative error below 2^-23) and one
+// third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - d y.
+__device__ __forceinline__ double rcp_pos(double d)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// Positive and normal, below 2^1000: on the exponent bits (false for NaN).
+__device__ __forceinline__ bool plain_pos(double v)
+{
+    return (unsigned)(__double2hiint(v) - 0x00100000) < 0x7e600000u;
+}
+
+// sqrt(x) and 1/sqrt(x) of a sum of squares: a square root and a division are about 25 float64 instructions,
+// the reciprocal root 6.
+__device__ __forceinline__ void root_and_inverse(double x, double *root, double *inverse)
+{
+    if (plain_pos(x)) {
+        *inverse = rsqrt_pos(x);
+        *root = x * *inverse;
+    } else {
+        *root = sqrt(x);
+        *inverse = 1.0 / *root;
+    }
+}
+#endif
+
 // Geometry constants of the pair formula, in units where velocities carry 1/(8 pi eta).
 template <typename R>
 struct PairConsts {
