@@ -36,6 +36,13 @@ struct InstDesc {
     double *out;      // U (product)
 };
 
+// A block's share of an instance in the kernels over chunks of kGsChunk spheres, which are numbered instance by
+// instance.
+struct ChunkDesc {
+    int inst, first;    // instance, its first sphere (instance-local)
+    int chunk0, count;  // the instance's first chunk and its number of chunks
+};
+
 struct BlockDesc {
     int inst;
     int first;  // first target (instance-local) of this 128-target block
@@ -379,21 +386,31 @@ __device__ __forceinline__ uint4 philox4x32_10_b(uint4 c, uint32_t k0, uint32_t 
     return c;
 }
 
-// Element (c, i) of the packed vector: normal k = 3 il + c of instance inst_of[i] (il local index).
-__global__ void batch_philox_kernel(const InstDesc *__restrict__ inst, const int *__restrict__ inst_of, int64_t total,
-                                    uint32_t sid, double *__restrict__ out)
+// Normals k = 2p and 2p + 1 (k = 3 il + c, il local index) of both noise streams (blockIdx.y: 0 into W, 1 into
+// Wt), one block per chunk.  One thread per counter: the logarithm, square root and sincospi (about 80 float64 instructions, which
+// bound this kernel) serve the two normals they give; a thread per normal did them twice.
+__global__ void __launch_bounds__(256) batch_philox_kernel(const InstDesc *__restrict__ inst,
+                                                           const ChunkDesc *__restrict__ chunks, int64_t total,
+                                                           double *__restrict__ W, double *__restrict__ Wt)
 {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < 3 * total; r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = r / total, i = r - c * total;
-        const InstDesc &d = inst[inst_of[i]];
-        const int64_t k = 3 * (i - d.off) + c;
-        const uint4 w = philox4x32_10_b(make_uint4((uint32_t)(k >> 1), d.step, sid, 0u), d.seed_lo, d.seed_hi);
+    // a chunk of 256 spheres holds normals 768 q .. 768 q + 767 of its instance: 384 counters
+    const ChunkDesc c = chunks[blockIdx.x];
+    const InstDesc d = inst[c.inst];
+    const uint32_t sid = blockIdx.y;
+    double *out = sid ? Wt : W;
+    const int n = 3 * d.N, p0 = 3 * c.first / 2;
+    const int p1 = min((n + 1) / 2, p0 + 3 * kGsChunk / 2);
+    for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
+        const uint4 w = philox4x32_10_b(make_uint4((uint32_t)p, d.step, sid, 0u), d.seed_lo, d.seed_hi);
         const double two26 = 67108864.0, two_m53 = 1.1102230246251565e-16;
         const double u1 = ((double)(w.x >> 5) * two26 + (double)(w.y >> 6) + 1.0) * two_m53;
         const double u2 = ((double)(w.z >> 5) * two26 + (double)(w.w >> 6) + 1.0) * two_m53;
+        const double rad = sqrt(-2.0 * log(u1));
         double sn, cs;
         sincospi(2.0 * u2, &sn, &cs);
-        out[r] = sqrt(-2.0 * log(u1)) * ((k & 1) ? sn : cs);
+        const int ka = 2 * p, kb = ka + 1;
+        out[(int64_t)(ka % 3) * total + d.off + ka / 3] = rad * cs;
+        if (kb < n) out[(int64_t)(kb % 3) * total + d.off + kb / 3] = rad * sn;
     }
 }
 
@@ -439,10 +456,6 @@ __global__ void batch_rfd_combine_kernel(double *__restrict__ up_drift, const do
 // fixed order, so nothing depends on the companions.  (One block per instance left the largest instances
 // to one SM: of a served mix with suspensions of up to 32768 spheres, 24 instances, the dot products and
 // projections took 18% of a step; 7.7 of 42 ms.)
-struct ChunkDesc {
-    int inst, first;    // instance, its first sphere (instance-local)
-    int chunk0, count;  // the instance's first chunk and its number of chunks
-};
 
 __device__ __forceinline__ GsSpan chunk_span(const ChunkDesc &c, const InstDesc &d, int64_t total)
 {
@@ -536,16 +549,35 @@ __global__ void __launch_bounds__(128) batch_norm_init_kernel(const double *__re
     active[b] = nw > 0.0 ? 1 : 0;
 }
 
-// v[r] = w[r] * status_b[idx] for rows of active instances (all instances when active is null).
-__global__ void batch_scale_kernel(const double *__restrict__ w, const InstDesc *__restrict__ inst,
-                                   const int *__restrict__ inst_of, const int *__restrict__ active, int64_t total,
-                                   const double *__restrict__ lz, size_t lz_stride, size_t status_off, int idx,
-                                   double *__restrict__ v)
+// v = w * status_b[idx] for the active instances (all when active is null), and s_i v into the packed sources
+// of the next product, whose positions stay packed through a solve.
+__global__ void __launch_bounds__(kGsThreads) batch_scale_kernel(const double *__restrict__ w,
+                                                                 const InstDesc *__restrict__ inst,
+                                                                 const ChunkDesc *__restrict__ chunks,
+                                                                 const int *__restrict__ active, int64_t total,
+                                                                 const double *__restrict__ lz, size_t lz_stride,
+                                                                 size_t status_off, int idx, double *__restrict__ v,
+                                                                 const double *__restrict__ s, void *__restrict__ src,
+                                                                 int fp64)
 {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < 3 * total; r += (int64_t)gridDim.x * blockDim.x) {
-        const int b = inst_of[r % total];
-        if (active && !active[b]) continue;
-        v[r] = w[r] * lz[(size_t)b * lz_stride + status_off + idx];
+    const ChunkDesc c = chunks[blockIdx.x];
+    if (active && !active[c.inst]) return;
+    const double inv = lz[(size_t)c.inst * lz_stride + status_off + idx];
+    int64_t row[kGsRows];
+    gs_rows(chunk_span(c, inst[c.inst], total), row);
+#pragma unroll
+    for (int u = 0; u < kGsRows; ++u) {
+        const int64_t r = row[u];
+        if (r < 0) continue;
+        const double x = w[r] * inv;
+        v[r] = x;
+        const int q = r < total ? 0 : (r < 2 * total ? 1 : 2);
+        const int64_t i = r - q * total;
+        const double f = s[i] * x;
+        if (fp64)
+            reinterpret_cast<double *>((SrcF64 *)src + i)[3 + q] = f;
+        else
+            reinterpret_cast<float *>((SrcF32 *)src + i)[5 + q] = (float)f;
     }
 }
 
@@ -773,25 +805,25 @@ static int batch_gather(rpb_batch *bt, int which, double *packed, int to_caller)
     return cuda_fail(cudaGetLastError(), "batch gather");
 }
 
-// U = M_tt F + M_tr T over the packed layout; F or T may be null; active masks instances.
+// U = M_tt F + M_tr T over the packed layout; F or T may be null; active masks instances.  packed: the packed
+// sources hold these positions and s F already (T null).
 static int batch_product(rpb_batch *bt, const double *pos, const double *F, const double *T, double *U,
-                         const int *active)
+                         const int *active, bool packed = false)
 {
     const int64_t total = bt->total;
     const double a = bt->p.a;
     const double scale = 1.0 / (8.0 * kPi * bt->p.eta);
     const int pb = 256;
     const int gpack = (int)((total + pb - 1) / pb);
-    const SelfCoefs none = {nullptr, 0, 0.0, PairConsts<double>{}};  // the one-way kernels evaluate their self terms
+    const SelfCoefs sc = {bt->selfc, total, scale, make_consts<double>(a)};
     if (bt->p.precision == RPB_FP32 && bt->sym_ok) {
         SrcF32 *src = (SrcF32 *)bt->src;
-        const SelfCoefs sc = {bt->selfc, total, scale, make_consts<double>(a)};
-        pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, sc);
-        count_launches(1);
+        if (!packed) pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, sc);
+        count_launches(!packed);
         return batch_sym_apply(bt->sym, bt->stream, src, total, F, T, U, active, a, sc);
     } else if (bt->p.precision == RPB_FP32) {
         SrcF32 *src = (SrcF32 *)bt->src;
-        pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, none);
+        if (!packed) pack_f32_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, sc);
         const X2Consts c = make_x2_consts(a);
         const PairConsts<double> cd = make_consts<double>(a);
         if (T)
@@ -802,7 +834,7 @@ static int batch_product(rpb_batch *bt, const double *pos, const double *F, cons
                 src, bt->d_inst, bt->d_blocks, active, total, c, cd, a, scale, pos, F, T, U);
     } else {
         SrcF64 *src = (SrcF64 *)bt->src;
-        pack_f64_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, none);
+        if (!packed) pack_f64_kernel<<<gpack, pb, 0, bt->stream>>>(pos, F, T, (int)total, a, 1, src, sc);
         const PairConsts<double> c = make_consts<double>(a);
         if (T)
             batch_pair_f64_kernel<true><<<bt->nblocks, kPairThreads, 0, bt->stream>>>(
@@ -811,7 +843,7 @@ static int batch_product(rpb_batch *bt, const double *pos, const double *F, cons
             batch_pair_f64_kernel<false><<<bt->nblocks, kPairThreads, 0, bt->stream>>>(
                 src, bt->d_inst, bt->d_blocks, active, total, c, a, scale, pos, F, T, U);
     }
-    count_launches(2);
+    count_launches(packed ? 1 : 2);
     return cuda_fail(cudaGetLastError(), "batch pair kernels");
 }
 
@@ -867,8 +899,9 @@ static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, doub
     batch_dots_kernel<<<nc, kGsThreads, 0, main_st>>>(W, 0, 1, W, bt->d_inst, bt->d_chunks, nullptr, total, bt->red);
     batch_norm_init_kernel<<<(B + 3) / 4, 128, 0, main_st>>>(bt->red, bt->d_inst_chunks, B, bt->lz, bt->lz_stride,
                                                              L.status, bt->d_active);
-    batch_scale_kernel<<<ge, 256, 0, main_st>>>(W, bt->d_inst, bt->d_inst_of, nullptr, total, bt->lz, bt->lz_stride,
-                                                L.status, ST_INV_NW, V);
+    const int fp64 = bt->p.precision == RPB_FP64;
+    batch_scale_kernel<<<nc, kGsThreads, 0, main_st>>>(W, bt->d_inst, bt->d_chunks, nullptr, total, bt->lz,
+                                                       bt->lz_stride, L.status, ST_INV_NW, V, bt->selfc, bt->src, fp64);
     count_launches(3);
     for (int k = 0; k < max_iter; ++k) {
         const bool cond = graph && k >= 1;
@@ -879,7 +912,7 @@ static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, doub
         cudaStream_t st = bt->stream;
         const uint64_t before = rpb_launch_count();
         const double *vk = V + (size_t)k * ld;
-        rc = batch_product(bt, pos, vk, nullptr, w, bt->d_active);
+        rc = batch_product(bt, pos, vk, nullptr, w, bt->d_active, true);
         const int nv = k + 1;
         if (!rc) {
             batch_dots_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, nv, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
@@ -908,8 +941,9 @@ static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, doub
                 if (*bt->h_nactive == 0) break;
             }
             if (k + 1 < max_iter) {
-                batch_scale_kernel<<<ge, 256, 0, st>>>(w, bt->d_inst, bt->d_inst_of, bt->d_active, total, bt->lz,
-                                                       bt->lz_stride, L.status, ST_INV_BETA, V + (size_t)(k + 1) * ld);
+                batch_scale_kernel<<<nc, kGsThreads, 0, st>>>(w, bt->d_inst, bt->d_chunks, bt->d_active, total, bt->lz,
+                                                              bt->lz_stride, L.status, ST_INV_BETA,
+                                                              V + (size_t)(k + 1) * ld, bt->selfc, bt->src, fp64);
                 count_launches(1);
             }
             rc = cuda_fail(cudaGetLastError(), "batch lanczos kernels");
@@ -963,9 +997,8 @@ static int batch_step_body(rpb_batch *bt, double dt, double delta, double tol, i
     batch_fill3_kernel<<<ge, 256, 0, st>>>(v[V_T], total, fp->torque[0], fp->torque[1], fp->torque[2]);
     count_launches(2);
     if ((rc = batch_product(bt, v[V_POS], v[V_F], v[V_T], v[V_UN], nullptr))) return rc;
-    batch_philox_kernel<<<ge, 256, 0, st>>>(bt->d_inst, bt->d_inst_of, total, 0u, v[V_W]);
-    batch_philox_kernel<<<ge, 256, 0, st>>>(bt->d_inst, bt->d_inst_of, total, 1u, v[V_WT]);
-    count_launches(2);
+    batch_philox_kernel<<<dim3(bt->nchunks, 2), 256, 0, st>>>(bt->d_inst, bt->d_chunks, total, v[V_W], v[V_WT]);
+    count_launches(1);
     if ((rc = batch_lanczos(bt, v[V_POS], v[V_W], v[V_G], tol, max_iter, graph))) return rc;
     // RFD: two products at the displaced configurations, regularised anew
     batch_displace_kernel<<<ge, 256, 0, st>>>(v[V_POS], v[V_WT], n, 0.5 * delta, v[V_PA], v[V_PB]);
