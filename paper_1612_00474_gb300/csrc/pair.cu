@@ -1868,6 +1868,104 @@ __global__ void __launch_bounds__(128) forces_kernel(const double *__restrict__ 
     }
 }
 
+// Small suspensions: sixteen spheres per block, eight threads each, in one launch without cell lists.  The
+// sources are screened in float32 against the same radius, kGroupChunk at a time; every thread marks its
+// candidates in a bit mask, the eight threads of a sphere write theirs to its list one after another (a
+// list holds a whole chunk, so it cannot overflow), and the list is evaluated in float64 by the eight in
+// turn.  What bounds it: the float64 chain of the pairs (about 40 instructions each, 64 cycles a warp
+// instruction whatever the active lanes): about 15 near pairs a sphere are two or three a thread here, where a
+// thread per sphere took the whole list of the longest in its warp, after six short launches that built
+// the cells (62 us a call from 64 to 4096 spheres; the pseudo-periodic all-pairs kernel 52 us at 256).  Twenty
+// steps of 256 spheres: 7.75 -> 7.03 ms in float64, 23.1 -> 22.0 ms pseudo-periodic.
+constexpr int kGroupTargets = 16, kGroupThreads = 8, kGroupChunk = 1024;
+constexpr int64_t kGroupMaxN = 8192;  // beyond, screening all pairs costs more than the cell lists
+
+template <bool PER>
+__global__ void __launch_bounds__(kGroupTargets * kGroupThreads) forces_group_kernel(
+    const double *__restrict__ pos, int N, double a, double weight, double U0, double b, float cut2,
+    double *__restrict__ F, double Lx, double Ly)
+{
+    constexpr int kMask = kGroupChunk / kGroupThreads / 32;
+    __shared__ float sx[kGroupChunk], sy[kGroupChunk], sz[kGroupChunk];
+    __shared__ unsigned short list[kGroupTargets][kGroupChunk];
+    const int tid = threadIdx.x, g = tid / kGroupThreads, p = tid % kGroupThreads;
+    const int i = blockIdx.x * kGroupTargets + g, ic = min(i, N - 1);
+    const double xi = pos[ic], yi = pos[N + ic], zi = pos[2 * N + ic];
+    const float xf = (float)xi, yf = (float)yi, zf = (float)zi;
+    const double f0 = U0 / b, inv_b = 1.0 / b;
+    const float fLx = (float)Lx, fLy = (float)Ly;
+    const float fiLx = PER ? 1.f / fLx : 0.f, fiLy = PER ? 1.f / fLy : 0.f;
+    double fx = 0.0, fy = 0.0, fz = 0.0;
+    for (int base = 0; base < N; base += kGroupChunk) {
+        const int n = min(kGroupChunk, N - base);
+        for (int j = tid; j < n; j += kGroupTargets * kGroupThreads) {
+            sx[j] = (float)pos[base + j];
+            sy[j] = (float)pos[N + base + j];
+            sz[j] = (float)pos[2 * N + base + j];
+        }
+        __syncthreads();
+        unsigned mask[kMask];
+        int cnt = 0;
+#pragma unroll
+        for (int w = 0; w < kMask; ++w) {
+            unsigned m = 0;
+            const int j0 = p + 32 * w * kGroupThreads;
+            if (j0 - p < n) {
+#pragma unroll 8
+                for (int k = 0; k < 32; ++k) {
+                    const int j = j0 + k * kGroupThreads;
+                    float dx = xf - sx[j], dy = yf - sy[j];
+                    const float dz = zf - sz[j];
+                    if (PER) {
+                        dx -= fLx * rintf(dx * fiLx);
+                        dy -= fLy * rintf(dy * fiLy);
+                    }
+                    if (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < cut2 && j < n && base + j != i) m |= 1u << k;
+                }
+            }
+            mask[w] = m;
+            cnt += __popc(m);
+        }
+        // places of this thread's candidates in its sphere's list
+        int end = cnt;
+        for (int o = 1; o < kGroupThreads; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, end, o, kGroupThreads);
+            if (p >= o) end += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, end, kGroupThreads - 1, kGroupThreads);
+        int at = end - cnt;
+#pragma unroll
+        for (int w = 0; w < kMask; ++w)
+            for (unsigned m = mask[w]; m; m &= m - 1)
+                list[g][at++] = (unsigned short)(p + (32 * w + __ffs(m) - 1) * kGroupThreads);
+        __syncwarp();
+        for (int e = p; e < total; e += kGroupThreads) {
+            const int j = base + list[g][e];
+            double dx = xi - pos[j], dy = yi - pos[N + j];
+            const double dz = zi - pos[2 * N + j];
+            if (PER) {
+                dx -= Lx * rint(dx / Lx);
+                dy -= Ly * rint(dy / Ly);
+            }
+            const double m = steric_pair_factor(dx * dx + dy * dy + dz * dz, 2.0 * a, f0, inv_b);
+            fx += m * dx;
+            fy += m * dy;
+            fz += m * dz;
+        }
+        __syncthreads();  // the tile and the lists are written again
+    }
+    for (int o = kGroupThreads / 2; o > 0; o >>= 1) {
+        fx += __shfl_xor_sync(0xffffffffu, fx, o);
+        fy += __shfl_xor_sync(0xffffffffu, fy, o);
+        fz += __shfl_xor_sync(0xffffffffu, fz, o);
+    }
+    if (p == 0 && i < N) {
+        F[i] = fx;
+        F[N + i] = fy;
+        F[2 * N + i] = fz + ((zi < a ? f0 : f0 * exp(-(zi - a) / b)) - weight);
+    }
+}
+
 int forces_impl(rpb_ctx *ctx, int64_t N, const double *pos, const rpb_force_params *fp, double *F)
 {
     const double a = ctx->p.a;
@@ -1875,13 +1973,24 @@ int forces_impl(rpb_ctx *ctx, int64_t N, const double *pos, const rpb_force_para
     const double rcm = r_cut * 1.01 + 0.01 * a;
     const float cut2 = (float)(rcm * rcm);
     const int n = (int)N;
+    const unsigned groups = (unsigned)((N + kGroupTargets - 1) / kGroupTargets);
     cudaStream_t st = ctx->stream;
     if (ctx->Lx > 0.0) {
         const int pb = 256;
         wrap_kernel<<<(unsigned)((N + pb - 1) / pb), pb, 0, st>>>(pos, n, ctx->Lx, ctx->Ly, ctx->ws.pos_w);
-        forces_kernel<true><<<(unsigned)((N + 127) / 128), 128, 0, st>>>(ctx->ws.pos_w, n, a, fp->weight, fp->U0,
-                                                                         fp->b, cut2, F, ctx->Lx, ctx->Ly);
+        if (N <= kGroupMaxN)
+            forces_group_kernel<true><<<groups, kGroupTargets * kGroupThreads, 0, st>>>(
+                ctx->ws.pos_w, n, a, fp->weight, fp->U0, fp->b, cut2, F, ctx->Lx, ctx->Ly);
+        else
+            forces_kernel<true><<<(unsigned)((N + 127) / 128), 128, 0, st>>>(ctx->ws.pos_w, n, a, fp->weight, fp->U0,
+                                                                             fp->b, cut2, F, ctx->Lx, ctx->Ly);
         count_launches(2);
+        return cuda_fail(cudaGetLastError(), "forces kernel");
+    }
+    if (N <= kGroupMaxN) {
+        forces_group_kernel<false><<<groups, kGroupTargets * kGroupThreads, 0, st>>>(pos, n, a, fp->weight, fp->U0,
+                                                                                     fp->b, cut2, F, 0.0, 0.0);
+        count_launches(1);
         return cuda_fail(cudaGetLastError(), "forces kernel");
     }
     // buckets of cells of side = the screen radius, then the bucket force pass; the all-pairs kernel
@@ -1897,7 +2006,7 @@ int forces_impl(rpb_ctx *ctx, int64_t N, const double *pos, const rpb_force_para
     cell_scan_kernel<<<1, 1024, 0, st>>>(L.count, nb, L.start, L.fill);
     cell_fill_kernel<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(n, L.cellof, L.fill, L.idx);
     cell_sort_kernel<<<nb / 256, 256, 0, st>>>(pos, n, nb, L.start, L.idx, L.posf, L.hdr);
-    // small systems in 32-sphere blocks: their float64 near pairs then spread over more SMs
+    // up to 128 x SMs spheres in 32-sphere blocks: their float64 near pairs then spread over more SMs
     const int fb = N < 128 * ctx->num_sms ? 32 : 128;
     forces_cell_kernel<<<(unsigned)((N + fb - 1) / fb), fb, 0, st>>>(pos, n, a, fp->weight, fp->U0, fp->b, cut2, inv_h,
                                                                      G, L.hdr, L.start, L.idx, L.posf, F);
