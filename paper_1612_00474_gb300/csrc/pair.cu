@@ -360,7 +360,9 @@ __device__ __forceinline__ float2 shift2(float2 d, float n, float Lh, float Ll)
 // PER: pseudo-periodic boundaries (Appendix B): each pair's offset is taken at its minimum image and
 // the block is summed over that image and its eight shifts by one period (reciprocity holds image by
 // image: the reversed pair's image at -s is the transposed block); the sphere's own unshifted image
-// is the self term of the reduce kernel.
+// is the self term of the reduce kernel.  Three images share one vote on the overlap branch, so that
+// their blocks are straight-line code with three chains in flight: small cells have one warp per
+// scheduler and wait for latencies (a step of 256 spheres 1.11 -> 0.93 ms; in order, so the same bits).
 // BATCH: the tiles belong to many suspensions packed one after another (sinst: one record per
 // suspension; a segment's pad field names its suspension, whose tiles are numbered from tile0);
 // segments of suspensions with active[] == 0 are skipped.
@@ -379,7 +381,6 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
 {
     constexpr int P = kTile / 2;
     constexpr int NC = RHS2 ? 6 : 3;
-    constexpr int NS = PER ? 9 : 1;  // image shifts per pair
     static_assert(!(PER && RHS2), "the two-right-hand-side form has no pseudo-periodic variant");
     static_assert(!(BATCH && (PER || RHS2)), "the batched form is the plain or the torque form");
     // G source pairs (2G sources) are evaluated per step and then reduce-scattered over the warp
@@ -523,27 +524,58 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
                 const float2 g = TORQUE ? make_float2(sG[k].x, sG[k].y) : zero2;
                 float2 rx0 = add2(sub2(txh, make_float2(a.x, a.y)), sub2(txl, make_float2(b.x, b.y)));
                 float2 ry0 = add2(sub2(tyh, make_float2(a.z, a.w)), sub2(tyl, make_float2(b.z, b.w)));
-                if (PER) {
+                if constexpr (PER) {
                     rx0 = min_image2(rx0, pl.xh, pl.xl, pl.ix);
                     ry0 = min_image2(ry0, pl.yh, pl.yl, pl.iy);
-                }
-                for (int sh = 0; sh < NS; ++sh) {
-                    const float2 rx = PER ? shift2(rx0, (float)(sh / 3 - 1), pl.xh, pl.xl) : rx0;
-                    const float2 ry = PER ? shift2(ry0, (float)(sh % 3 - 1), pl.yh, pl.yl) : ry0;
+                    const float2 zj = make_float2(cc.x, cc.y), rz = sub2(tz2, zj);
+                    for (int sx = -1; sx <= 1; ++sx) {
+                        const float2 rx = shift2(rx0, (float)sx, pl.xh, pl.xl);
+                        float2 ry[3], rho2[3], r2[3];
+                        bool near = false;
+#pragma unroll
+                        for (int q = 0; q < 3; ++q) {
+                            ry[q] = shift2(ry0, (float)(q - 1), pl.yh, pl.yl);
+                            rho2[q] = fma2(rx, rx, mul2(ry[q], ry[q]));
+                            r2[q] = fma2(rz, rz, rho2[q]);
+                            near = near || r2[q].x < c.four_a2 || r2[q].y < c.four_a2;
+                        }
+                        auto images = [&](bool close) {
+#pragma unroll
+                            for (int im = 0; im < 3; ++im) {
+                                float2 dd[3] = {zero2, zero2, zero2};
+                                pair_velocity_x2_geo<TORQUE>(rx, ry[im], rz, rho2[im], r2[im], close, tz2, zj,
+                                                             make_float2(cc.z, cc.w), make_float2(d.x, d.y),
+                                                             make_float2(d.z, d.w), make_float2(e.x, e.y),
+                                                             make_float2(e.z, e.w), g, c, dd[0], dd[1], dd[2]);
+                                // source 2k + hh is this thread's own sphere: its unshifted image is the self term
+                                const bool self = k == pp && sx == 0 && im == 1;
+#pragma unroll
+                                for (int q = 0; q < 3; ++q) {
+                                    if (self && hh == 0) dd[q].x = 0.f;
+                                    if (self && hh == 1) dd[q].y = 0.f;
+                                    u[q] = add2(u[q], dd[q]);
+                                }
+                            }
+                        };
+                        if (__any_sync(0xffffffffu, near))
+                            images(true);
+                        else
+                            images(false);
+                    }
+                } else {
                     float2 dd[NC];
 #pragma unroll
                     for (int q = 0; q < NC; ++q) dd[q] = zero2;
-                    pair_velocity_x2<TORQUE>(rx, ry, tz2, make_float2(cc.x, cc.y), make_float2(cc.z, cc.w),
+                    pair_velocity_x2<TORQUE>(rx0, ry0, tz2, make_float2(cc.x, cc.y), make_float2(cc.z, cc.w),
                                              make_float2(d.x, d.y), make_float2(d.z, d.w), make_float2(e.x, e.y),
                                              make_float2(e.z, e.w), g, c, dd[0], dd[1], dd[2]);
                     if (RHS2) {
                         const float4 pv = sP[k];
-                        pair_velocity_x2<false>(rx, ry, tz2, make_float2(cc.x, cc.y), make_float2(pv.x, pv.y),
+                        pair_velocity_x2<false>(rx0, ry0, tz2, make_float2(cc.x, cc.y), make_float2(pv.x, pv.y),
                                                 make_float2(pv.z, pv.w), sQ[k], zero2, zero2, zero2, c, dd[3 % NC],
                                                 dd[4 % NC], dd[5 % NC]);
                     }
-                    // source 2k + hh is this thread's own sphere: its unshifted image is the self term
-                    if (k == pp && (!PER || sh == 4)) {
+                    if (k == pp) {  // source 2k + hh is this thread's own sphere
 #pragma unroll
                         for (int q = 0; q < NC; ++q) {
                             if (hh == 0)
@@ -593,21 +625,34 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
                         const float2 rz = sub2(tz2, zj);
 #pragma unroll
                         for (int q = 0; q < NC; ++q) v[h][q] = zero2;
-                        for (int sh = 0; sh < 9; ++sh) {
-                            const float2 rx = shift2(rx0, (float)(sh / 3 - 1), pl.xh, pl.xl);
-                            const float2 ry = shift2(ry0, (float)(sh % 3 - 1), pl.yh, pl.yl);
-                            const float2 rho2 = fma2(rx, rx, mul2(ry, ry));
-                            const float2 r2 = fma2(rz, rz, rho2);
-                            const bool close = __any_sync(0xffffffffu, r2.x < c.four_a2 || r2.y < c.four_a2);
-                            float2 vx, vy, vz;
-                            pair_sym_x2<TORQUE>(rx, ry, rz, rho2, r2, close, tz2, zj, m2zj, m4zj2, six_zi, six_zj,
-                                                make_float2(cc.z, cc.w),
-                                                make_float2(d.x, d.y), make_float2(d.z, d.w), Gx, Gy, Gz,
-                                                make_float2(e.x, e.y), make_float2(e.z, e.w), g, Hx, Hy, Hz, c,
-                                                u[0], u[1], u[2], vx, vy, vz);
-                            v[h][0] = add2(v[h][0], vx);
-                            v[h][1] = add2(v[h][1], vy);
-                            v[h][2] = add2(v[h][2], vz);
+                        for (int sx = -1; sx <= 1; ++sx) {
+                            const float2 rx = shift2(rx0, (float)sx, pl.xh, pl.xl);
+                            float2 ry[3], rho2[3], r2[3];
+                            bool near = false;
+#pragma unroll
+                            for (int im = 0; im < 3; ++im) {
+                                ry[im] = shift2(ry0, (float)(im - 1), pl.yh, pl.yl);
+                                rho2[im] = fma2(rx, rx, mul2(ry[im], ry[im]));
+                                r2[im] = fma2(rz, rz, rho2[im]);
+                                near = near || r2[im].x < c.four_a2 || r2[im].y < c.four_a2;
+                            }
+                            auto images = [&](bool close) {
+#pragma unroll
+                                for (int im = 0; im < 3; ++im) {
+                                    float2 vx, vy, vz;
+                                    pair_sym_x2<TORQUE>(rx, ry[im], rz, rho2[im], r2[im], close, tz2, zj, m2zj, m4zj2, six_zi,
+                                                        six_zj, make_float2(cc.z, cc.w), make_float2(d.x, d.y),
+                                                        make_float2(d.z, d.w), Gx, Gy, Gz, make_float2(e.x, e.y),
+                                                        make_float2(e.z, e.w), g, Hx, Hy, Hz, c, u[0], u[1], u[2], vx, vy, vz);
+                                    v[h][0] = add2(v[h][0], vx);
+                                    v[h][1] = add2(v[h][1], vy);
+                                    v[h][2] = add2(v[h][2], vz);
+                                }
+                            };
+                            if (__any_sync(0xffffffffu, near))
+                                images(true);
+                            else
+                                images(false);
                         }
                     }
                 }
@@ -748,7 +793,13 @@ constexpr int kTtMinBlocks = 5;     // resident CTAs per SM of the translation-t
                                     // with the polynomial coefficient form; 4 CTAs measured 2.6% slower)
 constexpr int kFusedMinBlocks = 4;  // resident CTAs per SM of the form with torques
 constexpr int kRhs2MinBlocks = 3;  // resident CTAs per SM of the two-right-hand-side form
-constexpr int kPerMinBlocks = 4;   // resident CTAs per SM of the pseudo-periodic forms
+// Resident CTAs per SM of the pseudo-periodic forms (the form with torques spills at 4; at 12000 spheres,
+// one image per block against three: 1590 -> 1463 us, with torques 2236 -> 2079 us)
+constexpr int kPerMinBlocks = 4, kPerFusedMinBlocks = 3;
+// Where the schedule has at most two CTAs per SM, the forms compiled for two: occupancy buys nothing there
+// and the registers keep the constants and more of a step in flight (a step of 1024 spheres 426 -> 411 us,
+// pseudo-periodic 256 spheres 930 -> 905 us; with full waves they are 3% slower, 5.58 ms a product at 65536).
+constexpr int kSmallMinBlocks = 2;
 
 // Capacity of the schedule: at most kSymMaxCtaPerSm x SMs CTAs and that many plus nb segments.
 constexpr int kSymMaxCtaPerSm = 64;
@@ -846,6 +897,9 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
         if (T)
             pair_f32x2_sym_kernel<kFusedMinBlocks, true><<<sc->ncta, kPairThreads, 0, st>>>(src, N, ctas, segs, c, cs,
                                                                                             w.sym_tgt, w.sym_src);
+        else if (sc->ncta <= kSmallMinBlocks * ctx->num_sms)
+            pair_f32x2_sym_kernel<kSmallMinBlocks, false><<<sc->ncta, kPairThreads, 0, st>>>(
+                src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src);
         else
             pair_f32x2_sym_kernel<kTtMinBlocks, false><<<sc->ncta, kPairThreads, 0, st>>>(src, N, ctas, segs, c, cs,
                                                                                           w.sym_tgt, w.sym_src);
@@ -884,12 +938,19 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
     pl.ix = 1.f / pl.xh;
     pl.iy = 1.f / pl.yh;
     if (sc->ncta > 0) {
-        if (T)
-            pair_f32x2_sym_kernel<kPerMinBlocks, true, false, true><<<sc->ncta, kPairThreads, 0, st>>>(
-                src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, pl);
+        const bool small = sc->ncta <= kSmallMinBlocks * ctx->num_sms;
+        auto run = [&](auto kernel) {
+            kernel<<<sc->ncta, kPairThreads, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, pl, nullptr,
+                                                      nullptr);
+        };
+        if (T && small)
+            run(pair_f32x2_sym_kernel<kSmallMinBlocks, true, false, true>);
+        else if (T)
+            run(pair_f32x2_sym_kernel<kPerFusedMinBlocks, true, false, true>);
+        else if (small)
+            run(pair_f32x2_sym_kernel<kSmallMinBlocks, false, false, true>);
         else
-            pair_f32x2_sym_kernel<kPerMinBlocks, false, false, true><<<sc->ncta, kPairThreads, 0, st>>>(
-                src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, pl);
+            run(pair_f32x2_sym_kernel<kPerMinBlocks, false, false, true>);
     }
     pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
         w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
