@@ -1,5 +1,6 @@
 // api.cu -- the extern "C" entry points declared in include/rpb.h: argument checks, context and
 // scratch management, and the sequence of the Adams-Bashforth step.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -7,7 +8,9 @@
 #include <cstring>
 #include <atomic>
 #include <new>
+#include <utility>
 
+#include "grid_plan.h"
 #include "rpb_internal.cuh"
 #include "sym64_plan.h"
 
@@ -106,18 +109,88 @@ int check_step_args(rpb_ctx *ctx, int64_t N, const double *pos, const double *U_
     return RPB_OK;
 }
 
+// Largest suspensions whose drift runs beside the Lanczos iterations: those whose products leave most of the
+// GPU idle (up to a wave of CTAs), so that the drift's two products, their packing and their noise cost
+// little: 20 steps of 256 spheres 7.03 -> 6.21 ms in float64 and 17.5 -> 14.4 ms pseudo-periodic in float32, a
+// float32 step of 4096 spheres 807 -> 765 us.  Beyond, both are bound by the arithmetic (a float64 step of
+// 4096: 15.46 and 15.41 ms) and the side scratch would only take memory.
+constexpr int64_t kSideMaxF32 = 4096, kSideMaxF64 = 1024;
+static int64_t side_max(const rpb_params &p, int64_t max_N)
+{
+    return std::min<int64_t>(max_N, p.precision == RPB_FP64 ? kSideMaxF64 : kSideMaxF32);
+}
+
+// While it lives, the context's products use the side scratch and its stream (host state only: the kernels
+// enqueued meanwhile keep the pointers they were given).
+struct SideScope {
+    rpb_ctx *c;
+    cudaStream_t stream;
+    explicit SideScope(rpb_ctx *ctx) : c(ctx), stream(ctx->stream)
+    {
+        swap();
+        c->stream = c->side_stream;
+    }
+    ~SideScope()
+    {
+        swap();
+        c->stream = stream;
+    }
+    void swap()
+    {
+        Workspace &w = c->ws;
+        SideSpace &q = c->side;
+        std::swap(w.src, q.src);
+        std::swap(w.partial, q.partial);
+        std::swap(w.partial_bytes, q.partial_bytes);
+        std::swap(w.selfc, q.selfc);
+        std::swap(w.w, q.w);
+        std::swap(w.pos_w, q.pos_w);
+        std::swap(w.sym64, q.sym64);
+        std::swap(w.sym64_N, q.sym64_N);
+        std::swap(w.sym_tgt, q.sym_tgt);
+        std::swap(w.sym_tgt_bytes, q.sym_tgt_bytes);
+        std::swap(w.sym_src, q.sym_src);
+        std::swap(w.sym_src_bytes, q.sym_src_bytes);
+    }
+};
+
+// The drift of a step enqueued beside what follows on the context's stream (noise W~, the two displaced
+// products, their combination); side_join() orders the stream after it.
+static int side_drift(rpb_ctx *ctx, int64_t N, const double *pos, uint64_t seed, uint32_t step,
+                      const unsigned int *d_step, double delta, int one_sided)
+{
+    int rc;
+    if (!ctx->side_stream &&
+        ((rc = cuda_fail(cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking), "side stream")) ||
+         (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->side_fork, cudaEventDisableTiming), "side event")) ||
+         (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->side_join, cudaEventDisableTiming), "side event"))))
+        return rc;
+    if ((rc = pair_prepare(ctx, N)) ||  // the symmetric schedule is shared by both streams
+        (rc = cuda_fail(cudaEventRecord(ctx->side_fork, ctx->stream), "event record")) ||
+        (rc = cuda_fail(cudaStreamWaitEvent(ctx->side_stream, ctx->side_fork, 0), "stream wait")))
+        return rc;
+    {
+        SideScope side(ctx);
+        rc = philox_impl(ctx, N, seed, step, 1u, 0u, ctx->ws.vec_e, d_step);
+        if (!rc) rc = rfd_impl(ctx, N, pos, ctx->ws.vec_e, delta, ctx->ws.vec_g, one_sided);
+    }
+    const int jrc = cuda_fail(cudaEventRecord(ctx->side_join, ctx->side_stream), "event record");
+    return rc ? rc : jrc;
+}
+
 // One time step (Eq. AB, or Eq. EM with scheme = RPB_SCHEME_EM), enqueued on ctx->stream.  gr == null:
 // the Lanczos stop is read back per iteration and stats are written.  gr != null: the step is being
 // captured into a graph (rpb_run): the step index and the first-step flag come from gr->state on the
 // device, Lanczos iterations after the first are conditional nodes, and nothing is read back.
-int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t step, uint64_t seed, double dt,
-              double delta, double tol, int max_iter, const rpb_force_params *fp, int scheme, int rfd,
-              rpb_step_stats *stats, LzGraph *gr)
+static int step_body(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t step, uint64_t seed, double dt,
+                     double delta, double tol, int max_iter, const rpb_force_params *fp, int scheme, int rfd,
+                     rpb_step_stats *stats, LzGraph *gr, bool beside)
 {
     int rc;
     Workspace &w = ctx->ws;
     const unsigned int *d_step = gr ? &gr->state->step : nullptr;
     double *F = w.vec_a, *T = w.vec_b, *Un = w.vec_c, *W = w.vec_d, *Wt = w.vec_e, *g = w.vec_f, *drift = w.vec_g;
+    if (beside && (rc = side_drift(ctx, N, pos, seed, step, d_step, delta, rfd == RPB_RFD_ONE_SIDED))) return rc;
     if ((rc = forces_impl(ctx, N, pos, fp, F))) return rc;
     if ((rc = fill_torque(ctx, N, fp->torque, T))) return rc;
     int iters = 0, conv = 0;
@@ -125,7 +198,7 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
     int lrc = RPB_OK;
     if (ctx->p.kT > 0.0) {
         if ((rc = philox_impl(ctx, N, seed, step, 0u, 0u, W, d_step))) return rc;
-        if ((rc = philox_impl(ctx, N, seed, step, 1u, 0u, Wt, d_step))) return rc;
+        if (!beside && (rc = philox_impl(ctx, N, seed, step, 1u, 0u, Wt, d_step))) return rc;
         if (mobility_apply2_ok(ctx, N)) {
             // the deterministic velocity and the first Lanczos product M v_0 share one pair pass
             if ((rc = lanczos_precond_prepare(ctx, N, pos)) || (rc = lanczos_init(ctx, N, W, false, gr)) ||
@@ -137,7 +210,11 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
             lrc = lanczos_impl(ctx, N, pos, W, g, tol, max_iter, ctx->hook == nullptr, &iters, &err, &conv, gr);
         }
         if (lrc != RPB_OK && lrc != RPB_ENOCONV) return lrc;
-        if ((rc = rfd_impl(ctx, N, pos, Wt, delta, drift, rfd == RPB_RFD_ONE_SIDED))) return rc;
+        if (beside)
+            rc = cuda_fail(cudaStreamWaitEvent(ctx->stream, ctx->side_join, 0), "stream wait");
+        else
+            rc = rfd_impl(ctx, N, pos, Wt, delta, drift, rfd == RPB_RFD_ONE_SIDED);
+        if (rc) return rc;
     } else {
         if ((rc = mobility_apply_impl(ctx, N, pos, F, T, Un))) return rc;
         // kT = 0: no Brownian increment and no drift (both carry a factor kT); the deterministic
@@ -164,6 +241,18 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
         return RPB_ENOCONV;
     }
     return RPB_OK;
+}
+
+int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t step, uint64_t seed, double dt,
+              double delta, double tol, int max_iter, const rpb_force_params *fp, int scheme, int rfd,
+              rpb_step_stats *stats, LzGraph *gr)
+{
+    const bool beside = ctx->p.kT > 0.0 && !ctx->hook && N <= ctx->side.max_N;
+    const int rc = step_body(ctx, N, pos, U_prev, step, seed, dt, delta, tol, max_iter, fp, scheme, rfd, stats, gr, beside);
+    // a step that failed half way: the stream is still ordered after the drift's reads of pos
+    if (rc && rc != RPB_ENOCONV && beside && !gr && ctx->side_join)
+        cudaStreamWaitEvent(ctx->stream, ctx->side_join, 0);
+    return rc;
 }
 
 }  // namespace rpb
@@ -239,6 +328,18 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
         sym64_bytes = sizeof(double) * (size_t)(sym64_tgt_elems(max_N, c->num_sms) + sym64_src_elems(max_N, c->num_sms));
         if (sym64_bytes > ((size_t)8 << 30)) sym64_bytes = 0;
     }
+    w.sym64_N = max_N;
+    SideSpace &side = c->side;
+    const int64_t ns = side_max(*p, max_N);
+    const size_t svb = (size_t)3 * ns * sizeof(double);
+    const bool f32 = p->precision == RPB_FP32;
+    side.max_N = ns;
+    side.sym64_N = ns;
+    side.partial_bytes = f32 ? (size_t)kMaxSplitsF32 * svb : pair_partial_bytes(ns, c->num_sms);
+    side.sym_tgt_bytes = f32 ? sym_tgt_part_bytes(ns, c->num_sms) : 0;
+    side.sym_src_bytes = f32 ? sym_src_part_bytes(ns) : 0;
+    const size_t side64 =
+        f32 ? 0 : sizeof(double) * (size_t)(sym64_tgt_elems(ns, c->num_sms) + sym64_src_elems(ns, c->num_sms));
     struct {
         void **ptr;
         size_t bytes;
@@ -263,6 +364,14 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
         {(void **)&w.vec_f, vb},
         {(void **)&w.vec_g, vb},
         {(void **)&w.sym64, sym64_bytes},
+        {&side.src, (size_t)ns * sizeof(SrcF64)},
+        {&side.partial, side.partial_bytes},
+        {(void **)&side.selfc, (size_t)4 * ns * sizeof(double)},
+        {(void **)&side.w, svb},
+        {(void **)&side.pos_w, svb},
+        {(void **)&side.sym64, side64},
+        {(void **)&side.sym_tgt, side.sym_tgt_bytes},
+        {(void **)&side.sym_src, side.sym_src_bytes},
     };
     // one allocation, each array on a 256-byte boundary
     size_t total = 0;
@@ -333,6 +442,10 @@ int rpb_destroy(rpb_ctx *ctx)
     g_err[0] = 0;
     int rc = cuda_fail(cudaStreamSynchronize(ctx->stream), "rpb_destroy sync");
     run_free(ctx);
+    if (ctx->side_stream) cudaStreamSynchronize(ctx->side_stream);
+    if (ctx->side_fork) cudaEventDestroy(ctx->side_fork);
+    if (ctx->side_join) cudaEventDestroy(ctx->side_join);
+    if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
     if (ctx->lz_ev) cudaEventDestroy(ctx->lz_ev);
     free_ws(ctx->ws);
     delete ctx;

@@ -583,7 +583,8 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
             stopped = hs[ST_STOP] != 0.0;
         }
     }
-    combine_kernel<<<blas_grid(n, ctx->num_sms), kBlasThreads, 0, main_st>>>(
+    const int tb = elem_threads(n, ctx->num_sms);
+    combine_kernel<<<tb == 32 ? (unsigned)((n + 31) / 32) : blas_grid(n, ctx->num_sms), tb, 0, main_st>>>(
         w.V, A.ld, n, m, w.lz + A.L.y, g, gr ? &gr->state->m : nullptr);
     count_launches(1);
     if (ctx->precond && (rc = precond_scale(ctx, N, g, g, true))) return rc;  // g = D^{1/2} y

@@ -810,16 +810,23 @@ size_t sym_src_part_bytes(int64_t max_N)
     return (size_t)(nb * (nb - 1) / 2) * 3 * kTile * sizeof(float);
 }
 
+// CTAs of any schedule up to max_N spheres: no more than the triangle has units.
+static int64_t sym_max_ctas(int64_t max_N, int num_sms)
+{
+    const int64_t nb = (max_N + kTile - 1) / kTile;
+    return std::min<int64_t>((int64_t)kSymMaxCtaPerSm * num_sms, nb * (nb + 1) / 2);
+}
+
 size_t sym_tgt_part_bytes(int64_t max_N, int num_sms)
 {
     const int64_t nb = (max_N + kTile - 1) / kTile;
-    return (size_t)(nb + (int64_t)kSymMaxCtaPerSm * num_sms + 1) * 3 * kTile * sizeof(double);
+    return (size_t)(nb + sym_max_ctas(max_N, num_sms) + 1) * 3 * kTile * sizeof(double);
 }
 
 size_t sym_index_ints(int64_t max_N, int num_sms)
 {
     const int64_t nb = (max_N + kTile - 1) / kTile;
-    const int64_t maxcta = (int64_t)kSymMaxCtaPerSm * num_sms;
+    const int64_t maxcta = sym_max_ctas(max_N, num_sms);
     return (size_t)(4 * maxcta + 4 * (maxcta + nb + 1) + 4 * (nb + 1));
 }
 
@@ -886,7 +893,7 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
     if ((rc = sym_prepare(ctx, N, &sc, part, nparts))) return rc;
     const double a = ctx->p.a;
     SrcF32 *src = (SrcF32 *)w.src;
-    const int pb = 256;
+    const int pb = elem_threads(N, ctx->num_sms);
     const SelfCoefs self = self_coefs(ctx, N);
     if (!packed) pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, self);
     const SymCta *ctas = (const SymCta *)sc->index;
@@ -923,7 +930,7 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
     if ((rc = sym_prepare(ctx, N, &sc, part, nparts))) return rc;
     const double a = ctx->p.a;
     SrcF32 *src = (SrcF32 *)w.src;
-    const int pb = 256;
+    const int pb = elem_threads(N, ctx->num_sms);
     const SelfCoefs self = self_coefs(ctx, N);
     if (!packed) pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos_w, F, T, N, a, 1, src, self);
     const SymCta *ctas = (const SymCta *)sc->index;
@@ -1102,7 +1109,7 @@ int mobility_apply2_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const dou
     const double a = ctx->p.a;
     SrcF32 *src = (SrcF32 *)w.src;
     float4 *src2 = (float4 *)w.src2;
-    const int pb = 256;
+    const int pb = elem_threads(N, ctx->num_sms);
     const SelfCoefs self = self_coefs(ctx, N);
     pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, 1, src, self);
     pack_rhs2_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, P, N, a, src2);
@@ -1462,7 +1469,7 @@ int mobility_rows_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
         return RPB_EINVAL;
     }
     double *part = (double *)ctx->ws.partial;
-    const int pb = 256;
+    const int pb = elem_threads(N, ctx->num_sms);
     const dim3 grid((unsigned)((nt + kPairThreads - 1) / kPairThreads), (unsigned)splits);
     const bool torque = T != nullptr;
     if (fp64) {
@@ -1530,7 +1537,7 @@ int mobility_part_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
     const bool sym = ctx->sym_enabled && ctx->p.wall && F && N >= 2 * kTile && (!T || ctx->sym_fused);
     if (sym && !(ctx->Lx > 0.0)) return mobility_sym(ctx, N, pos, F, T, U, false, part, nparts);
     if (sym && ctx->p.precision == RPB_FP32) {
-        const int pb = 256;
+        const int pb = elem_threads(N, ctx->num_sms);
         wrap_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, N, ctx->Lx, ctx->Ly, ctx->ws.pos_w);
         count_launches(1);
         return mobility_sym_periodic(ctx, N, ctx->ws.pos_w, pos, F, T, U, false, part, nparts);
@@ -1566,7 +1573,7 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
         return RPB_EINVAL;
     }
     double *part = (double *)ctx->ws.partial;
-    const int pb = 256;
+    const int pb = elem_threads(N, ctx->num_sms);
     const dim3 grid((unsigned)((N + kPairThreads - 1) / kPairThreads), (unsigned)splits);
     const bool torque = T != nullptr;
     const SelfCoefs self = self_coefs(ctx, N);
@@ -2037,7 +2044,7 @@ int forces_impl(rpb_ctx *ctx, int64_t N, const double *pos, const rpb_force_para
     const unsigned groups = (unsigned)((N + kGroupTargets - 1) / kGroupTargets);
     cudaStream_t st = ctx->stream;
     if (ctx->Lx > 0.0) {
-        const int pb = 256;
+        const int pb = elem_threads(N, ctx->num_sms);
         wrap_kernel<<<(unsigned)((N + pb - 1) / pb), pb, 0, st>>>(pos, n, ctx->Lx, ctx->Ly, ctx->ws.pos_w);
         if (N <= kGroupMaxN)
             forces_group_kernel<true><<<groups, kGroupTargets * kGroupThreads, 0, st>>>(
@@ -2226,7 +2233,7 @@ extern "C" int rpb_mobility_apply_noalloc(int64_t N64, const double *pos, const 
     int64_t chunk;
     noalloc_grid_plan(N64, sms, p->precision == RPB_FP64, kTile, kNoAllocPartialElems, &splits, &chunk);
     double *part = (double *)((unsigned char *)base + kNoAllocSrcBytes);
-    const int pb = 256;
+    const int pb = elem_threads(N, sms);
     const dim3 grid((unsigned)((N + kPairThreads - 1) / kPairThreads), (unsigned)splits);
     const double a = p->a;
     if (p->precision == RPB_FP32) {

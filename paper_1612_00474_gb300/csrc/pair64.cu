@@ -291,9 +291,10 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
     const SelfCoefs self = self_coefs(ctx, N);
     const Sym64Consts c64 = make_sym64_consts(a);
     const Sym64Plan pl = sym64_plan(N, ctx->num_sms);
-    double *tgt = ctx->ws.sym64, *col = tgt + sym64_tgt_elems(ctx->max_N, ctx->num_sms);
+    double *tgt = ctx->ws.sym64, *col = tgt + sym64_tgt_elems(ctx->ws.sym64_N, ctx->num_sms);
     SrcF64 *src = (SrcF64 *)ctx->ws.src;
-    if (!packed) pack_f64_kernel<<<(N + 255) / 256, 256, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
+    const int pb = elem_threads(N, ctx->num_sms);
+    if (!packed) pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
     const dim3 grid((unsigned)pl.runs, (unsigned)pl.qs);
     const int nt = 32 * kSym64Warps;
     if (ctx->p.wall && T)

@@ -185,7 +185,7 @@ struct SymSched {
 
 // Scratch owned by a context.
 struct Workspace {
-    void *slab = nullptr;         // the allocation of the arrays down to vec_g, and of sym64
+    void *slab = nullptr;         // the allocation of the arrays down to vec_g, of sym64 and of the SideSpace
     void *src = nullptr;          // packed sources, max_N records (SrcF64 size)
     void *partial = nullptr;      // pair-kernel partial sums
     size_t partial_bytes = 0;
@@ -218,9 +218,28 @@ struct Workspace {
     size_t sym_src_bytes = 0;
     void *src2 = nullptr;          // second right-hand side of the two-RHS symmetric pass (float4 per sphere)
     double *sym64 = nullptr;       // float64 contexts: row and column partials of the symmetric pass (pair64.cu)
+    int64_t sym64_N = 0;           // ... sized for this many spheres
     SymSched sym;       // the whole triangle
     SymSched sym_part;  // one share of it (rpb_mobility_apply_part)
 };
+
+// What one product writes besides its result, for the products of a step's drift when they run beside the
+// Lanczos iterations (step_impl): the fields of Workspace of the same names, for up to max_N spheres.
+struct SideSpace {
+    int64_t max_N = 0, sym64_N = 0;
+    void *src = nullptr, *partial = nullptr;
+    size_t partial_bytes = 0, sym_tgt_bytes = 0, sym_src_bytes = 0;
+    double *selfc = nullptr, *w = nullptr, *pos_w = nullptr, *sym64 = nullptr, *sym_tgt = nullptr;
+    float *sym_src = nullptr;
+};
+
+// Threads per block of an elementwise kernel over n items: single warps while they leave room on the SMs (a
+// float64 warp instruction takes 64 cycles of its scheduler, so a small vector is spread over all of
+// them), 256 beyond.
+inline int elem_threads(int64_t n, int num_sms)
+{
+    return n <= 32 * 8 * (int64_t)num_sms ? 32 : 256;
+}
 
 constexpr int kRunMaxIter = 64;  // = kMaxIter of the Lanczos state
 
@@ -271,6 +290,9 @@ struct rpb_ctx {
     void *hook_user = nullptr;
     int in_hook = 0;                  // inside the hook: products are computed here
     int gs_cluster = 8;               // blocks of the Lanczos cluster kernel at most (lanczos_setup)
+    rpb::SideSpace side;              // scratch, stream and events of a step's drift beside its Lanczos solve
+    cudaStream_t side_stream = nullptr;
+    cudaEvent_t side_fork = nullptr, side_join = nullptr;
     cudaEvent_t lz_ev = nullptr;      // host-driven Lanczos: an iteration's status has been written
 };
 

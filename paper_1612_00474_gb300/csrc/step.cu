@@ -1,4 +1,5 @@
 // step.cu -- Philox noise, random-finite-difference drift and the Adams-Bashforth update.
+#include <algorithm>
 #include <cmath>
 
 #include "rpb_internal.cuh"
@@ -51,9 +52,9 @@ int philox_impl(rpb_ctx *ctx, int64_t N, uint64_t seed, uint32_t step, uint32_t 
                 double *out, const unsigned int *d_step)
 {
     const int64_t npairs = (3 * N + 1) / 2;
-    int grid = (int)((npairs + 255) / 256);
-    if (grid > 8 * ctx->num_sms) grid = 8 * ctx->num_sms;
-    philox_normal_kernel<<<grid, 256, 0, ctx->stream>>>((int)N, (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32),
+    const int tb = elem_threads(npairs, ctx->num_sms);
+    const int grid = (int)std::min<int64_t>((npairs + tb - 1) / tb, 8 * ctx->num_sms);
+    philox_normal_kernel<<<grid, tb, 0, ctx->stream>>>((int)N, (uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32),
                                                         step, stream_id, instance, out, d_step);
     count_launches(1);
     return cuda_fail(cudaGetLastError(), "philox kernel");
@@ -78,7 +79,8 @@ __global__ void rfd_combine_kernel(double *__restrict__ up_drift, const double *
 
 static int elem_grid(int64_t n, int num_sms)
 {
-    int64_t g = (n + 255) / 256;
+    const int tb = elem_threads(n, num_sms);
+    int64_t g = (n + tb - 1) / tb;
     if (g > 8 * (int64_t)num_sms) g = 8 * num_sms;
     return g < 1 ? 1 : (int)g;
 }
@@ -86,16 +88,16 @@ static int elem_grid(int64_t n, int num_sms)
 int rfd_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *Wt, double delta, double *drift, int one_sided)
 {
     const int64_t n = 3 * N;
-    const int G = elem_grid(n, ctx->num_sms);
+    const int G = elem_grid(n, ctx->num_sms), tb = elem_threads(n, ctx->num_sms);
     // centred: q +- delta/2 W~; one-sided: q + delta W~ and q itself
-    displace_kernel<<<G, 256, 0, ctx->stream>>>(pos, Wt, n, one_sided ? delta : 0.5 * delta, ctx->ws.pos_a,
+    displace_kernel<<<G, tb, 0, ctx->stream>>>(pos, Wt, n, one_sided ? delta : 0.5 * delta, ctx->ws.pos_a,
                                                 ctx->ws.pos_b);
     count_launches(1);
     int rc;
     if ((rc = cuda_fail(cudaGetLastError(), "rfd displace"))) return rc;
     if ((rc = mobility_apply_impl(ctx, N, ctx->ws.pos_a, Wt, nullptr, drift))) return rc;
     if ((rc = mobility_apply_impl(ctx, N, one_sided ? pos : ctx->ws.pos_b, Wt, nullptr, ctx->ws.w))) return rc;
-    rfd_combine_kernel<<<G, 256, 0, ctx->stream>>>(drift, ctx->ws.w, n, ctx->p.kT / delta);
+    rfd_combine_kernel<<<G, tb, 0, ctx->stream>>>(drift, ctx->ws.w, n, ctx->p.kT / delta);
     count_launches(1);
     return cuda_fail(cudaGetLastError(), "rfd combine");
 }
@@ -125,7 +127,7 @@ int ab_update_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, const d
                    const double *drift, double dt, double noise_scale, int first, const int *d_first)
 {
     const int64_t n = 3 * N;
-    ab_update_kernel<<<elem_grid(n, ctx->num_sms), 256, 0, ctx->stream>>>(pos, U_prev, Un, g, drift, n, dt,
+    ab_update_kernel<<<elem_grid(n, ctx->num_sms), elem_threads(n, ctx->num_sms), 0, ctx->stream>>>(pos, U_prev, Un, g, drift, n, dt,
                                                                             noise_scale, first, d_first);
     count_launches(1);
     return cuda_fail(cudaGetLastError(), "ab update");
@@ -133,7 +135,7 @@ int ab_update_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, const d
 
 int fill_torque(rpb_ctx *ctx, int64_t N, const double *t, double *T)
 {
-    fill3_kernel<<<elem_grid(3 * N, ctx->num_sms), 256, 0, ctx->stream>>>(T, (int)N, t[0], t[1], t[2]);
+    fill3_kernel<<<elem_grid(3 * N, ctx->num_sms), elem_threads(3 * N, ctx->num_sms), 0, ctx->stream>>>(T, (int)N, t[0], t[1], t[2]);
     count_launches(1);
     return cuda_fail(cudaGetLastError(), "fill torque");
 }
