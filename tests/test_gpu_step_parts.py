@@ -36,9 +36,12 @@ def test_step_is_its_parts(gpu_lib, precision, N, periodic):
     finally:
         ctx.close()
     assert st["m"] == m
-    # the same kernels on the same inputs, up to the order of float64 sums; float32 pairs in a step share a pass
-    # whose accumulation is the same
-    assert float((U - Un).abs().max()) <= 1e-12 * float(Un.abs().max())
+    # the same kernels on the same inputs, up to the order of float64 sums; a float32 step of 256 spheres and more
+    # takes the velocity and the first Lanczos product in one pass, whose float32 rounding is its own (a product's
+    # relative rounding is below 1e-6)
+    shared = precision == "fp32" and N >= 256 and not periodic
+    assert float((U - Un).abs().max()) <= (1e-6 if shared else 1e-12) * float(Un.abs().max())
     ref = dt * Un + math.sqrt(2.0 * dt) * g + dt * d
     # the drift amplifies a product's rounding by 1/delta
-    assert float((q - q0 - ref).abs().max()) <= (1e-11 + 1e-15 / delta) * float(ref.abs().max())
+    bound = 1e-6 if shared else 1e-11 + 1e-15 / delta
+    assert float((q - q0 - ref).abs().max()) <= bound * float(ref.abs().max())
