@@ -75,7 +75,7 @@ static int check_vec(const void *p, const char *name, bool nullable)
 
 static void free_ws(Workspace &w)
 {
-    void *dev[] = {w.slab, w.sym_index, w.sym_tgt, w.sym_src, w.src2, w.pc};
+    void *dev[] = {w.slab, w.blocks64, w.sym_index, w.sym_tgt, w.sym_src, w.src2, w.pc};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (w.host_status) cudaFreeHost(w.host_status);
@@ -206,7 +206,7 @@ static int step_body(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint3
                 return rc;
             lrc = lanczos_run(ctx, N, pos, g, tol, max_iter, true, true, &iters, &err, &conv, gr);
         } else {
-            if ((rc = mobility_apply_impl(ctx, N, pos, F, T, Un))) return rc;
+            if ((rc = mobility_apply_impl(ctx, N, pos, F, T, Un, kKeep))) return rc;
             lrc = lanczos_impl(ctx, N, pos, W, g, tol, max_iter, ctx->hook == nullptr, &iters, &err, &conv, gr);
         }
         if (lrc != RPB_OK && lrc != RPB_ENOCONV) return lrc;
@@ -417,6 +417,14 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
                 return RPB_ENOMEM;
             }
         }
+    }
+    // the blocks of the float64 pairs (32 N^2 bytes) make the later products of a Lanczos solve about five
+    // times cheaper; kept while they stay below 8 GB and the device has the room, else every product
+    // evaluates its pairs
+    if (w.sym64 && blocks64_bytes(max_N) <= ((size_t)8 << 30) &&
+        cudaMalloc(&w.blocks64, blocks64_bytes(max_N)) != cudaSuccess) {
+        cudaGetLastError();
+        w.blocks64 = nullptr;
     }
     if (cudaMallocHost((void **)&w.host_status, 8 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();

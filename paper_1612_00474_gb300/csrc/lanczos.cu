@@ -522,8 +522,8 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
     GsArgs A = gs_args(ctx, N, pk, gr);
     A.tol = tol;
     A.max_iter = max_iter;
-    auto product = [&](bool is_packed) {
-        return mobility_apply_impl(ctx, N, pos, w.vf, nullptr, w.w, is_packed && pk);
+    auto product = [&](bool again) {
+        return mobility_apply_impl(ctx, N, pos, w.vf, nullptr, w.w, !pk ? kPlain : (again ? kAgain : kKeep));
     };
     if (gr) {
         // iteration 0 with the step; the others are the body of a loop node that an iteration's
@@ -560,7 +560,7 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
             (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->lz_ev, cudaEventDisableTiming), "lanczos event")))
             return rc;
         const double t_product = (ctx->Lx > 0.0 ? 9.0 : 1.0) * (double)N * (double)N *
-                                 (ctx->p.precision == RPB_FP64 ? 8e-11 : 1.3e-12);
+                                 (ctx->p.precision == RPB_FP32 ? 1.3e-12 : (w.blocks64 ? 1.6e-11 : 8e-11));
         const bool speculate = t_product < 1e-4;
         A.hs = w.host_status;
         bool have = first_done;

@@ -1502,10 +1502,10 @@ int mobility_rows_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
 }
 
 static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const double *F, const double *T,
-                           double *U, bool packed = false);
+                           double *U, ProductMode mode = kPlain);
 
 int mobility_apply_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const double *F, const double *T, double *U,
-                        bool packed)
+                        ProductMode mode)
 {
     if (ctx->hook && !ctx->in_hook) {  // the product is delegated (e.g. shared out among processes)
         ctx->in_hook = 1;
@@ -1514,7 +1514,7 @@ int mobility_apply_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doub
         if (rc != RPB_OK && rpb_last_error()[0] == 0) set_error("product hook returned %d", rc);
         return rc;
     }
-    return mobility_direct(ctx, N64, pos, F, T, U, packed);
+    return mobility_direct(ctx, N64, pos, F, T, U, mode);
 }
 
 // Rows [r0, r1) of share `part` of `nparts`: whole 128-row tiles, as equal as the tiles allow.
@@ -1557,12 +1557,13 @@ int mobility_part_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doubl
 }
 
 static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const double *F, const double *T,
-                           double *U, bool packed)
+                           double *U, ProductMode mode)
 {
     const int N = (int)N64;
+    const bool packed = mode == kAgain;
     if (ctx->sym_enabled && ctx->p.wall && !(ctx->Lx > 0.0) && F && N >= 2 * kTile && (!T || ctx->sym_fused))
         return mobility_sym(ctx, N, pos, F, T, U, packed);
-    if (mobility_sym64_ok(ctx, F)) return mobility_sym64(ctx, N, pos, F, T, U, packed);
+    if (mobility_sym64_ok(ctx, F)) return mobility_sym64(ctx, N, pos, F, T, U, mode);
     cudaStream_t st = ctx->stream;
     const double a = ctx->p.a;
     int splits;

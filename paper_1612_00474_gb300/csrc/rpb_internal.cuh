@@ -30,18 +30,18 @@ struct alignas(16) SrcF64 {
 };
 
 #ifdef __CUDACC__
-// 1/sqrt(x) for a positive normal x: the hardware's approximation, then one fourth-order step of the
-// binomial series, y (1 + e/2 + 3 e^2/8 + 5 e^3/16) with e = 1 - x y^2 (Householder's iteration).
+// 1/sqrt(x) for a positive normal x: the hardware's approximation (relative error measured at 2^-20.0), then one
+// third-order step of the binomial series, y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (Householder's
+// iteration): it leaves 5 e^3/16 = 2^-58.7, below rounding.
 __device__ __forceinline__ double rsqrt_pos(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-(x * y), y, 1.0);
-    const double p = fma(e, fma(e, 0.3125, 0.375), 0.5);
-    return fma(e * y, p, y);
+    return fma(e * y, fma(e, 0.375, 0.5), y);
 }
 
-// 1/d for a positive normal d: the hardware's approximation (relative error below 2^-23) and one
+// 1/d for a positive normal d: the hardware's approximation (relative error measured at 2^-19.9) and one
 // third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - d y.
 __device__ __forceinline__ double rcp_pos(double d)
 {
@@ -219,6 +219,7 @@ struct Workspace {
     void *src2 = nullptr;          // second right-hand side of the two-RHS symmetric pass (float4 per sphere)
     double *sym64 = nullptr;       // float64 contexts: row and column partials of the symmetric pass (pair64.cu)
     int64_t sym64_N = 0;           // ... sized for this many spheres
+    double *blocks64 = nullptr;    // the pairs' translation blocks at a Lanczos solve's positions (blocks64_bytes)
     SymSched sym;       // the whole triangle
     SymSched sym_part;  // one share of it (rpb_mobility_apply_part)
 };
@@ -305,10 +306,13 @@ void count_launches(int n);
 int cuda_fail(cudaError_t e, const char *what);
 
 // Pair product: U = M_tt F + M_tr T with the context's precision.  F or T may be null.
-// All pointers device, SoA float64.  Enqueued on ctx->stream.  packed: the context's packed sources hold
-// these positions and s F already (F is still read for the self terms; T must be null).
+// All pointers device, SoA float64.  Enqueued on ctx->stream.  mode (a Lanczos solve makes many products at the
+// same positions): kPlain; kKeep, a first one that leaves what the others can use (the packed positions, and
+// in float64 the pairs' blocks, pair64.cu); kAgain, another one at those positions, with no product of the
+// context in between: the packed sources hold s F already (F is still read for the self terms; T null).
+enum ProductMode { kPlain, kKeep, kAgain };
 int mobility_apply_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *F, const double *T,
-                        double *U, bool packed = false);
+                        double *U, ProductMode mode = kPlain);
 // Rows t0 .. t1 - 1 of the product (component stride ldu, ldu < 0: t1 - t0), one-way kernels over a
 // target range.
 int mobility_rows_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *F, const double *T, int64_t t0,
@@ -319,7 +323,8 @@ int mobility_part_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double 
 // The float64 product with each unordered pair evaluated once (pair64.cu): whether it can be taken (a
 // float64 context with its scratch, forces given, no periodic images), and the product.
 bool mobility_sym64_ok(const rpb_ctx *ctx, const double *F);
-int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U, bool packed);
+int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U, ProductMode mode);
+size_t blocks64_bytes(int64_t max_N);
 // Whether mobility_apply2_impl can take this product (float32 symmetric pass with two right-hand sides).
 bool mobility_apply2_ok(const rpb_ctx *ctx, int64_t N);
 // U = M_tt F + M_tr T and U2 = M_tt P in one symmetric pass (F, T, P non-null).

@@ -71,3 +71,18 @@ def test_not_finite(gpu_lib):
             assert torch.equal(torch.isfinite(U), torch.isfinite(R))
     finally:
         ctx.close()
+
+
+# the products of a solve after the first read the blocks that it stored
+@pytest.mark.parametrize("N", [1, 2, 31, 33, 64, 100, 300, 1000])
+@pytest.mark.parametrize("wall", [True, False])
+def test_lanczos_from_stored_blocks(gpu_lib, N, wall):
+    pos, W = _config(N), inputs.vectors(N, 3)
+    ctx = gpu_lib.Context(max_N=N + 40, precision="fp64", max_iter=16, wall=wall)
+    try:
+        ctx.lanczos_sqrt_apply(_dev(inputs.monolayer(N, seed=1)), _dev(W), tol=0.0, max_iter=3, raise_on_noconv=False)
+        g, m, _, _ = ctx.lanczos_sqrt_apply(_dev(pos), _dev(W), tol=0.0, max_iter=5, raise_on_noconv=False)
+    finally:
+        ctx.close()
+    ref, mr, _, _ = O.lanczos_sqrt(pos, W, exact_iters=5, wall=wall)
+    assert m == mr and O.rel_err(inputs.from_soa(g.cpu().numpy(), N), ref) <= 1e-10  # the float64 path's bound
