@@ -596,11 +596,12 @@ __global__ void __launch_bounds__(kTailThreads) batch_tail_kernel(double *__rest
     double s = 0.0;  // |w|^2 from the chunks' parts (every warp, the same in every thread)
     for (int q = threadIdx.x & 31; q < c.y; q += 32) s += norm2[c.x + q];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    lanczos_tail_block(lzb, L, k, tol, lzb[L.c1 + k] + lzb[L.c2 + k], sqrt(s), nodes, sh);
+    const TailRegs reg = lanczos_tail_load(lzb, L, k, nodes, sh, threadIdx.x);
+    const TailResult r = lanczos_tail_y(lzb, L, k, lzb[L.c1 + k] + lzb[L.c2 + k], reg, sh, threadIdx.x);
     if (threadIdx.x == 0) {
         double *st = lzb + L.status;
         st[6] = k + 1;
-        if (st[ST_STOP] != 0.0) {
+        if (lanczos_tail_stop(lzb, L, k, tol, sqrt(s), r, reg.nW, nullptr)) {
             st[7] = 1.0;
             active[b] = 0;
         } else {

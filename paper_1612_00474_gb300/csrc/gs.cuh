@@ -16,6 +16,12 @@ constexpr int kGsWarps = kGsThreads / 32;
 constexpr int kGsChunk = 256;                              // spheres of a chunk at most
 constexpr int kGsRows = 3 * kGsChunk / kGsThreads;         // rows (sphere, component) of a thread
 
+// Barrier 2 among a block's first kGsThreads threads (a block may have others beside them).
+__device__ __forceinline__ void gs_sync()
+{
+    asm volatile("bar.sync 2, %0;" ::"n"(kGsThreads) : "memory");
+}
+
 // Rows of a chunk: components x, y, z of `cnt` spheres at offsets base + c stride + i.
 struct GsSpan {
     int64_t base, stride;
@@ -65,11 +71,12 @@ __device__ __forceinline__ double gs_block_sum(double v, int nu, int nw, double 
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) sh[threadIdx.x >> 5] = v;
     }
-    __syncthreads();
+    gs_sync();
     double s = 0.0;
     if (threadIdx.x < 32) {
         s = lane < nw ? sh[lane] : 0.0;
         for (int o = kGsWarps / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        s = __shfl_sync(0xffffffffu, s, 0);  // the first kGsWarps lanes hold the sum
     }
     return s;
 }
@@ -109,7 +116,7 @@ __device__ __forceinline__ double gs_dots(const double *__restrict__ V, size_t l
         gs_dots_rows<2>(V, ld, nvec, row, w, mine);
     else if (nu == 3)
         gs_dots_rows<3>(V, ld, nvec, row, w, mine);
-    __syncthreads();
+    gs_sync();
     double s = 0.0;
     if (threadIdx.x < nvec)
         for (int k = 0; k < nw; ++k) s += sh[k][threadIdx.x];
@@ -153,7 +160,7 @@ __device__ __forceinline__ void gs_coefs(const double *__restrict__ red, size_t 
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) coef[j] = s;
     }
-    __syncthreads();
+    gs_sync();
 }
 
 }  // namespace rpb

@@ -98,8 +98,13 @@ struct GsArgs {
     RunState *rs;      // graph-replayed run: k and the loop's state live here
     cudaGraphConditionalHandle loop;
     __device__ __forceinline__ int iter() const { return rs ? rs->k : k; }
-    // v_{k+1} (row r = c N + i, i a sphere of component c) into the basis and the next product's load
-    __device__ __forceinline__ void store(double *v, int64_t r, double x) const
+    // s_i of row r's sphere (r = c N + i)
+    __device__ __forceinline__ double factor(int64_t r) const
+    {
+        return src ? sc[r < N ? r : (r < 2 * N ? r - N : r - 2 * N)] : 0.0;
+    }
+    // v_{k+1} (row r, s_i = si) into the basis and the next product's load
+    __device__ __forceinline__ void store(double *v, int64_t r, double x, double si) const
     {
         v[r] = x;
         const double f = P ? x * P[r] : x;
@@ -107,7 +112,7 @@ struct GsArgs {
         if (!src) return;
         const int c = r < N ? 0 : (r < 2 * N ? 1 : 2);
         const int64_t i = r - c * N;
-        const double s = sc[i] * f;
+        const double s = si * f;
         if (fp64)
             reinterpret_cast<double *>((SrcF64 *)src + i)[3 + c] = s;
         else
@@ -125,17 +130,15 @@ struct GsArgs {
         status[ST_BREAK] = 0.0;
         if (rs) rs->k = 0;
     }
-    // after the tridiagonal step of iteration k, by the thread that wrote the status words
-    __device__ __forceinline__ void end(int k) const
+    // after the tridiagonal step of iteration k, by one thread
+    __device__ __forceinline__ void end(int k, double beta_k, const TailResult &r, double nW) const
     {
-        const double *status = lz + L.status;
-        if (hs)
-            for (int q = 0; q < 8; ++q) hs[q] = status[q];
+        const bool stop = lanczos_tail_stop(lz, L, k, tol, beta_k, r, nW, hs);
         if (rs) {
             rs->m = k + 1;
             rs->k = k + 1;
-            if (k > 0) rs->loops += 1ull;
-            if (max_iter > 1) cudaGraphSetConditional(loop, status[ST_STOP] == 0.0 && k + 1 < max_iter ? 1u : 0u);
+            if (k > 0) atomicAdd(&rs->loops, 1ull);
+            if (max_iter > 1) cudaGraphSetConditional(loop, !stop && k + 1 < max_iter ? 1u : 0u);
         }
     }
 };
@@ -145,76 +148,116 @@ static_assert(sizeof(SrcF32) == 48 && sizeof(SrcF64) == 80, "packed source recor
 // ------------------------------------------------------------------ small suspensions: one cluster
 constexpr int kGsCluster = 16;  // blocks of the cluster at most (8 where the device schedules no 16)
 
-// coef_j = sum over the cluster's blocks of their part[j], four threads per j; ends with a block barrier
-__device__ __forceinline__ void cluster_coefs(cg::cluster_group &cl, double *part, int nvec, double *coef)
+constexpr int kGsClusterThreads = kGsThreads + kTailThreads;
+
+// Exchange of the cluster: every block writes its partial sums into all blocks' arrays before the barrier, so
+// that the sums read their own shared memory (a read of another block's costs about 600 cycles).
+struct ClusterShared {
+    double part[2][kGsCluster][kMaxIter];  // dot products of the two passes, by block
+    double norm[kGsCluster];
+    double coef[kMaxIter];
+    double alpha[2];                       // the last vector's coefficients: alpha_k is their sum
+};
+
+// coef_j = sum over the cluster's blocks of part[block][j], four threads per j; ends with a barrier of the rows'
+// threads
+__device__ __forceinline__ void cluster_coefs(const double (*part)[kMaxIter], int blocks, int nvec, double *coef)
 {
-    const int j = threadIdx.x >> 2, q = threadIdx.x & 3, n = (int)cl.num_blocks();
+    const int j = threadIdx.x >> 2, q = threadIdx.x & 3;
     double s = 0.0;
     if (j < nvec)
-        for (int r = q; r < n; r += 4) s += cl.map_shared_rank(part, r)[j];
+        for (int r = q; r < blocks; r += 4) s += part[r][j];
     s += __shfl_xor_sync(0xffffffffu, s, 2);
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     if (q == 0 && j < nvec) coef[j] = s;
-    __syncthreads();
+    gs_sync();
 }
 
-// One cluster, block r holding spheres [r per, (r + 1) per): Gram-Schmidt on w, v_{k+1}, and the tridiagonal
-// step in the first block.  init: v_0 = W / |W| instead.
-__global__ void __launch_bounds__(kGsThreads) gs_cluster_kernel(GsArgs A, int per, int init)
+// One cluster, block r holding spheres [r per, (r + 1) per): Gram-Schmidt on w and v_{k+1} by the first
+// kGsThreads threads of every block; the tridiagonal step by the other kTailThreads of the first block, which
+// have loaded its state before alpha_k is known and run beside the second projection, the norm and the
+// stores (T has no beta_k): 15.9 -> 13.7 us a launch at 256 spheres, of which the tridiagonal step was about 5.
+// init: v_0 = W / |W| instead.
+// Every thread of the cluster arrives at its four barriers (two when init) and waits for each; warps are
+// converged at all of them.
+__global__ void __launch_bounds__(kGsClusterThreads) gs_cluster_kernel(GsArgs A, int per, int init)
 {
     static_assert(kGsThreads >= 4 * kMaxIter, "four threads per coefficient");
     __shared__ double sh[kGsWarps][kMaxIter + 8];
-    __shared__ double part[2][kMaxIter], norm[1], coef[kMaxIter];
+    __shared__ ClusterShared cs;
     __shared__ TailShared ts;
     cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+    const int rank = (int)cl.block_rank(), blocks = (int)cl.num_blocks(), tid = threadIdx.x;
     const int k = init ? -1 : A.iter();
+    cl.sync();  // every block of the cluster runs: its shared memory may be written
+    if (tid >= kGsThreads) {
+        const int t = tid - kGsThreads;
+        TailRegs reg = {};
+        if (rank == 0 && !init) reg = lanczos_tail_load(A.lz, A.L, k, A.lz + A.L.total, ts, t);
+        if (!init) {
+            cl.sync();
+            cl.sync();
+        }
+        cl.barrier_arrive();
+        TailResult r = {};
+        if (rank == 0 && !init) {
+            asm volatile("bar.sync 3, %0;" ::"n"(kGsClusterThreads) : "memory");  // alpha is there
+            r = lanczos_tail_y(A.lz, A.L, k, cs.alpha[0] + cs.alpha[1], reg, ts, t);
+        }
+        __syncwarp();
+        cl.barrier_wait();
+        if (rank == 0 && t == 0) {
+            double bn = 0.0, nb, inv;
+            for (int q = 0; q < blocks; ++q) bn += cs.norm[q];
+            root_and_inverse(bn, &nb, &inv);
+            if (init)
+                A.begin(bn);
+            else
+                A.end(k, nb, r, reg.nW);
+        }
+        return;
+    }
     const int first = rank * per;
     const int left = (int)A.N - first;
     int64_t row[kGsRows];
-    double x[kGsRows];
+    double x[kGsRows], si[kGsRows];
     const GsSpan span = {first, A.N, max(0, min(per, left))};
     const int nu = gs_rows(span, row), nw = gs_warps(span);
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) {
         x[u] = row[u] < 0 ? 0.0 : (init ? A.W[row[u]] : A.w[row[u]]);
+        si[u] = row[u] < 0 ? 0.0 : A.factor(row[u]);
         if (A.P && !init && row[u] >= 0) x[u] *= A.P[row[u]];
     }
     for (int pass = 0; pass < 2 && !init; ++pass) {
         const double s = gs_dots(A.V, A.ld, k + 1, row, nu, nw, x, sh);
-        if (tid <= k) part[pass][tid] = s;
+        if (tid <= k)
+            for (int q = 0; q < blocks; ++q) cl.map_shared_rank(&cs, q)->part[pass][rank][tid] = s;
+        __syncwarp();
         cl.sync();
-        cluster_coefs(cl, part[pass], k + 1, coef);
-        if (rank == 0 && tid <= k) A.lz[(pass ? A.L.c2 : A.L.c1) + tid] = coef[tid];
-        gs_project(A.V, A.ld, k + 1, row, nu, coef, x);
+        cluster_coefs(cs.part[pass], blocks, k + 1, cs.coef);
+        if (rank == 0) {
+            if (tid == k) cs.alpha[pass] = cs.coef[k];
+            __syncwarp();
+            if (pass == 1) asm volatile("bar.arrive 3, %0;" ::"n"(kGsClusterThreads) : "memory");
+        }
+        gs_project(A.V, A.ld, k + 1, row, nu, cs.coef, x);
     }
     double s = 0.0;
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u) s = fma(x[u], x[u], s);
     s = gs_block_sum(s, nu, nw, sh[0]);
-    if (tid == 0) norm[0] = s;
+    if (tid < blocks) cl.map_shared_rank(&cs, tid)->norm[rank] = s;  // (the sum is in the first warp's threads)
+    __syncwarp();
     cl.sync();
-    const int lane = tid & (kGsCluster - 1);
-    double bn = lane < (int)cl.num_blocks() ? cl.map_shared_rank(norm, lane)[0] : 0.0;
-    for (int o = kGsCluster / 2; o > 0; o >>= 1) bn += __shfl_xor_sync(0xffffffffu, bn, o);
-    cl.barrier_arrive();  // nothing of another block's memory is read from here on
-    double nb, inv;
+    double bn = 0.0, nb, inv;
+    for (int q = 0; q < blocks; ++q) bn += cs.norm[q];
     root_and_inverse(bn, &nb, &inv);
     if (init && !(nb > 0.0)) inv = 0.0;
     double *v = A.V + (size_t)(k + 1) * A.ld;
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u)
-        if (row[u] >= 0) A.store(v, row[u], x[u] * inv);
-    if (rank == 0) {
-        if (init) {
-            if (tid == 0) A.begin(bn);
-        } else if (tid < kTailThreads) {
-            // (c1 and c2 of the last vector were stored by other threads of this block, before a barrier)
-            lanczos_tail_block(A.lz, A.L, k, A.tol, A.lz[A.L.c1 + k] + A.lz[A.L.c2 + k], nb, A.lz + A.L.total, ts);
-            if (tid == 0) A.end(k);
-        }
-    }
-    cl.barrier_wait();
+        if (row[u] >= 0) A.store(v, row[u], x[u] * inv, si[u]);
 }
 
 // ------------------------------------------------------------------ larger suspensions: chunks over the GPU
@@ -302,7 +345,7 @@ __global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(GsArgs A, int chun
     const double *w = init ? A.W : A.w;
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u)
-        if (row[u] >= 0) A.store(v, row[u], w[row[u]] * inv);
+        if (row[u] >= 0) A.store(v, row[u], w[row[u]] * inv, A.factor(row[u]));
     if (init && blockIdx.x == 0 && threadIdx.x == 0) A.begin(bn);
 }
 
@@ -313,8 +356,9 @@ __global__ void __launch_bounds__(kTailThreads) lanczos_tail_kernel(GsArgs A, in
     double bn = 0.0;  // the same in every warp
     for (int b = threadIdx.x & 31; b < parts; b += 32) bn += A.norm2[b];
     for (int o = 16; o > 0; o >>= 1) bn += __shfl_xor_sync(0xffffffffu, bn, o);
-    lanczos_tail_block(A.lz, A.L, k, A.tol, A.lz[A.L.c1 + k] + A.lz[A.L.c2 + k], sqrt(bn), A.lz + A.L.total, ts);
-    if (threadIdx.x == 0) A.end(k);
+    const TailRegs reg = lanczos_tail_load(A.lz, A.L, k, A.lz + A.L.total, ts, threadIdx.x);
+    const TailResult r = lanczos_tail_y(A.lz, A.L, k, A.lz[A.L.c1 + k] + A.lz[A.L.c2 + k], reg, ts, threadIdx.x);
+    if (threadIdx.x == 0) A.end(k, sqrt(bn), r, reg.nW);
 }
 
 // g[r] = sum_{k < m} y[k] V[k][r]   (y already carries |W|); d_m (optional): read m from the device
@@ -394,7 +438,7 @@ static int query_cluster()
     int n = 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kGsCluster);
-    cfg.blockDim = dim3(kGsThreads);
+    cfg.blockDim = dim3(kGsClusterThreads);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = kGsCluster;
@@ -454,7 +498,7 @@ static int gs_cluster_launch(cudaStream_t st, const GsArgs &A, int blocks, int i
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(kGsThreads);
+    cfg.blockDim = dim3(kGsClusterThreads);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;

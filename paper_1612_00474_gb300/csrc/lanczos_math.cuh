@@ -125,7 +125,7 @@ constexpr int kTailThreads = kSqrtNodes;  // one node per thread
 constexpr int kTailRows = 16;             // entries of y summed over the nodes at a time
 struct TailShared {
     double al[kMaxIter], be[kMaxIter], b2[kMaxIter];  // the entries of T, beta^2
-    double y[kMaxIter];
+    double y[kMaxIter], yprev[kMaxIter];
     double q0[kMaxIter], sl[kMaxIter];                // eigen-decomposition
     double z[kTailRows][kSqrtNodes + 8];              // the nodes' terms (padded: the sums read 8 columns of
                                                       // four rows at a time)
@@ -160,9 +160,27 @@ __device__ __forceinline__ bool tail_any(bool p)
     return r != 0;
 }
 
-// The tridiagonal step of one Krylov space by the first kTailThreads threads of a block: stores alpha_k,
-// beta_k, y, eps and the stopping decision in its state block lz.  nodes: kSqrtNodes shifts, then as
-// many weights (sqrt_nodes.h).
+// The tridiagonal step of one Krylov space by kTailThreads threads (tid: 0 .. kTailThreads - 1), in three parts.
+// lanczos_tail_load fetches what is known before iteration k's projections: the nodes (kSqrtNodes shifts, then as
+// many weights, sqrt_nodes.h), the entries of T_k, the last y and |W|.
+struct TailRegs {
+    double s, w, nW;
+};
+__device__ __forceinline__ TailRegs lanczos_tail_load(const double *__restrict__ lz, const LzLayout &L, int k,
+                                                      const double *__restrict__ nodes, TailShared &sh, int tid)
+{
+    if (tid < k) {
+        const double b = lz[L.beta + tid];
+        sh.al[tid] = lz[L.alpha + tid];
+        sh.be[tid] = b;
+        sh.b2[tid] = b * b;
+        sh.yprev[tid] = lz[L.yprev + tid];
+    }
+    if (tid == k) sh.be[k] = sh.b2[k] = sh.yprev[k] = 0.0;
+    return TailRegs{nodes[tid], nodes[kSqrtNodes + tid], lz[L.status + ST_NW]};
+}
+
+// lanczos_tail_y: with alpha_k, stores alpha_k and y; thread 0 returns eps and the largest entry of T.
 //
 // With T = tridiag(beta, alpha, beta) scaled by M, the power of four above its Gershgorin bound (its square
 // root is exact and costs nothing), y = |W| T^{1/2} e_1 ~ |W| sqrt(M) sum_j w_j T (T + M s_j)^{-1} e_1.  Thread j solves its shifted system by eliminating from
@@ -179,24 +197,20 @@ __device__ __forceinline__ bool tail_any(bool p)
 // iterations of a converging solve of 8 dimensions and 164 us over one of 19; with the nodes a
 // 3001-sphere free-space solve (18 iterations, float32 pairs) went from 3251 to 1211 us and a step of 4096
 // spheres from 1103 to 1004 us.
-__device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, const LzLayout &L, int k, double tol,
-                                                   double alpha_k, double beta_k, const double *__restrict__ nodes,
-                                                   TailShared &sh)
+struct TailResult {
+    double eps, tnorm;
+};
+__device__ __forceinline__ TailResult lanczos_tail_y(double *__restrict__ lz, const LzLayout &L, int k, double alpha_k,
+                                                     const TailRegs &reg, TailShared &sh, int tid)
 {
-    const int tid = threadIdx.x, lane = tid & 31;
-    double *status = lz + L.status;
+    const int lane = tid & 31;
     const int n = k + 1;
-    if (tid < n) {
-        const double b = tid < k ? lz[L.beta + tid] : 0.0;
-        sh.al[tid] = tid < k ? lz[L.alpha + tid] : alpha_k;
-        sh.be[tid] = b;
-        sh.b2[tid] = b * b;
-    }
-    const double sj = nodes[tid], wj = nodes[kSqrtNodes + tid];
-    const double nW = status[ST_NW];
+    const double sj = reg.s, wj = reg.w, nW = reg.nW;
+    TailResult res = {-1.0, 0.0};
+    if (tid == 0) sh.al[k] = alpha_k;
     tail_sync();
     // Gershgorin bound and largest entry (every warp, over the entries lane and lane + 32)
-    double mb = 0.0, mt = fabs(beta_k);
+    double mb = 0.0, mt = 0.0;
     for (int i = lane; i < n; i += 32) {
         const double a = fabs(sh.al[i]), b = fabs(sh.be[i]);
         mb = fmax(mb, a + b + (i > 0 ? fabs(sh.be[i - 1]) : 0.0));
@@ -206,7 +220,7 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
     const double bound = warp_max_pos(mb);
     const int e4 = plain_pos(bound) ? ((__double2hiint(bound) >> 20) - 1023 + 2) >> 1 : 0;
     const double M = __hiloint2double((1023 + 2 * e4) << 20, 0), rootM = __hiloint2double((1023 + e4) << 20, 0);
-    const double tnorm = warp_max_pos(mt);
+    res.tnorm = warp_max_pos(mt);
     const double s = M * sj;
     double r[kMaxIter];
     double c = sh.al[k];
@@ -222,7 +236,7 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
         r[i] = ri;
     }
     if (tail_any(!ok)) {
-        if (tid >= 32) return;  // (no barrier follows for the first warp on this path)
+        if (tid >= 32) return res;  // (no barrier follows for the first warp on this path)
         double y0, y1;
         tridiag_sqrt_ql(sh.al, sh.be, k, nW, sh.q0, sh.sl, &y0, &y1);
         if (lane < n) sh.y[lane] = y0;
@@ -250,36 +264,49 @@ __device__ __forceinline__ void lanczos_tail_block(double *__restrict__ lz, cons
             if (p == 0 && row < m) sh.y[base + row] = v * scale;
             tail_sync();
         }
-        if (tid >= 32) return;
+        if (tid >= 32) return res;
     }
     // eps_k = |y - (yprev, 0)| / |yprev|: lanes 0 .. 15 sum the numerator, 16 .. 31 the denominator
     const bool upper = lane >= 16;
     double sq = 0.0;
     for (int i = lane & 15; i < n; i += 16) {
-        const double p = i < k ? lz[L.yprev + i] : 0.0;
+        const double p = sh.yprev[i];
         const double d = upper ? p : sh.y[i] - p;
         sq = fma(d, d, sq);
     }
-    __syncwarp();  // yprev has been read
     for (int i = lane; i < n; i += 32) lz[L.y + i] = lz[L.yprev + i] = sh.y[i];
     for (int o = 8; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
     const double den = __shfl_sync(0xffffffffu, sq, 16);
     const double num = sq;  // in lane 0
     if (lane == 0) {
         lz[L.alpha + k] = alpha_k;
-        lz[L.beta + k] = beta_k;
-        double eps = -1.0;
         if (k >= 1 && den > 0.0) {
             const double q = plain_pos(den) ? num * rcp_pos(den) : num / den;
-            eps = plain_pos(q) ? q * rsqrt_pos(q) : sqrt(q);
+            res.eps = plain_pos(q) ? q * rsqrt_pos(q) : sqrt(q);
         }
-        const bool brk = beta_k <= 1e-14 * tnorm;
-        const bool conv = (tol > 0.0 && k >= 1 && eps <= tol);
-        status[ST_EPS] = eps;
-        status[ST_BREAK] = brk ? 1.0 : 0.0;
-        status[ST_STOP] = (brk || conv) ? 1.0 : 0.0;
-        status[ST_INV_BETA] = brk ? 0.0 : (plain_pos(beta_k) ? rcp_pos(beta_k) : 1.0 / beta_k);
     }
+    return res;
+}
+
+// lanczos_tail_stop, by one thread: with beta_k, stores it and the stopping decision (*hs: also there, null:
+// nowhere); returns whether the iteration stops.
+__device__ __forceinline__ bool lanczos_tail_stop(double *__restrict__ lz, const LzLayout &L, int k, double tol,
+                                                  double beta_k, const TailResult &r, double nW, double *hs)
+{
+    double *status = lz + L.status;
+    lz[L.beta + k] = beta_k;
+    const bool brk = beta_k <= 1e-14 * fmax(r.tnorm, beta_k);
+    const bool stop = brk || (tol > 0.0 && k >= 1 && r.eps <= tol);
+    status[ST_EPS] = r.eps;
+    status[ST_BREAK] = brk ? 1.0 : 0.0;
+    status[ST_STOP] = stop ? 1.0 : 0.0;
+    status[ST_INV_BETA] = brk ? 0.0 : (plain_pos(beta_k) ? rcp_pos(beta_k) : 1.0 / beta_k);
+    if (hs) {
+        hs[ST_EPS] = r.eps;
+        hs[ST_NW] = nW;
+        hs[ST_STOP] = stop ? 1.0 : 0.0;
+    }
+    return stop;
 }
 
 }  // namespace rpb
