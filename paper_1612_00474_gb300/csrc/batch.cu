@@ -462,8 +462,15 @@ __device__ __forceinline__ GsSpan chunk_span(const ChunkDesc &c, const InstDesc 
     return GsSpan{d.off + c.first, total, min(kGsChunk, d.N - c.first)};
 }
 
-// red[j nchunks + chunk] = the chunk's part of <V_j, w>, j < nvec
-__global__ void __launch_bounds__(kGsThreads) batch_dots_kernel(const double *__restrict__ V, size_t ld, int nvec,
+// The iteration a kernel of the loop works on: k, or in a replayed graph the one the device is at.
+__device__ __forceinline__ int batch_iter(int k, const int *__restrict__ d_k)
+{
+    return d_k ? *d_k : k;
+}
+
+// red[j nchunks + chunk] = the chunk's part of <V_j, w>, j <= k
+__global__ void __launch_bounds__(kGsThreads) batch_dots_kernel(const double *__restrict__ V, size_t ld, int k,
+                                                                const int *__restrict__ d_k,
                                                                 const double *__restrict__ w,
                                                                 const InstDesc *__restrict__ inst,
                                                                 const ChunkDesc *__restrict__ chunks,
@@ -473,6 +480,7 @@ __global__ void __launch_bounds__(kGsThreads) batch_dots_kernel(const double *__
     __shared__ double sh[kGsWarps][kMaxIter + 8];
     const ChunkDesc c = chunks[blockIdx.x];
     if (active && !active[c.inst]) return;  // uniform per block
+    const int nvec = batch_iter(k, d_k) + 1;
     int64_t row[kGsRows];
     double x[kGsRows];
     const GsSpan span = chunk_span(c, inst[c.inst], total);
@@ -486,7 +494,8 @@ __global__ void __launch_bounds__(kGsThreads) batch_dots_kernel(const double *__
 // w -= sum_j c_j V_j with c_j from the partials `red`; the instance's first chunk stores c in its state block
 // (lz_b + coef_off).  Then, with red2, the dot products of the new w (the second pass of Gram-Schmidt) as
 // batch_dots_kernel, or the chunk's part of |w|^2 in norm2.
-__global__ void __launch_bounds__(kGsThreads) batch_project_kernel(const double *__restrict__ V, size_t ld, int nvec,
+__global__ void __launch_bounds__(kGsThreads) batch_project_kernel(const double *__restrict__ V, size_t ld, int k,
+                                                                   const int *__restrict__ d_k,
                                                                    double *__restrict__ w,
                                                                    const InstDesc *__restrict__ inst,
                                                                    const ChunkDesc *__restrict__ chunks,
@@ -500,6 +509,7 @@ __global__ void __launch_bounds__(kGsThreads) batch_project_kernel(const double 
     __shared__ double coef[kMaxIter];
     const ChunkDesc c = chunks[blockIdx.x];
     if (active && !active[c.inst]) return;
+    const int nvec = batch_iter(k, d_k) + 1;
     int64_t row[kGsRows];
     double x[kGsRows];
     const GsSpan span = chunk_span(c, inst[c.inst], total);
@@ -549,19 +559,22 @@ __global__ void __launch_bounds__(128) batch_norm_init_kernel(const double *__re
     active[b] = nw > 0.0 ? 1 : 0;
 }
 
-// v = w * status_b[idx] for the active instances (all when active is null), and s_i v into the packed sources
-// of the next product, whose positions stay packed through a solve.
+// Basis vector row0 (in a replayed graph the one after the iteration's) = w * status_b[idx] for the active
+// instances (all when active is null); also into vf, the next product's load, and times s_i into its
+// packed sources, whose positions stay packed through a solve.
 __global__ void __launch_bounds__(kGsThreads) batch_scale_kernel(const double *__restrict__ w,
                                                                  const InstDesc *__restrict__ inst,
                                                                  const ChunkDesc *__restrict__ chunks,
                                                                  const int *__restrict__ active, int64_t total,
                                                                  const double *__restrict__ lz, size_t lz_stride,
-                                                                 size_t status_off, int idx, double *__restrict__ v,
-                                                                 const double *__restrict__ s, void *__restrict__ src,
-                                                                 int fp64)
+                                                                 size_t status_off, int idx, double *__restrict__ V,
+                                                                 size_t ld, int row0, const int *__restrict__ d_k,
+                                                                 double *__restrict__ vf, const double *__restrict__ s,
+                                                                 void *__restrict__ src, int fp64)
 {
     const ChunkDesc c = chunks[blockIdx.x];
     if (active && !active[c.inst]) return;
+    double *v = V + (size_t)(d_k ? *d_k + 1 : row0) * ld;
     const double inv = lz[(size_t)c.inst * lz_stride + status_off + idx];
     int64_t row[kGsRows];
     gs_rows(chunk_span(c, inst[c.inst], total), row);
@@ -571,6 +584,7 @@ __global__ void __launch_bounds__(kGsThreads) batch_scale_kernel(const double *_
         if (r < 0) continue;
         const double x = w[r] * inv;
         v[r] = x;
+        vf[r] = x;
         const int q = r < total ? 0 : (r < 2 * total ? 1 : 2);
         const int64_t i = r - q * total;
         const double f = s[i] * x;
@@ -583,7 +597,8 @@ __global__ void __launch_bounds__(kGsThreads) batch_scale_kernel(const double *_
 
 // One block per instance: the tridiagonal step; converged instances leave the active set.
 __global__ void __launch_bounds__(kTailThreads) batch_tail_kernel(double *__restrict__ lz, size_t lz_stride, LzLayout L,
-                                                                  int k, double tol, const double *__restrict__ norm2,
+                                                                  int k, const int *__restrict__ d_k, double tol,
+                                                                  const double *__restrict__ norm2,
                                                                   const int2 *__restrict__ inst_chunks,
                                                                   const double *__restrict__ nodes,
                                                                   int *__restrict__ active, int *__restrict__ n_active)
@@ -591,6 +606,7 @@ __global__ void __launch_bounds__(kTailThreads) batch_tail_kernel(double *__rest
     __shared__ TailShared sh;
     const int b = blockIdx.x;
     if (!active[b]) return;  // the whole block leaves together
+    k = batch_iter(k, d_k);
     double *lzb = lz + (size_t)b * lz_stride;
     const int2 c = inst_chunks[b];
     double s = 0.0;  // |w|^2 from the chunks' parts (every warp, the same in every thread)
@@ -645,7 +661,7 @@ struct rpb_batch {
     int *d_active = nullptr;
     int *d_nactive = nullptr;
     void *src = nullptr;
-    double *vec[12] = {};  // pos, Up, F, T, Un, W, Wt, g, drift, pos_a, pos_b, w
+    double *vec[13] = {};  // pos, Up, F, T, Un, W, Wt, g, drift, pos_a, pos_b, w, the next product's load
     double *V = nullptr;
     double *lz = nullptr;
     double *red = nullptr;
@@ -670,13 +686,13 @@ struct rpb_batch {
     cudaEvent_t join = nullptr;
     unsigned long long *d_unconv = nullptr;
     unsigned long long *h_unconv = nullptr;
-    // graph-replayed Lanczos: iterations after the first run inside conditional (IF) nodes of the
-    // graph, captured on `body`; d_iter_runs[k] counts how often iteration k ran (for the launch
-    // count), iter_launches[k] is the number of kernels of iteration k's body
+    // graph-replayed Lanczos: the iterations after the first run in a loop node of the graph, captured on
+    // `body`; d_k is the iteration, d_loops counts the body's runs (for the launch count)
     cudaStream_t body = nullptr;
-    unsigned long long *d_iter_runs = nullptr;
-    unsigned long long *h_iter_runs = nullptr;
-    int iter_launches[kMaxIter] = {};
+    int *d_k = nullptr;
+    unsigned long long *d_loops = nullptr;
+    unsigned long long *h_loops = nullptr;
+    int body_launches = 0;
     // float32 products by the symmetric pass (both directions of a pair from one evaluation):
     // schedule and partial-sum scratch for the current batch sizes
     bool sym_enabled = false;
@@ -688,7 +704,7 @@ struct rpb_batch {
 
 namespace rpb {
 
-enum { V_POS, V_UP, V_F, V_T, V_UN, V_W, V_WT, V_G, V_DRIFT, V_PA, V_PB, V_WORK };
+enum { V_POS, V_UP, V_F, V_T, V_UN, V_W, V_WT, V_G, V_DRIFT, V_PA, V_PB, V_WORK, V_VF };
 
 static void batch_free(rpb_batch *bt)
 {
@@ -702,8 +718,9 @@ static void batch_free(rpb_batch *bt)
     for (void *p : host)
         if (p) cudaFreeHost(p);
     if (bt->d_unconv) cudaFree(bt->d_unconv);
-    if (bt->d_iter_runs) cudaFree(bt->d_iter_runs);
-    if (bt->h_iter_runs) cudaFreeHost(bt->h_iter_runs);
+    if (bt->d_k) cudaFree(bt->d_k);
+    if (bt->d_loops) cudaFree(bt->d_loops);
+    if (bt->h_loops) cudaFreeHost(bt->h_loops);
     if (bt->body) cudaStreamDestroy(bt->body);
     batch_sym_free(bt->sym);
     if (bt->join) cudaEventDestroy(bt->join);
@@ -848,22 +865,24 @@ static int batch_product(rpb_batch *bt, const double *pos, const double *F, cons
     return cuda_fail(cudaGetLastError(), "batch pair kernels");
 }
 
-// Inside a replayed graph: count this run of iteration k and, unless it is the last one, let the
-// conditional node of iteration k + 1 run only while some instance is still active.
-__global__ void batch_iter_kernel(cudaGraphConditionalHandle next, int has_next, const int *__restrict__ n_active,
-                                  unsigned long long *__restrict__ runs_k)
+// Inside a replayed graph, the end of an iteration: the next one, counted, and the loop node's body runs again
+// while some instance is still active and iterations are left.
+__global__ void batch_iter_kernel(cudaGraphConditionalHandle loop, int max_iter, const int *__restrict__ n_active,
+                                  int *__restrict__ d_k, unsigned long long *__restrict__ loops)
 {
-    *runs_k += 1ull;
-    if (has_next) cudaGraphSetConditional(next, *n_active > 0 ? 1u : 0u);
+    const int k = *d_k;
+    *d_k = k + 1;
+    if (k > 0) *loops += 1ull;
+    if (max_iter > 1) cudaGraphSetConditional(loop, *n_active > 0 && k + 1 < max_iter ? 1u : 0u);
 }
 
 // Lanczos for every instance at once; per-instance m, eps and convergence land in h_lz statuses.
 // graph == false: the host reads the number of still-active instances after every iteration and stops
 // when it reaches zero, then copies the per-instance statuses to h_lz.  graph == true (inside a CUDA
-// graph capture): iteration 0 is captured as is and iterations 1 .. max_iter - 1 each inside a
-// conditional node that runs only while some instance is still active (the previous iteration's
-// last kernel sets its condition), so a replay does the iterations the step needs, at most max_iter;
-// converged instances are masked out of every kernel, and nothing is read back.
+// graph capture): iteration 0 is captured as is and the others as the body of a loop (WHILE) node that runs
+// while some instance is still active (the end of an iteration sets its condition), so a replay does the
+// iterations the step needs, at most max_iter; converged instances are masked out of every kernel, and
+// nothing is read back.
 static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, double *g, double tol, int max_iter,
                          bool graph = false)
 {
@@ -872,91 +891,79 @@ static int batch_lanczos(rpb_batch *bt, const double *pos, const double *W, doub
     const int64_t total = bt->total;
     const size_t ld = (size_t)3 * bt->max_total;
     const LzLayout L(bt->max_iter);
-    double *V = bt->V, *w = bt->vec[V_WORK];
-    const int ge = grid_for(3 * total, bt->num_sms);
+    double *V = bt->V, *w = bt->vec[V_WORK], *vf = bt->vec[V_VF];
+    const int ge = grid_for(3 * total, bt->num_sms), nc = bt->nchunks;
+    const int fp64 = bt->p.precision == RPB_FP64;
+    double *red2 = bt->red + (size_t)bt->max_iter * nc;
+    const int *d_k = graph ? bt->d_k : nullptr;
     int rc;
-    cudaGraphConditionalHandle hnd[kMaxIter] = {};
+    cudaGraphConditionalHandle loop = 0;
     if (graph) {
         cudaStreamCaptureStatus cs;
         cudaGraph_t cg = nullptr;
         if ((rc = cuda_fail(cudaStreamGetCaptureInfo(main_st, &cs, nullptr, &cg, nullptr, nullptr, nullptr),
-                            "capture info")))
+                            "capture info")) ||
+            (rc = cuda_fail(cudaGraphConditionalHandleCreate(&loop, cg, 0u, cudaGraphCondAssignDefault),
+                            "conditional handle")) ||
+            (rc = cuda_fail(cudaMemsetAsync(bt->d_k, 0, sizeof(int), main_st), "memset")))
             return rc;
-        CondSet cs_all = {};
-        for (int k = 1; k < max_iter; ++k) {
-            if ((rc = cuda_fail(cudaGraphConditionalHandleCreate(&hnd[k], cg, 0u, cudaGraphCondAssignDefault),
-                                "conditional handle")))
-                return rc;
-            cs_all.h[k - 1] = hnd[k];
-        }
-        // the iterations' conditions start at 0 in every step (the graph runs the step in a loop)
-        if (max_iter > 1) {
-            graph_reset_conds_kernel<<<1, 64, 0, main_st>>>(cs_all, max_iter - 1);
-            count_launches(1);
-        }
     }
-    const int nc = bt->nchunks;
-    double *red2 = bt->red + (size_t)bt->max_iter * nc;
-    batch_dots_kernel<<<nc, kGsThreads, 0, main_st>>>(W, 0, 1, W, bt->d_inst, bt->d_chunks, nullptr, total, bt->red);
+    batch_dots_kernel<<<nc, kGsThreads, 0, main_st>>>(W, 0, 0, nullptr, W, bt->d_inst, bt->d_chunks, nullptr, total,
+                                                      bt->red);
     batch_norm_init_kernel<<<(B + 3) / 4, 128, 0, main_st>>>(bt->red, bt->d_inst_chunks, B, bt->lz, bt->lz_stride,
                                                              L.status, bt->d_active);
-    const int fp64 = bt->p.precision == RPB_FP64;
     batch_scale_kernel<<<nc, kGsThreads, 0, main_st>>>(W, bt->d_inst, bt->d_chunks, nullptr, total, bt->lz,
-                                                       bt->lz_stride, L.status, ST_INV_NW, V, bt->selfc, bt->src, fp64);
+                                                       bt->lz_stride, L.status, ST_INV_NW, V, ld, 0, nullptr, vf,
+                                                       bt->selfc, bt->src, fp64);
     count_launches(3);
-    for (int k = 0; k < max_iter; ++k) {
-        const bool cond = graph && k >= 1;
-        if (cond) {
-            if ((rc = graph_begin_if(main_st, bt->body, hnd[k]))) return rc;
-            bt->stream = bt->body;
-        }
+    // everything of an iteration but the host's reading of n_active
+    auto iteration = [&](int k, bool scale) {
         cudaStream_t st = bt->stream;
-        const uint64_t before = rpb_launch_count();
-        const double *vk = V + (size_t)k * ld;
-        rc = batch_product(bt, pos, vk, nullptr, w, bt->d_active, true);
-        const int nv = k + 1;
-        if (!rc) {
-            batch_dots_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, nv, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
-                                                         bt->red);
-            batch_project_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, nv, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
-                                                            bt->red, bt->lz, bt->lz_stride, L.c1, red2, nullptr);
-            batch_project_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, nv, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
-                                                            red2, bt->lz, bt->lz_stride, L.c2, nullptr, bt->norm2);
-            rc = cuda_fail(cudaMemsetAsync(bt->d_nactive, 0, sizeof(int), st), "memset");
+        int r = batch_product(bt, pos, vf, nullptr, w, bt->d_active, true);
+        if (r) return r;
+        batch_dots_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, k, d_k, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
+                                                     bt->red);
+        batch_project_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, k, d_k, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
+                                                        bt->red, bt->lz, bt->lz_stride, L.c1, red2, nullptr);
+        batch_project_kernel<<<nc, kGsThreads, 0, st>>>(V, ld, k, d_k, w, bt->d_inst, bt->d_chunks, bt->d_active, total,
+                                                        red2, bt->lz, bt->lz_stride, L.c2, nullptr, bt->norm2);
+        if ((r = cuda_fail(cudaMemsetAsync(bt->d_nactive, 0, sizeof(int), st), "memset"))) return r;
+        batch_tail_kernel<<<B, kTailThreads, 0, st>>>(bt->lz, bt->lz_stride, L, k, d_k, tol, bt->norm2,
+                                                      bt->d_inst_chunks, bt->nodes, bt->d_active, bt->d_nactive);
+        count_launches(4);
+        if (scale) {
+            batch_scale_kernel<<<nc, kGsThreads, 0, st>>>(w, bt->d_inst, bt->d_chunks, bt->d_active, total, bt->lz,
+                                                          bt->lz_stride, L.status, ST_INV_BETA, V, ld, k + 1, d_k, vf,
+                                                          bt->selfc, bt->src, fp64);
+            count_launches(1);
         }
-        if (!rc) {
-            batch_tail_kernel<<<B, kTailThreads, 0, st>>>(bt->lz, bt->lz_stride, L, k, tol, bt->norm2,
-                                                          bt->d_inst_chunks, bt->nodes, bt->d_active, bt->d_nactive);
-            count_launches(4);
-            if (graph) {
-                const bool has_next = k + 1 < max_iter;
-                batch_iter_kernel<<<1, 1, 0, st>>>(has_next ? hnd[k + 1] : 0ull, has_next ? 1 : 0, bt->d_nactive,
-                                                   bt->d_iter_runs + k);
-                count_launches(1);
-            } else {
-                if ((rc = cuda_fail(cudaMemcpyAsync(bt->h_nactive, bt->d_nactive, sizeof(int),
-                                                    cudaMemcpyDeviceToHost, st),
-                                    "n_active copy")))
-                    return rc;
-                if ((rc = cuda_fail(cudaStreamSynchronize(st), "batch lanczos iteration"))) return rc;
-                if (*bt->h_nactive == 0) break;
-            }
-            if (k + 1 < max_iter) {
-                batch_scale_kernel<<<nc, kGsThreads, 0, st>>>(w, bt->d_inst, bt->d_chunks, bt->d_active, total, bt->lz,
-                                                              bt->lz_stride, L.status, ST_INV_BETA,
-                                                              V + (size_t)(k + 1) * ld, bt->selfc, bt->src, fp64);
-                count_launches(1);
-            }
-            rc = cuda_fail(cudaGetLastError(), "batch lanczos kernels");
+        if (graph) {
+            batch_iter_kernel<<<1, 1, 0, st>>>(loop, max_iter, bt->d_nactive, bt->d_k, bt->d_loops);
+            count_launches(1);
         }
-        if (cond) {
-            bt->iter_launches[k] = (int)(rpb_launch_count() - before);
-            cudaGraph_t body_graph = nullptr;
+        return cuda_fail(cudaGetLastError(), "batch lanczos kernels");
+    };
+    if (graph) {
+        if ((rc = iteration(0, max_iter > 1))) return rc;
+        if (max_iter > 1) {
+            if ((rc = graph_begin_cond(main_st, bt->body, loop, cudaGraphCondTypeWhile))) return rc;
+            bt->stream = bt->body;
+            const uint64_t before = rpb_launch_count();
+            rc = iteration(0, true);
+            bt->body_launches = (int)(rpb_launch_count() - before);
+            cudaGraph_t body_graph = nullptr;  // owned by the node
             const int erc = cuda_fail(cudaStreamEndCapture(bt->body, &body_graph), "body capture end");
             bt->stream = main_st;
-            if (!rc) rc = erc;
+            if (rc || (rc = erc)) return rc;
         }
-        if (rc) return rc;
+    }
+    for (int k = 0; k < max_iter && !graph; ++k) {
+        if ((rc = iteration(k, k + 1 < max_iter)) ||
+            (rc = cuda_fail(cudaMemcpyAsync(bt->h_nactive, bt->d_nactive, sizeof(int), cudaMemcpyDeviceToHost, main_st),
+                            "n_active copy")) ||
+            (rc = cuda_fail(cudaStreamSynchronize(main_st), "batch lanczos iteration")))
+            return rc;
+        if (*bt->h_nactive == 0) break;
     }
     batch_combine_kernel<<<ge, 256, 0, main_st>>>(V, ld, bt->d_inst_of, total, bt->lz, bt->lz_stride, L, g);
     count_launches(1);
@@ -1036,7 +1043,7 @@ static int batch_read_stats(rpb_batch *bt, double tol, rpb_step_stats *stats)
 }
 
 // nsteps AB steps of the batch: one gather, one launch of a CUDA graph whose WHILE node runs a step
-// (fixed Lanczos iteration count, converged instances masked) nsteps times without host
+// (converged instances masked) nsteps times without host
 // synchronisation, one scatter.
 static int batch_run_impl(rpb_batch *bt, int B, const int64_t *N, double *const *pos, double *const *U_prev,
                           const int64_t *steps, const uint64_t *seeds, int nsteps, double dt, double delta, double tol,
@@ -1048,9 +1055,9 @@ static int batch_run_impl(rpb_batch *bt, int B, const int64_t *N, double *const 
     double **v = bt->vec;
     if ((rc = batch_gather(bt, 0, v[V_POS], 0)) || (rc = batch_gather(bt, 1, v[V_UP], 0))) return rc;
     if ((rc = cuda_fail(cudaMemsetAsync(bt->d_unconv, 0, sizeof(unsigned long long), st), "memset")) ||
-        (rc = cuda_fail(cudaMemsetAsync(bt->d_iter_runs, 0, kMaxIter * sizeof(unsigned long long), st), "memset")))
+        (rc = cuda_fail(cudaMemsetAsync(bt->d_loops, 0, sizeof(unsigned long long), st), "memset")))
         return rc;
-    for (int k = 0; k < kMaxIter; ++k) bt->iter_launches[k] = 0;
+    bt->body_launches = 0;
     int per_step = 0;
     if (nsteps > 0) {
         // one graph launch for all nsteps: a WHILE node whose body is a step, counted down on the device
@@ -1100,19 +1107,13 @@ static int batch_run_impl(rpb_batch *bt, int B, const int64_t *N, double *const 
         (rc = cuda_fail(cudaMemcpyAsync(bt->h_unconv, bt->d_unconv, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                         st),
                         "count copy")) ||
-        (rc = cuda_fail(cudaMemcpyAsync(bt->h_iter_runs, bt->d_iter_runs, kMaxIter * sizeof(unsigned long long),
-                                        cudaMemcpyDeviceToHost, st),
+        (rc = cuda_fail(cudaMemcpyAsync(bt->h_loops, bt->d_loops, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st),
                         "iteration count copy")) ||
         (rc = cuda_fail(cudaStreamSynchronize(st), "batch run")))
         return rc;
-    if (nsteps > 0) {  // kernels executed: the unconditional part every step, each iteration body per run
-        int64_t cond_part = 0, executed = 0;
-        for (int k = 1; k < kMaxIter; ++k) {
-            cond_part += bt->iter_launches[k];
-            executed += (int64_t)bt->iter_launches[k] * (int64_t)bt->h_iter_runs[k];
-        }
-        count_launches((int)((per_step - cond_part) * (int64_t)nsteps + executed));
-    }
+    if (nsteps > 0)  // kernels executed: the unconditional part every step, the loop's body once per run of it
+        count_launches((int)((int64_t)(per_step - bt->body_launches) * nsteps +
+                             (int64_t)bt->body_launches * (int64_t)*bt->h_loops));
     batch_read_stats(bt, tol, stats);
     if (unconverged) *unconverged = (int64_t)*bt->h_unconv;
     if (*bt->h_unconv && tol > 0.0) {
@@ -1195,8 +1196,9 @@ int rpb_batch_create(rpb_batch **out, const rpb_params *p, int64_t max_total_N, 
               cudaStreamCreateWithFlags(&bt->loop, cudaStreamNonBlocking) == cudaSuccess &&
               cudaMalloc(&bt->d_left, sizeof(int)) == cudaSuccess &&
               cudaStreamCreateWithFlags(&bt->body, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaMalloc(&bt->d_iter_runs, kMaxIter * sizeof(unsigned long long)) == cudaSuccess &&
-              cudaMallocHost(&bt->h_iter_runs, kMaxIter * sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMalloc(&bt->d_k, sizeof(int)) == cudaSuccess &&
+              cudaMalloc(&bt->d_loops, sizeof(unsigned long long)) == cudaSuccess &&
+              cudaMallocHost(&bt->h_loops, sizeof(unsigned long long)) == cudaSuccess &&
               cudaEventCreateWithFlags(&bt->join, cudaEventDisableTiming) == cudaSuccess;
     for (double *&v : bt->vec) ok = ok && cudaMalloc(&v, vb) == cudaSuccess;
     if (!ok) {

@@ -369,19 +369,11 @@ int philox_impl(rpb_ctx *ctx, int64_t N, uint64_t seed, uint32_t step, uint32_t 
                 double *out, const unsigned int *d_step = nullptr);
 // Open a conditional node after the work captured so far on `st` and start capturing its body on
 // `body`; an IF node runs its body when `h` was set non-zero, a WHILE node as long as it is.
-int graph_begin_if(cudaStream_t st, cudaStream_t body, cudaGraphConditionalHandle h);
 int graph_begin_cond(cudaStream_t st, cudaStream_t body, cudaGraphConditionalHandle h,
                      cudaGraphConditionalNodeType type);
 // Adds a WHILE node (its handle created with the default value 1) after the capture dependencies of
 // st and begins capturing its body on `body`; the body ends with graph_loop_tail_kernel.
 int graph_begin_loop(cudaStream_t st, cudaStream_t body, cudaGraphConditionalHandle *h);
-// The conditions of a set of conditional nodes, all set to 0 by graph_reset_conds_kernel: a condition
-// keeps its value from one pass of a loop body to the next (the default is applied only when the
-// graph is launched), so a body that decides its conditional nodes as it goes clears them first.
-struct CondSet {
-    cudaGraphConditionalHandle h[kRunMaxIter];
-};
-__global__ void graph_reset_conds_kernel(CondSet s, int n);
 // *left = n (before the loop's graph is launched)
 __global__ void graph_loop_init_kernel(int *left, int n);
 // End of one pass of a loop body: --*left, and the loop runs again while *left > 0.

@@ -31,16 +31,6 @@ struct RunCtx {
     double *h_status = nullptr;   // pinned host copy of the Lanczos status words
 };
 
-int graph_begin_if(cudaStream_t st, cudaStream_t body, cudaGraphConditionalHandle h)
-{
-    return graph_begin_cond(st, body, h, cudaGraphCondTypeIf);
-}
-
-__global__ void graph_reset_conds_kernel(CondSet s, int n)
-{
-    for (int k = threadIdx.x; k < n; k += blockDim.x) cudaGraphSetConditional(s.h[k], 0u);
-}
-
 __global__ void graph_loop_init_kernel(int *left, int n)
 {
     *left = n;
