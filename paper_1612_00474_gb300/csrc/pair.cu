@@ -178,6 +178,120 @@ __global__ void __launch_bounds__(kPairThreads) pair_f32_kernel(const SrcF32 *__
     }
 }
 
+// Float32 pair pass without the wall for chunks of several tiles (more than 2048 spheres): two targets per
+// lane with packed arithmetic, every source read by the whole warp, because the scalar kernel is bound by
+// issue (two targets' instructions per source instead of one's for half of the loads and votes).  Block of 64
+// threads: targets tid and tid + 64 of 128.  The operations of a pair and the order of a target's sums are
+// those of pair_f32_kernel, so the results are the same bits.
+// tile_sums (chunk = one tile): the float32 sums of every tile instead of the chunk's, tile_sums[(tile 3 + q) N
+// + i], for pair_reduce_tiles_kernel.
+// Products in us, scalar kernel -> this one, without / with torques: N = 3001 35.3 -> 31.1 / 35.4 -> 35.3,
+// 8000 111 -> 93 / 130 -> 116, 40000 1782 -> 1459 / 2232 -> 1937.  With one tile per CTA a warp is alone on
+// its scheduler and two targets per lane double its chain: N = 2048 24.8 -> 29.4, 300 22.8 -> 26.8, so the
+// scalar kernel keeps those.
+template <bool TORQUE>
+__global__ void __launch_bounds__(64) pair_f32_free_kernel(const SrcF32 *__restrict__ src, int N, int chunk, X2Consts c,
+                                                           double *__restrict__ part, float *__restrict__ tile_sums)
+{
+    __shared__ float4 sp[kTile], sf[kTile];
+    __shared__ float4 st[TORQUE ? kTile : 1];
+    const int tid = threadIdx.x;
+    const int i0 = blockIdx.x * kTile + tid, i1 = i0 + 64;
+    const int j0 = blockIdx.y * chunk;
+    const int j1 = min(N, j0 + chunk);
+    const float2 zero2 = make_float2(0.f, 0.f), one2 = make_float2(1.f, 1.f);
+    float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
+    float2 tz = one2;
+    if (i0 < N) {
+        p0 = src[i0].p;
+        tz.x = src[i0].f.x;
+    }
+    if (i1 < N) {
+        p1 = src[i1].p;
+        tz.y = src[i1].f.x;
+    }
+    const float2 tx = make_float2(p0.x, p1.x), ty = make_float2(p0.y, p1.y);
+    const float2 txl = make_float2(p0.z, p1.z), tyl = make_float2(p0.w, p1.w);
+    float2 s[3] = {zero2, zero2, zero2}, comp[3] = {zero2, zero2, zero2};
+    auto dup = [](float v) { return make_float2(v, v); };
+    // the targets' velocities from source k added to u
+    auto pair = [&](int k, float2 &ux, float2 &uy, float2 &uz) {
+        const float4 p = sp[k], f = sf[k];
+        const float2 rx = add2(sub2(tx, dup(p.x)), sub2(txl, dup(p.z)));
+        const float2 ry = add2(sub2(ty, dup(p.y)), sub2(tyl, dup(p.w)));
+        const float2 rz = sub2(tz, dup(f.x));
+        const float2 r2 = fma2(rz, rz, fma2(rx, rx, mul2(ry, ry)));
+        const float2 ir = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
+        const float2 ir2 = mul2(ir, ir), ir3 = mul2(ir, ir2);
+        float2 c1 = mul2(ir, fma2(c.two_3_a2, ir2, one2));
+        float2 c2 = mul2(ir3, fma2(c.m_two_a2, ir2, one2));
+        float2 ct = ir3;
+        const bool n0 = r2.x < c.four_a2, n1 = r2.y < c.four_a2;
+        if (__any_sync(0xffffffffu, n0 || n1)) {
+            if (n0) near_fix(r2.x, ir.x, 0.f, c, c1.x, c2.x, ct.x);
+            if (n1) near_fix(r2.y, ir.y, 0.f, c, c1.y, c2.y, ct.y);
+        }
+        const float2 Fx = dup(f.y), Fy = dup(f.z), Fz = dup(f.w);
+        const float2 k2 = mul2(c2, fma2(rz, Fz, fma2(rx, Fx, mul2(ry, Fy))));
+        ux = fma2(c1, Fx, fma2(k2, rx, ux));
+        uy = fma2(c1, Fy, fma2(k2, ry, uy));
+        uz = fma2(c1, Fz, fma2(k2, rz, uz));
+        if (TORQUE) {
+            const float4 q = st[k];
+            const float2 Tx = dup(q.x), Ty = dup(q.y), Tz = dup(q.z);
+            ux = fma2(ct, fma2(Ty, rz, neg2(mul2(Tz, ry))), ux);
+            uy = fma2(ct, fma2(Tz, rx, neg2(mul2(Tx, rz))), uy);
+            uz = fma2(ct, fma2(Tx, ry, neg2(mul2(Ty, rx))), uz);
+        }
+    };
+    for (int base = j0; base < j1; base += kTile) {
+        const int cnt = min(kTile, j1 - base);
+        for (int k = tid; k < cnt; k += 64) {
+            sp[k] = src[base + k].p;
+            sf[k] = src[base + k].f;
+            if (TORQUE) st[k] = src[base + k].t;
+        }
+        __syncthreads();
+        float2 u[3] = {zero2, zero2, zero2};
+        if (base != (int)blockIdx.x * kTile) {
+#pragma unroll 4
+            for (int k = 0; k < cnt; ++k) pair(k, u[0], u[1], u[2]);
+        } else {
+            for (int k = 0; k < cnt; ++k) {
+                float2 d[3] = {zero2, zero2, zero2};
+                pair(k, d[0], d[1], d[2]);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    if (k != tid) u[q].x += d[q].x;
+                    if (k != tid + 64) u[q].y += d[q].y;
+                }
+            }
+        }
+        if (tile_sums) {
+            float *o = tile_sums + (size_t)blockIdx.y * 3 * N;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                if (i0 < N) o[(size_t)q * N + i0] = u[q].x;
+                if (i1 < N) o[(size_t)q * N + i1] = u[q].y;
+            }
+            return;
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {  // compensated (Kahan) accumulation of the tile sums
+            const float2 y = sub2(u[q], comp[q]), t = add2(s[q], y);
+            comp[q] = sub2(sub2(t, s[q]), y);
+            s[q] = t;
+        }
+        __syncthreads();
+    }
+    double *o = part + (size_t)blockIdx.y * 3 * N;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        if (i0 < N) o[(size_t)q * N + i0] = (double)s[q].x - (double)comp[q].x;
+        if (i1 < N) o[(size_t)q * N + i1] = (double)s[q].y - (double)comp[q].y;
+    }
+}
+
 // Float32 pair pass evaluating two sources per lane and iteration with packed float32x2 arithmetic.
 // The shared tile holds the 128 sources as 64 interleaved pairs: float4 (x_hi[2p], x_hi[2p+1],
 // y_hi[2p], y_hi[2p+1]), (x_lo.., y_lo..), (z~.., Fx..), (Fy.., Fz..), and for torques (Tx.., Ty..)
@@ -1403,6 +1517,41 @@ __global__ void __launch_bounds__(128) pair_reduce_warp_kernel(const double *__r
     U[2 * ldu + li] = k * uz;
 }
 
+// The same from float32 tile sums: per chunk of `per` tiles the compensated chain that pair_f32_kernel runs over
+// them, then the chunks in order, so that the result does not depend on which kernel took the tiles.
+// For products without the wall whose chunks make too few CTAs: two tiles per CTA leave 288 CTAs to 3001
+// spheres, one makes 576; the pair kernel takes 18.1 us instead of 22.9, this one 6.9 instead of 5.5 and a
+// Lanczos solve 920 us instead of 1053.
+__global__ void __launch_bounds__(64) pair_reduce_tiles_kernel(const float *__restrict__ tile_sums, int tiles, int per,
+                                                               int N, const double *__restrict__ F,
+                                                               const double *__restrict__ T, SelfCoefs sc,
+                                                               double *__restrict__ U)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
+    if (i >= N) return;
+    const float *p = tile_sums + (size_t)q * N + i;
+    double sum = 0.0;
+    float s = 0.f, c = 0.f;
+    for (int t0 = 0, left = per; t0 < tiles; t0 += 8) {
+        float x[8];  // eight loads in flight
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = t0 + u < tiles ? p[(size_t)(t0 + u) * 3 * N] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (t0 + u >= tiles) break;
+            const float y = x[u] - c, v = s + y;
+            c = (v - s) - y;
+            s = v;
+            if (--left == 0 || t0 + u + 1 == tiles) {  // the end of a chunk
+                sum += (double)s - (double)c;
+                s = c = 0.f;
+                left = per;
+            }
+        }
+    }
+    U[(size_t)q * N + i] = sc.velocity(i, q, sum, F, T, N);
+}
+
 // Chunk partials -> U (targets t0 .. t0 + nt - 1, nt < 0: all N; U's component stride ldu, ldu < 0:
 // nt): a thread per target for few chunks (coalesced loads), a warp per target for many.  With the
 // spheres' self coefficients in sc, or without (sc.s null) evaluating the self terms.
@@ -1622,11 +1771,34 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
         SrcF32 *src = (SrcF32 *)ctx->ws.src;
         if (!packed) pack_f32_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
         if (!ctx->p.wall) {
-            const PairConsts<float> c = make_consts<float>(a);
-            if (torque)
-                pair_f32_kernel<true, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
-            else
-                pair_f32_kernel<false, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
+            if (chunk == kTile) {
+                const PairConsts<float> c = make_consts<float>(a);
+                if (torque)
+                    pair_f32_kernel<true, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
+                else
+                    pair_f32_kernel<false, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
+            } else {
+                const X2Consts c = make_x2_consts(a);
+                auto run = [&](const dim3 &g, int len, double *chunks, float *tile_sums) {
+                    if (torque)
+                        pair_f32_free_kernel<true><<<g, 64, 0, st>>>(src, N, len, c, chunks, tile_sums);
+                    else
+                        pair_f32_free_kernel<false><<<g, 64, 0, st>>>(src, N, len, c, chunks, tile_sums);
+                };
+                // chunks that leave fewer CTAs than four per SM: a CTA per tile (their float32 sums need half
+                // of the chunks' float64 ones per tile; one that finds no room takes the chunks)
+                const int tiles = (int)grid.x, per = (int)(chunk / kTile);
+                if ((int64_t)grid.x * grid.y < 4 * ctx->num_sms &&
+                    (size_t)tiles * 3 * N * sizeof(float) <= ctx->ws.partial_bytes) {
+                    float *sums = (float *)part;
+                    run(dim3(grid.x, (unsigned)tiles), kTile, nullptr, sums);
+                    pair_reduce_tiles_kernel<<<dim3((unsigned)((N + 63) / 64), 3), 64, 0, st>>>(sums, tiles, per, N,
+                                                                                               F, T, self, U);
+                    count_launches(packed ? 2 : 3);
+                    return cuda_fail(cudaGetLastError(), "pair kernels");
+                }
+                run(grid, (int)chunk, part, nullptr);
+            }
         } else if (ctx->fp32_variant == 1) {
             const X2Consts c = make_x2_consts(a);
             if (torque)
