@@ -30,9 +30,13 @@
 #include <cstdio>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "grid_plan.h"
 #include "pair_math.cuh"
 #include "sym_schedule.h"
+
+namespace cg = cooperative_groups;
 
 namespace rpb {
 
@@ -815,6 +819,181 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
     }
 }
 
+// The pseudo-periodic pass of a small cell, one pair per lane.  A schedule of few one-tile runs leaves most of
+// the chip idle while each of its warps works through 32 targets x 128 sources x 9 images (a cell of 256
+// spheres: 3 CTAs, one warp per scheduler).  Here a cluster of eight CTAs takes a tile: CTA w and CTA w + 4 the
+// targets [32 w, 32 w + 32), the first their sums, the second the velocities of the sources.  Its warps take
+// parts that are independent in the sums of pair_f32x2_sym_kernel, so that the results are the same bits:
+//   targets   a lane per target; four warps for the even sources and four for the odd ones (the halves of that
+//             kernel's packed sums), in the lane's order there.  A warp forms the factors of every fourth
+//             source's nine blocks, waits for its turn and adds them to the sums, which go from warp to warp
+//             in shared memory.
+//   sources   a lane per source; eight warps for four groups of 32 sources and two halves of the targets.  The
+//             sum over the 32 targets runs through them in the order of that kernel's exchange between lanes (a
+//             binary tree); the four CTAs' sums are added as the four warps' there.
+// What bounds it: the instructions of 32 x 9 blocks (one direction, about 56 each) per scheduler.
+template <bool TORQUE>
+__global__ void __cluster_dims__(8) __launch_bounds__(256, TORQUE ? 1 : 2) pair_sym_lanes_kernel(
+    const SrcF32 *__restrict__ src, int N, const SymCta *__restrict__ ctas, const SymSeg *__restrict__ segs, X2Consts c,
+    const int *__restrict__ col_start, double *__restrict__ tgt_part, float *__restrict__ src_part, PerLen pl)
+{
+    __shared__ SrcF32 ss[kTile], st[32];
+    __shared__ float us[2][3][32], sv[2][3][kTile];
+    cg::cluster_group cl = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int w = (int)cl.block_rank() & 3;
+    const bool targets = cl.block_rank() < 4;
+    const int sg = ctas[blockIdx.x / 8].s0;
+    const int b = segs[sg].b, t = segs[sg].t0;
+    const bool diag = b == t;  // the same in the whole cluster
+    if (diag && !targets) return;
+    const int nsrc = min(kTile, N - t * kTile);
+    if (tid < kTile + 32) {
+        const bool s = tid < kTile;
+        const int j = s ? t * kTile + tid : b * kTile + 32 * w + (tid - kTile);
+        SrcF32 v;
+        v.p = make_float4(s ? 1e18f : 0.f, 0.f, 0.f, 0.f);
+        v.f = make_float4(1.f, 0.f, 0.f, 0.f);
+        v.t = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (j < N) v = src[j];
+        (s ? ss[tid] : st[tid - kTile]) = v;
+    }
+    __syncthreads();
+    // the nine images of target T and source S under one vote, so that their blocks are straight-line code with
+    // nine chains in flight (three to a vote 54 us a product, nine 46, before warps took turns);
+    // eval(image, rx, ry, rz, rho2, r2, close), image 4 the unshifted one
+    auto images = [&](const SrcF32 &T, const SrcF32 &S, auto &&eval) {
+        const float rx0 = min_image_f(add2(sub2(T.p.x, S.p.x), sub2(T.p.z, S.p.z)), pl.xh, pl.xl, pl.ix);
+        const float ry0 = min_image_f(add2(sub2(T.p.y, S.p.y), sub2(T.p.w, S.p.w)), pl.yh, pl.yl, pl.iy);
+        const float rz = sub2(T.f.x, S.f.x);
+        float rx[3], ry[3], yy[3], rho2[9], r2[9];
+        bool near = false;
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            rx[s] = fmaf((float)(s - 1), pl.xl, fmaf((float)(s - 1), pl.xh, rx0));
+            ry[s] = fmaf((float)(s - 1), pl.yl, fmaf((float)(s - 1), pl.yh, ry0));
+            yy[s] = mul2(ry[s], ry[s]);
+        }
+#pragma unroll
+        for (int s = 0; s < 9; ++s) {
+            rho2[s] = fma2(rx[s / 3], rx[s / 3], yy[s % 3]);
+            r2[s] = fma2(rz, rz, rho2[s]);
+            near = near || r2[s] < c.four_a2;
+        }
+        if (__any_sync(0xffffffffu, near)) {
+#pragma unroll
+            for (int s = 0; s < 9; ++s) eval(s, rx[s / 3], ry[s % 3], rz, rho2[s], r2[s], true);
+        } else {
+#pragma unroll
+            for (int s = 0; s < 9; ++s) eval(s, rx[s / 3], ry[s % 3], rz, rho2[s], r2[s], false);
+        }
+    };
+    if (targets) {
+        const int e = warp & 1, turn = warp >> 1;
+        const SrcF32 T = st[lane];
+        const int pk = diag ? 0 : (2 * ((lane >> 4) & 1)) ^ ((lane >> 3) & 1);
+        const int K = diag ? ((nsrc + 1) / 2 + 3) / 4 * 4 : (nsrc + 7) / 8 * 4;  // at most kTile / 2
+        float u[3] = {0.f, 0.f, 0.f};
+        // turns: the 32 threads of the warp before arrive at one of barriers 1 .. 8 when they have added their
+        // source, ours wait there
+        for (int k = turn; k < K; k += 4) {
+            const int j = 2 * (k ^ pk) + e;
+            const SrcF32 S = ss[j];
+            TTTerms<float> tt[9];
+            TRTerms<float> tr[9];
+            images(T, S, [&](int s, float rx, float ry, float rz, float rho2, float r2, bool close) {
+                TTBlock<float> m;
+                TRBlock<float> tb;
+                pair_block_x2<TORQUE>(rx, ry, rz, rho2, r2, close, T.f.x, S.f.x, -2.f * S.f.x, -4.f * (S.f.x * S.f.x),
+                                      6.f * T.f.x, 6.f * S.f.x, c, m, tb);
+                tt[s] = tt_target_terms(m, S.f.y, S.f.z, S.f.w);
+                if (TORQUE) tr[s] = tr_target_terms(m, tb, S.t.x, S.t.y, S.t.z);
+            });
+            float d[9][3];
+            if (diag) {  // here every image's velocity is rounded before it is added, the self term's left out
+                const bool self = j == 32 * w + lane;
+#pragma unroll
+                for (int s = 0; s < 9; ++s) {
+                    d[s][0] = d[s][1] = d[s][2] = 0.f;
+                    tt_target_add(tt[s], S.f.y, S.f.z, S.f.w, d[s][0], d[s][1], d[s][2]);
+                    if (TORQUE) tr_target_add(tr[s], S.t.x, S.t.y, d[s][0], d[s][1], d[s][2]);
+                    if (s == 4 && self) d[s][0] = d[s][1] = d[s][2] = 0.f;
+                }
+            }
+            if (k > 0) {
+                asm volatile("bar.sync %0, 64;" ::"r"(1 + 4 * e + turn) : "memory");
+#pragma unroll
+                for (int q = 0; q < 3; ++q) u[q] = us[e][q][lane];
+            }
+            if (diag) {
+#pragma unroll
+                for (int s = 0; s < 9; ++s)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) u[q] = add2(u[q], d[s][q]);
+            } else {
+#pragma unroll
+                for (int s = 0; s < 9; ++s) {
+                    tt_target_add(tt[s], S.f.y, S.f.z, S.f.w, u[0], u[1], u[2]);
+                    if (TORQUE) tr_target_add(tr[s], S.t.x, S.t.y, u[0], u[1], u[2]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) us[e][q][lane] = u[q];
+            if (k + 1 < K) asm volatile("bar.arrive %0, 64;" ::"r"(1 + 4 * e + ((turn + 1) & 3)) : "memory");
+        }
+        __syncthreads();
+        if (warp < 3) tgt_part[((size_t)sg * 3 + warp) * kTile + 32 * w + lane] = (double)add2(us[0][warp][lane], us[1][warp][lane]);
+    } else {
+        const int half = warp >> 2, j = 32 * (warp & 3) + lane;
+        const SrcF32 S = ss[j];
+        float tree[4][3], x[3];
+        for (int n = 0; n < 16; ++n) {
+            const SrcF32 T = st[__brev(16 * half + n) >> 27];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) x[q] = 0.f;
+            images(T, S, [&](int, float rx, float ry, float rz, float rho2, float r2, bool close) {
+                TTBlock<float> m;
+                TRBlock<float> tb;
+                float v[3];
+                pair_block_x2<TORQUE>(rx, ry, rz, rho2, r2, close, T.f.x, S.f.x, -2.f * S.f.x, -4.f * (S.f.x * S.f.x),
+                                      6.f * T.f.x, 6.f * S.f.x, c, m, tb);
+                tt_apply_source(m, T.f.y, T.f.z, T.f.w, v[0], v[1], v[2]);
+                if (TORQUE) tr_apply_source(m, tb, T.t.x, T.t.y, T.t.z, v[0], v[1], v[2]);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) x[q] = add2(x[q], v[q]);
+            });
+            // add the finished left subtrees that end here, keep the result as its level's left one
+            bool kept = false;
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                if (!kept && ((n >> l) & 1)) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) x[q] = add2(tree[l][q], x[q]);
+                } else if (!kept) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) tree[l][q] = x[q];
+                    kept = true;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) sv[half][q][j] = x[q];
+    }
+    if (diag) return;
+    cl.sync();  // the sums of the four CTAs are there
+    if (!targets && tid < 96) {
+        const int q = tid >> 5, j = 32 * w + lane;
+        float x[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float *o = cl.map_shared_rank(&sv[0][0][0], 4 + r) + q * kTile + j;
+            x[r] = add2(o[0], o[3 * kTile]);
+        }
+        src_part[((size_t)(col_start[t] + b) * 3 + q) * kTile + j] = add2(add2(x[0], x[1]), add2(x[2], x[3]));
+    }
+    cl.sync();  // no CTA leaves while another reads its sums
+}
+
 // Row partials of the targets plus column partials of the sources, fixed order, and the float64 self term
 // from the spheres' coefficients (left out when self_term is 0, for all but one share of a shared
 // product).  col_rows: the rows [r0, r1) of each column that the schedule wrote (null: all rows above the
@@ -914,6 +1093,11 @@ constexpr int kPerMinBlocks = 4, kPerFusedMinBlocks = 3;
 // and the registers keep the constants and more of a step in flight (a step of 1024 spheres 426 -> 411 us,
 // pseudo-periodic 256 spheres 930 -> 905 us; with full waves they are 3% slower, 5.58 ms a product at 65536).
 constexpr int kSmallMinBlocks = 2;
+// Pseudo-periodic tiles that take pair_sym_lanes_kernel's cluster of eight CTAs: while these make at most three
+// CTAs per SM (1280 spheres at 152 SMs).  A product in us, one CTA of packed arithmetic a tile -> a cluster, without
+// / with torques: 256 spheres 79 -> 34 / 99 -> 37, 700 80 -> 44 / 101 -> 54, 1024 80 -> 46 / 101 -> 74,
+// 1280 80 -> 70 / 101 -> 95, 1500 82 -> 79 / 103 -> 113.
+constexpr int kLanesCtasPerSm = 3;
 
 // Capacity of the schedule: at most kSymMaxCtaPerSm x SMs CTAs and that many plus nb segments.
 constexpr int kSymMaxCtaPerSm = 64;
@@ -1060,11 +1244,16 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
     pl.iy = 1.f / pl.yh;
     if (sc->ncta > 0) {
         const bool small = sc->ncta <= kSmallMinBlocks * ctx->num_sms;
+        const bool lanes = 8 * sc->ncta <= kLanesCtasPerSm * ctx->num_sms;  // then a run is one tile
         auto run = [&](auto kernel) {
             kernel<<<sc->ncta, kPairThreads, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, pl, nullptr,
                                                       nullptr);
         };
-        if (T && small)
+        if (T && lanes)
+            pair_sym_lanes_kernel<true><<<8 * sc->ncta, 256, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, pl);
+        else if (lanes)
+            pair_sym_lanes_kernel<false><<<8 * sc->ncta, 256, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, pl);
+        else if (T && small)
             run(pair_f32x2_sym_kernel<kSmallMinBlocks, true, false, true>);
         else if (T)
             run(pair_f32x2_sym_kernel<kPerFusedMinBlocks, true, false, true>);

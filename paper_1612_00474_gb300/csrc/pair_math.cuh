@@ -421,6 +421,50 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b)
     return __fadd2_rn(a, neg2(b));
 }
 
+// The same operations on one value: the pair functions below take either a float2 (two pairs per lane) or a
+// float (one pair per lane, for kernels that spread few pairs over many warps), bit for bit alike.
+__device__ __forceinline__ float fma2(float a, float b, float c)
+{
+    return __fmaf_rn(a, b, c);
+}
+__device__ __forceinline__ float mul2(float a, float b)
+{
+    return __fmul_rn(a, b);
+}
+__device__ __forceinline__ float add2(float a, float b)
+{
+    return __fadd_rn(a, b);
+}
+__device__ __forceinline__ float neg2(float a)
+{
+    return -a;
+}
+__device__ __forceinline__ float sub2(float a, float b)
+{
+    return __fadd_rn(a, -b);
+}
+__device__ __forceinline__ float2 rsqrt2(float2 a)
+{
+    return make_float2(rsqrt_ftz(a.x), rsqrt_ftz(a.y));
+}
+__device__ __forceinline__ float rsqrt2(float a)
+{
+    return rsqrt_ftz(a);
+}
+// a constant (both halves alike) in the pair functions' type
+template <typename V>
+__device__ __forceinline__ V konst(float2 v);
+template <>
+__device__ __forceinline__ float2 konst<float2>(float2 v)
+{
+    return v;
+}
+template <>
+__device__ __forceinline__ float konst<float>(float2 v)
+{
+    return v.x;
+}
+
 // Overlap branch (r < 2a) of the free-space coefficients for one pair: c1 - u (u = 1/|R| of the
 // image), c2 and the rotlet coefficient c_t.  r^2 below the smallest normal float is a coincident
 // pair (the self form).
@@ -432,6 +476,18 @@ __device__ __forceinline__ void near_fix(float r2, float inv_r, float u, const X
     c1mu = fmaf(c.near_c1, fmaf(-c.near_r, r, 1.f), -u);
     c2 = c.near_c2 * ir;
     ct = c.near_tr * fmaf(-c.near_tr_r, r, 1.f);
+}
+
+// Pairs with r^2 below 4a^2 among a lane's two (or its one) take the overlap branch.
+__device__ __forceinline__ void near_fix2(float2 r2, float2 inv_r, float2 u, const X2Consts &c, float2 &c1mu, float2 &c2,
+                                          float2 &ct)
+{
+    if (r2.x < c.four_a2) near_fix(r2.x, inv_r.x, u.x, c, c1mu.x, c2.x, ct.x);
+    if (r2.y < c.four_a2) near_fix(r2.y, inv_r.y, u.y, c, c1mu.y, c2.y, ct.y);
+}
+__device__ __forceinline__ void near_fix2(float r2, float inv_r, float u, const X2Consts &c, float &c1mu, float &c2, float &ct)
+{
+    if (r2 < c.four_a2) near_fix(r2, inv_r, u, c, c1mu, c2, ct);
 }
 
 // Offsets of the target from two sources (packed), from the high parts of the positions; the low
@@ -461,52 +517,51 @@ __device__ __forceinline__ bool pair_offsets_x2(float2 txh, float2 tyh, float2 t
 
 // Coefficients of a translation-translation pair block (packed pairs): M F = c_F F + c2 (r.F) r +
 // (B3 w + C3 F_z) R + (D3 w + E3 F_z) z_hat with w = R.F, c_FE = c_F + E3.
+template <typename V>
 struct TTBlock {
-    float2 rx, ry, rz, Rz, c2, cF, cFE, B3, C3, D3;
+    V rx, ry, rz, Rz, c2, cF, cFE, B3, C3, D3;
 };
 // Direction-independent factors of the translation-rotation coupling: dcp = c_t - u^3; m2, kappa and
 // the z factor (dcp - 2a^2 u^5 - kappa R_z) for the pair (t) and the reversed pair (s).
+template <typename V>
 struct TRBlock {
-    float2 dcp, m2t, m2s, kt, ks, zt, zs;
+    V dcp, m2t, m2s, kt, ks, zt, zs;
 };
 
 // The block of two pairs from their geometry: in-plane offset (rx, ry), rz = zi - zj, rho2 = rx^2 +
 // ry^2, r2 = rho2 + rz^2; `close` true (warp-uniformly) when some lane may hold an overlapping pair
 // (r < 2a), the overlap branch then being taken per pair.  m2zj = -2 z_j, m4zj2 = -4 z_j^2; six_zi,
 // six_zj = 6 z_i, 6 z_j (read only with TORQUE; six_zj only for the reversed pair's factors).
-template <bool TORQUE>
-__device__ __forceinline__ void pair_block_x2(float2 rx, float2 ry, float2 rz, float2 rho2, float2 r2, bool close,
-                                              float2 zi, float2 zj, float2 m2zj, float2 m4zj2, float2 six_zi,
-                                              float2 six_zj, const X2Consts &c, TTBlock &m, TRBlock &tb)
+template <bool TORQUE, typename V>
+__device__ __forceinline__ void pair_block_x2(V rx, V ry, V rz, V rho2, V r2, bool close,
+                                              V zi, V zj, V m2zj, V m4zj2, V six_zi,
+                                              V six_zj, const X2Consts &c, TTBlock<V> &m, TRBlock<V> &tb)
 {
-    const float2 ir = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-    const float2 Rz = add2(zi, zj);
-    const float2 Z = mul2(Rz, Rz);
-    const float2 R2 = add2(rho2, Z);
-    const float2 u = make_float2(rsqrt_ftz(R2.x), rsqrt_ftz(R2.y));
-    const float2 ir2 = mul2(ir, ir);
-    const float2 ir3 = mul2(ir, ir2);
-    float2 c1mu = fma2(c.two_3_a2, ir3, sub2(ir, u));  // (1 + 2a^2/(3 r^2)) / r - u
-    float2 c2 = fma2(c.m_two_a2, mul2(ir3, ir2), ir3);  // (1 - 2a^2/r^2) / r^3
-    float2 ct = ir3;
-    if (close) {
-        if (r2.x < c.four_a2) near_fix(r2.x, ir.x, u.x, c, c1mu.x, c2.x, ct.x);
-        if (r2.y < c.four_a2) near_fix(r2.y, ir.y, u.y, c, c1mu.y, c2.y, ct.y);
-    }
-    const float2 s = mul2(u, u);
-    const float2 u3 = mul2(s, u);
-    const float2 u5 = mul2(u3, s);
-    const float2 sZ = mul2(s, Z);
-    const float2 p = fma2(m2zj, zi, c.m2_3_a2);
-    const float2 q = fma2(c.two_a2, Z, c.two_3_a4);
-    const float2 XA = fma2(s, fma2(sZ, c.m10_3_a4, q), p);
-    const float2 XB2 = fma2(s, fma2(sZ, c.c140_3_a4, fma2(c.m20_a2, Z, c.m20_3_a4)), mul2(c.m6, p));
-    const float2 Eh = fma2(s, fma2(sZ, c.c20_a4, fma2(c.m4_a2, Z, c.m8_3_a4)), m4zj2);
-    const float2 b2 = mul2(u5, XB2);
-    const float2 T2 = neg2(mul2(u3, m2zj));  // 2 u^3 z_j
-    const float2 u5Rz = mul2(u5, Rz);
-    const float2 u7Rz = mul2(u5Rz, s);
-    const float2 cF = fma2(u3, XA, c1mu);
+    const V ir = rsqrt2(r2);
+    const V Rz = add2(zi, zj);
+    const V Z = mul2(Rz, Rz);
+    const V R2 = add2(rho2, Z);
+    const V u = rsqrt2(R2);
+    const V ir2 = mul2(ir, ir);
+    const V ir3 = mul2(ir, ir2);
+    V c1mu = fma2(konst<V>(c.two_3_a2), ir3, sub2(ir, u));  // (1 + 2a^2/(3 r^2)) / r - u
+    V c2 = fma2(konst<V>(c.m_two_a2), mul2(ir3, ir2), ir3);  // (1 - 2a^2/r^2) / r^3
+    V ct = ir3;
+    if (close) near_fix2(r2, ir, u, c, c1mu, c2, ct);
+    const V s = mul2(u, u);
+    const V u3 = mul2(s, u);
+    const V u5 = mul2(u3, s);
+    const V sZ = mul2(s, Z);
+    const V p = fma2(m2zj, zi, konst<V>(c.m2_3_a2));
+    const V q = fma2(konst<V>(c.two_a2), Z, konst<V>(c.two_3_a4));
+    const V XA = fma2(s, fma2(sZ, konst<V>(c.m10_3_a4), q), p);
+    const V XB2 = fma2(s, fma2(sZ, konst<V>(c.c140_3_a4), fma2(konst<V>(c.m20_a2), Z, konst<V>(c.m20_3_a4))), mul2(konst<V>(c.m6), p));
+    const V Eh = fma2(s, fma2(sZ, konst<V>(c.c20_a4), fma2(konst<V>(c.m4_a2), Z, konst<V>(c.m8_3_a4))), m4zj2);
+    const V b2 = mul2(u5, XB2);
+    const V T2 = neg2(mul2(u3, m2zj));  // 2 u^3 z_j
+    const V u5Rz = mul2(u5, Rz);
+    const V u7Rz = mul2(u5Rz, s);
+    const V cF = fma2(u3, XA, c1mu);
     m.rx = rx;
     m.ry = ry;
     m.rz = rz;
@@ -514,17 +569,17 @@ __device__ __forceinline__ void pair_block_x2(float2 rx, float2 ry, float2 rz, f
     m.c2 = c2;
     m.cF = cF;
     m.cFE = fma2(u3, Eh, cF);
-    m.B3 = fma2(b2, c.half, neg2(u3));
-    m.C3 = fma2(neg2(Rz), b2, fma2(u7Rz, c.c20_3_a4, T2));
-    m.D3 = fma2(u7Rz, c.m20_3_a4, T2);
+    m.B3 = fma2(b2, konst<V>(c.half), neg2(u3));
+    m.C3 = fma2(neg2(Rz), b2, fma2(u7Rz, konst<V>(c.c20_3_a4), T2));
+    m.D3 = fma2(u7Rz, konst<V>(c.m20_3_a4), T2);
     if (TORQUE) {
-        const float2 dcp = sub2(ct, u3);
-        const float2 dcprz = mul2(dcp, rz);
-        const float2 w10 = mul2(c.m10_a2, u7Rz);
-        const float2 d2 = fma2(c.m_two_a2, u5, dcp);
+        const V dcp = sub2(ct, u3);
+        const V dcprz = mul2(dcp, rz);
+        const V w10 = mul2(konst<V>(c.m10_a2), u7Rz);
+        const V d2 = fma2(konst<V>(c.m_two_a2), u5, dcp);
         tb.dcp = dcp;
-        tb.m2t = fma2(u5Rz, c.two_a2, dcprz);
-        tb.m2s = fma2(u5Rz, c.two_a2, neg2(dcprz));
+        tb.m2t = fma2(u5Rz, konst<V>(c.two_a2), dcprz);
+        tb.m2s = fma2(u5Rz, konst<V>(c.two_a2), neg2(dcprz));
         tb.kt = fma2(six_zi, u5, w10);
         tb.ks = fma2(six_zj, u5, w10);
         tb.zt = fma2(neg2(Rz), tb.kt, d2);
@@ -532,50 +587,79 @@ __device__ __forceinline__ void pair_block_x2(float2 rx, float2 ry, float2 rz, f
     }
 }
 
-// target side: u += M_ij F_j
-__device__ __forceinline__ void tt_apply_target(const TTBlock &m, float2 Fx, float2 Fy, float2 Fz, float2 &ux,
-                                                float2 &uy, float2 &uz)
+// target side: u += M_ij F_j, as the factors of one block and the chain of multiply-adds into u (apart for the
+// kernel whose warps take turns at u)
+template <typename V>
+struct TTTerms {
+    V rx, ry, rz, Rz, cF, cFE, kk, k2, ke, D3, w;
+};
+template <typename V>
+__device__ __forceinline__ TTTerms<V> tt_target_terms(const TTBlock<V> &m, V Fx, V Fy, V Fz)
 {
-    const float2 pF = fma2(m.rx, Fx, mul2(m.ry, Fy));
-    const float2 w = fma2(m.Rz, Fz, pF);
-    const float2 k2 = mul2(m.c2, fma2(m.rz, Fz, pF));
-    const float2 ke = fma2(m.B3, w, mul2(m.C3, Fz));
-    const float2 kk = add2(k2, ke);
-    ux = fma2(m.cF, Fx, fma2(kk, m.rx, ux));
-    uy = fma2(m.cF, Fy, fma2(kk, m.ry, uy));
-    uz = fma2(m.cFE, Fz, fma2(k2, m.rz, fma2(ke, m.Rz, fma2(m.D3, w, uz))));
+    const V pF = fma2(m.rx, Fx, mul2(m.ry, Fy));
+    const V w = fma2(m.Rz, Fz, pF);
+    const V k2 = mul2(m.c2, fma2(m.rz, Fz, pF));
+    const V ke = fma2(m.B3, w, mul2(m.C3, Fz));
+    return {m.rx, m.ry, m.rz, m.Rz, m.cF, m.cFE, add2(k2, ke), k2, ke, m.D3, w};
+}
+template <typename V>
+__device__ __forceinline__ void tt_target_add(const TTTerms<V> &t, V Fx, V Fy, V Fz, V &ux, V &uy, V &uz)
+{
+    ux = fma2(t.cF, Fx, fma2(t.kk, t.rx, ux));
+    uy = fma2(t.cF, Fy, fma2(t.kk, t.ry, uy));
+    uz = fma2(t.cFE, Fz, fma2(t.k2, t.rz, fma2(t.ke, t.Rz, fma2(t.D3, t.w, uz))));
+}
+template <typename V>
+__device__ __forceinline__ void tt_apply_target(const TTBlock<V> &m, V Fx, V Fy, V Fz, V &ux, V &uy, V &uz)
+{
+    tt_target_add(tt_target_terms(m, Fx, Fy, Fz), Fx, Fy, Fz, ux, uy, uz);
 }
 // source side: v = M_ij^T G_i (C3 and D3 exchanged)
-__device__ __forceinline__ void tt_apply_source(const TTBlock &m, float2 Gx, float2 Gy, float2 Gz, float2 &vx,
-                                                float2 &vy, float2 &vz)
+template <typename V>
+__device__ __forceinline__ void tt_apply_source(const TTBlock<V> &m, V Gx, V Gy, V Gz, V &vx,
+                                                V &vy, V &vz)
 {
-    const float2 pF = fma2(m.rx, Gx, mul2(m.ry, Gy));
-    const float2 w = fma2(m.Rz, Gz, pF);
-    const float2 k2 = mul2(m.c2, fma2(m.rz, Gz, pF));
-    const float2 ke = fma2(m.B3, w, mul2(m.D3, Gz));
-    const float2 kk = add2(k2, ke);
+    const V pF = fma2(m.rx, Gx, mul2(m.ry, Gy));
+    const V w = fma2(m.Rz, Gz, pF);
+    const V k2 = mul2(m.c2, fma2(m.rz, Gz, pF));
+    const V ke = fma2(m.B3, w, mul2(m.D3, Gz));
+    const V kk = add2(k2, ke);
     vx = fma2(m.cF, Gx, mul2(kk, m.rx));
     vy = fma2(m.cF, Gy, mul2(kk, m.ry));
     vz = fma2(m.cFE, Gz, fma2(k2, m.rz, fma2(ke, m.Rz, mul2(m.C3, w))));
 }
-// target side of the translation-rotation coupling: u += M_tr(i, j) T_j
-__device__ __forceinline__ void tr_apply_target(const TTBlock &m, const TRBlock &tb, float2 Tx, float2 Ty, float2 Tz,
-                                                float2 &ux, float2 &uy, float2 &uz)
+// target side of the translation-rotation coupling: u += M_tr(i, j) T_j, likewise
+template <typename V>
+struct TRTerms {
+    V rx, ry, m2, dTz, kt, tz3, zt;
+};
+template <typename V>
+__device__ __forceinline__ TRTerms<V> tr_target_terms(const TTBlock<V> &m, const TRBlock<V> &tb, V Tx, V Ty, V Tz)
 {
-    const float2 tz3 = fma2(Tx, m.ry, neg2(mul2(Ty, m.rx)));
-    const float2 dTz = mul2(tb.dcp, Tz);
-    const float2 kt = mul2(tb.kt, tz3);
-    ux = fma2(Ty, tb.m2t, fma2(neg2(dTz), m.ry, fma2(neg2(kt), m.rx, ux)));
-    uy = fma2(neg2(Tx), tb.m2t, fma2(dTz, m.rx, fma2(neg2(kt), m.ry, uy)));
-    uz = fma2(tz3, tb.zt, uz);
+    const V tz3 = fma2(Tx, m.ry, neg2(mul2(Ty, m.rx)));
+    return {m.rx, m.ry, tb.m2t, mul2(tb.dcp, Tz), mul2(tb.kt, tz3), tz3, tb.zt};
+}
+template <typename V>
+__device__ __forceinline__ void tr_target_add(const TRTerms<V> &t, V Tx, V Ty, V &ux, V &uy, V &uz)
+{
+    ux = fma2(Ty, t.m2, fma2(neg2(t.dTz), t.ry, fma2(neg2(t.kt), t.rx, ux)));
+    uy = fma2(neg2(Tx), t.m2, fma2(t.dTz, t.rx, fma2(neg2(t.kt), t.ry, uy)));
+    uz = fma2(t.tz3, t.zt, uz);
+}
+template <typename V>
+__device__ __forceinline__ void tr_apply_target(const TTBlock<V> &m, const TRBlock<V> &tb, V Tx, V Ty, V Tz, V &ux, V &uy,
+                                                V &uz)
+{
+    tr_target_add(tr_target_terms(m, tb, Tx, Ty, Tz), Tx, Ty, ux, uy, uz);
 }
 // source side: v += M_tr(j, i) H_i (the reversed pair: r -> -r, z_i <-> z_j)
-__device__ __forceinline__ void tr_apply_source(const TTBlock &m, const TRBlock &tb, float2 Hx, float2 Hy, float2 Hz,
-                                                float2 &vx, float2 &vy, float2 &vz)
+template <typename V>
+__device__ __forceinline__ void tr_apply_source(const TTBlock<V> &m, const TRBlock<V> &tb, V Hx, V Hy, V Hz,
+                                                V &vx, V &vy, V &vz)
 {
-    const float2 tau = fma2(Hx, m.ry, neg2(mul2(Hy, m.rx)));
-    const float2 dHz = mul2(tb.dcp, Hz);
-    const float2 ks = mul2(tb.ks, tau);
+    const V tau = fma2(Hx, m.ry, neg2(mul2(Hy, m.rx)));
+    const V dHz = mul2(tb.dcp, Hz);
+    const V ks = mul2(tb.ks, tau);
     vx = fma2(Hy, tb.m2s, fma2(dHz, m.ry, fma2(neg2(ks), m.rx, vx)));
     vy = fma2(neg2(Hx), tb.m2s, fma2(neg2(dHz), m.rx, fma2(neg2(ks), m.ry, vy)));
     vz = fma2(neg2(tau), tb.zs, vz);
@@ -583,18 +667,18 @@ __device__ __forceinline__ void tr_apply_source(const TTBlock &m, const TRBlock 
 
 // Target velocity of two sources (one-way), from the geometry of pair_offsets_x2 (close: some lane
 // may overlap); the per-source factors are formed here.  In units of 1/(8 pi eta); F, T with s_j.
-template <bool TORQUE>
-__device__ __forceinline__ void pair_velocity_x2_geo(float2 rx, float2 ry, float2 rz, float2 rho2, float2 r2,
-                                                     bool close, float2 zi, float2 zj, float2 Fx, float2 Fy,
-                                                     float2 Fz, float2 Tx, float2 Ty, float2 Tz, const X2Consts &c,
-                                                     float2 &ux, float2 &uy, float2 &uz)
+template <bool TORQUE, typename V>
+__device__ __forceinline__ void pair_velocity_x2_geo(V rx, V ry, V rz, V rho2, V r2,
+                                                     bool close, V zi, V zj, V Fx, V Fy,
+                                                     V Fz, V Tx, V Ty, V Tz, const X2Consts &c,
+                                                     V &ux, V &uy, V &uz)
 {
-    const float2 zj2 = add2(zj, zj);
-    const float2 six = make_float2(6.f, 6.f);
-    TTBlock m;
-    TRBlock tb;
+    const V zj2 = add2(zj, zj);
+    const V six = konst<V>(make_float2(6.f, 6.f));
+    TTBlock<V> m;
+    TRBlock<V> tb;
     pair_block_x2<TORQUE>(rx, ry, rz, rho2, r2, close, zi, zj, neg2(zj2), neg2(mul2(zj2, zj2)), mul2(six, zi),
-                          make_float2(0.f, 0.f), c, m, tb);
+                          V{}, c, m, tb);
     tt_apply_target(m, Fx, Fy, Fz, ux, uy, uz);
     if (TORQUE) tr_apply_target(m, tb, Tx, Ty, Tz, ux, uy, uz);
 }
@@ -620,18 +704,18 @@ __device__ __forceinline__ void pair_velocity_x2(float2 rx, float2 ry, float2 zi
 // m4zj2 = -4 z_j^2, six_zj = 6 z_j and the target's six_zi = 6 z_i come precomputed.
 // RHS2: a second translation-translation right-hand side applied with the same block, P (sources)
 // and Q (targets) -> u2 (target side, accumulated) and v2 (source side, returned).
-template <bool TORQUE, bool RHS2 = false>
-__device__ __forceinline__ void pair_sym_x2(float2 rx, float2 ry, float2 rz, float2 rho2, float2 r2, bool close,
-                                            float2 zi, float2 zj, float2 m2zj, float2 m4zj2, float2 six_zi,
-                                            float2 six_zj, float2 Fx, float2 Fy, float2 Fz, float2 Gx,
-                                            float2 Gy, float2 Gz, float2 Tx, float2 Ty, float2 Tz, float2 Hx,
-                                            float2 Hy, float2 Hz, const X2Consts &c, float2 &ux, float2 &uy,
-                                            float2 &uz, float2 &vx, float2 &vy, float2 &vz, float2 Px = {},
-                                            float2 Py = {}, float2 Pz = {}, float2 Qx = {}, float2 Qy = {},
-                                            float2 Qz = {}, float2 *u2 = nullptr, float2 *v2 = nullptr)
+template <bool TORQUE, bool RHS2 = false, typename V>
+__device__ __forceinline__ void pair_sym_x2(V rx, V ry, V rz, V rho2, V r2, bool close,
+                                            V zi, V zj, V m2zj, V m4zj2, V six_zi,
+                                            V six_zj, V Fx, V Fy, V Fz, V Gx,
+                                            V Gy, V Gz, V Tx, V Ty, V Tz, V Hx,
+                                            V Hy, V Hz, const X2Consts &c, V &ux, V &uy,
+                                            V &uz, V &vx, V &vy, V &vz, V Px = {},
+                                            V Py = {}, V Pz = {}, V Qx = {}, V Qy = {},
+                                            V Qz = {}, V *u2 = nullptr, V *v2 = nullptr)
 {
-    TTBlock m;
-    TRBlock tb;
+    TTBlock<V> m;
+    TRBlock<V> tb;
     pair_block_x2<TORQUE>(rx, ry, rz, rho2, r2, close, zi, zj, m2zj, m4zj2, six_zi, six_zj, c, m, tb);
     tt_apply_target(m, Fx, Fy, Fz, ux, uy, uz);
     tt_apply_source(m, Gx, Gy, Gz, vx, vy, vz);
