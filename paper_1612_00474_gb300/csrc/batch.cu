@@ -20,6 +20,7 @@
 #include <new>
 #include <vector>
 
+#include "cells.cuh"
 #include "gs.cuh"
 #include "pair_math.cuh"
 
@@ -261,113 +262,12 @@ __global__ void __launch_bounds__(kPairThreads) batch_pair_f64_kernel(
     }
 }
 
-// Forces of Sec. III within each instance (same screening as the single-suspension kernel).
+// Forces of Sec. III within each instance: the cell lists of cells.cuh over the whole batch.
 // Pairs farther apart than 2a + kFarB b, whose repulsion is below e^-kFarB U0/b (~2e-9 U0/b), take it
 // in float32 (IEEE square root and division, expf: a relative error of a few 1e-6 on a term that small
 // is below 1e-14 U0/b) and are summed in float32 before their total joins the float64 sum; nearer
-// pairs are evaluated in float64.  The two kinds are queued apart so that a warp runs the float64 loop
-// only as long as its longest near queue (a float64 warp instruction costs the same whatever the
-// number of active lanes).
-constexpr float kFarB = 20.f;
-
-__global__ void __launch_bounds__(128) batch_forces_kernel(const double *__restrict__ pos, const InstDesc *__restrict__ inst,
-                                                           const BlockDesc *__restrict__ blocks, int64_t total, double a,
-                                                           double weight, double U0, double b, float cut2,
-                                                           float near2, double *__restrict__ F)
-{
-    // the screen of forces_kernel, within the block's own instance: the float32 screen takes two
-    // sources per lane (packed); near pairs are queued from the front of one array, far pairs from its
-    // back, and each kind is evaluated together, in index order
-    __shared__ float4 sp[64];
-    __shared__ float2 sz[64];
-    const BlockDesc bd = blocks[blockIdx.x];
-    const InstDesc d = inst[bd.inst];
-    const int tid = threadIdx.x;
-    const int il = bd.first + tid;
-    const int64_t i = d.off + il;
-    const bool valid = il < d.N;
-    double xi = 0.0, yi = 0.0, zi = 0.0;
-    if (valid) {
-        xi = pos[i];
-        yi = pos[total + i];
-        zi = pos[2 * total + i];
-    }
-    const float xf = (float)xi, yf = (float)yi, zf = (float)zi;
-    const double f0 = U0 / b, inv_b = 1.0 / b;
-    const float f0f = (float)f0, inv_bf = (float)inv_b, two_af = (float)(2.0 * a);
-    double fx = 0.0, fy = 0.0, fz = 0.0;
-    float gx = 0.f, gy = 0.f, gz = 0.f;  // far pairs
-    constexpr int kQ = 32;
-    int queue[kQ];
-    int nn = 0, nf = 0;  // near pairs at queue[0 .. nn), far pairs at queue[kQ - nf .. kQ)
-    auto flush = [&]() {
-        for (int q = 0; q < nn; ++q) {
-            const int64_t j = d.off + queue[q];
-            const double dx = xi - pos[j], dy = yi - pos[total + j], dz = zi - pos[2 * total + j];
-            const double m = steric_pair_factor(dx * dx + dy * dy + dz * dz, 2.0 * a, f0, inv_b);
-            fx += m * dx;
-            fy += m * dy;
-            fz += m * dz;
-        }
-        for (int q = kQ - nf; q < kQ; ++q) {
-            const int64_t j = d.off + queue[q];
-            const float dx = (float)(xi - pos[j]), dy = (float)(yi - pos[total + j]), dz = (float)(zi - pos[2 * total + j]);
-            const float r = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-            const float m = f0f * expf((two_af - r) * inv_bf) / r;
-            gx = fmaf(m, dx, gx);
-            gy = fmaf(m, dy, gy);
-            gz = fmaf(m, dz, gz);
-        }
-        nn = 0;
-        nf = 0;
-    };
-    float *fxy = reinterpret_cast<float *>(sp);
-    float *fz2 = reinterpret_cast<float *>(sz);
-    const float2 X = make_float2(xf, xf), Y = make_float2(yf, yf), Z = make_float2(zf, zf);
-    const int pp = tid >> 1, hh = tid & 1;
-    for (int base = 0; base < d.N; base += 128) {
-        const int jl = base + tid;
-        const int64_t jt = d.off + jl;
-        // slots past the instance's end hold a point far above the wall (never inside the screen)
-        const bool in = jl < d.N;
-        fxy[4 * pp + hh] = in ? (float)pos[jt] : 0.f;
-        fxy[4 * pp + 2 + hh] = in ? (float)pos[total + jt] : 0.f;
-        fz2[2 * pp + hh] = in ? (float)pos[2 * total + jt] : 1e18f;
-        __syncthreads();
-#pragma unroll 8
-        for (int k = 0; k < 64; ++k) {
-            const float4 p = sp[k];
-            const float2 dx = sub2(X, make_float2(p.x, p.y)), dy = sub2(Y, make_float2(p.z, p.w));
-            const float2 dz = sub2(Z, sz[k]);
-            const float2 d2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-            if (d2.x < cut2 || d2.y < cut2) {
-                const int j0 = base + 2 * k;
-                if (d2.x < cut2 && j0 != il && j0 < d.N) {
-                    if (d2.x < near2)
-                        queue[nn++] = j0;
-                    else
-                        queue[kQ - ++nf] = j0;
-                    if (nn + nf == kQ) flush();
-                }
-                if (d2.y < cut2 && j0 + 1 != il && j0 + 1 < d.N) {
-                    if (d2.y < near2)
-                        queue[nn++] = j0 + 1;
-                    else
-                        queue[kQ - ++nf] = j0 + 1;
-                    if (nn + nf == kQ) flush();
-                }
-            }
-        }
-        __syncthreads();
-    }
-    flush();
-    if (valid) {
-        fz += (zi < a ? f0 : f0 * exp(-(zi - a) / b)) - weight;
-        F[i] = fx + (double)gx;
-        F[total + i] = fy + (double)gy;
-        F[2 * total + i] = fz + (double)gz;
-    }
-}
+// pairs are evaluated in float64.
+constexpr double kFarB = 20.0;
 
 // ------------------------------------------------------------------ noise and elementwise steps
 __device__ __forceinline__ uint4 philox4x32_10_b(uint4 c, uint32_t k0, uint32_t k1)
@@ -667,6 +567,7 @@ struct rpb_batch {
     double *red = nullptr;
     double *norm2 = nullptr;
     double *selfc = nullptr;  // self coefficients of the packed positions (SelfCoefs), 4 max_total_N
+    void *cells = nullptr;    // cell lists of the force pass (cell_lists_bytes)
     double *nodes = nullptr;  // nodes and weights of the Lanczos square root
     // host (pinned)
     InstDesc *h_inst = nullptr;
@@ -709,7 +610,7 @@ enum { V_POS, V_UP, V_F, V_T, V_UN, V_W, V_WT, V_G, V_DRIFT, V_PA, V_PB, V_WORK,
 static void batch_free(rpb_batch *bt)
 {
     void *dev[] = {bt->d_inst, bt->d_blocks, bt->d_chunks, bt->d_inst_chunks, bt->d_inst_of, bt->d_active, bt->d_nactive, bt->src, bt->V, bt->lz, bt->red,
-                   bt->norm2, bt->selfc, bt->nodes, bt->d_left};
+                   bt->norm2, bt->selfc, bt->nodes, bt->cells, bt->d_left};
     for (void *p : dev)
         if (p) cudaFree(p);
     for (double *p : bt->vec)
@@ -999,11 +900,11 @@ static int batch_step_body(rpb_batch *bt, double dt, double delta, double tol, i
     int rc;
     const double a = bt->p.a;
     const double rcut = (2.0 * a + kForceCutoffB * fp->b) * 1.01 + 0.01 * a;
-    const double rnear = 2.0 * a + (double)kFarB * fp->b;
-    batch_forces_kernel<<<bt->nblocks, 128, 0, st>>>(v[V_POS], bt->d_inst, bt->d_blocks, total, a, fp->weight, fp->U0,
-                                                     fp->b, (float)(rcut * rcut), (float)(rnear * rnear), v[V_F]);
+    if ((rc = cell_forces<InstDesc>(st, cell_lists(bt->cells, bt->max_total), v[V_POS], total, a, fp->weight, fp->U0, fp->b,
+                                    rcut, 2.0 * a + kFarB * fp->b, bt->d_inst, bt->d_inst_of, v[V_F])))
+        return rc;
     batch_fill3_kernel<<<ge, 256, 0, st>>>(v[V_T], total, fp->torque[0], fp->torque[1], fp->torque[2]);
-    count_launches(2);
+    count_launches(1);
     if ((rc = batch_product(bt, v[V_POS], v[V_F], v[V_T], v[V_UN], nullptr))) return rc;
     batch_philox_kernel<<<dim3(bt->nchunks, 2), 256, 0, st>>>(bt->d_inst, bt->d_chunks, total, v[V_W], v[V_WT]);
     count_launches(1);
@@ -1185,6 +1086,7 @@ int rpb_batch_create(rpb_batch **out, const rpb_params *p, int64_t max_total_N, 
               cudaMallocHost(&bt->h_chunks, max_chunks * sizeof(ChunkDesc)) == cudaSuccess &&
               cudaMallocHost(&bt->h_inst_chunks, max_B * sizeof(int2)) == cudaSuccess &&
               cudaMalloc(&bt->selfc, (size_t)4 * max_total_N * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&bt->cells, cell_lists_bytes(max_total_N)) == cudaSuccess &&
               cudaMalloc(&bt->nodes, 2 * kSqrtNodes * sizeof(double)) == cudaSuccess &&
               cudaMallocHost(&bt->h_inst, max_B * sizeof(InstDesc)) == cudaSuccess &&
               cudaMallocHost(&bt->h_blocks, max_blocks * sizeof(BlockDesc)) == cudaSuccess &&

@@ -107,10 +107,9 @@ inline PairConsts<R> make_consts(double a)
 // e^{-40} U0/b ~ 4e-18 U0/b, far under the float64 rounding of any force it would be added to.
 constexpr double kForceCutoffB = 40.0;
 
-// Cell lists of the force pass (pair.cu): header, then int arrays in one allocation.
-constexpr int kCellGrid = 256;                  // at most kCellGrid x kCellGrid buckets (cells hashed modulo G)
-constexpr int kCells = kCellGrid * kCellGrid;
-constexpr int kCellMaxSorted = 512;             // a fuller cell hands the force pass to the all-pairs kernel
+// Cell lists of the force pass (cells.cuh): header, then the arrays in one allocation.
+constexpr int kCellGrid = 1024;     // at most kCellGrid x kCellGrid buckets (cells hashed modulo G)
+constexpr int kCellMaxSorted = 512;  // a fuller cell hands the force pass to the all-pairs kernel
 struct CellHeader {
     int overfull, pad[15];  // 64 bytes, followed by the bucket counts
 };
@@ -120,31 +119,36 @@ __device__ __forceinline__ bool cell_overfull(const CellHeader *h)
 }
 struct CellLists {
     CellHeader *hdr;
-    int *count, *start, *fill, *cellof, *idx;
-    float4 *posf;  // float32 copies (x, y, z, index bits) in bucket order
+    int *count, *start;  // G^2 and G^2 + 1 entries
+    float4 *posf;        // in bucket order: float32 copies (x, y, z, index bits)
+    double *posd;        // ... the positions (SoA)
+    int2 *cellof;
+    int *any;
 };
-// count, start and fill hold kCells + 1 entries each and are read and written as int4, so each array
-// starts on a 16-byte boundary: stride kCellStride (a multiple of 4 ints) after a 64-byte header, in
-// an allocation that cudaMalloc aligns to 256 bytes.
-constexpr int kCellStride = kCells + 4;
-static_assert(kCellStride % 4 == 0 && kCellStride >= kCells + 1, "bucket array stride");
+inline int cell_grid(int64_t N)
+{
+    int G = 64;
+    while (G < kCellGrid && (int64_t)G * G < N) G *= 2;
+    return G;
+}
 inline size_t cell_lists_bytes(int64_t max_N)
 {
-    return 64 + sizeof(int) * (size_t)3 * kCellStride + sizeof(float4) * (size_t)max_N +
-           sizeof(int) * (size_t)2 * max_N;
+    const size_t nb = (size_t)cell_grid(max_N) * cell_grid(max_N);
+    return sizeof(CellHeader) + sizeof(int) * (2 * nb + 4) +
+           (sizeof(float4) + 3 * sizeof(double) + sizeof(int2) + sizeof(int)) * (size_t)max_N;
 }
+// Lists for up to max_N spheres at base (256-byte aligned); count, start and posf begin on 16-byte boundaries.
 inline CellLists cell_lists(void *base, int64_t max_N)
 {
+    const size_t nb = (size_t)cell_grid(max_N) * cell_grid(max_N);
     CellLists L;
-    char *p = (char *)base;
-    L.hdr = (CellHeader *)p;
-    int *q = (int *)(p + 64);
-    L.count = q;
-    L.start = q + kCellStride;
-    L.fill = q + 2 * kCellStride;
-    L.posf = (float4 *)(q + 3 * kCellStride);  // 64 + 12 kCellStride bytes: 16-byte aligned
-    L.cellof = (int *)(L.posf + max_N);
-    L.idx = L.cellof + max_N;
+    L.hdr = (CellHeader *)base;
+    L.count = (int *)(L.hdr + 1);
+    L.start = L.count + nb;
+    L.posf = (float4 *)(L.start + nb + 4);
+    L.posd = (double *)(L.posf + max_N);
+    L.cellof = (int2 *)(L.posd + 3 * max_N);
+    L.any = (int *)(L.cellof + max_N);
     return L;
 }
 
