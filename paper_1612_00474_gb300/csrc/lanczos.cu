@@ -596,16 +596,17 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
             if (rc || (rc = erc)) return rc;
         }
     } else {
-        // Host-driven: the tridiagonal step leaves its status in pinned memory and an event tells when.  Where
-        // a product is short the next one is enqueued before the host knows whether this iteration
-        // stopped (then it is discarded): the stream would otherwise idle for the host's answer, about 15 us
-        // an iteration.  The estimate uses the measured per-pair times of the symmetric kernels.
+        // Host-driven: the tridiagonal step leaves its status in pinned memory and an event tells when.  The next
+        // product is enqueued before the host knows whether this iteration stopped: the stream would otherwise
+        // idle for the host's answer, about 15 us an iteration.  Its kernels read the status and leave if it did;
+        // those that do not ask (one-way passes) are enqueued where the product is short, from the measured
+        // per-pair times.
         if (!ctx->lz_ev &&
             (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->lz_ev, cudaEventDisableTiming), "lanczos event")))
             return rc;
         const double t_product = (ctx->Lx > 0.0 ? 9.0 : 1.0) * (double)N * (double)N *
                                  (ctx->p.precision == RPB_FP32 ? 1.3e-12 : (w.blocks64 ? 1.6e-11 : 8e-11));
-        const bool speculate = t_product < 1e-4;
+        const bool asks = pk && product_stops(ctx, N), speculate = asks || t_product < 1e-4;
         A.hs = w.host_status;
         bool have = first_done;
         for (int k = 0; k < max_iter && !stopped; ++k) {
@@ -614,7 +615,12 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
             if ((rc = gs_iteration(ctx, A)) || (rc = cuda_fail(cudaEventRecord(ctx->lz_ev, main_st), "event record")))
                 return rc;
             have = speculate && k + 1 < max_iter;
-            if (have && (rc = product(true))) return rc;
+            if (have) {
+                if (asks) ctx->stop = w.lz + A.L.status + ST_STOP;
+                rc = product(true);
+                ctx->stop = nullptr;
+                if (rc) return rc;
+            }
             if ((rc = cuda_fail(cudaEventSynchronize(ctx->lz_ev), "lanczos iteration"))) return rc;
             if (k == 0 && hs[ST_NW] == 0.0) {  // W = 0
                 if (iters_out) *iters_out = 0;

@@ -100,14 +100,25 @@ static SelfCoefs no_self_coefs()
     return SelfCoefs{nullptr, 0, 0.0, PairConsts<double>{}};
 }
 
+// A product enqueued before the host knows whether the Lanczos iteration before it stopped: stop is that
+// iteration's status word, and the pair kernels leave when it is set (null: none to ask).  They test it after their
+// first loads, beside which it arrives.  A step of 10000 spheres 2145 -> 2095 us, a float64 solve of 2000 1164 ->
+// 1122 (there the stream waited for the host); a short discarded product mostly ran while the host answered.
+__device__ __forceinline__ bool stopped(const double *stop)
+{
+    return stop && *stop != 0.0;
+}
+
 // ------------------------------------------------------------------ pair kernels
 // grid = (ceil(N/128), splits); block (bx, by) covers targets [128 bx, 128 bx + 128) and sources
 // [by chunk, (by + 1) chunk); chunk is a multiple of 128, so the tile holding the block's own
 // targets (where j == i can occur) is the one starting at 128 bx.
 template <bool TORQUE, bool WALL = true>
 __global__ void __launch_bounds__(kPairThreads) pair_f32_kernel(const SrcF32 *__restrict__ src, int N, int chunk,
-                                                                 PairConsts<float> c, double *__restrict__ part)
+                                                                 PairConsts<float> c, double *__restrict__ part,
+                                                                 const double *__restrict__ stop = nullptr)
 {
+    const bool quit = stopped(stop);
     __shared__ float4 sp[kTile];
     __shared__ float4 sf[kTile];
     __shared__ float4 st[TORQUE ? kTile : 1];
@@ -131,6 +142,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_f32_kernel(const SrcF32 *__
             if (TORQUE) st[tid] = src[j].t;
         }
         __syncthreads();
+        if (quit) return;
         const int cnt = min(kTile, j1 - base);
         float ux = 0.f, uy = 0.f, uz = 0.f;
         if (base != diag) {
@@ -196,8 +208,10 @@ __global__ void __launch_bounds__(kPairThreads) pair_f32_kernel(const SrcF32 *__
 // scalar kernel keeps those.
 template <bool TORQUE>
 __global__ void __launch_bounds__(64) pair_f32_free_kernel(const SrcF32 *__restrict__ src, int N, int chunk, X2Consts c,
-                                                           double *__restrict__ part, float *__restrict__ tile_sums)
+                                                           double *__restrict__ part, float *__restrict__ tile_sums,
+                                                           const double *__restrict__ stop)
 {
+    const bool quit = stopped(stop);
     __shared__ float4 sp[kTile], sf[kTile];
     __shared__ float4 st[TORQUE ? kTile : 1];
     const int tid = threadIdx.x;
@@ -257,6 +271,7 @@ __global__ void __launch_bounds__(64) pair_f32_free_kernel(const SrcF32 *__restr
             if (TORQUE) st[k] = src[base + k].t;
         }
         __syncthreads();
+        if (quit) return;
         float2 u[3] = {zero2, zero2, zero2};
         if (base != (int)blockIdx.x * kTile) {
 #pragma unroll 4
@@ -496,8 +511,10 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
                                                                              const float4 *__restrict__ src2 = nullptr,
                                                                              PerLen pl = PerLen{},
                                                                              const SymInst *__restrict__ sinst = nullptr,
-                                                                             const int *__restrict__ active = nullptr)
+                                                                             const int *__restrict__ active = nullptr,
+                                                                             const double *__restrict__ stop = nullptr)
 {
+    const bool quit = !BATCH && stopped(stop);
     constexpr int P = kTile / 2;
     constexpr int NC = RHS2 ? 6 : 3;
     static_assert(!(PER && RHS2), "the two-right-hand-side form has no pseudo-periodic variant");
@@ -580,6 +597,7 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
         nsp = src[j0].p;
         nsf = src[j0].f;
     }
+    if (quit) return;  // after the loads above, beside which the word arrives
     for (int t = seg.t0; t < seg.t1; ++t) {
         const int lj = (t - tb) * kTile + tid;
         const long long j = off + lj;
@@ -836,8 +854,10 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
 template <bool TORQUE>
 __global__ void __cluster_dims__(8) __launch_bounds__(256, TORQUE ? 1 : 2) pair_sym_lanes_kernel(
     const SrcF32 *__restrict__ src, int N, const SymCta *__restrict__ ctas, const SymSeg *__restrict__ segs, X2Consts c,
-    const int *__restrict__ col_start, double *__restrict__ tgt_part, float *__restrict__ src_part, PerLen pl)
+    const int *__restrict__ col_start, double *__restrict__ tgt_part, float *__restrict__ src_part, PerLen pl,
+    const double *__restrict__ stop)
 {
+    const bool quit = stopped(stop);  // the same for the whole cluster
     __shared__ SrcF32 ss[kTile], st[32];
     __shared__ float us[2][3][32], sv[2][3][kTile];
     cg::cluster_group cl = cg::this_cluster();
@@ -860,6 +880,7 @@ __global__ void __cluster_dims__(8) __launch_bounds__(256, TORQUE ? 1 : 2) pair_
         (s ? ss[tid] : st[tid - kTile]) = v;
     }
     __syncthreads();
+    if (quit) return;
     // the nine images of target T and source S under one vote, so that their blocks are straight-line code with
     // nine chains in flight (three to a vote 54 us a product, nine 46, before warps took turns);
     // eval(image, rx, ry, rz, rho2, r2, close), image 4 the unshifted one
@@ -1205,10 +1226,10 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
                                                                                             w.sym_tgt, w.sym_src);
         else if (sc->ncta <= kSmallMinBlocks * ctx->num_sms)
             pair_f32x2_sym_kernel<kSmallMinBlocks, false><<<sc->ncta, kPairThreads, 0, st>>>(
-                src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src);
+                src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, PerLen{}, nullptr, nullptr, ctx->stop);
         else
-            pair_f32x2_sym_kernel<kTtMinBlocks, false><<<sc->ncta, kPairThreads, 0, st>>>(src, N, ctas, segs, c, cs,
-                                                                                          w.sym_tgt, w.sym_src);
+            pair_f32x2_sym_kernel<kTtMinBlocks, false><<<sc->ncta, kPairThreads, 0, st>>>(
+                src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, PerLen{}, nullptr, nullptr, ctx->stop);
     }
     pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
         w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
@@ -1248,12 +1269,14 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
         const bool lanes = 8 * sc->ncta <= kLanesCtasPerSm * ctx->num_sms;  // then a run is one tile
         auto run = [&](auto kernel) {
             kernel<<<sc->ncta, kPairThreads, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, pl, nullptr,
-                                                      nullptr);
+                                                      nullptr, ctx->stop);
         };
         if (T && lanes)
-            pair_sym_lanes_kernel<true><<<8 * sc->ncta, 256, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, pl);
+            pair_sym_lanes_kernel<true><<<8 * sc->ncta, 256, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, pl,
+                                                                      ctx->stop);
         else if (lanes)
-            pair_sym_lanes_kernel<false><<<8 * sc->ncta, 256, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, pl);
+            pair_sym_lanes_kernel<false><<<8 * sc->ncta, 256, 0, st>>>(src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, pl,
+                                                                       ctx->stop);
         else if (T && small)
             run(pair_f32x2_sym_kernel<kSmallMinBlocks, true, false, true>);
         else if (T)
@@ -1856,6 +1879,13 @@ int mobility_apply_impl(rpb_ctx *ctx, int64_t N64, const double *pos, const doub
     return mobility_direct(ctx, N64, pos, F, T, U, mode);
 }
 
+// The product of a force on N spheres leaves early when ctx->stop tells it to.
+bool product_stops(const rpb_ctx *ctx, int64_t N)
+{
+    if (ctx->p.precision == RPB_FP64) return mobility_sym64_ok(ctx, ctx->ws.vf);
+    return ctx->p.wall ? ctx->sym_enabled && N >= 2 * kTile : !(ctx->Lx > 0.0);
+}
+
 // Rows [r0, r1) of share `part` of `nparts`: whole 128-row tiles, as equal as the tiles allow.
 static void part_rows(int64_t N, int part, int nparts, int64_t *r0, int64_t *r1)
 {
@@ -1964,16 +1994,16 @@ static int mobility_direct(rpb_ctx *ctx, int64_t N64, const double *pos, const d
             if (chunk == kTile) {
                 const PairConsts<float> c = make_consts<float>(a);
                 if (torque)
-                    pair_f32_kernel<true, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
+                    pair_f32_kernel<true, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part, ctx->stop);
                 else
-                    pair_f32_kernel<false, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part);
+                    pair_f32_kernel<false, false><<<grid, kPairThreads, 0, st>>>(src, N, (int)chunk, c, part, ctx->stop);
             } else {
                 const X2Consts c = make_x2_consts(a);
                 auto run = [&](const dim3 &g, int len, double *chunks, float *tile_sums) {
                     if (torque)
-                        pair_f32_free_kernel<true><<<g, 64, 0, st>>>(src, N, len, c, chunks, tile_sums);
+                        pair_f32_free_kernel<true><<<g, 64, 0, st>>>(src, N, len, c, chunks, tile_sums, ctx->stop);
                     else
-                        pair_f32_free_kernel<false><<<g, 64, 0, st>>>(src, N, len, c, chunks, tile_sums);
+                        pair_f32_free_kernel<false><<<g, 64, 0, st>>>(src, N, len, c, chunks, tile_sums, ctx->stop);
                 };
                 // chunks that leave fewer CTAs than four per SM: a CTA per tile (their float32 sums need half
                 // of the chunks' float64 ones per tile; one that finds no room takes the chunks)

@@ -238,8 +238,10 @@ template <bool TORQUE, bool WALL, PairSource PAIRS>
 __global__ void __launch_bounds__(32 * kSym64Warps) pair_sym64_kernel(const SrcF64 *__restrict__ src, int N, Sym64Plan pl,
                                                                        Sym64Consts c, double *__restrict__ tgt_part,
                                                                        double *__restrict__ src_part,
-                                                                       double *__restrict__ blocks)
+                                                                       double *__restrict__ blocks,
+                                                                       const double *__restrict__ stop)
 {
+    const bool quit = stop && *stop != 0.0;  // see stopped() in pair.cu
     static_assert(!(TORQUE && PAIRS == kRead), "the blocks are the translation part");
     constexpr int NS = TORQUE ? 11 : 8;
     // 2 z_j, -4 z_j^2, x, y, z~, F, T of the source tile
@@ -290,6 +292,7 @@ __global__ void __launch_bounds__(32 * kSym64Warps) pair_sym64_kernel(const SrcF
             S[1][lane] = -(z2 * z2);
         }
         __syncthreads();
+        if (quit) return;
         Vec3 v = zero;
 #pragma unroll 1
         for (int q = q0; q < q1; ++q) {
@@ -393,7 +396,7 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
     if (mode != kAgain)
         pack_f64_kernel<<<(N + pb - 1) / pb, pb, 0, st>>>(pos, F, T, N, a, ctx->p.wall, src, self);
     const dim3 grid((unsigned)pl.runs, (unsigned)pl.qs);
-    auto run = [&](auto kernel) { kernel<<<grid, 32 * kSym64Warps, 0, st>>>(src, N, pl, c64, tgt, col, blocks); };
+    auto run = [&](auto kernel) { kernel<<<grid, 32 * kSym64Warps, 0, st>>>(src, N, pl, c64, tgt, col, blocks, ctx->stop); };
     const PairSource pairs = !blocks || mode == kPlain ? kEvaluate : (mode == kKeep ? kStore : kRead);
     if (pairs == kRead)
         run(pair_sym64_kernel<false, true, kRead>);

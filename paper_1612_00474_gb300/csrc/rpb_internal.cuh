@@ -299,6 +299,7 @@ struct rpb_ctx {
     cudaStream_t side_stream = nullptr;
     cudaEvent_t side_fork = nullptr, side_join = nullptr;
     cudaEvent_t lz_ev = nullptr;      // host-driven Lanczos: an iteration's status has been written
+    const double *stop = nullptr;     // set while a Lanczos solve enqueues a product it may discard: the stop word
 };
 
 namespace rpb {
@@ -315,6 +316,7 @@ int cuda_fail(cudaError_t e, const char *what);
 // in float64 the pairs' blocks, pair64.cu); kAgain, another one at those positions, with no product of the
 // context in between: the packed sources hold s F already (F is still read for the self terms; T null).
 enum ProductMode { kPlain, kKeep, kAgain };
+bool product_stops(const rpb_ctx *ctx, int64_t N);
 int mobility_apply_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double *F, const double *T,
                         double *U, ProductMode mode = kPlain);
 // Rows t0 .. t1 - 1 of the product (component stride ldu, ldu < 0: t1 - t0), one-way kernels over a
