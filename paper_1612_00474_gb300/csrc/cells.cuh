@@ -129,8 +129,7 @@ __global__ void __launch_bounds__(256) cell_order_kernel(const double *__restric
     posd[k] = x;
     posd[N + k] = y;
     posd[2 * N + k] = z;
-    const double h = z - a, e = h * inv_b;
-    Fz[i] = (z < a ? f0 : f0 * exp_neg(-fma(fma(-e, b, h), inv_b, e))) - weight;  // e^{-(z - a) / b}
+    Fz[i] = wall_force(z, a, weight, f0, b, inv_b);
 }
 
 // Force pass over the buckets, kCellLanes threads per sphere in bucket order (neighbouring groups search the same

@@ -2169,7 +2169,7 @@ constexpr int64_t kGroupMaxN = 4096, kGroupMaxNPer = 8192;
 
 template <bool PER>
 __global__ void __launch_bounds__(kGroupTargets * kGroupThreads) forces_group_kernel(
-    const double *__restrict__ pos, int N, double a, double weight, double U0, double b, float cut2,
+    const double *__restrict__ pos, int N, double a, double weight, double f0, double b, double inv_b, float cut2,
     double *__restrict__ F, double Lx, double Ly)
 {
     constexpr int kMask = kGroupChunk / kGroupThreads / 32;
@@ -2179,9 +2179,9 @@ __global__ void __launch_bounds__(kGroupTargets * kGroupThreads) forces_group_ke
     const int i = blockIdx.x * kGroupTargets + g, ic = min(i, N - 1);
     const double xi = pos[ic], yi = pos[N + ic], zi = pos[2 * N + ic];
     const float xf = (float)xi, yf = (float)yi, zf = (float)zi;
-    const double f0 = U0 / b, inv_b = 1.0 / b;
     const float fLx = (float)Lx, fLy = (float)Ly;
     const float fiLx = PER ? 1.f / fLx : 0.f, fiLy = PER ? 1.f / fLy : 0.f;
+    const double two_a = a + a;
     double fx = 0.0, fy = 0.0, fz = 0.0;
     for (int base = 0; base < N; base += kGroupChunk) {
         const int n = min(kGroupChunk, N - base);
@@ -2234,7 +2234,7 @@ __global__ void __launch_bounds__(kGroupTargets * kGroupThreads) forces_group_ke
                 dx -= Lx * rint(dx / Lx);
                 dy -= Ly * rint(dy / Ly);
             }
-            const double m = steric_pair_factor(dx * dx + dy * dy + dz * dz, 2.0 * a, f0, inv_b);
+            const double m = steric_pair_factor(dx * dx + dy * dy + dz * dz, two_a, f0, inv_b);
             fx += m * dx;
             fy += m * dy;
             fz += m * dz;
@@ -2249,7 +2249,7 @@ __global__ void __launch_bounds__(kGroupTargets * kGroupThreads) forces_group_ke
     if (p == 0 && i < N) {
         F[i] = fx;
         F[N + i] = fy;
-        F[2 * N + i] = fz + ((zi < a ? f0 : f0 * exp(-(zi - a) / b)) - weight);
+        F[2 * N + i] = fz + wall_force(zi, a, weight, f0, b, inv_b);
     }
 }
 
@@ -2259,6 +2259,7 @@ int forces_impl(rpb_ctx *ctx, int64_t N, const double *pos, const rpb_force_para
     const double r_cut = 2.0 * a + kForceCutoffB * fp->b;
     const double rcm = r_cut * 1.01 + 0.01 * a;
     const float cut2 = (float)(rcm * rcm);
+    const double f0 = fp->U0 / fp->b, inv_b = 1.0 / fp->b;
     const int n = (int)N;
     const unsigned groups = (unsigned)((N + kGroupTargets - 1) / kGroupTargets);
     cudaStream_t st = ctx->stream;
@@ -2267,7 +2268,7 @@ int forces_impl(rpb_ctx *ctx, int64_t N, const double *pos, const rpb_force_para
         wrap_kernel<<<(unsigned)((N + pb - 1) / pb), pb, 0, st>>>(pos, n, ctx->Lx, ctx->Ly, ctx->ws.pos_w);
         if (N <= kGroupMaxNPer)
             forces_group_kernel<true><<<groups, kGroupTargets * kGroupThreads, 0, st>>>(
-                ctx->ws.pos_w, n, a, fp->weight, fp->U0, fp->b, cut2, F, ctx->Lx, ctx->Ly);
+                ctx->ws.pos_w, n, a, fp->weight, f0, fp->b, inv_b, cut2, F, ctx->Lx, ctx->Ly);
         else
             forces_kernel<true><<<(unsigned)((N + 127) / 128), 128, 0, st>>>(ctx->ws.pos_w, n, a, fp->weight, fp->U0,
                                                                              fp->b, cut2, F, ctx->Lx, ctx->Ly);
@@ -2275,8 +2276,8 @@ int forces_impl(rpb_ctx *ctx, int64_t N, const double *pos, const rpb_force_para
         return cuda_fail(cudaGetLastError(), "forces kernel");
     }
     if (N <= kGroupMaxN) {
-        forces_group_kernel<false><<<groups, kGroupTargets * kGroupThreads, 0, st>>>(pos, n, a, fp->weight, fp->U0,
-                                                                                     fp->b, cut2, F, 0.0, 0.0);
+        forces_group_kernel<false><<<groups, kGroupTargets * kGroupThreads, 0, st>>>(pos, n, a, fp->weight, f0, fp->b,
+                                                                                     inv_b, cut2, F, 0.0, 0.0);
         count_launches(1);
         return cuda_fail(cudaGetLastError(), "forces kernel");
     }

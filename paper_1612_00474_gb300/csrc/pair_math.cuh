@@ -813,6 +813,15 @@ __device__ __forceinline__ double steric_pair_factor(double r2, double two_a, do
     return f0 * exp_neg(x) * ir;
 }
 
+// Force of the wall, f0 below contact and f0 e^{-(z - a)/b} above (the quotient from inv_b and one correction), less
+// the weight.
+__device__ __forceinline__ double wall_force(double z, double a, double weight, double f0, double b, double inv_b)
+{
+    const double h = z - a, e = h * inv_b;
+    const bool plain = (__double2hiint(e) & 0x7fffffff) < 0x40900000;  // below 1024: no overflow, no infinity
+    return (z < a ? f0 : f0 * exp_neg(-(plain ? fma(fma(-e, b, h), inv_b, e) : e))) - weight;
+}
+
 __device__ __forceinline__ double H0(double x)
 {
     return x > 1.0 ? 1.0 : (x >= 0.0 ? x : 0.0);

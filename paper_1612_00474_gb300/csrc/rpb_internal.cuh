@@ -128,7 +128,7 @@ struct CellLists {
 inline int cell_grid(int64_t N)
 {
     int G = 64;
-    while (G < kCellGrid && (int64_t)G * G < N) G *= 2;
+    while (G < kCellGrid && (int64_t)2 * G * G < N) G *= 2;  // about 5 spheres a cell: at least one bucket for 2
     return G;
 }
 inline size_t cell_lists_bytes(int64_t max_N)

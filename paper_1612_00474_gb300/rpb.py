@@ -429,10 +429,13 @@ class BatchContext:
             if nullable:
                 return None
             raise ValueError(f"{name} is required")
-        arr = (ctypes.c_void_p * len(ts))()
-        for k, t in enumerate(ts):
-            arr[k] = _ptr(t, None, f"{name}[{k}]").value
-        return arr
+        import torch
+
+        # one pass over the attributes; _ptr names the tensor that is not as it must be
+        tensor, f64 = torch.Tensor, torch.float64
+        return (ctypes.c_void_p * len(ts))(*[
+            t.data_ptr() if isinstance(t, tensor) and t.is_cuda and t.dtype == f64 and t.is_contiguous() else
+            _ptr(t, None, f"{name}[{k}]").value for k, t in enumerate(ts)])
 
     def mobility_apply(self, pos, F=None, T=None, out=None):
         """U_b = M_tt F_b + M_tr T_b for each instance (rpb_batch_mobility_apply); lists of tensors."""
