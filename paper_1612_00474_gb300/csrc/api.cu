@@ -113,51 +113,18 @@ int check_step_args(rpb_ctx *ctx, int64_t N, const double *pos, const double *U_
 // GPU idle (up to a wave of CTAs), so that the drift's two products, their packing and their noise cost
 // little: 20 steps of 256 spheres 7.03 -> 6.21 ms in float64 and 17.5 -> 14.4 ms pseudo-periodic in float32, a
 // float32 step of 4096 spheres 807 -> 765 us.  Beyond, both are bound by the arithmetic (a float64 step of
-// 4096: 15.46 and 15.41 ms) and the side scratch would only take memory.
-constexpr int64_t kSideMaxF32 = 4096, kSideMaxF64 = 1024;
+// 4096: 15.46 and 15.41 ms).
+constexpr int64_t kBesideMaxF32 = 4096, kBesideMaxF64 = 1024;
+// The side scratch reaches further for float32: a drift's two products beside each other (rfd_impl) fill the last
+// waves of each other's CTAs.
+constexpr int64_t kSideMaxF32 = 32768;
 static int64_t side_max(const rpb_params &p, int64_t max_N)
 {
-    return std::min<int64_t>(max_N, p.precision == RPB_FP64 ? kSideMaxF64 : kSideMaxF32);
+    return std::min<int64_t>(max_N, p.precision == RPB_FP64 ? kBesideMaxF64 : kSideMaxF32);
 }
 
-// While it lives, the context's products use the side scratch and its stream (host state only: the kernels
-// enqueued meanwhile keep the pointers they were given).
-struct SideScope {
-    rpb_ctx *c;
-    cudaStream_t stream;
-    explicit SideScope(rpb_ctx *ctx) : c(ctx), stream(ctx->stream)
-    {
-        swap();
-        c->stream = c->side_stream;
-    }
-    ~SideScope()
-    {
-        swap();
-        c->stream = stream;
-    }
-    void swap()
-    {
-        Workspace &w = c->ws;
-        SideSpace &q = c->side;
-        std::swap(w.src, q.src);
-        std::swap(w.partial, q.partial);
-        std::swap(w.partial_bytes, q.partial_bytes);
-        std::swap(w.selfc, q.selfc);
-        std::swap(w.w, q.w);
-        std::swap(w.pos_w, q.pos_w);
-        std::swap(w.sym64, q.sym64);
-        std::swap(w.sym64_N, q.sym64_N);
-        std::swap(w.sym_tgt, q.sym_tgt);
-        std::swap(w.sym_tgt_bytes, q.sym_tgt_bytes);
-        std::swap(w.sym_src, q.sym_src);
-        std::swap(w.sym_src_bytes, q.sym_src_bytes);
-    }
-};
-
-// The drift of a step enqueued beside what follows on the context's stream (noise W~, the two displaced
-// products, their combination); side_join() orders the stream after it.
-static int side_drift(rpb_ctx *ctx, int64_t N, const double *pos, uint64_t seed, uint32_t step,
-                      const unsigned int *d_step, double delta, int one_sided)
+// The side stream, ordered after what is enqueued on the context's stream.
+int side_fork(rpb_ctx *ctx, int64_t N)
 {
     int rc;
     if (!ctx->side_stream &&
@@ -166,9 +133,25 @@ static int side_drift(rpb_ctx *ctx, int64_t N, const double *pos, uint64_t seed,
          (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->side_join, cudaEventDisableTiming), "side event"))))
         return rc;
     if ((rc = pair_prepare(ctx, N)) ||  // the symmetric schedule is shared by both streams
-        (rc = cuda_fail(cudaEventRecord(ctx->side_fork, ctx->stream), "event record")) ||
-        (rc = cuda_fail(cudaStreamWaitEvent(ctx->side_stream, ctx->side_fork, 0), "stream wait")))
+        (rc = cuda_fail(cudaEventRecord(ctx->side_fork, ctx->stream), "event record")))
         return rc;
+    return cuda_fail(cudaStreamWaitEvent(ctx->side_stream, ctx->side_fork, 0), "stream wait");
+}
+
+// The context's stream ordered after what is enqueued on the side stream.
+int side_join(rpb_ctx *ctx)
+{
+    const int rc = cuda_fail(cudaEventRecord(ctx->side_join, ctx->side_stream), "event record");
+    return rc ? rc : cuda_fail(cudaStreamWaitEvent(ctx->stream, ctx->side_join, 0), "stream wait");
+}
+
+// The drift of a step enqueued beside what follows on the context's stream (noise W~, the two displaced
+// products, their combination); the step waits for ctx->side_join before it reads the drift.
+static int side_drift(rpb_ctx *ctx, int64_t N, const double *pos, uint64_t seed, uint32_t step,
+                      const unsigned int *d_step, double delta, int one_sided)
+{
+    int rc;
+    if ((rc = side_fork(ctx, N))) return rc;
     {
         SideScope side(ctx);
         rc = philox_impl(ctx, N, seed, step, 1u, 0u, ctx->ws.vec_e, d_step);
@@ -247,7 +230,8 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
               double delta, double tol, int max_iter, const rpb_force_params *fp, int scheme, int rfd,
               rpb_step_stats *stats, LzGraph *gr)
 {
-    const bool beside = ctx->p.kT > 0.0 && !ctx->hook && N <= ctx->side.max_N;
+    const bool beside = ctx->p.kT > 0.0 && !ctx->hook &&
+                        N <= (ctx->p.precision == RPB_FP64 ? kBesideMaxF64 : kBesideMaxF32);
     const int rc = step_body(ctx, N, pos, U_prev, step, seed, dt, delta, tol, max_iter, fp, scheme, rfd, stats, gr, beside);
     // a step that failed half way: the stream is still ordered after the drift's reads of pos
     if (rc && rc != RPB_ENOCONV && beside && !gr && ctx->side_join)

@@ -1,6 +1,8 @@
 // rpb_internal.cuh -- shared declarations of the CUDA translation units (not part of the ABI).
 #pragma once
 
+#include <utility>
+
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -228,8 +230,9 @@ struct Workspace {
     SymSched sym_part;  // one share of it (rpb_mobility_apply_part)
 };
 
-// What one product writes besides its result, for the products of a step's drift when they run beside the
-// Lanczos iterations (step_impl): the fields of Workspace of the same names, for up to max_N spheres.
+// What one product writes besides its result, for products on the side stream (a step's drift beside its Lanczos
+// iterations, a drift's second product beside its first): the fields of Workspace of the same names, for up to
+// max_N spheres.
 struct SideSpace {
     int64_t max_N = 0, sym64_N = 0;
     void *src = nullptr, *partial = nullptr;
@@ -297,6 +300,7 @@ struct rpb_ctx {
     int gs_cluster = 8;               // blocks of the Lanczos cluster kernel at most (lanczos_setup)
     rpb::SideSpace side;              // scratch, stream and events of a step's drift beside its Lanczos solve
     cudaStream_t side_stream = nullptr;
+    bool in_side = false;             // a SideScope lives
     cudaEvent_t side_fork = nullptr, side_join = nullptr;
     cudaEvent_t lz_ev = nullptr;      // host-driven Lanczos: an iteration's status has been written
     const double *stop = nullptr;     // set while a Lanczos solve enqueues a product it may discard: the stop word
@@ -309,6 +313,45 @@ void set_error(const char *fmt, ...);
 // Count kernel launches enqueued by the library (reported by rpb_launch_count).
 void count_launches(int n);
 int cuda_fail(cudaError_t e, const char *what);
+
+// While it lives, the context's products use the side scratch and its stream (host state only: the kernels
+// enqueued meanwhile keep the pointers they were given).
+struct SideScope {
+    rpb_ctx *c;
+    cudaStream_t stream;
+    explicit SideScope(rpb_ctx *ctx) : c(ctx), stream(ctx->stream)
+    {
+        swap();
+        c->stream = c->side_stream;
+        c->in_side = true;
+    }
+    ~SideScope()
+    {
+        swap();
+        c->stream = stream;
+        c->in_side = false;
+    }
+    void swap()
+    {
+        Workspace &w = c->ws;
+        SideSpace &q = c->side;
+        std::swap(w.src, q.src);
+        std::swap(w.partial, q.partial);
+        std::swap(w.partial_bytes, q.partial_bytes);
+        std::swap(w.selfc, q.selfc);
+        std::swap(w.w, q.w);
+        std::swap(w.pos_w, q.pos_w);
+        std::swap(w.sym64, q.sym64);
+        std::swap(w.sym64_N, q.sym64_N);
+        std::swap(w.sym_tgt, q.sym_tgt);
+        std::swap(w.sym_tgt_bytes, q.sym_tgt_bytes);
+        std::swap(w.sym_src, q.sym_src);
+        std::swap(w.sym_src_bytes, q.sym_src_bytes);
+    }
+};
+
+int side_fork(rpb_ctx *ctx, int64_t N);
+int side_join(rpb_ctx *ctx);
 
 // Pair product: U = M_tt F + M_tr T with the context's precision.  F or T may be null.
 // All pointers device, SoA float64.  Enqueued on ctx->stream.  mode (a Lanczos solve makes many products at the
