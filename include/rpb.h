@@ -83,8 +83,9 @@ typedef struct {
 
 /* Create a context for up to max_N spheres and Lanczos runs of up to max_iter iterations.
  * stream: a cudaStream_t (NULL = legacy default stream).  The device is the current one.
- * Allocates all scratch now (about (max_iter + 12) * 24 * max_N bytes plus partial-sum
- * buffers); returns RPB_ENOMEM if that fails.  *ctx is NULL on failure. */
+ * Allocates all scratch now (about (max_iter + 14) * 24 * max_N bytes plus partial-sum
+ * buffers; float64 contexts also room for the pairs' translation blocks, 32 max_N^2 bytes, while
+ * that is below 8 GB and free); returns RPB_ENOMEM if that fails.  *ctx is NULL on failure. */
 int rpb_create(rpb_ctx **ctx, const rpb_params *p, int64_t max_N, int max_iter, void *stream);
 
 /* Free the context's scratch (after synchronising its stream).  NULL is accepted. */
@@ -278,7 +279,7 @@ uint64_t rpb_launch_count(void);
 typedef struct rpb_batch rpb_batch;
 
 /* Create a batch context for at most max_B instances totalling at most max_total_N spheres.
- * Allocates all scratch now (about (max_iter + 14) * 24 * max_total_N bytes). */
+ * Allocates all scratch now (about (max_iter + 22) * 24 * max_total_N bytes). */
 int rpb_batch_create(rpb_batch **bt, const rpb_params *p, int64_t max_total_N, int max_B, int max_iter,
                      void *stream);
 int rpb_batch_destroy(rpb_batch *bt);
@@ -300,8 +301,9 @@ int rpb_batch_ab_step(rpb_batch *bt, int B, const int64_t *N, double *const *pos
 
 /* nsteps AB steps of every instance (as repeated rpb_batch_ab_step) with one gather and one scatter
  * of the state, the step captured once as the body of a loop (WHILE) node of a CUDA graph that is
- * launched once, running nsteps steps with no host synchronisation in between.  Inside the graph each Lanczos iteration after the first is a
- * conditional node that runs while some instance is still active (decided on the device), up to
+ * launched once, running nsteps steps with no host synchronisation in between.  Inside the graph the
+ * Lanczos iterations after the first are the body of a second loop node, which runs while some
+ * instance is still active (decided on the device), up to
  * lanczos_iters iterations per step, with converged instances masked out (so lanczos_iters caps the
  * iteration count the tolerance needs; *unconverged, if not NULL, receives the number of
  * instance-steps that did not reach tol, and RPB_ENOCONV is returned if it is nonzero with tol > 0).  steps: each instance's

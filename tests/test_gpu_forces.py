@@ -1,5 +1,5 @@
 """Steric forces at the edges of the two kernels' ranges: all pairs by groups of sixteen spheres and chunks of 1024
-sources up to 8192 spheres, hashed cells beyond, and its all-pairs fallback."""
+sources up to 4096 spheres (8192 pseudo-periodic), hashed cells beyond, and its all-pairs fallback."""
 import math
 
 import numpy as np
@@ -58,7 +58,7 @@ def test_periodic(gpu_lib, N, many):
 
 
 def test_far_clusters_share_buckets(gpu_lib):
-    """Beyond 8192 spheres: clusters many grid periods apart fall into the same hashed buckets."""
+    """Clusters many grid periods apart fall into the same hashed buckets."""
     pos = inputs.monolayer(9000, seed=12)
     pos[3000:6000, 0] += 256 * 6.07 * 40
     pos[6000:, 1] -= 256 * 6.07 * 77
