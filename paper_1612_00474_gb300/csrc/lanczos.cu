@@ -188,8 +188,9 @@ __global__ void __launch_bounds__(kGsClusterThreads) gs_cluster_kernel(GsArgs A,
     __shared__ TailShared ts;
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), blocks = (int)cl.num_blocks(), tid = threadIdx.x;
-    const int k = init ? -1 : A.iter();
     cl.sync();  // every block of the cluster runs: its shared memory may be written
+    wait_for_before();
+    const int k = init ? -1 : A.iter();
     if (tid >= kGsThreads) {
         const int t = tid - kGsThreads;
         TailRegs reg = {};
@@ -496,18 +497,9 @@ static GsArgs gs_args(rpb_ctx *ctx, int64_t N, bool pack, LzGraph *gr)
 
 static int gs_cluster_launch(cudaStream_t st, const GsArgs &A, int blocks, int init)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(kGsClusterThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = blocks;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
     count_launches(1);
-    return cuda_fail(cudaLaunchKernelEx(&cfg, gs_cluster_kernel, A, (int)((A.N + blocks - 1) / blocks), init),
+    return cuda_fail(launch_after(!init, gs_cluster_kernel, dim3(blocks), kGsClusterThreads, blocks, st, A,
+                                  (int)((A.N + blocks - 1) / blocks), init),
                      "lanczos cluster kernel");
 }
 

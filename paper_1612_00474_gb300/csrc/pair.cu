@@ -514,6 +514,7 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
                                                                              const int *__restrict__ active = nullptr,
                                                                              const double *__restrict__ stop = nullptr)
 {
+    if (!BATCH) after_may_start();
     const bool quit = !BATCH && stopped(stop);
     constexpr int P = kTile / 2;
     constexpr int NC = RHS2 ? 6 : 3;
@@ -857,6 +858,7 @@ __global__ void __cluster_dims__(8) __launch_bounds__(256, TORQUE ? 1 : 2) pair_
     const int *__restrict__ col_start, double *__restrict__ tgt_part, float *__restrict__ src_part, PerLen pl,
     const double *__restrict__ stop)
 {
+    after_may_start();
     const bool quit = stopped(stop);  // the same for the whole cluster
     __shared__ SrcF32 ss[kTile], st[32];
     __shared__ float us[2][3][32], sv[2][3][kTile];
@@ -1043,6 +1045,10 @@ __global__ void __launch_bounds__(BATCH ? 384 : 768, BATCH ? 5 : 2) pair_sym_red
     __shared__ double s1[NC][kTile];
     const int nb = gridDim.x;
     const int b = BATCH ? (int)blockIdx.x : nb - 1 - (int)blockIdx.x;
+    if (!BATCH) {
+        after_may_start();
+        wait_for_before();
+    }
     long long off = 0;
     int Ni = N, tb = 0;
     if (BATCH) {
@@ -1231,11 +1237,12 @@ static int mobility_sym(rpb_ctx *ctx, int N, const double *pos, const double *F,
             pair_f32x2_sym_kernel<kTtMinBlocks, false><<<sc->ncta, kPairThreads, 0, st>>>(
                 src, N, ctas, segs, c, cs, w.sym_tgt, w.sym_src, nullptr, PerLen{}, nullptr, nullptr, ctx->stop);
     }
-    pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
-        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
-        sc->index + sc->rows_off, part == 0);
+    const cudaError_t e = launch_after(
+        packed && N <= kAfterMaxN, pair_sym_reduce_kernel<3>, dim3((N + kTile - 1) / kTile), 6 * kTile, 0, st, w.sym_tgt, w.sym_src,
+        sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr, sc->index + sc->rows_off,
+        part == 0);
     count_launches((sc->ncta > 0 ? 2 : 1) + !packed);
-    return cuda_fail(cudaGetLastError(), "symmetric pair kernels");
+    return cuda_fail(e == cudaSuccess ? cudaGetLastError() : e, "symmetric pair kernels");
 }
 
 // The symmetric product in pseudo-periodic mode: positions already folded into the unit cell
@@ -1286,11 +1293,12 @@ static int mobility_sym_periodic(rpb_ctx *ctx, int N, const double *pos_w, const
         else
             run(pair_f32x2_sym_kernel<kPerMinBlocks, false, false, true>);
     }
-    pair_sym_reduce_kernel<3><<<(N + kTile - 1) / kTile, 6 * kTile, 0, st>>>(
-        w.sym_tgt, w.sym_src, sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr,
-        sc->index + sc->rows_off, part == 0);
+    const cudaError_t e = launch_after(
+        packed && N <= kAfterMaxN, pair_sym_reduce_kernel<3>, dim3((N + kTile - 1) / kTile), 6 * kTile, 0, st, w.sym_tgt, w.sym_src,
+        sc->index + sc->row_off, cs, N, F, T, self, U, nullptr, nullptr, nullptr, nullptr, nullptr, sc->index + sc->rows_off,
+        part == 0);
     count_launches((sc->ncta > 0 ? 2 : 1) + !packed);
-    return cuda_fail(cudaGetLastError(), "periodic symmetric pair kernels");
+    return cuda_fail(e == cudaSuccess ? cudaGetLastError() : e, "periodic symmetric pair kernels");
 }
 
 // ------------------------------------------------------------------ batched symmetric pass

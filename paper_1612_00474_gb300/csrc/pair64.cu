@@ -241,6 +241,7 @@ __global__ void __launch_bounds__(32 * kSym64Warps) pair_sym64_kernel(const SrcF
                                                                        double *__restrict__ blocks,
                                                                        const double *__restrict__ stop)
 {
+    after_may_start();
     const bool quit = stop && *stop != 0.0;  // see stopped() in pair.cu
     static_assert(!(TORQUE && PAIRS == kRead), "the blocks are the translation part");
     constexpr int NS = TORQUE ? 11 : 8;
@@ -362,6 +363,8 @@ __global__ void __launch_bounds__(kRed64Threads) pair_sym64_reduce_kernel(
     const int64_t r0 = sym64_row_run(pl, b) * pl.qs;
     const int nr = (int)((pl.nb - b + pl.L - 1) / pl.L) * pl.qs, nc = b * pl.qs;
     const double *row = tgt_part + r0 * 96 + e, *col = src_part + sym64_col_slot(pl, 0, b, 0) * 96 + e;
+    after_may_start();
+    wait_for_before();
     double x[2] = {0.0, 0.0};
 #pragma unroll 4
     for (int k = g; k < nr; k += kRed64Groups) x[0] += row[(int64_t)k * 96];
@@ -408,9 +411,10 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
         pairs == kStore ? run(pair_sym64_kernel<true, false, kStore>) : run(pair_sym64_kernel<true, false, kEvaluate>);
     else
         pairs == kStore ? run(pair_sym64_kernel<false, false, kStore>) : run(pair_sym64_kernel<false, false, kEvaluate>);
-    pair_sym64_reduce_kernel<<<pl.nb, kRed64Threads, 0, st>>>(tgt, col, pl, N, F, T, self, U);
+    const cudaError_t e = launch_after(mode == kAgain && N <= kAfterMaxN, pair_sym64_reduce_kernel, dim3(pl.nb), kRed64Threads, 0, st, tgt, col, pl, N,
+                                       F, T, self, U);
     count_launches(mode == kAgain ? 2 : 3);
-    return cuda_fail(cudaGetLastError(), "float64 symmetric pair kernels");
+    return cuda_fail(e == cudaSuccess ? cudaGetLastError() : e, "float64 symmetric pair kernels");
 }
 
 }  // namespace rpb

@@ -241,6 +241,51 @@ struct SideSpace {
     float *sym_src = nullptr;
 };
 
+// Programmatic dependent launch along the chain of a Lanczos iteration, product -> reduce -> cluster kernel: a kernel
+// launched by launch_after() may start while the one before it runs, once every CTA of that one has passed
+// after_may_start(), and waits in wait_for_before() until it is complete and its writes are visible, before it
+// reads or writes any global memory.  Every kernel launched this way waits, so completion is transitive along the
+// chain; started otherwise, wait_for_before() returns at once.  Products of a solve after the first, of at most kAfterMaxN spheres: there a kernel's launch is a good
+// part of its time, and waiting CTAs take no room that running ones need.  A float32 step of 4096 spheres 747 -> 698 us, a
+// float64 one of 256 358 -> 316, twenty replayed ones 5.18 -> 4.85 ms, a solve of 3001 spheres 436 -> 403 us.
+constexpr int64_t kAfterMaxN = 4096;
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_may_start()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_before()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_after(bool early, void (*kernel)(P...), dim3 grid, unsigned threads, unsigned cluster, cudaStream_t st,
+                                A... args)
+{
+    if (!early && !cluster) {  // half the host time of the call below
+        kernel<<<grid, threads, 0, st>>>(static_cast<P>(args)...);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    if (early) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[cfg.numAttrs].val.clusterDim.x = cluster;
+        at[cfg.numAttrs].val.clusterDim.y = at[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    cfg.attrs = at;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 // Threads per block of an elementwise kernel over n items: single warps while they leave room on the SMs (a
 // float64 warp instruction takes 64 cycles of its scheduler, so a small vector is spread over all of
 // them), 256 beyond.
