@@ -184,8 +184,10 @@ int rpb_mobility_apply2(rpb_ctx *ctx, int64_t N, const double *pos, const double
  * tol <= 0, runs exactly max_iter iterations (for comparisons at equal m).  Stops early (exact
  * result) if the Krylov space becomes invariant.  max_iter must be in [1, context max_iter].
  * W = 0 gives g = 0, m = 0.  W, g: 3N; g must not alias W or pos.  iters_out, err_out: host
- * pointers (may be NULL).  Waits on the host once per iteration for the stopping test (short products of
- * the next iteration may already be enqueued then and are discarded at the stop).  Returns RPB_ENOCONV
+ * pointers (may be NULL).  Waits on the host once per iteration for the stopping test (the next
+ * iteration's product may already be enqueued then and is discarded at the stop: its kernels leave early
+ * where they can, else, and through a product hook, only short ones are enqueued, and an error of a
+ * discarded call of the hook is dropped).  Returns RPB_ENOCONV
  * if tol > 0 and max_iter was reached without convergence (g is still written). */
 int rpb_lanczos_sqrt_apply(rpb_ctx *ctx, int64_t N, const double *pos, const double *W, double *g,
                            double tol, int max_iter, int *iters_out, double *err_out);

@@ -590,14 +590,17 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
     } else {
         // Host-driven: the tridiagonal step leaves its status in pinned memory and an event tells when.  The next
         // product is enqueued before the host knows whether this iteration stopped: the stream would otherwise
-        // idle for the host's answer, about 15 us an iteration.  Its kernels read the status and leave if it did;
-        // those that do not ask (one-way passes) are enqueued where the product is short, from the measured
-        // per-pair times.
+        // idle for the host's answer, about 15 us an iteration.  Its kernels read the status and leave if it did.
+        // Products that do not ask (one-way kernels, a caller's) are enqueued where a discarded one costs less than the
+        // idling of a solve, from what the evaluated pairs take: float32 1.3 ps, float64 150 ps one-way, 200 ps an image
+        // of a pseudo-periodic pair (300, 500 and 800 such spheres discarding one 1.58, 2.89 and 6.81 ms, now 1.49, 2.64
+        // and 6.07).
         if (!ctx->lz_ev &&
             (rc = cuda_fail(cudaEventCreateWithFlags(&ctx->lz_ev, cudaEventDisableTiming), "lanczos event")))
             return rc;
-        const double t_product = (ctx->Lx > 0.0 ? 9.0 : 1.0) * (double)N * (double)N *
-                                 (ctx->p.precision == RPB_FP32 ? 1.3e-12 : (w.blocks64 ? 1.6e-11 : 8e-11));
+        const bool per = ctx->Lx > 0.0;
+        const double t_product = (per ? 9.0 : 1.0) * (double)N * (double)N *
+                                 (ctx->p.precision == RPB_FP32 ? 1.3e-12 : (per ? 2e-10 : 1.5e-10));
         const bool asks = pk && product_stops(ctx, N), speculate = asks || t_product < 1e-4;
         A.hs = w.host_status;
         bool have = first_done;
@@ -607,11 +610,12 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
             if ((rc = gs_iteration(ctx, A)) || (rc = cuda_fail(cudaEventRecord(ctx->lz_ev, main_st), "event record")))
                 return rc;
             have = speculate && k + 1 < max_iter;
+            int ahead = RPB_OK;
             if (have) {
                 if (asks) ctx->stop = w.lz + A.L.status + ST_STOP;
-                rc = product(true);
+                ahead = product(true);
                 ctx->stop = nullptr;
-                if (rc) return rc;
+                if (ahead && pk) return ahead;
             }
             if ((rc = cuda_fail(cudaEventSynchronize(ctx->lz_ev), "lanczos iteration"))) return rc;
             if (k == 0 && hs[ST_NW] == 0.0) {  // W = 0
@@ -623,6 +627,8 @@ int lanczos_run(rpb_ctx *ctx, int64_t N, const double *pos, double *g, double to
             m = k + 1;
             eps = hs[ST_EPS];
             stopped = hs[ST_STOP] != 0.0;
+            if (ahead && !stopped) return ahead;
+            if (ahead) set_error("%s", "");  // a caller's product failed that the solve does not need
         }
     }
     const int tb = elem_threads(n, ctx->num_sms);
