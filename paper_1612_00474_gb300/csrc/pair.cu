@@ -2087,8 +2087,10 @@ __global__ void __launch_bounds__(128) forces_kernel(const double *__restrict__ 
     const double f0 = U0 / b;
     double fx = 0.0, fy = 0.0, fz = 0.0;
     // Near pairs found by the float32 screen are queued per thread and evaluated in float64 together
-    // after the screen (or when the queue is full), so a warp pays for the slowest lane's list rather
-    // than for every lane's pairs one after another.
+    // after the screen (or when the queue cannot take two more), so a warp pays for the slowest lane's list
+    // rather than for every lane's pairs one after another.  One place evaluates a full queue: with one after
+    // each of the two sources the screen of a pseudo-periodic cell took twice as long (8193 spheres 823 -> 434 us,
+    // 65536 6848 -> 3587; open, a column of 5000 spheres 1544 -> 1205).
     constexpr int kQ = 32;
     int queue[kQ];
     int nq = 0;
@@ -2140,14 +2142,9 @@ __global__ void __launch_bounds__(128) forces_kernel(const double *__restrict__ 
             const float2 d2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
             if (d2.x < cut2 || d2.y < cut2) {  // rare: a near pair (or the sphere itself)
                 const int j0 = base + 2 * k;
-                if (d2.x < cut2 && j0 != i && j0 < N) {
-                    queue[nq++] = j0;
-                    if (nq == kQ) flush();
-                }
-                if (d2.y < cut2 && j0 + 1 != i && j0 + 1 < N) {
-                    queue[nq++] = j0 + 1;
-                    if (nq == kQ) flush();
-                }
+                if (d2.x < cut2 && j0 != i && j0 < N) queue[nq++] = j0;
+                if (d2.y < cut2 && j0 + 1 != i && j0 + 1 < N) queue[nq++] = j0 + 1;
+                if (nq >= kQ - 1) flush();
             }
         }
         __syncthreads();
@@ -2171,9 +2168,11 @@ __global__ void __launch_bounds__(128) forces_kernel(const double *__restrict__ 
 // the cells (62 us a call from 64 to 4096 spheres; the pseudo-periodic all-pairs kernel 52 us at 256).  Twenty
 // steps of 256 spheres: 7.75 -> 7.03 ms in float64, 23.1 -> 22.0 ms pseudo-periodic.
 constexpr int kGroupTargets = 16, kGroupThreads = 8, kGroupChunk = 1024;
-// Up to here; beyond, screening all pairs costs more than the cell lists (41 us a call at 4096, 100 at 8192, where
-// the cell lists take 49); in pseudo-periodic mode it takes over from the kernel of a thread per sphere.
-constexpr int64_t kGroupMaxN = 4096, kGroupMaxNPer = 8192;
+// Up to here; beyond, screening all pairs costs more than the cell lists (40 us a call at 4096, 100 at 8192, where
+// the cell lists take 46 from 4097 spheres on and 49 at 8192).  Pseudo-periodic cells have no cell lists, and up to
+// 40000 spheres the kernel of a thread per sphere is slower: 8193 434 us against 131, 16384 801 against 406, 32768
+// 1704 against 1333, 40000 2104 against 1924, 65536 3587 against 4573 (with many near pairs a sphere far slower).
+constexpr int64_t kGroupMaxN = 4096, kGroupMaxNPer = 40000;
 
 template <bool PER>
 __global__ void __launch_bounds__(kGroupTargets * kGroupThreads) forces_group_kernel(
