@@ -84,8 +84,12 @@ typedef struct {
 /* Create a context for up to max_N spheres and Lanczos runs of up to max_iter iterations.
  * stream: a cudaStream_t (NULL = legacy default stream).  The device is the current one.
  * Allocates all scratch now (about (max_iter + 14) * 24 * max_N bytes plus partial-sum
- * buffers; float64 contexts also room for the pairs' translation blocks, 32 max_N^2 bytes, while
- * that is below 8 GB and free); returns RPB_ENOMEM if that fails.  *ctx is NULL on failure. */
+ * buffers; float64 contexts up to 1400 spheres another 32 max_N^2 bytes for the pairs' translation
+ * blocks, float32 ones up to 100 MB for a drift beside other work); returns RPB_ENOMEM if that fails.
+ * *ctx is NULL on failure.  One exception: in a larger float64 context the first Lanczos solve, step or
+ * run (without periods and without a product hook) of N spheres asks for the room for its pairs' blocks,
+ * 32 N^2 bytes, kept for later ones; above 8 GB, or where less than an eighth of the device would stay
+ * free, its products evaluate their pairs instead. */
 int rpb_create(rpb_ctx **ctx, const rpb_params *p, int64_t max_N, int max_iter, void *stream);
 
 /* Free the context's scratch (after synchronising its stream).  NULL is accepted. */

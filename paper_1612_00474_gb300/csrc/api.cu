@@ -75,6 +75,7 @@ static int check_vec(const void *p, const char *name, bool nullable)
 
 static void free_ws(Workspace &w)
 {
+    if (w.blocks64_small) w.blocks64 = nullptr;  // part of the slab
     void *dev[] = {w.slab, w.blocks64, w.sym_index, w.sym_tgt, w.sym_src, w.src2, w.pc};
     for (void *p : dev)
         if (p) cudaFree(p);
@@ -232,6 +233,7 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
 {
     const bool beside = ctx->p.kT > 0.0 && !ctx->hook &&
                         N <= (ctx->p.precision == RPB_FP64 ? kBesideMaxF64 : kBesideMaxF32);
+    if (ctx->p.kT > 0.0 && max_iter > 1 && !gr) blocks64_prepare(ctx, N);
     const int rc = step_body(ctx, N, pos, U_prev, step, seed, dt, delta, tol, max_iter, fp, scheme, rfd, stats, gr, beside);
     // a step that failed half way: the stream is still ordered after the drift's reads of pos
     if (rc && rc != RPB_ENOCONV && beside && !gr && ctx->side_join)
@@ -313,6 +315,8 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
         if (sym64_bytes > ((size_t)8 << 30)) sym64_bytes = 0;
     }
     w.sym64_N = max_N;
+    w.blocks64_small = sym64_bytes && blocks64_bytes(max_N) <= kBlocks64SmallBytes;
+    if (w.blocks64_small) w.blocks64_N = max_N;
     SideSpace &side = c->side;
     const int64_t ns = side_max(*p, max_N);
     const size_t svb = (size_t)3 * ns * sizeof(double);
@@ -348,6 +352,7 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
         {(void **)&w.vec_f, vb},
         {(void **)&w.vec_g, vb},
         {(void **)&w.sym64, sym64_bytes},
+        {(void **)&w.blocks64, w.blocks64_small ? (size_t)blocks64_bytes(max_N) : 0},
         {&side.src, (size_t)ns * sizeof(SrcF64)},
         {&side.partial, side.partial_bytes},
         {(void **)&side.selfc, (size_t)4 * ns * sizeof(double)},
@@ -401,14 +406,6 @@ int rpb_create(rpb_ctx **out, const rpb_params *p, int64_t max_N, int max_iter, 
                 return RPB_ENOMEM;
             }
         }
-    }
-    // the blocks of the float64 pairs (32 N^2 bytes) make the later products of a Lanczos solve about five
-    // times cheaper; kept while they stay below 8 GB and the device has the room, else every product
-    // evaluates its pairs
-    if (w.sym64 && blocks64_bytes(max_N) <= ((size_t)8 << 30) &&
-        cudaMalloc(&w.blocks64, blocks64_bytes(max_N)) != cudaSuccess) {
-        cudaGetLastError();
-        w.blocks64 = nullptr;
     }
     if (cudaMallocHost((void **)&w.host_status, 8 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
@@ -609,6 +606,7 @@ int rpb_lanczos_sqrt_apply(rpb_ctx *ctx, int64_t N, const double *pos, const dou
         set_error("g aliases an input");
         return RPB_EINVAL;
     }
+    if (max_iter > 1) blocks64_prepare(ctx, N);
     return lanczos_impl(ctx, N, pos, W, g, tol, max_iter, false, iters_out, err_out, nullptr);
 }
 

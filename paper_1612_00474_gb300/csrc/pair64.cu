@@ -219,12 +219,6 @@ __device__ __forceinline__ double *block_rows(double *blocks, int b, int t, int 
     return blocks + (((int64_t)t * (t + 1) / 2 + b) * 32 + q) * (8 * 32);
 }
 
-size_t blocks64_bytes(int64_t max_N)
-{
-    const int64_t nb = (max_N + kTile64 - 1) / kTile64;
-    return (size_t)(nb * (nb + 1) / 2) * 32 * 8 * 32 * sizeof(double);
-}
-
 constexpr int kSym64Warps = 4;
 
 // How a product gets its pairs: evaluated, evaluated and their blocks stored, or read from those blocks.
@@ -385,6 +379,42 @@ bool mobility_sym64_ok(const rpb_ctx *ctx, const double *F)
     return ctx->ws.sym64 != nullptr && F != nullptr && !(ctx->Lx > 0.0);
 }
 
+// Room for the blocks of a solve of N spheres where the context's scratch has none: asked for by the first solve that
+// can read them (a context that makes products only, or pseudo-periodic or hooked ones, takes none), kept, and
+// enlarged for a larger one.  What is not granted is not asked for again: those solves evaluate their pairs.
+void blocks64_prepare(rpb_ctx *ctx, int64_t N)
+{
+    Workspace &w = ctx->ws;
+    if (ctx->hook || !mobility_sym64_ok(ctx, w.vf) || N <= w.blocks64_N || N >= w.blocks64_refused) return;
+    // another thread may be capturing; this one does so only where the solve is refused
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    size_t avail = 0, total = 0;
+    int64_t room = 0;
+    if (cudaMemGetInfo(&avail, &total) == cudaSuccess)
+        room = blocks64_room(N, w.blocks64_N, ctx->max_N, (int64_t)avail, (int64_t)total);
+    if (room > 0) {
+        if (w.blocks64) {  // kernels that read the old ones have ended
+            cudaStreamSynchronize(ctx->stream);
+            cudaFree(w.blocks64);
+        }
+        w.blocks64 = nullptr;
+        w.blocks64_N = 0;
+        if (cudaMalloc(&w.blocks64, (size_t)blocks64_bytes(room)) == cudaSuccess)
+            w.blocks64_N = room;
+        else
+            w.blocks64 = nullptr;
+    }
+    if (N > w.blocks64_N) w.blocks64_refused = N;
+    cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
 int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U, ProductMode mode)
 {
     cudaStream_t st = ctx->stream;
@@ -393,7 +423,7 @@ int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, cons
     const Sym64Consts c64 = make_sym64_consts(a);
     const Sym64Plan pl = sym64_plan(N, ctx->num_sms);
     double *tgt = ctx->ws.sym64, *col = tgt + sym64_tgt_elems(ctx->ws.sym64_N, ctx->num_sms);
-    double *blocks = ctx->ws.blocks64;
+    double *blocks = N <= ctx->ws.blocks64_N ? ctx->ws.blocks64 : nullptr;
     SrcF64 *src = (SrcF64 *)ctx->ws.src;
     const int pb = elem_threads(N, ctx->num_sms);
     if (mode != kAgain)

@@ -191,7 +191,8 @@ struct SymSched {
 
 // Scratch owned by a context.
 struct Workspace {
-    void *slab = nullptr;         // the allocation of the arrays down to vec_g, of sym64 and of the SideSpace
+    void *slab = nullptr;         // the allocation of the arrays down to vec_g, of sym64, of small blocks64 and of the
+                                  // SideSpace
     void *src = nullptr;          // packed sources, max_N records (SrcF64 size)
     void *partial = nullptr;      // pair-kernel partial sums
     size_t partial_bytes = 0;
@@ -225,7 +226,10 @@ struct Workspace {
     void *src2 = nullptr;          // second right-hand side of the two-RHS symmetric pass (float4 per sphere)
     double *sym64 = nullptr;       // float64 contexts: row and column partials of the symmetric pass (pair64.cu)
     int64_t sym64_N = 0;           // ... sized for this many spheres
-    double *blocks64 = nullptr;    // the pairs' translation blocks at a Lanczos solve's positions (blocks64_bytes)
+    double *blocks64 = nullptr;    // the pairs' translation blocks at a Lanczos solve's positions (blocks64_prepare)
+    int64_t blocks64_N = 0;                // ... sized for this many spheres
+    int64_t blocks64_refused = INT64_MAX;  // ... no room for this many or more
+    bool blocks64_small = false;           // ... part of the slab
     SymSched sym;       // the whole triangle
     SymSched sym_part;  // one share of it (rpb_mobility_apply_part)
 };
@@ -418,7 +422,7 @@ int mobility_part_impl(rpb_ctx *ctx, int64_t N, const double *pos, const double 
 // float64 context with its scratch, forces given, no periodic images), and the product.
 bool mobility_sym64_ok(const rpb_ctx *ctx, const double *F);
 int mobility_sym64(rpb_ctx *ctx, int N, const double *pos, const double *F, const double *T, double *U, ProductMode mode);
-size_t blocks64_bytes(int64_t max_N);
+void blocks64_prepare(rpb_ctx *ctx, int64_t N);
 // Whether mobility_apply2_impl can take this product (float32 symmetric pass with two right-hand sides).
 bool mobility_apply2_ok(const rpb_ctx *ctx, int64_t N);
 // U = M_tt F + M_tr T and U2 = M_tt P in one symmetric pass (F, T, P non-null).

@@ -175,6 +175,7 @@ extern "C" int rpb_run(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, int
     RunCtx *r = ctx->run;
     const cudaStream_t user = ctx->stream;
     // host-side preparation before the capture, then the run ordered after the caller's stream
+    if (ctx->p.kT > 0.0 && max_iter > 1) blocks64_prepare(ctx, N);
     if ((rc = pair_prepare(ctx, N)) || (rc = cuda_fail(cudaEventRecord(r->ev, user), "event record")) ||
         (rc = cuda_fail(cudaStreamWaitEvent(r->st, r->ev, 0), "stream wait")))
         return rc;

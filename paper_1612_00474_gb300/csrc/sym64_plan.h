@@ -100,4 +100,27 @@ inline int64_t sym64_src_elems(int64_t max_N, int num_sms)
     return 96 * (units > small ? units : small);
 }
 
+// A Lanczos solve in float64 keeps the blocks of its pairs (pair64.cu): 64 bytes for each pair of lanes of each unit.
+inline int64_t blocks64_bytes(int64_t N)
+{
+    const int64_t nb = (N + kTile64 - 1) / kTile64;
+    return nb * (nb + 1) / 2 * 32 * 8 * 32 * (int64_t)sizeof(double);
+}
+
+// Contexts whose blocks take no more than this (1,400 spheres) hold them from the start, as part of their scratch: a
+// first solve of 300 spheres takes 345 us, and the allocation would be 100 of its own.
+constexpr int64_t kBlocks64SmallBytes = (int64_t)64 << 20;
+// Spheres that a solve of N makes room for when there is room for `held` of at most max_N: N at first, then with some
+// to spare, so that a slowly growing suspension does not ask each time; 0: none, evaluate the pairs.  Up to 8 GB
+// (16,000 spheres), and an eighth of the device stays free for others.
+constexpr int64_t kBlocks64MaxBytes = (int64_t)8 << 30;
+inline int64_t blocks64_room(int64_t N, int64_t held, int64_t max_N, int64_t free_bytes, int64_t total_bytes)
+{
+    const int64_t more = held + held / 4 < max_N ? held + held / 4 : max_N;
+    const int64_t left = free_bytes + (held > 0 ? blocks64_bytes(held) : 0) - total_bytes / 8;
+    const int64_t most = left < kBlocks64MaxBytes ? left : kBlocks64MaxBytes;
+    if (more > N && blocks64_bytes(more) <= most) return more;
+    return blocks64_bytes(N) <= most ? N : 0;
+}
+
 }  // namespace rpb
