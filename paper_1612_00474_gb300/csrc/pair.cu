@@ -1031,7 +1031,7 @@ __global__ void __cluster_dims__(8) __launch_bounds__(256, TORQUE ? 1 : 2) pair_
 // of loads and additions for a single small suspension.
 template <int NC, bool BATCH = false>
 __global__ void __launch_bounds__(BATCH ? 384 : 768, BATCH ? 5 : 2) pair_sym_reduce_kernel(
-    const double *__restrict__ tgt_part, const float *__restrict__ src_part, const int *__restrict__ row_seg,
+    const double *tgt_part, const float *src_part, const int *__restrict__ row_seg,
     const int *__restrict__ col_start, int N, const double *__restrict__ F, const double *__restrict__ T, SelfCoefs sc,
     double *__restrict__ U, const double *__restrict__ P = nullptr, double *__restrict__ U2 = nullptr,
     const SymInst *__restrict__ sinst = nullptr, const int *__restrict__ tile_inst = nullptr,

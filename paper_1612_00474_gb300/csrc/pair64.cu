@@ -347,7 +347,7 @@ constexpr int kRed64Groups = 8;
 constexpr int kRed64Threads = 96 * kRed64Groups;
 
 __global__ void __launch_bounds__(kRed64Threads) pair_sym64_reduce_kernel(
-    const double *__restrict__ tgt_part, const double *__restrict__ src_part, Sym64Plan pl, int N,
+    const double *tgt_part, const double *src_part, Sym64Plan pl, int N,
     const double *__restrict__ F, const double *__restrict__ T, SelfCoefs sc, double *__restrict__ U)
 {
     __shared__ double sum[kRed64Groups][96];

@@ -248,8 +248,10 @@ struct SideSpace {
 // Programmatic dependent launch along the chain of a Lanczos iteration, product -> reduce -> cluster kernel: a kernel
 // launched by launch_after() may start while the one before it runs, once every CTA of that one has passed
 // after_may_start(), and waits in wait_for_before() until it is complete and its writes are visible, before it
-// reads or writes any global memory.  Every kernel launched this way waits, so completion is transitive along the
-// chain; started otherwise, wait_for_before() returns at once.  Products of a solve after the first, of at most kAfterMaxN spheres: there a kernel's launch is a good
+// reads or writes any global memory.  What the one before writes is no `const __restrict__` parameter of such a
+// kernel: that would promise that nothing changes it while the kernel runs, and allow its loads ahead of the wait.
+// Every kernel launched this way waits, so completion is transitive along the chain; started otherwise,
+// wait_for_before() returns at once.  Products of a solve after the first, of at most kAfterMaxN spheres: there a kernel's launch is a good
 // part of its time, and waiting CTAs take no room that running ones need.  A float32 step of 4096 spheres 747 -> 698 us, a
 // float64 one of 256 358 -> 316, twenty replayed ones 5.18 -> 4.85 ms, a solve of 3001 spheres 436 -> 403 us.
 constexpr int64_t kAfterMaxN = 4096;
