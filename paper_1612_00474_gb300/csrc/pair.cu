@@ -33,6 +33,7 @@
 #include <cooperative_groups.h>
 
 #include "cells.cuh"
+#include "float_sums.h"
 #include "grid_plan.h"
 #include "pair_math.cuh"
 #include "sym_schedule.h"
@@ -1043,6 +1044,7 @@ __global__ void __launch_bounds__(BATCH ? 384 : 768, BATCH ? 5 : 2) pair_sym_red
     // that twice as many tiles are resident at once)
     constexpr int HALVES = BATCH ? 1 : 6 / NC;
     __shared__ double s1[NC][kTile];
+    __shared__ FloatSum f1[NC][kTile];
     const int nb = gridDim.x;
     const int b = BATCH ? (int)blockIdx.x : nb - 1 - (int)blockIdx.x;
     if (!BATCH) {
@@ -1082,25 +1084,25 @@ __global__ void __launch_bounds__(BATCH ? 384 : 768, BATCH ? 5 : 2) pair_sym_red
             }
         }
     }
-    // the four sums as one float32 pair (Knuth's exact two-sum, the errors gathered in the low part:
-    // 2^-48 of the largest), so that one sum, not eight numbers, is converted
-    float hi = cs[0], lo = -cc[0];
-#pragma unroll
-    for (int u = 1; u < 4; ++u) {
-        const float t = hi + cs[u], z = t - hi;
-        lo += (hi - (t - z)) + (cs[u] - z) - cc[u];
-        hi = t;
-    }
-    double v = (double)hi + (double)lo;
+    FloatSum f = join_sums(cs, cc);
+    int k = row_seg[b] + half;
+    const int k1 = row_seg[b + 1];
+    double v = k < k1 ? tgt_part[((size_t)k * NC + q) * kTile + l] : 0.0;
 #pragma unroll 4
-    for (int k = row_seg[b] + half; k < row_seg[b + 1]; k += HALVES) v += tgt_part[((size_t)k * NC + q) * kTile + l];
+    for (k += HALVES; k < k1; k += HALVES) v += tgt_part[((size_t)k * NC + q) * kTile + l];
     if (HALVES == 2) {
-        if (half == 1) s1[q][l] = v;
+        if (half == 1) {
+            s1[q][l] = v;
+            f1[q][l] = f;
+        }
         __syncthreads();
-        if (half == 0) v += s1[q][l];
+        if (half != 0) return;
+        v += s1[q][l];
+        f.add(f1[q][l]);
     }
     const int lb = (b - tb) * kTile + l;
-    if (half != 0 || lb >= Ni) return;
+    if (lb >= Ni) return;
+    v += f.value();
     const long long i = off + lb;
     if (NC == 6 && q >= 3)
         U2[(q - 3) * (int64_t)N + i] = sc.velocity(i, q - 3, v, P, nullptr, N);
