@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kGsClusterThreads) gs_cluster_kernel(GsArgs A,
     double bn = 0.0, nb, inv;
     for (int q = 0; q < blocks; ++q) bn += cs.norm[q];
     root_and_inverse(bn, &nb, &inv);
-    if (init && !(nb > 0.0)) inv = 0.0;
+    if (init && !(bn > 0.0)) inv = 0.0;
     double *v = A.V + (size_t)(k + 1) * A.ld;
 #pragma unroll
     for (int u = 0; u < kGsRows; ++u)
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kGsThreads) gs_scale_kernel(GsArgs A, int chun
     gs_coefs(A.norm2, 0, gridDim.x, 1, &bn);
     double nb, inv;
     root_and_inverse(bn, &nb, &inv);
-    if (init && !(nb > 0.0)) inv = 0.0;
+    if (init && !(bn > 0.0)) inv = 0.0;
     const int k = init ? -1 : A.iter();
     int64_t row[kGsRows];
     gs_rows(gs_chunk_span(A, chunk), row);

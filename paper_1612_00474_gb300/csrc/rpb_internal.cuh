@@ -34,17 +34,19 @@ struct alignas(16) SrcF64 {
 #ifdef __CUDACC__
 // 1/sqrt(x) for a positive normal x: the hardware's approximation (relative error measured at 2^-20.0), then one
 // third-order step of the binomial series, y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (Householder's
-// iteration): it leaves 5 e^3/16 = 2^-58.7, below rounding.
+// iteration): it leaves 5 e^3/16 = 2^-58.7, below rounding.  The approximation has zeros in its lower 32 bits, so its
+// square is exact and e is rounded once: within 0.53 ulp.  (With e from x y, rounded, it was 0.95 ulp, and the
+// float64 products of 500 spheres had 3.7e-16 of error where the library's root had given 3.4e-16.)
 __device__ __forceinline__ double rsqrt_pos(double x)
 {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
+    const double e = fma(-x, y * y, 1.0);
     return fma(e * y, fma(e, 0.375, 0.5), y);
 }
 
 // 1/d for a positive normal d: the hardware's approximation (relative error measured at 2^-19.9) and one
-// third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - d y.
+// third-order step of Householder's iteration, y (1 + e + e^2) with e = 1 - d y: within 0.52 ulp.
 __device__ __forceinline__ double rcp_pos(double d)
 {
     double y;
@@ -60,12 +62,13 @@ __device__ __forceinline__ bool plain_pos(double v)
 }
 
 // sqrt(x) and 1/sqrt(x) of a sum of squares: a square root and a division are about 25 float64 instructions,
-// the reciprocal root 6.
+// the reciprocal root 5 and the root 4 more (one Newton step: within 0.51 ulp while its residual is a normal number).
 __device__ __forceinline__ void root_and_inverse(double x, double *root, double *inverse)
 {
     if (plain_pos(x)) {
-        *inverse = rsqrt_pos(x);
-        *root = x * *inverse;
+        const double y = rsqrt_pos(x), r = x * y;
+        *inverse = y;
+        *root = __double2hiint(x) >= 0x04000000 ? fma(fma(-r, r, x), 0.5 * y, r) : sqrt(x);  // from 2^-959 on
     } else {
         *root = sqrt(x);
         *inverse = 1.0 / *root;
