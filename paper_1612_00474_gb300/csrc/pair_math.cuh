@@ -765,8 +765,8 @@ static __device__ const double2 kExp2Table[64] = {
     {0x1.f50765b6e4540p+0, 0x1.9d3e12dd8a18bp-54}, {0x1.fa7c1819e90d8p+0, 0x1.74853f3a5931ep-55}};
 
 // e^x for -700 <= x <= 0: x = (64 k + i) ln 2 / 64 + r with |r| <= ln 2 / 128, e^x = 2^k 2^(i/64) e^r (Tang's
-// table-driven method), e^r - 1 by its series to r^5 (the next term is below 2^-54).  Eleven float64
-// instructions; the table's low parts keep the result within 0.52 ulp.
+// table-driven method), e^r - 1 by its series to r^5 (the next term is below 2^-54, up to 0.32 ulp of the result).
+// Eleven float64 instructions; with the table's low parts the result is within 0.83 ulp.
 __device__ __forceinline__ double exp_table(double x)
 {
     const double shift = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the nearest integer

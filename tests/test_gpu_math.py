@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1612_00474_gb300", "csrc")
-FUNCTIONS = ("rsqrt_pos", "rcp_pos", "root", "inverse")
+FUNCTIONS = ("rsqrt_pos", "rcp_pos", "root", "inverse", "exp_table", "exp_neg")
 SRC = r"""
 #include "pair_math.cuh"
 using namespace rpb;
@@ -23,7 +23,10 @@ __global__ void evaluate(int which, const double *x, double *y, int n)
     if (i >= n) return;
     double root, inverse;
     root_and_inverse(x[i], &root, &inverse);
-    y[i] = which == 0 ? rsqrt_pos(x[i]) : which == 1 ? rcp_pos(x[i]) : which == 2 ? root : inverse;
+    if (which >= 4)
+        y[i] = which == 4 ? exp_table(x[i]) : exp_neg(x[i]);
+    else
+        y[i] = which == 0 ? rsqrt_pos(x[i]) : which == 1 ? rcp_pos(x[i]) : which == 2 ? root : inverse;
 }
 extern "C" int run(int which, const void *x, void *y, int n)
 {
@@ -74,3 +77,23 @@ def test_roots_and_reciprocals(evaluate, name, of, bound):
     x = _positive(-1021, 998)  # plain_pos: 2^-1022 .. 2^1000 (a reciprocal's result is normal up to 2^1021)
     y = evaluate(name, x)
     assert float(_ulps(y, of(x.astype(np.longdouble))).max()) <= bound
+
+
+# one rounding, 0.5; the series' next term, (ln 2 / 128)^6 / 720, 0.32 where the result's last place counts least; 0.01 for
+# the roundings before the last
+def test_exponential(evaluate):
+    rng = np.random.default_rng(8)
+    n = np.arange(0, 64639)  # every table entry and exponent: in the middle, and where the nearest entry changes
+    x = -np.concatenate([n * np.log(2.0) / 64, (n + 0.5) * np.log(2.0) / 64 - 1e-9, (n + 0.5) * np.log(2.0) / 64 + 1e-9,
+                         rng.random(200000) * 40, rng.random(200000) * 700, rng.random(20000) * 1e-3,
+                         2.0 ** -rng.integers(1, 1000, 2000), [0.0, 700.0]])
+    x = x[x >= -700.0]
+    exact = np.exp(x.astype(np.longdouble))
+    y = evaluate("exp_table", x)
+    assert float(_ulps(y, exact).max()) <= 0.83
+    inside = (x > -700.0) & (x < 0.0)
+    assert np.array_equal(evaluate("exp_neg", x)[inside], y[inside])
+    far = np.array([0.0, 1.0, -700.0, -720.0, -745.0, -1e4, -np.inf, np.inf, np.nan])  # the library's
+    z = evaluate("exp_neg", far)
+    assert np.array_equal(z[[0, 5, 6, 7]], [1.0, 0.0, 0.0, np.inf]) and np.isnan(z[8])
+    assert np.allclose(z[1:5], np.exp(far[1:5]), rtol=1e-15, atol=5e-324)
