@@ -522,12 +522,12 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
     static_assert(!(PER && RHS2), "the two-right-hand-side form has no pseudo-periodic variant");
     static_assert(!(BATCH && (PER || RHS2)), "the batched form is the plain or the torque form");
     // G source pairs (2G sources) are evaluated per step and then reduce-scattered over the warp
-    // (G = 2 is kept as an option: every form measured faster with four).  Each source array holds
-    // the tile's pairs (2p, 2p+1) at [p] and the same pairs swapped at [SW + p]; lanes with bit 3
-    // (G = 2) or bit 2 (G = 4) set read the swapped copy, so that the element each lane keeps in the
-    // reduce-scatter is always .x (SW puts the two copies in different banks for the 2G lane groups)
+    // (two pairs measured slower in every form).  Each source array holds the tile's pairs (2p, 2p+1) at [p]
+    // and the same pairs swapped at [SW + p]; lanes with bit 2 set read the swapped copy, so that the element
+    // each lane keeps in the reduce-scatter is always .x (SW puts the two copies in different banks for the 2G
+    // lane groups)
     constexpr int G = 4;
-    constexpr int SW = G == 4 ? P + 4 : P + 2;
+    constexpr int SW = P + 4;
     __shared__ float4 sA[SW + P], sB[SW + P], sC[SW + P], sD[SW + P];
     __shared__ float4 sE[TORQUE ? SW + P : 1];
     __shared__ float4 sG[TORQUE ? SW + P : 1];  // (T_z, T_z', 6 z_j, 6 z_j')
@@ -543,11 +543,9 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
     // pk: the pair of a step this lane keeps in the reduce-scatter (it evaluates pairs in the order
     // h ^ pk, so v[0] is that pair and the pairs it sends come in the order its partners keep them);
     // swz: its copy of the source arrays
-    const int pk = G == 4 ? ((2 * (int)bit4) ^ (int)bit3) : (int)bit4;
-    const bool bsw = G == 4 ? (lane >> 2) & 1 : bit3;  // the lane reads the swapped copy
+    const int pk = (2 * (int)bit4) ^ (int)bit3;
+    const bool bsw = (lane >> 2) & 1;  // the lane reads the swapped copy
     const int swz = bsw ? SW : 0;
-    // G = 2: offsets of the pair this lane keeps (k0) and of the pair it sends (k1)
-    const int k0 = (int)bit4 + (bit3 ? SW : 0), k1 = 1 - (int)bit4 + (bit3 ? SW : 0);
     float *fA = reinterpret_cast<float *>(sA);
     float *fB = reinterpret_cast<float *>(sB);
     float *fC = reinterpret_cast<float *>(sC);
@@ -733,7 +731,7 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
                 float2 v[G][NC];
 #pragma unroll
                 for (int h = 0; h < G; ++h) {
-                    const int kh = G == 2 ? k + (h ? k1 : k0) : k + (h ^ pk) + swz;
+                    const int kh = k + (h ^ pk) + swz;
                     const float4 a = sA[kh], cc = sC[kh], d = sD[kh];
                     const float4 e = TORQUE ? sE[kh] : make_float4(0.f, 0.f, 0.f, 0.f);
                     const float4 g4 = TORQUE ? sG[kh] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -800,22 +798,13 @@ __global__ void __launch_bounds__(kPairThreads, MINB) pair_f32x2_sym_kernel(cons
                 // with source 2(k + pk) + bit2(L), stored by lanes 0, 4, .., 28
 #pragma unroll
                 for (int q = 0; q < NC; ++q) {
-                    float w;
-                    if (G == 2) {
-                        const float2 w2 = add2(v[0][q], shfl_xor2(v[1 % G][q], 16));
-                        w = w2.x + __shfl_xor_sync(0xffffffffu, w2.y, 8);
-                    } else {
-                        const float2 a0 = add2(v[0][q], shfl_xor2(v[2 % G][q], 16));
-                        const float2 a1 = add2(v[1 % G][q], shfl_xor2(v[3 % G][q], 16));
-                        const float2 x2 = add2(a0, shfl_xor2(a1, 8));
-                        w = x2.x + __shfl_xor_sync(0xffffffffu, x2.y, 4);
-                    }
-                    if (G == 2) w += __shfl_xor_sync(0xffffffffu, w, 4);
+                    const float2 a0 = add2(v[0][q], shfl_xor2(v[2][q], 16));
+                    const float2 a1 = add2(v[1][q], shfl_xor2(v[3][q], 16));
+                    const float2 x2 = add2(a0, shfl_xor2(a1, 8));
+                    float w = x2.x + __shfl_xor_sync(0xffffffffu, x2.y, 4);
                     w += __shfl_xor_sync(0xffffffffu, w, 2);
                     w += __shfl_xor_sync(0xffffffffu, w, 1);
-                    // (the two-pair index is spelled 2k + 2 bit4 + bit3: the equal 2(k + pk) + bit3 cost the
-                    // two-right-hand-side form, at its 128-register cap, 14% in time)
-                    if ((lane & (G == 4 ? 3 : 7)) == 0) sv[warp][q][G == 4 ? 2 * (k + pk) + bsw : 2 * k + 2 * bit4 + bit3] = w;
+                    if ((lane & 3) == 0) sv[warp][q][2 * (k + pk) + bsw] = w;
                 }
             }
         }
