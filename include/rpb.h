@@ -43,8 +43,9 @@ extern "C" {
 #define RPB_ECUDA 3     /* a CUDA runtime call or kernel launch failed (message has the CUDA error) */
 #define RPB_ENOCONV 4   /* Lanczos reached max_iter with eps > tol: results are still written */
 #define RPB_ETIMEOUT 5  /* a bounded device-side wait expired.  Reserved: no kernel of this library waits
-                           on another (the Lanczos stop and the step loop are graph conditions, the
-                           stages plain stream order), so no call returns it */
+                           for a flag or a word that another writes (the Lanczos stop and the step loop are
+                           graph conditions, the stages stream order or programmatic dependencies, which
+                           end with the kernel before them), so no call returns it */
 
 #define RPB_FP64 0      /* pair arithmetic in float64 */
 #define RPB_FP32 1      /* pair arithmetic in float32 (hi/lo split positions, compensated tile sums,

@@ -113,11 +113,15 @@ int check_step_args(rpb_ctx *ctx, int64_t N, const double *pos, const double *U_
 // Largest suspensions whose drift runs beside the Lanczos iterations: those whose products leave most of the
 // GPU idle (up to a wave of CTAs), so that the drift's two products, their packing and their noise cost
 // little: 20 steps of 256 spheres 7.03 -> 6.21 ms in float64 and 17.5 -> 14.4 ms pseudo-periodic in float32, a
-// float32 step of 4096 spheres 807 -> 765 us.  Beyond, both are bound by the arithmetic (a float64 step of
-// 4096: 15.46 and 15.41 ms).
+// float32 step of 4096 spheres 807 -> 765 us.  Host-driven steps now, after each other / beside, float32: 300 spheres
+// 432 / 417 us, 1000 453 / 445, 3000 581 / 571, 4096 729 / 731; float64: 300 380 / 376, 600 512 / 500, 1000 788 / 780.
+// Float32 steps beyond would still gain, with the scratch that is there (4500 spheres 967 / 933 us, 8192 1616 / 1591,
+// 32768 15613 / 15500); float64 ones would (1500 1329 / 1292, 4096 6880 / 6812) for scratch that grows as N^2.
 constexpr int64_t kBesideMaxF32 = 4096, kBesideMaxF64 = 1024;
 // The side scratch reaches further for float32: a drift's two products beside each other (rfd_impl) fill the last
-// waves of each other's CTAs.
+// waves of each other's CTAs.  A drift on one stream / two: 4097 spheres 124 / 102 us, 6000 178 / 148, 10007 348 /
+// 319, 16384 778 / 747, 20000 1113 / 1080, 28000 2073 / 2036, 32768 2813 / 2760; the scratch, which grows as N^2, is
+// 92 MB there, and beyond the gain is below 2%.
 constexpr int64_t kSideMaxF32 = 32768;
 static int64_t side_max(const rpb_params &p, int64_t max_N)
 {

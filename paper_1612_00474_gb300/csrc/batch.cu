@@ -9,8 +9,9 @@
 //
 //   pair products : one 128-target block of one instance per CTA, all of that instance's sources
 //                   in 128-source tiles; the float64 self term and s_i/(8 pi eta) in the epilogue.
-//   Lanczos       : per-instance dot products / Gram-Schmidt and tridiagonal step (one CTA per
-//                   instance), instances drop out as they converge.
+//   Lanczos       : dot products and Gram-Schmidt over chunks of 256 spheres (one CTA each), the
+//                   tridiagonal step by one CTA per instance, instances drop out as they converge.
+//   forces        : the cell lists of cells.cuh over the whole batch.
 //   noise         : Philox keyed by each instance's seed, counter (k/2, step_b, stream, 0) -- the
 //                   same numbers the single-suspension path draws for that seed and step.
 #include <algorithm>
@@ -261,13 +262,6 @@ __global__ void __launch_bounds__(kPairThreads) batch_pair_f64_kernel(
         U[2 * total + i] = k * uz;
     }
 }
-
-// Forces of Sec. III within each instance: the cell lists of cells.cuh over the whole batch.
-// Pairs farther apart than 2a + kFarB b, whose repulsion is below e^-kFarB U0/b (~2e-9 U0/b), take it
-// in float32 (IEEE square root and division, expf: a relative error of a few 1e-6 on a term that small
-// is below 1e-14 U0/b) and are summed in float32 before their total joins the float64 sum; nearer
-// pairs are evaluated in float64.
-constexpr double kFarB = 20.0;
 
 // ------------------------------------------------------------------ noise and elementwise steps
 __device__ __forceinline__ uint4 philox4x32_10_b(uint4 c, uint32_t k0, uint32_t k1)

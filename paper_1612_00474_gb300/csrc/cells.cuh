@@ -139,7 +139,10 @@ __global__ void __launch_bounds__(256) cell_order_kernel(const double *__restric
 // for 76% of its time): a thread per sphere paid for the longest list of 32 and left four warps on some schedulers
 // and three on others.  65536 spheres: this kernel 111 -> 86 us, the forces 182 -> 119 (8 threads a sphere 121,
 // 2 128, 1 173); 8193: 78 -> 49.
-// In a batch, pairs beyond near2 take the float32 form (see kFarB) from the list's other end.
+// In a batch, pairs farther apart than 2a + kFarB b (near2), whose repulsion is below e^-kFarB U0/b (~2e-9 U0/b),
+// take it in float32 from the list's other end (IEEE square root and division, expf: a relative error of a few 1e-6 on
+// a term that small is below 1e-14 U0/b) and are summed in float32 before their total joins the float64 sum.
+constexpr double kFarB = 20.0;
 constexpr int kCellLanes = 4, kCellList = 64;
 
 template <class Inst>

@@ -17,8 +17,8 @@
 // writes it into the packed sources of the next product (whose positions stay packed), and its first
 // block does the tridiagonal step.  Separate kernels for the two projections, their dot products, the
 // scaling, the packing and the tridiagonal step were seven launches, about 25 us of an iteration at 256
-// spheres; 20 steps of 256 spheres in float64 went from 13.7 to 8.8 ms, a step of 4096 in float32 from 960 to
-// 849 us.  Larger suspensions spread the same steps over the GPU (gs.cuh).
+// spheres; 20 steps of 256 spheres in float64 went from 13.7 to 8.4 ms, a step of 4096 in float32 from 960 to
+// 845 us.  Larger suspensions spread the same steps over the GPU (gs.cuh).
 // Reductions are summed in a fixed order: results do not depend on scheduling.  The stopping decision
 // is written to pinned host memory, or, inside a graph-replayed run, taken on the device: the
 // iterations after the first are the body of a loop node that each iteration keeps running or ends.
@@ -469,7 +469,10 @@ int lanczos_setup(rpb_ctx *ctx)
 
 // Blocks of the cluster for N spheres, 0 for the kernels over the whole GPU.  Up to kGsChunk spheres a
 // block; 64 and fewer for a small suspension, whose time is the latency of the steps and not their
-// arithmetic.
+// arithmetic.  Solves in us by 1 / 4 / 8 blocks, float64: 64 spheres 270 / 264 / 263, 200 292 / 264 / 270, 300 314 /
+// 320 / 311, 512 349 / 355 / 345; float32, 256: 394 / 365 / 360.  By 4 / 8 / 16, 800 spheres 459 / 453 / 451, 1024
+// 539 / 527 / 523, without the wall in float32 700 / 664 / 645.  Up to 32 spheres (two warps of rows) one block and
+// eight do not differ.
 static int gs_cluster_blocks(const rpb_ctx *ctx, int64_t N)
 {
     if (N <= 32) return 1;

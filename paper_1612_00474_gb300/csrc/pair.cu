@@ -1536,8 +1536,8 @@ __global__ void wrap_kernel(const double *__restrict__ pos, int N, double Lx, do
 }
 
 // Appendix B: periodic in x and y; each source is taken at its minimum image and at the eight shifts of
-// it by one period (the unit cell and its eight neighbour cells).  One-way kernels (the symmetric
-// pass is not used in this mode).  The pack kernel has wrapped every position into the unit cell, so
+// it by one period (the unit cell and its eight neighbour cells).  One-way kernels, for float64, products
+// without forces or without the wall, and fewer than 256 spheres in float32.  The pack kernel has wrapped every position into the unit cell, so
 // in-plane offsets lie in (-L, L) and the minimum-image correction is 0 or +-L.  The sphere's own
 // unshifted image is the self term (added by the reduce kernel); its eight shifted images are pairs.
 template <bool TORQUE, bool WALL>
@@ -2159,8 +2159,8 @@ __global__ void __launch_bounds__(128) forces_kernel(const double *__restrict__ 
 // the cells (62 us a call from 64 to 4096 spheres; the pseudo-periodic all-pairs kernel 52 us at 256).  Twenty
 // steps of 256 spheres: 7.75 -> 7.03 ms in float64, 23.1 -> 22.0 ms pseudo-periodic.
 constexpr int kGroupTargets = 16, kGroupThreads = 8, kGroupChunk = 1024;
-// Up to here; beyond, screening all pairs costs more than the cell lists (40 us a call at 4096, 100 at 8192, where
-// the cell lists take 46 from 4097 spheres on and 49 at 8192).  Pseudo-periodic cells have no cell lists, and up to
+// Up to here; beyond, screening all pairs costs more than the cell lists (this kernel 41 us at 4096, 43 at 4300, 46
+// at 4600, 56 at 5000, 67 at 6000, 100 at 8192; the cell lists 46 from 4097 to 5000, 49 at 8192).  Pseudo-periodic cells have no cell lists, and up to
 // 40000 spheres the kernel of a thread per sphere is slower: 8193 434 us against 131, 16384 801 against 406, 32768
 // 1704 against 1333, 40000 2104 against 1924, 65536 3587 against 4573 (with many near pairs a sphere far slower).
 constexpr int64_t kGroupMaxN = 4096, kGroupMaxNPer = 40000;

@@ -254,9 +254,13 @@ struct SideSpace {
 // reads or writes any global memory.  What the one before writes is no `const __restrict__` parameter of such a
 // kernel: that would promise that nothing changes it while the kernel runs, and allow its loads ahead of the wait.
 // Every kernel launched this way waits, so completion is transitive along the chain; started otherwise,
-// wait_for_before() returns at once.  Products of a solve after the first, of at most kAfterMaxN spheres: there a kernel's launch is a good
-// part of its time, and waiting CTAs take no room that running ones need.  A float32 step of 4096 spheres 747 -> 698 us, a
-// float64 one of 256 358 -> 316, twenty replayed ones 5.18 -> 4.85 ms, a solve of 3001 spheres 436 -> 403 us.
+// wait_for_before() returns at once.  Products of a solve after the first, of at most kAfterMaxN spheres, the range of
+// the cluster kernel: there a kernel's launch is a good part of its time, and waiting CTAs take no room that running ones
+// need.  A float32 step of 4096 spheres 747 -> 698 us, a float64 one of 256 358 -> 316, twenty replayed ones 5.18 ->
+// 4.85 ms, a solve of 3001 spheres 436 -> 403 us.  Host-driven solves without / with, float64: 300 spheres 330 / 311 us,
+// 800 472 / 450, 2000 1175 / 1153, 4096 3554 / 3535; float32: 300 390 / 368, 4096 606 / 589.  The line is no crossing:
+// with the reduce kernels of larger solves launched early too, float32 solves of 4500 and 8192 spheres take 778 and
+// 1251 us instead of 800 and 1270, float64 ones of 4500 4331 instead of 4354.
 constexpr int64_t kAfterMaxN = 4096;
 #ifdef __CUDACC__
 __device__ __forceinline__ void after_may_start()
