@@ -187,6 +187,7 @@ static int step_body(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint3
     if (ctx->p.kT > 0.0) {
         if ((rc = philox_impl(ctx, N, seed, step, 0u, 0u, W, d_step))) return rc;
         if (!beside && (rc = philox_impl(ctx, N, seed, step, 1u, 0u, Wt, d_step))) return rc;
+        if (max_iter > 1 && !gr) blocks64_prepare(ctx, N);  // while the GPU works on the forces
         if (mobility_apply2_ok(ctx, N)) {
             // the deterministic velocity and the first Lanczos product M v_0 share one pair pass
             if ((rc = lanczos_precond_prepare(ctx, N, pos)) || (rc = lanczos_init(ctx, N, W, false, gr)) ||
@@ -237,7 +238,6 @@ int step_impl(rpb_ctx *ctx, int64_t N, double *pos, double *U_prev, uint32_t ste
 {
     const bool beside = ctx->p.kT > 0.0 && !ctx->hook &&
                         N <= (ctx->p.precision == RPB_FP64 ? kBesideMaxF64 : kBesideMaxF32);
-    if (ctx->p.kT > 0.0 && max_iter > 1 && !gr) blocks64_prepare(ctx, N);
     const int rc = step_body(ctx, N, pos, U_prev, step, seed, dt, delta, tol, max_iter, fp, scheme, rfd, stats, gr, beside);
     // a step that failed half way: the stream is still ordered after the drift's reads of pos
     if (rc && rc != RPB_ENOCONV && beside && !gr && ctx->side_join)

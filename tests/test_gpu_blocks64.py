@@ -1,5 +1,7 @@
 """Device memory of float64 contexts: the pairs' blocks are taken by the first Lanczos solve that reads them, for its own
 size, and a solve gives the same bits in every context that holds them."""
+import gc
+
 import pytest
 
 from paper_1612_00474_gb300 import inputs
@@ -16,6 +18,7 @@ def _dev(x):
 
 
 def _used():
+    gc.collect()  # contexts that earlier tests left behind
     torch.cuda.synchronize()
     free, total = torch.cuda.mem_get_info()
     return total - free
